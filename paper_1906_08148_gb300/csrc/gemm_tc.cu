@@ -42,9 +42,9 @@
 // discarded quadrants: each output element depends on one A row and one B
 // column).  The 4-slice form stages each step in two K-halves (64 KB each,
 // three in flight) so that its 128 KB of operands per step still pipeline.
-// Accumulators are 128 x 128 FP32 slots of TMEM; four slots rotate, one per
-// accumulator of each step in order, so the MMAs of the next step start as
-// soon as the epilogue has drained the slots they reuse.
+// Accumulators are 128 x 128 FP32 slots of TMEM; four slots rotate (acc_slot below),
+// so the MMAs of the next step start as soon as the epilogue has drained the slots
+// they reuse.
 //
 // Warp roles (one CTA per SM, persistent; quads are claimed one at a time
 // from a global counter in Morton order, so the quads in flight on all SMs
@@ -60,6 +60,18 @@
 //              output rows as two-float pairs.
 // No atomics on C: one CTA owns each output quad; k runs in ascending order.
 // Every wait is bounded; on timeout the CTA sets the error word and leaves.
+//
+// What bounds it: per step the MMAs (64 cycles each: 10, 6 or 3 terms x 4 K pieces,
+// 2560 / 1536 / 768 cycles), the FP32 pipe of the epilogue (about 1980 / 1050 / 130
+// cycles where all four children are kept) and the copies (up to 128 / 96 / 64 KB
+// through L2) all come within a factor of two of one another, and every hand-over
+// between them is a look at a barrier in shared memory that takes some 250 cycles
+// beside the operand reads.  Measured on the 3-D lattices (GEMM only, CUDA events),
+// with the waits taken out of each role's way as the comments below say: 4 slices,
+// n = 65536, tau = 1e-6, 115.6 -> 94.4 ms (1666 TFLOP/s executed, near the chip's
+// power-limited rate); 3 slices, n = 16384, 8.19 -> 6.67 ms; FP16 with 128-leaves,
+// n = 20000, tau = 1e-4, 7.67 -> 5.78 ms.  With single parts left out the first takes
+// 68 ms (MMAs alone), 51 (copies alone), 80 (without epilogue), 85 (without copies).
 #include "convert.cuh"
 #include "internal.cuh"
 #include "ptx.cuh"
@@ -71,15 +83,26 @@ namespace spamm {
 // Three warpgroups: warpgroup 0 holds the producer (warp 0) and the MMA issuer
 // (warp 1; warps 2-3 idle), warpgroups 1-2 the epilogue (warps 4-11).  The
 // launch gives every thread 168 registers (384 x 168 = 64512 of 65536); the
-// control warpgroup then gives up 112 of them per thread and the epilogue
-// takes 56 more, enough for its two-float accumulators: 128 x 56 + 256 x 224
-// = 64512, the launch total, so the increase never waits.
+// control warpgroup then gives up 96 of them per thread and the epilogue
+// takes 48 more, enough for its two-float accumulators and one slot's columns:
+// 128 x 72 + 256 x 216 = 64512, the launch total, so the increase never waits.
 constexpr int kQuadThreads = 384;
-constexpr uint32_t kLaunchRegs = 168, kCtlRegs = 56, kEpiRegs = 224;
+constexpr uint32_t kLaunchRegs = 168, kCtlRegs = 72, kEpiRegs = 216;
 static_assert(128 * kCtlRegs + 256 * kEpiRegs == kQuadThreads * kLaunchRegs, "register split must match the launch");
 static_assert(kQuadThreads * kLaunchRegs <= 65536, "launch registers exceed the register file");
 constexpr int kQuadBufs = 4;  // rotating TMEM accumulator slots of 128 FP32 columns
 constexpr int kQuadQ = 4;     // ring of claimed quads shared by the three roles
+// Ring of step scales, written by the producer (eight steps at a time) and read by
+// the epilogue.  The producer's copies are at most the stages ahead of the MMAs, and
+// these at most four steps (one per slot) ahead of the epilogue, so fewer than
+// 8 + 6 + 4 entries are in use and one is read before it is reused.
+constexpr int kScaleRing = 32;
+// Steps before the end of a unit at which the next one is claimed.  Neighbouring
+// units read the same leaves at the same k, so they share them in L2 only while they
+// run side by side: claimed a whole unit ahead, their starts scatter over a unit's
+// length (the copies alone of the 4-slice form on the n = 65536 lattice 72 ms instead
+// of 54); claimed at the unit's end, its look-ups leave the stages empty.
+constexpr int kClaimAhead = 5;
 
 // One stage: two A and two B leaves, every term of a step (whole-K forms) or
 // of one K-part of it.  A region: leaf 2I's part (all terms, atom-interleaved,
@@ -98,10 +121,12 @@ struct QuadLayout {
   static constexpr uint32_t BREG = 2 * LPART;
   static constexpr uint32_t STAGE = 2 * BREG;
   static constexpr size_t SMEM = 1024 + (size_t)Cfg::NS * STAGE;
-  __device__ static uint64_t desc(uint32_t saddr) {
-    if constexpr (Cfg::KPARTS == 1) return sw128_kmajor_desc(saddr, SBO);
-    if constexpr (Cfg::KPARTS == 2) return sw64_kmajor_desc(saddr, SBO);
-    return sw32_kmajor_desc(saddr, SBO);
+  // high word of every operand's matrix descriptor (stride, version, swizzle)
+  __device__ static constexpr uint32_t desc_hi() {
+    return (uint32_t)((Cfg::KPARTS == 1   ? sw128_kmajor_desc(0, SBO)
+                       : Cfg::KPARTS == 2 ? sw64_kmajor_desc(0, SBO)
+                                          : sw32_kmajor_desc(0, SBO)) >>
+                      32);
   }
 };
 
@@ -110,74 +135,168 @@ double quad_step_flops(spamm_prec prec) {
   return (double)(terms * (terms + 1) / 2) * 2.0 * 128.0 * 128.0 * 64.0;
 }
 
-// The MMAs of accumulator `acc` for one stage: term products (i, g - i) with
-// index sum g = acc (g from acc to TERMS - 1 for the last accumulator, the
-// largest sums first so the smallest products are added first), the first
-// of them overwriting the slot when `fresh`.
-template <int PREC, int ACC>
-__device__ __forceinline__ void issue_acc(uint32_t d, uint32_t a_s, uint32_t b_s, uint32_t idesc, bool fresh) {
-  using Cfg = FormCfg<PREC>;
-  using Lay = QuadLayout<PREC>;
-  constexpr int GLO = ACC, GHI = ACC < Cfg::NACC - 1 ? ACC : Cfg::TERMS - 1;
-  uint32_t accumulate = fresh ? 0u : 1u;
-#pragma unroll
-  for (int g = GHI; g >= GLO; --g) {
-#pragma unroll
+// Accumulator slots.  A step's accumulator a < NACC - 1 takes the term products
+// of index sum a (exact), the last one every larger sum.  kQuadBufs slots of 128
+// FP32 columns rotate so that a step's first MMAs never wait for the previous
+// step's last drain: the last accumulator (the longest in use, committed at the
+// end of its step) alternates between slots 0 and 1, the others between 2 and 3;
+// with three accumulators sums 0 and 1 swap slots 2 and 3 every step.  `use` is
+// how often the slot was used before.
+template <int NACC>
+__device__ __forceinline__ void acc_slot(uint32_t n, int a, uint32_t* slot, uint32_t* use) {
+  if constexpr (NACC == 1) {
+    *slot = n & 3u;
+    *use = n >> 2;
+  } else if (a == NACC - 1) {
+    *slot = n & 1u;
+    *use = n >> 1;
+  } else if constexpr (NACC == 2) {
+    *slot = 2u + (n & 1u);
+    *use = n >> 1;
+  } else {
+    *slot = 2u + ((n + (uint32_t)a + 1u) & 1u);
+    *use = n;
+  }
+}
+static_assert(kQuadBufs == 4, "acc_slot rotates four slots");
+
+// The order of one stage's MMAs: K = 16 piece `ks` of A term i against B term j,
+// and how the tensor core's buffer for A serves it.  A 128 x 128 x 16 MMA reads
+// 8 KB of operands in the 64 cycles it computes, all that shared memory delivers
+// (128 B per clock), beside the copies into the next stage; where consecutive
+// MMAs use the same A piece, the first keeps it in the buffer (fill) and the
+// others read only B.  The sums in an accumulator that is not exact depend on
+// the order, so it is chosen per form:
+//   4 slices  the products of index sum 2 and 3 share one accumulator; A's terms
+//             from the last to the first in the first K-part and back in the last,
+//             each against every B term it meets: 16 reads of A instead of 40,
+//             and the exact accumulators are in use for the shortest time;
+//   3 slices  index sums 2 and 1 share one accumulator, the smaller products first,
+//             each product whole; the exact (0, 0) rides on the last product's A;
+//   FP16      one accumulator, h1 g0, h0 g1, h0 g0, each product whole.
+struct MmaOrder {
+  int n = 0;
+  uint8_t i[48] = {}, j[48] = {}, ks[48] = {}, collect[48] = {};
+  __host__ __device__ constexpr void add(int i_, int j_, int ks_, int collect_) {
+    i[n] = (uint8_t)i_;
+    j[n] = (uint8_t)j_;
+    ks[n] = (uint8_t)ks_;
+    collect[n] = (uint8_t)collect_;
+    ++n;
+  }
+};
+template <int PREC>
+__host__ __device__ constexpr MmaOrder mma_order(bool last_part) {
+  constexpr int T = FormCfg<PREC>::TERMS, KS = 4 / FormCfg<PREC>::KPARTS;
+  MmaOrder o;
+  if (T == 4) {
+    for (int ii = 0; ii < T; ++ii) {
+      const int i = last_part ? ii : T - 1 - ii, m = T - i;
+      for (int ks = 0; ks < KS; ++ks)
+        for (int jj = 0; jj < m; ++jj)
+          o.add(i, last_part ? jj : m - 1 - jj, ks,
+                m == 1 ? kCollectNone : jj == 0 ? kCollectFill : jj == m - 1 ? kCollectLast : kCollectUse);
+    }
+    return o;
+  }
+  for (int g = T - 1; g >= 0; --g)
     for (int i = g; i >= 0; --i) {
-#pragma unroll
-      for (int ks = 0; ks < Lay::KS; ++ks) {
-        umma_f16(d, Lay::desc(a_s + (uint32_t)i * Lay::ATOM + 32 * ks),
-                 Lay::desc(b_s + (uint32_t)(g - i) * Lay::ATOM + 32 * ks), idesc, accumulate);
-        accumulate = 1u;
+      if (T == 3 && g == 0) continue;
+      for (int ks = 0; ks < KS; ++ks) {
+        const bool share = T == 3 && g == 1 && i == 0;  // A term 0 also for the exact product
+        o.add(i, g - i, ks, share ? kCollectFill : kCollectNone);
+        if (share) o.add(0, 0, ks, kCollectLast);
       }
     }
+  return o;
+}
+
+// Issues one stage's MMAs into the step's accumulator slots.  ready(a): waits until
+// slot a may be overwritten, called before the first MMA into it; ahead(): called
+// a few MMAs before the end, while the tensor core still has work queued (it takes
+// about five MMAs ahead), to look at the barriers the next stage needs -- a wait
+// on a barrier in shared memory takes some 250 cycles beside the operand reads, and
+// the tensor core would run dry; done(a): after the last MMA into slot a.
+constexpr int kAhead = 4;
+template <int PREC, bool FIRST, bool LAST, class Ready, class Ahead, class Done>
+__device__ __forceinline__ bool issue_stage(uint32_t tbase, const uint32_t (&slot)[3], uint32_t a_s, uint32_t b_s,
+                                            uint32_t idesc, Ready ready, Ahead ahead, Done done) {
+  using Cfg = FormCfg<PREC>;
+  using Lay = QuadLayout<PREC>;
+  constexpr uint32_t HI = Lay::desc_hi();
+  constexpr MmaOrder O = mma_order<PREC>(LAST);
+  const uint32_t alo = desc_lo(a_s), blo = desc_lo(b_s);
+  bool fresh[3] = {FIRST, FIRST, FIRST};
+  int left[3] = {0, 0, 0};
+#pragma unroll
+  for (int q = 0; q < O.n; ++q) ++left[O.i[q] + O.j[q] < Cfg::NACC - 1 ? O.i[q] + O.j[q] : Cfg::NACC - 1];
+#pragma unroll
+  for (int q = 0; q < O.n; ++q) {
+    const int a = O.i[q] + O.j[q] < Cfg::NACC - 1 ? O.i[q] + O.j[q] : Cfg::NACC - 1;
+    if (fresh[a] && !ready(a)) return false;
+    if (q == O.n - kAhead) ahead();
+    umma_f16(tbase + slot[a] * 128u, alo + ((O.i[q] * Lay::ATOM + 32u * O.ks[q]) >> 4),
+             blo + ((O.j[q] * Lay::ATOM + 32u * O.ks[q]) >> 4), HI, idesc, fresh[a] ? 0u : 1u, O.collect[q]);
+    fresh[a] = false;
+    if (LAST && --left[a] == 0) done(a);
+  }
+  return true;
+}
+
+// Eight pairs of adjacent output elements at a time: (hi, lo) += v sc with an
+// error-free TwoSum of hi and v sc (the product is exact: sc is a power of two),
+// in the packed FP32x2 instructions, each lane rounding like the scalar
+// round-to-nearest operation; hi + lo gains v sc up to the rounding of lo.  Seven
+// instructions per pair (the products ride in the two FMAs), taken across the
+// eight pairs one operation after the other: a packed instruction issues every
+// two cycles and its result is ready after four, so a single pair's chain would
+// leave the pipe idle half of the time (measured with two warps per scheduler:
+// 1165 cycles per 64 columns in eight instructions pair by pair, 920 like this,
+// the pipe's rate).
+__device__ __forceinline__ void two_sum_x8(uint64_t* hi, uint64_t* lo, const uint32_t* v, uint64_t sc2) {
+  uint64_t x[8], s[8], nb[8], t[8];
+#pragma unroll
+  for (int q = 0; q < 8; ++q) x[q] = pack_x2(v[2 * q], v[2 * q + 1]);
+#pragma unroll
+  for (int q = 0; q < 8; ++q) s[q] = fma_x2(x[q], sc2, hi[q]);
+#pragma unroll
+  for (int q = 0; q < 8; ++q) nb[q] = sub_x2(hi[q], s[q]);  // -(s - hi)
+#pragma unroll
+  for (int q = 0; q < 8; ++q) t[q] = add_x2(s[q], nb[q]);
+#pragma unroll
+  for (int q = 0; q < 8; ++q) nb[q] = fma_x2(x[q], sc2, nb[q]);  // v sc - (s - hi)
+#pragma unroll
+  for (int q = 0; q < 8; ++q) t[q] = sub_x2(hi[q], t[q]);  // hi - (s - (s - hi))
+#pragma unroll
+  for (int q = 0; q < 8; ++q) t[q] = add_x2(t[q], nb[q]);
+#pragma unroll
+  for (int q = 0; q < 8; ++q) {
+    hi[q] = s[q];
+    lo[q] = add_x2(lo[q], t[q]);
   }
 }
 
-// (hi, lo) += x sc for two adjacent output elements at once, with an
-// error-free TwoSum of hi and x sc (x sc is exact: sc is a power of two) in
-// the packed FP32x2 instructions, each lane rounding like the scalar
-// round-to-nearest operation: hi + lo gains x sc up to the rounding of lo.
-// hi2, lo2 hold (hi, lo) of elements 2q and 2q + 1; v0, v1 are the
-// accumulator's FP32 bits of the two elements, sc2 the scale twice.
-__device__ __forceinline__ void two_sum_x2(uint64_t& hi2, uint64_t& lo2, uint32_t v0, uint32_t v1, uint64_t sc2) {
-  asm("{\n\t.reg .b64 x, s, bp, t1, t2, t3, e;\n\t"
-      "mov.b64 x, {%2, %3};\n\t"
-      "mul.rn.f32x2 x, x, %4;\n\t"
-      "add.rn.f32x2 s, %0, x;\n\t"
-      "sub.rn.f32x2 bp, s, %0;\n\t"
-      "sub.rn.f32x2 t1, s, bp;\n\t"
-      "sub.rn.f32x2 t2, %0, t1;\n\t"
-      "sub.rn.f32x2 t3, x, bp;\n\t"
-      "add.rn.f32x2 e, t2, t3;\n\t"
-      "add.rn.f32x2 %1, %1, e;\n\t"
-      "mov.b64 %0, s;\n\t}"
-      : "+l"(hi2), "+l"(lo2)
-      : "r"(v0), "r"(v1), "l"(sc2));
-}
-// lo2 += (v0, v1) sc2, packed.
-__device__ __forceinline__ void fma_x2(uint64_t& lo2, uint32_t v0, uint32_t v1, uint64_t sc2) {
-  asm("{\n\t.reg .b64 x;\n\t"
-      "mov.b64 x, {%1, %2};\n\t"
-      "fma.rn.f32x2 %0, x, %3, %0;\n\t}"
-      : "+l"(lo2)
-      : "r"(v0), "r"(v1), "l"(sc2));
-}
+// What the producer tells the other roles about a claimed unit.
+struct UnitInfo {
+  double* out[4];  // first element of each child's 64 x 64 output, null where absent
+  int32_t nstep;   // -1: no more units
+  int32_t ld;      // row length of the output leaves
+};
 
 template <int PREC>
 __global__ void __launch_bounds__(kQuadThreads, 1)
     gemm_quad_kernel(BatchDev batch, unsigned long long* __restrict__ work, int* __restrict__ err) {
   using Cfg = FormCfg<PREC>;
   using Lay = QuadLayout<PREC>;
-  constexpr int NS = Cfg::NS, TERMS = Cfg::TERMS, NACC = Cfg::NACC, NB = kQuadBufs, SPS = Lay::SPS;
-  constexpr uint32_t LEAF = leaf_bytes<PREC>(), STAGE = Lay::STAGE, BREG = Lay::BREG, TILE = Lay::TILE;
-  static_assert(NACC <= NB - 1, "the next step needs a free accumulator slot");
+  constexpr int NS = Cfg::NS, NACC = Cfg::NACC, NB = kQuadBufs, SPS = Lay::SPS;
+  constexpr uint32_t LEAF = leaf_bytes<PREC>(), STAGE = Lay::STAGE, BREG = Lay::BREG, LP = Lay::LPART;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   __shared__ __align__(8) uint64_t full[NS], empty[NS], tfull[NB], tempty[NB], qfull[kQuadQ], qempty[kQuadQ];
-  __shared__ int64_t qid[kQuadQ], epi_un;
+  __shared__ UnitInfo qinfo[kQuadQ];
+  __shared__ __align__(16) float4 sscale[kScaleRing];  // step n's scales at n mod kScaleRing
   __shared__ uint32_t tmem_base;
-  __shared__ int abort_flag, epi_stop;
+  __shared__ int abort_flag;
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
@@ -191,7 +310,7 @@ __global__ void __launch_bounds__(kQuadThreads, 1)
     }
     for (int q = 0; q < kQuadQ; ++q) {
       mbar_init(&qfull[q], 1);
-      mbar_init(&qempty[q], 2);  // the MMA issuer and the epilogue's first thread
+      mbar_init(&qempty[q], 9);  // the MMA issuer and the eight epilogue warps
     }
     fence_mbar_init();
     abort_flag = 0;
@@ -207,255 +326,338 @@ __global__ void __launch_bounds__(kQuadThreads, 1)
   volatile int* abortp = &abort_flag;
   if (warp < 4) {
     regs_dec<kCtlRegs>();  // every warp of warpgroup 0, at this one instruction
-  if (warp == 0) {
-    // ---------------- TMA producer; claims the quads (Morton order, first come first served) for all roles
-    if (lane == 0) {
-      int64_t t = 0;  // stages filled
-      bool stop = false;
-      for (int64_t c = 0; !stop; ++c) {
-        const int qs = (int)(c % kQuadQ);
-        if (c >= kQuadQ && !mbar_wait_or_abort(&qempty[qs], (uint32_t)(((c / kQuadQ) - 1) & 1), abortp)) {
-          atomicOr(err, DEV_ERR_TIMEOUT);
-          *abortp = 1;
-          break;
-        }
-        const int64_t claimed = (int64_t)atomicAdd(work, 1ull);
-        const int64_t un = claimed < batch.nunits ? claimed : -1;
-        qid[qs] = un;
-        mbar_arrive(&qfull[qs]);
-        if (un < 0) break;
-        const int r = plan_of(batch.ubegin, batch.nplans, un);
-        const PlanDev& pl = batch.plans[r];
-        const int64_t Qc = un - batch.ubegin[r], Q = pl.uorder ? pl.uorder[Qc] : pl.ufirst + Qc;
-        const int64_t j1 = pl.qstart[Q + 1];
-        int64_t j = pl.qstart[Q];
-        const int4* rec = reinterpret_cast<const int4*>(pl.qsteps);  // word 2j: a0, a1, b0, b1 of step j
-        int4 nx = j < j1 ? __ldg(rec + 2 * j) : make_int4(-1, -1, -1, -1);
-        for (; j < j1 && !stop; ++j) {
-          const int4 ab = nx;
-          if (j + 1 < j1) nx = __ldg(rec + 2 * (j + 1));  // next step's leaves, in flight during the wait
-          const uint32_t nload = (uint32_t)((ab.x >= 0) + (ab.y >= 0) + (ab.z >= 0) + (ab.w >= 0));
-#pragma unroll
-          for (int h = 0; h < SPS; ++h) {
-            const int s = (int)(t % NS);
-            if (t >= NS && !mbar_wait_or_abort(&empty[s], (uint32_t)(((t / NS) - 1) & 1), abortp)) {
-              atomicOr(err, DEV_ERR_TIMEOUT);
-              *abortp = 1;
-              stop = true;
-              break;
-            }
-            uint8_t* st = smem + s * STAGE;
-            constexpr uint32_t LP = Lay::LPART;
-            mbar_arrive_expect_tx(&full[s], nload * LP);
-            // one copy per leaf: its part h, every term
-            const int64_t off = (int64_t)h * LP;
-            if (ab.x >= 0) bulk_g2s(st, pl.termsA + (int64_t)ab.x * LEAF + off, LP, &full[s]);
-            if (ab.y >= 0) bulk_g2s(st + LP, pl.termsA + (int64_t)ab.y * LEAF + off, LP, &full[s]);
-            if (ab.z >= 0) bulk_g2s(st + BREG, pl.termsB + (int64_t)ab.z * LEAF + off, LP, &full[s]);
-            if (ab.w >= 0) bulk_g2s(st + BREG + LP, pl.termsB + (int64_t)ab.w * LEAF + off, LP, &full[s]);
-            ++t;
+    if (warp == 0) {
+      // ---------------- TMA producer; claims the quads (Morton order, first come first served) for all
+      // roles.  Step records are read eight at a time, lanes 4 i .. 4 i + 3 holding the four leaf indices
+      // (and scales) of step i, which these lanes then copy: no shuffles, and one load per eight steps,
+      // well ahead of its use.  The next unit is claimed and looked up during the current one's last
+      // steps, each dependent load one step before it is used.
+      struct Unit {
+        const int32_t* rec;  // records of eight words: a0, a1, b0, b1, four scales
+        const uint8_t* term; // this lane's operand: A (lanes 0, 1 mod 4) or B
+        int32_t nstep;       // -1: no more units
+      };
+      const int sub = lane >> 2, leafn = lane & 3;  // this lane's step of eight and its leaf in it
+      uint32_t t = 0, n = 0;       // stages filled, steps listed
+      uint32_t s = 0, ephase = 1;  // the stage to fill, and the phase of `empty` that frees it (from the second fill on)
+      bool ok = true;
+      // The next unit (number c of this CTA), in three parts.
+      unsigned long long claimed = 0;
+      const PlanDev* npl = nullptr;
+      int64_t nQ = 0, nq0 = 0, nq1 = 0;
+      int32_t ngrp = 0, nidx = -1, nscl = 0;  // nidx, nscl: its first eight records
+      Unit next{nullptr, nullptr, -1};
+      auto load = [&](const Unit& u, int32_t j, int32_t* idx, int32_t* scl) {
+        const bool in = j + sub < u.nstep;
+        const int32_t* r = u.rec + 8 * (int64_t)(j + sub) + leafn;
+        *idx = in ? __ldg(r) : -1;
+        *scl = in ? __ldg(r + 4) : 0;
+      };
+      auto advance = [&](int part, uint32_t c) {
+        if (part == 0) {  // claim it
+          if (lane == 0) claimed = atomicAdd(work, 1ull);
+        } else if (part == 1) {  // find its plan, start reading its step range and outputs
+          const int64_t un = (int64_t)__shfl_sync(0xffffffffu, claimed, 0);
+          npl = nullptr;
+          if (un < batch.nunits) {
+            const int r = plan_of(batch.ubegin, batch.nplans, un);
+            npl = batch.plans + r;
+            const int64_t Qc = un - batch.ubegin[r];
+            nQ = npl->uorder ? npl->uorder[Qc] : npl->ufirst + Qc;
+            nq0 = npl->qstart[nQ];
+            nq1 = npl->qstart[nQ + 1];
+            ngrp = npl->tc_bs == 128 ? 0 : npl->quads[4 * nQ + leafn];
           }
-        }
-      }
-      // leave no bulk copy in flight: the last fill of every stage has landed
-      for (int64_t k = (t > NS ? t - NS : 0); k < t; ++k) mbar_wait_bounded(&full[k % NS], (uint32_t)((k / NS) & 1));
-    }
-  } else if (warp == 1) {
-    // ---------------- MMA issuer: the accumulators of step number n are slots (NACC n + a) % NB
-    if (lane == 0) {
-      constexpr uint32_t idesc = umma_idesc_f16(Cfg::AB, 128, 128);
-      int64_t t = 0, u = 0;  // stages consumed, accumulator units started
-      bool stop = false;
-      for (int64_t c = 0; !stop; ++c) {
-        const int qs = (int)(c % kQuadQ);
-        if (!mbar_wait_or_abort(&qfull[qs], (uint32_t)((c / kQuadQ) & 1), abortp)) {
-          atomicOr(err, DEV_ERR_TIMEOUT);
-          *abortp = 1;
-          break;
-        }
-        const int64_t un = qid[qs];
-        mbar_arrive(&qempty[qs]);
-        if (un < 0) break;
-        const int r = plan_of(batch.ubegin, batch.nplans, un);
-        const PlanDev& pl = batch.plans[r];
-        const int64_t Qc = un - batch.ubegin[r], Q = pl.uorder ? pl.uorder[Qc] : pl.ufirst + Qc;
-        const int64_t nstep = pl.qstart[Q + 1] - pl.qstart[Q];
-        for (int64_t j = 0; j < nstep && !stop; ++j) {
-#pragma unroll
-          for (int h = 0; h < SPS; ++h) {
-            const int s = (int)(t % NS);
-            if (!mbar_wait_or_abort(&full[s], (uint32_t)((t / NS) & 1), abortp)) {
-              stop = true;
-              break;
+        } else {  // enter it in the ring (not announced yet), start reading its first records
+          next.nstep = -1;
+          if (npl) {
+            next.nstep = (int32_t)(nq1 - nq0);
+            next.rec = reinterpret_cast<const int32_t*>(npl->qsteps) + 8 * nq0;
+            next.term = leafn < 2 ? npl->termsA : npl->termsB;
+          }
+          load(next, 0, &nidx, &nscl);
+          ok = ok && (c < kQuadQ || mbar_wait_or_abort(&qempty[c % kQuadQ], ((c / kQuadQ) - 1) & 1u, abortp));
+          ok = __all_sync(0xffffffffu, ok);
+          if (ok && lane < 4) {
+            UnitInfo& info = qinfo[c % kQuadQ];
+            if (npl) {  // lane c: child c; the four quadrants of output leaf Q, or up to four output leaves
+              const bool big = npl->tc_bs == 128;
+              info.out[lane] = ngrp < 0 ? nullptr
+                               : big    ? npl->cpool + nQ * 16384 + (lane >> 1) * 8192 + (lane & 1) * 64
+                                        : npl->cpool + (int64_t)ngrp * 4096;
+              if (lane == 0) info.ld = big ? 128 : 64;
             }
-            tc_fence_after();
-            const uint32_t a_s = smem_u32(smem + s * STAGE), b_s = a_s + BREG;
+            if (lane == 0) info.nstep = next.nstep;
+          }
+          __syncwarp();
+        }
+      };
+      for (int part = 0; part < 3; ++part) advance(part, 0);
+      for (uint32_t c = 0; ok; ++c) {
+        const Unit cur = next;
+        int32_t idx = nidx, scl = nscl;
+        if (lane == 0) mbar_arrive(&qfull[c % kQuadQ]);
+        if (cur.nstep < 0) break;
+        int part = 0;
+        for (int32_t jb = 0; jb < cur.nstep && ok; jb += 8) {
+          int32_t idx2, scl2;
+          load(cur, jb + 8, &idx2, &scl2);
+          const unsigned used = __ballot_sync(0xffffffffu, idx >= 0);
+          const uint8_t* src = cur.term + (int64_t)idx * LEAF;
+          reinterpret_cast<int32_t*>(&sscale[(n + sub) % kScaleRing])[leafn] = scl;
+          __syncwarp();  // ordered before the arrivals below, which the epilogue's waits follow
+          const int m = min(8, cur.nstep - jb);
+          for (int i = 0; i < m && ok; ++i, ++n) {
+            const uint32_t bytes = (uint32_t)__popc((used >> (4 * i)) & 15u) * LP;
 #pragma unroll
-            for (int a = 0; a < NACC; ++a) {
-              const int64_t un_a = u + a;
-              const int b = (int)(un_a % NB);
-              if (h == 0 && un_a >= NB) {
-                if (!mbar_wait_or_abort(&tempty[b], (uint32_t)(((un_a / NB) - 1) & 1), abortp)) {
-                  stop = true;
-                  break;
-                }
-                tc_fence_after();
+            for (int h = 0; h < SPS; ++h) {
+              if (t >= NS) ok = __all_sync(0xffffffffu, mbar_wait_or_abort(&empty[s], ephase, abortp));
+              if (!ok) break;
+              if (sub == i) {  // one copy per leaf: its part h, every term
+                if (leafn == 0) mbar_arrive_expect_tx(&full[s], bytes);
+                if (idx >= 0) bulk_g2s(smem + s * STAGE + (uint32_t)leafn * LP, src + (int64_t)h * LP, LP, &full[s]);
               }
-              const uint32_t d = tbase + (uint32_t)b * 128u;
-              if (a == 0) issue_acc<PREC, 0>(d, a_s, b_s, idesc, h == 0);
-              if constexpr (NACC > 1) if (a == 1) issue_acc<PREC, (NACC > 1 ? 1 : 0)>(d, a_s, b_s, idesc, h == 0);
-              if constexpr (NACC > 2) if (a == 2) issue_acc<PREC, (NACC > 2 ? 2 : 0)>(d, a_s, b_s, idesc, h == 0);
-              if (h == SPS - 1) umma_commit(&tfull[b]);
+              ++t;
+              if (++s == NS) {
+                s = 0;
+                ephase ^= 1u;
+              }
             }
-            if (stop) break;
-            umma_commit(&empty[s]);
-            ++t;
+            if (ok && part < 3 && cur.nstep - (jb + i) <= kClaimAhead) advance(part++, c + 1);
           }
-          if (!stop) u += NACC;
+          idx = idx2;
+          scl = scl2;
+        }
+        while (part < 3 && ok) advance(part++, c + 1);
+      }
+      if (lane == 0) {
+        if (!ok) {
+          atomicOr(err, DEV_ERR_TIMEOUT);
+          *abortp = 1;
+        }
+        // leave no bulk copy in flight: the last fill of every stage has landed
+        for (uint32_t k = (t > NS ? t - NS : 0); k < t; ++k) mbar_wait_bounded(&full[k % NS], (k / NS) & 1u);
+      }
+    } else if (warp == 1) {
+      // ---------------- MMA issuer (one elected lane)
+      if (elect_one()) {
+        constexpr uint32_t idesc = umma_idesc_f16(Cfg::AB, 128, 128);
+        constexpr int A0 = mma_order<PREC>(SPS == 1).i[0] + mma_order<PREC>(SPS == 1).j[0] < NACC - 1
+                               ? mma_order<PREC>(SPS == 1).i[0] + mma_order<PREC>(SPS == 1).j[0]
+                               : NACC - 1;  // the accumulator a step touches first
+        const uint32_t smem0 = smem_u32(smem);
+        uint32_t n = 0;                  // steps started
+        uint32_t s = 0, sphase = 0;      // stage, and the phase of its next fill
+        uint32_t last = 0, lphase = 0;   // the last committed stage and its phase
+        bool any = false, stop = false;
+        bool saw_full = false, saw_slot = false;  // the next stage / its first slot, seen ready ahead
+        for (uint32_t c = 0; !stop; ++c) {
+          const uint32_t qs = c % kQuadQ;
+          if (!mbar_wait_or_abort(&qfull[qs], (c / kQuadQ) & 1u, abortp)) {
+            stop = true;
+            break;
+          }
+          const int32_t nstep = qinfo[qs].nstep;
+          mbar_arrive(&qempty[qs]);
+          if (nstep < 0) break;
+          for (int32_t j = 0; j < nstep && !stop; ++j, ++n) {
+            uint32_t slot[3] = {0, 0, 0}, use[3] = {0, 0, 0};
+#pragma unroll
+            for (int a = 0; a < NACC; ++a) acc_slot<NACC>(n, a, &slot[a], &use[a]);
+            uint32_t nslot, nuse;  // the next step's first slot
+            acc_slot<NACC>(n + 1, A0, &nslot, &nuse);
+            auto ready = [&](int a) {
+              if (use[a] == 0) return true;
+              if (a == A0 && saw_slot) {
+                tc_fence_after();
+                return true;
+              }
+              if (!mbar_wait_or_abort(&tempty[slot[a]], (use[a] - 1u) & 1u, abortp)) return false;
+              tc_fence_after();
+              return true;
+            };
+            auto done = [&](int a) { umma_commit(&tfull[slot[a]]); };
+#pragma unroll
+            for (int h = 0; h < SPS; ++h) {
+              if (!saw_full && !mbar_wait_or_abort(&full[s], sphase, abortp)) {
+                stop = true;
+                break;
+              }
+              tc_fence_after();
+              const uint32_t a_s = smem0 + s * STAGE, b_s = a_s + BREG;
+              const uint32_t s1 = s + 1 == NS ? 0 : s + 1, p1 = s + 1 == NS ? sphase ^ 1u : sphase;
+              bool sf = false, ss = false;
+              auto ahead = [&] {
+                sf = mbar_test_wait(&full[s1], p1);
+                if (h == SPS - 1) ss = nuse > 0 && mbar_test_wait(&tempty[nslot], (nuse - 1u) & 1u);
+              };
+              bool ok;
+              if (SPS == 1)
+                ok = issue_stage<PREC, true, true>(tbase, slot, a_s, b_s, idesc, ready, ahead, done);
+              else if (h == 0)
+                ok = issue_stage<PREC, true, false>(tbase, slot, a_s, b_s, idesc, ready, ahead, done);
+              else if (h == SPS - 1)
+                ok = issue_stage<PREC, false, true>(tbase, slot, a_s, b_s, idesc, ready, ahead, done);
+              else
+                ok = issue_stage<PREC, false, false>(tbase, slot, a_s, b_s, idesc, ready, ahead, done);
+              umma_commit(&empty[s]);
+              saw_full = sf;
+              saw_slot = ss;
+              any = true;
+              last = s;
+              lphase = sphase;
+              s = s1;
+              sphase = p1;
+              if (!ok) {
+                stop = true;
+                break;
+              }
+            }
+          }
         }
         if (stop) {
           atomicOr(err, DEV_ERR_TIMEOUT);
           *abortp = 1;
         }
+        // leave no MMA in flight: everything issued before the last commit has completed
+        if (any) mbar_wait_bounded(&empty[last], lphase);
       }
-      // leave no MMA in flight: everything issued before the last commit has completed
-      if (t > 0) mbar_wait_bounded(&empty[(t - 1) % NS], (uint32_t)(((t - 1) / NS) & 1));
     }
-  }
   } else {
     regs_inc<kEpiRegs>();
-    // ---------------- epilogue: warps 4..11; column c = (warp - 4) / 4; TMEM lane = output row
+    // ---------------- epilogue: warps 4..11; column c = (warp - 4) / 4; TMEM lane = output row.  Each
+    // warp goes its own way (its own arrivals on the unit ring and the slots), so one warp's output
+    // stores overlap the others' sums.
     const int col = (warp - 4) >> 2;
     const int quarter = warp & 3;
     const int lrow = 32 * quarter + lane;
     const int half = lrow >> 6, row = lrow & 63;
     const int child = 2 * half + col;  // warp-uniform
-    const int te = threadIdx.x - 128;  // 0..255
     const uint32_t taddr0 = tbase + ((uint32_t)(32 * quarter) << 16) + 64u * (uint32_t)col;
-    int64_t u = 0;  // accumulator units drained
+    uint32_t n = 0;     // steps drained
+    bool seen = false;  // the next accumulator was seen complete ahead
     // FP16: one FP32 accumulator per element; BF16 splits: (hi, lo) pairs of
     // adjacent elements packed for the FP32x2 instructions
     constexpr int NHI = NACC == 1 ? 64 : 1, NPK = NACC == 1 ? 1 : 32;
     float hi[NHI];
     uint64_t hi2[NPK], lo2[NPK];
-    for (int64_t c = 0;; ++c) {
-      // one thread takes the next claimed quad for all 256 (-2: the wait gave up)
-      if (te == 0) {
-        const int qs = (int)(c % kQuadQ);
-        if (mbar_wait_or_abort(&qfull[qs], (uint32_t)((c / kQuadQ) & 1), abortp)) {
-          epi_un = qid[qs];
-          mbar_arrive(&qempty[qs]);
-        } else {
-          epi_un = -2;
-        }
-      }
-      named_barrier(2, 256);
-      const int64_t un = epi_un;  // rewritten only after the two barriers that end this quad
-      if (un < 0) {
-        if (un == -2 && te == 0) {
-          atomicOr(err, DEV_ERR_TIMEOUT);
-          *abortp = 1;
-        }
+    bool failed = false;
+    for (uint32_t c = 0; !failed; ++c) {
+      const uint32_t qs = c % kQuadQ;
+      bool ok = true;
+      if (lane == 0) ok = mbar_wait_or_abort(&qfull[qs], (c / kQuadQ) & 1u, abortp);
+      if (!__shfl_sync(0xffffffffu, ok ? 1 : 0, 0)) {
+        failed = true;
         break;
       }
-      const int r = plan_of(batch.ubegin, batch.nplans, un);
-      const PlanDev& pl = batch.plans[r];
-      const int64_t Qc = un - batch.ubegin[r], Q = pl.uorder ? pl.uorder[Qc] : pl.ufirst + Qc;
-      // children: four output leaves (64-leaves), or the four quadrants of output leaf Q (128-leaves)
-      const bool big = pl.tc_bs == 128;
-      const int32_t g[4] = {big ? (int32_t)Q : pl.quads[4 * Q], big ? (int32_t)Q : pl.quads[4 * Q + 1],
-                            big ? (int32_t)Q : pl.quads[4 * Q + 2], big ? (int32_t)Q : pl.quads[4 * Q + 3]};
+      const int32_t nstep = qinfo[qs].nstep, ld = qinfo[qs].ld;
+      double* const outp = qinfo[qs].out[child];
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&qempty[qs]);
+      if (nstep < 0) break;
 #pragma unroll
       for (int i = 0; i < NHI; ++i) hi[i] = 0.f;
 #pragma unroll
       for (int i = 0; i < NPK; ++i) hi2[i] = lo2[i] = 0ull;
-      const int64_t j1 = pl.qstart[Q + 1];
-      int64_t j = pl.qstart[Q];
-      float sc_next = j < j1 ? __ldg(&pl.qsteps[j].scale[child]) : 0.f;
-      bool failed = false;
-      for (; j < j1 && !failed; ++j) {
-        const float sc = sc_next;
-        if (j + 1 < j1) sc_next = __ldg(&pl.qsteps[j + 1].scale[child]);
-        // one accumulator at a time, in the order the MMAs commit them; a
-        // runtime loop, so the code holds one copy of each update kind
-#pragma unroll 1
+      auto wait_full = [&](uint32_t b, uint32_t use) {
+        bool done = true;
+        if (lane == 0) done = mbar_wait_or_abort(&tfull[b], use & 1u, abortp);
+        return __shfl_sync(0xffffffffu, done ? 1 : 0, 0) != 0;
+      };
+      auto release = [&](uint32_t b) {  // one arrival per warp, after all its lanes' loads
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&tempty[b]);
+      };
+      // 32 of the slot's columns, added to the accumulators of columns 32 hh ..
+      auto add_up = [&](int hh, const uint32_t (&v)[32], bool exact, float sc) {
+        const uint64_t sc2 = ((uint64_t)__float_as_uint(sc) << 32) | __float_as_uint(sc);
+        if constexpr (NACC == 1) {
+#pragma unroll
+          for (int i = 0; i < 32; ++i) hi[32 * hh + i] = fmaf(__uint_as_float(v[i]), sc, hi[32 * hh + i]);
+        } else if (exact) {  // an exact accumulator: TwoSum into (hi, lo)
+          two_sum_x8(hi2 + 16 * hh, lo2 + 16 * hh, v, sc2);
+          two_sum_x8(hi2 + 16 * hh + 8, lo2 + 16 * hh + 8, v + 16, sc2);
+        } else {
+#pragma unroll
+          for (int i = 0; i < 16; ++i)
+            lo2[16 * hh + i] = fma_x2(pack_x2(v[2 * i], v[2 * i + 1]), sc2, lo2[16 * hh + i]);
+        }
+      };
+      // One step: its accumulators in the order the MMAs commit them.  A slot's 64 columns of this
+      // thread's row are loaded in two halves and handed back to the MMAs before they are added up; the
+      // next accumulator's halves are loaded as soon as the registers of this one's are free, so their
+      // way from tensor memory passes behind the sums.
+      auto step = [&]() {
+        uint32_t b, use;
+        acc_slot<NACC>(n, 0, &b, &use);
+        if (!seen && !wait_full(b, use)) return false;
+        seen = false;
+        tc_fence_after();
+        const float sc = reinterpret_cast<const float*>(&sscale[n % kScaleRing])[child];
+        if (sc == 0.f) {  // no kept product of this warp's child at this k
+          release(b);
+#pragma unroll
+          for (int a = 1; a < NACC; ++a) {
+            acc_slot<NACC>(n, a, &b, &use);
+            if (!wait_full(b, use)) return false;
+            release(b);
+          }
+          return true;
+        }
+        uint32_t va[32], vb[32];
+        tmem_ld32_async(taddr0 + b * 128u, va);
+        tmem_ld32_async(taddr0 + b * 128u + 32u, vb);
+#pragma unroll
         for (int a = 0; a < NACC; ++a) {
-          const int b = (int)(u % NB);
-          bool ok = true;
-          if (lane == 0) ok = mbar_wait_or_abort(&tfull[b], (uint32_t)((u / NB) & 1), abortp);
-          ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
-          ++u;
-          if (!ok) {
-            // the epilogue still runs the barrier sequence below, then stops together
-            atomicOr(err, DEV_ERR_TIMEOUT);
-            *abortp = 1;
-            failed = true;
-            break;
+          tmem_wait32(va);  // waits for every load in flight
+          tmem_wait32(vb);
+          release(b);
+          add_up(0, va, a < NACC - 1, sc);
+          if (a + 1 < NACC) {
+            acc_slot<NACC>(n, a + 1, &b, &use);
+            if (!wait_full(b, use)) return false;
+            tc_fence_after();
+            tmem_ld32_async(taddr0 + b * 128u, va);
+          } else {
+            acc_slot<NACC>(n + 1, 0, &b, &use);
+            seen = __all_sync(0xffffffffu, mbar_test_wait(&tfull[b], use & 1u));
           }
-          tc_fence_after();
-          bool released = false;
-          if (sc != 0.f) {  // this warp's child has a kept product at this k
-            const bool exact = a < NACC - 1;  // an exact accumulator: TwoSum into (hi, lo)
-            const uint64_t sc2 = ((uint64_t)__float_as_uint(sc) << 32) | __float_as_uint(sc);
-            // the slot's 64 columns of this thread's row: four loads in flight
-            // at once, one wait; the slot is handed back to the MMAs before
-            // the registers are added up
-            const uint32_t ta = taddr0 + (uint32_t)b * 128u;
-            uint32_t buf[4][16];
-#pragma unroll
-            for (int hh = 0; hh < 4; ++hh) tmem_ld16_async(ta + 16u * hh, buf[hh]);
-#pragma unroll
-            for (int hh = 0; hh < 4; ++hh) tmem_wait16(buf[hh]);  // the first waits for all four
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(&tempty[b]);  // one arrival per warp, after all its lanes' loads
-            released = true;
-#pragma unroll
-            for (int hh = 0; hh < 4; ++hh) {
-              const uint32_t* v = buf[hh];
-              if constexpr (NACC == 1) {
-#pragma unroll
-                for (int i = 0; i < 16; ++i) hi[16 * hh + i] = fmaf(__uint_as_float(v[i]), sc, hi[16 * hh + i]);
-              } else if (exact) {
-#pragma unroll
-                for (int i = 0; i < 8; ++i) two_sum_x2(hi2[8 * hh + i], lo2[8 * hh + i], v[2 * i], v[2 * i + 1], sc2);
-              } else {
-#pragma unroll
-                for (int i = 0; i < 8; ++i) fma_x2(lo2[8 * hh + i], v[2 * i], v[2 * i + 1], sc2);
-              }
-            }
-          }
-          if (!released) {
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(&tempty[b]);
-          }
+          add_up(1, vb, a < NACC - 1, sc);
+          if (a + 1 < NACC) tmem_ld32_async(taddr0 + b * 128u + 32u, vb);
+        }
+        return true;
+      };
+      for (int32_t j = 0; j < nstep; ++j, ++n) {
+        if (!step()) {
+          failed = true;
+          break;
         }
       }
-      // output row `row` of leaf g[child], unconverted: each element's 8-byte
+      if (failed) break;
+      // output row `row` of this warp's child, unconverted: each element's 8-byte
       // slot receives its two-float pair (hi, lo) (FP16: (hi, 0)); the finishing
       // pass (tc_finish_kernel) turns the slots into FP64 and takes the leaf
       // norms, so no FP64 instruction runs here, where it would hold up the
-      // draining of the accumulators the next quad's MMAs wait for
-      const int gl = g[child];
-      if (gl >= 0) {
-        uint4* out = reinterpret_cast<uint4*>(big ? pl.cpool + (int64_t)gl * 16384 + (64 * half + row) * 128 + 64 * col
-                                                  : pl.cpool + (int64_t)gl * 4096 + row * 64);
+      // draining of the accumulators the next quad's MMAs wait for.  32 bytes
+      // (one sector) per lane and store.
+      if (outp) {
+        double* out = outp + row * ld;
 #pragma unroll
-        for (int q = 0; q < 64; q += 2) {
-          if constexpr (NACC == 1) {
-            out[q >> 1] = make_uint4(__float_as_uint(hi[q]), 0u, __float_as_uint(hi[q + 1]), 0u);
-          } else {
-            const uint64_t h = hi2[q / 2], l = lo2[q / 2];
-            out[q >> 1] = make_uint4((uint32_t)h, (uint32_t)l, (uint32_t)(h >> 32), (uint32_t)(l >> 32));
-          }
+        for (int q = 0; q < 64; q += 4) {
+          if constexpr (NACC == 1)
+            store_32(out + q, __float_as_uint(hi[q]), 0u, __float_as_uint(hi[q + 1]), 0u, __float_as_uint(hi[q + 2]), 0u,
+                     __float_as_uint(hi[q + 3]), 0u);
+          else
+            store_32(out + q, (uint32_t)hi2[q / 2], (uint32_t)lo2[q / 2], (uint32_t)(hi2[q / 2] >> 32),
+                     (uint32_t)(lo2[q / 2] >> 32), (uint32_t)hi2[q / 2 + 1], (uint32_t)lo2[q / 2 + 1],
+                     (uint32_t)(hi2[q / 2 + 1] >> 32), (uint32_t)(lo2[q / 2 + 1] >> 32));
         }
       }
-      if (te == 0) epi_stop = *abortp;
-      named_barrier(1, 256);
-      const bool stop = epi_stop != 0;
-      named_barrier(1, 256);
-      if (stop) break;
+    }
+    if (failed && lane == 0) {
+      atomicOr(err, DEV_ERR_TIMEOUT);
+      *abortp = 1;
     }
   }
   tc_fence_before();
