@@ -37,19 +37,27 @@ static unsigned grid_for(spamm_ctx ctx, int64_t items, int per_block, int max_pe
 // The FMA is the only FP64 instruction per element: this part issues two FP64
 // operations per clock per SM, so the non-zero and finiteness checks work on
 // the bit patterns in the integer pipe (any bit besides the sign set: non-zero;
-// exponent field all ones: Inf or NaN).
-template <class Get>
+// exponent field all ones: Inf or NaN).  U pairs per lane are read before the
+// first is used (bs^2 / 2 is a multiple of 512 pairs for every leaf size, so U
+// is at most 16): a lane that reads one pair at a time waits for memory 64 times
+// in a 64 x 64 leaf.
+template <int U, class Get>
 __device__ __forceinline__ void warp_leaf_sumsq(Get get, int bs, int lane, double* s_out, bool* nz_out, bool* bad_out) {
   const int pairs = bs * bs / 2;
   double s = 0.0;
   uint32_t bits = 0, emax = 0;
-  for (int i = lane; i < pairs; i += 32) {
-    double2 v = get(i);
-    s = __fma_rn(v.x, v.x, s);
-    s = __fma_rn(v.y, v.y, s);
-    const uint32_t hx = (uint32_t)__double2hiint(v.x), hy = (uint32_t)__double2hiint(v.y);
-    bits |= (uint32_t)__double2loint(v.x) | (uint32_t)__double2loint(v.y) | ((hx | hy) & 0x7fffffffu);
-    emax = max(emax, max(hx & 0x7ff00000u, hy & 0x7ff00000u));
+  for (int i = lane; i < pairs; i += 32 * U) {
+    double2 v[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) v[u] = get(i + 32 * u);
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      s = __fma_rn(v[u].x, v[u].x, s);
+      s = __fma_rn(v[u].y, v[u].y, s);
+      const uint32_t hx = (uint32_t)__double2hiint(v[u].x), hy = (uint32_t)__double2hiint(v[u].y);
+      bits |= (uint32_t)__double2loint(v[u].x) | (uint32_t)__double2loint(v[u].y) | ((hx | hy) & 0x7fffffffu);
+      emax = max(emax, max(hx & 0x7ff00000u, hy & 0x7ff00000u));
+    }
   }
 #pragma unroll
   for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
@@ -58,21 +66,20 @@ __device__ __forceinline__ void warp_leaf_sumsq(Get get, int bs, int lane, doubl
   *bad_out = __any_sync(0xffffffffu, emax == 0x7ff00000u);
 }
 
-// Block b takes leaves [64 b, 64 b + 64), each of its 8 warps every 8th of
-// them (a grid of about nleaves / 64 blocks spreads evenly over the SMs;
-// larger grids stride by whole blocks).
-constexpr int64_t kNormLeavesPerBlock = 64;
+// Block b takes leaves [8 b, 8 b + 8), one per warp (larger grids stride by whole
+// blocks): with 64 leaves per block a few thousand leaves kept only a third of
+// the SMs busy.
+constexpr int64_t kNormLeavesPerBlock = 8;
 __global__ void leaf_sqnorm_kernel(const double* __restrict__ pool, const int64_t* __restrict__ slot, int64_t m,
                                    int bs, double* __restrict__ sq, uint8_t* __restrict__ nonzero, int check_finite,
                                    int* err) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwb = blockDim.x >> 5;
   const int64_t e = (int64_t)bs * bs;
-  for (int64_t q0 = (int64_t)blockIdx.x * kNormLeavesPerBlock; q0 < m; q0 += (int64_t)gridDim.x * kNormLeavesPerBlock)
-  for (int64_t q = q0 + warp; q < q0 + kNormLeavesPerBlock && q < m; q += nwb) {
+  for (int64_t q = (int64_t)blockIdx.x * kNormLeavesPerBlock + warp; q < m; q += (int64_t)gridDim.x * nwb) {
     const double2* src = reinterpret_cast<const double2*>(pool + (slot ? slot[q] : q) * e);
     double s;
     bool nz, bad;
-    warp_leaf_sumsq([&](int i) { return __ldg(src + i); }, bs, lane, &s, &nz, &bad);
+    warp_leaf_sumsq<8>([&](int i) { return __ldg(src + i); }, bs, lane, &s, &nz, &bad);
     if (lane == 0) {
       sq[q] = s;
       if (nonzero) nonzero[q] = nz;
@@ -552,7 +559,7 @@ __global__ void candidate_stats_kernel(Elem elem, int64_t ncand, int bs, int64_t
     }
     double s;
     bool nz, bad;
-    warp_leaf_sumsq(
+    warp_leaf_sumsq<1>(
         [&](int i) {
           int e0 = 2 * i;
           double x = elem(r, c, e0 / bs, e0 % bs), y = elem(r, c, e0 / bs, e0 % bs + 1);
@@ -950,7 +957,7 @@ __global__ void error_x_kernel(const double* __restrict__ xpool, const int64_t* 
     const double2* ys = reinterpret_cast<const double2*>(ypool + yslot[p] * e);
     double s;
     bool nz, bad;
-    warp_leaf_sumsq(
+    warp_leaf_sumsq<4>(
         [&](int i) {
           double2 a = __ldg(xs + i), b = __ldg(ys + i);
           return make_double2(a.x - b.x, a.y - b.y);
