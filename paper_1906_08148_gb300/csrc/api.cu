@@ -87,7 +87,7 @@ double elapsed_ms(cudaEvent_t a, cudaEvent_t b) {
 }
 
 struct Events {
-  cudaEvent_t e[5] = {};
+  cudaEvent_t e[6] = {};
   Events() {
     for (auto& x : e) CK(cudaEventCreate(&x));
   }
@@ -282,15 +282,16 @@ spamm_status spamm_release(spamm_mat m) {
   return SPAMM_OK;
 }
 
+// The operands after the method's input truncation (enqueued only: their counts are
+// taken over by task_begin).
 static void run_truncation(spamm_mat A, spamm_mat B, double tau, spamm_mode mode, spamm_mat* At, spamm_mat* Bt,
-                           spamm_ctx on = nullptr) {
+                           spamm_ctx ctx) {
   if (mode == SPAMM_MODE_SPAMM) {
     *At = A;
     *Bt = B;
     return;
   }
-  *At = truncate_block(A, tau, on);
-  *Bt = (B == A) ? *At : truncate_block(B, tau, on);
+  truncate_pair(ctx, A, B, tau, At, Bt);
 }
 
 static void check_pair(spamm_mat A, spamm_mat B, double tau, spamm_mode mode) {
@@ -316,6 +317,7 @@ struct spamm_plan_s {
   BufP uorder;          // FP64 form: unit -> output leaf, longest first (empty: identity)
   int64_t nsteps = 0;
   std::vector<Level> cskel;  // output quadtree structure (codes, child links; no norms)
+  BufP cdcount;              // its node counts on the device
   int64_t na = 0, nb = 0;
   double ms_truncate = 0, ms_tasks = 0, ms_prep = 0;
   int64_t launches = 0;
@@ -364,27 +366,12 @@ spamm_plan make_plan(spamm_ctx ctx, spamm_mat A, spamm_mat B, double tau, spamm_
   run_truncation(A, B, tau, mode, &At, &Bt, ctx);
   std::unique_ptr<spamm_mat_s> ownA(At != A ? At : nullptr), ownB((Bt != B && Bt != At) ? Bt : nullptr);
   CK(cudaEventRecord(ev.e[1], ctx->stream));
-  p->T = build_tasks(At, Bt, tau, mode != SPAMM_MODE_TRUNCATE, ctx);
-  {
-    // the output structure is fixed by the kept set (Section 4.4): build it now
-    std::unique_ptr<spamm_mat_s> sk(new_mat(ctx, A->n, A->bs));
-    sk->lv[sk->L].count = p->T.ngroups;
-    sk->lv[sk->L].code = p->T.gcode;
-    build_skeleton(sk.get());
-    p->cskel = sk->lv;
-  }
-  CK(cudaEventRecord(ev.e[2], ctx->stream));
+  std::shared_ptr<TaskBuild> tb = task_begin(At, Bt, tau, mode != SPAMM_MODE_TRUNCATE, ctx, &p->T);
   p->na = At->nleaves;
   p->nb = Bt->nleaves;
-  if (prec == SPAMM_PREC_FP64) {
-    p->poolA = At->pool;
-    p->slotA = At->slot;
-    p->poolB = Bt->pool;
-    p->slotB = Bt->slot;
-    const bool longest = ctx->claim_order == SPAMM_ORDER_LONGEST_FIRST ||
-                         (ctx->claim_order == SPAMM_ORDER_AUTO && p->bs >= 128);
-    if (longest) p->uorder = unit_order_longest(ctx, P<int64_t>(p->T.gstart), p->T.ngroups);
-  } else {
+  CK(cudaEventRecord(ev.e[2], ctx->stream));
+  const bool tensor = prec != SPAMM_PREC_FP64;
+  if (tensor) {
     prep_terms(At, prec, 0, &p->termsA, &p->expA, ctx);
     // X times X with X symmetric: the B operand of leaf (k, j) is the transpose
     // of leaf (j, k), whose A terms are exactly the B terms of (k, j) (rows of
@@ -397,20 +384,47 @@ spamm_plan make_plan(spamm_ctx ctx, spamm_mat A, spamm_mat B, double tau, spamm_
       p->bmap.reset();
       prep_terms(Bt, prec, 1, &p->termsB, &p->expB, ctx);
     }
+  }
+  CK(cudaEventRecord(ev.e[3], ctx->stream));
+  {
+    const StepExps exps{P<int32_t>(p->expA), P<int32_t>(p->expB), P<int32_t>(p->bmap)};
+    const bool quads = tensor && p->bs == 64;
+    task_finish(ctx, tb.get(), &p->T, quads ? &exps : nullptr, &p->qstart, &p->qsteps);
+    p->nsteps = quads ? p->T.nsteps : 0;
+  }
+  // the output structure is fixed by the kept set (Section 4.4): build it now
+  std::unique_ptr<spamm_mat_s> sk(new_mat(ctx, A->n, A->bs));
+  sk->lv[sk->L].count = p->T.ngroups;
+  sk->lv[sk->L].code = p->T.gcode;
+  uint64_t* counts = static_cast<uint64_t*>(ctx->h_pinned);
+  if (p->T.ngroups > 0) {
+    tree_skeleton(ctx, sk.get());
+    tree_counts_async(ctx, sk.get(), counts);
+  }
+  CK(cudaEventRecord(ev.e[4], ctx->stream));
+  if (!tensor) {
+    p->poolA = At->pool;
+    p->slotA = At->slot;
+    p->poolB = Bt->pool;
+    p->slotB = Bt->slot;
+    const bool longest = ctx->claim_order == SPAMM_ORDER_LONGEST_FIRST ||
+                         (ctx->claim_order == SPAMM_ORDER_AUTO && p->bs >= 128);
+    if (longest) p->uorder = unit_order_longest(ctx, P<int64_t>(p->T.gstart), p->T.ngroups);
+  } else {
     if (p->bs == 128)
       p->nsteps = build_leaf128_steps(ctx, p->T, P<int32_t>(p->expA), P<int32_t>(p->expB), P<int32_t>(p->bmap),
                                       &p->qstart, &p->qsteps);
-    else
-      p->nsteps = build_quad_steps(ctx, p->T, P<uint32_t>(At->lv[At->L].code), P<int32_t>(p->expA),
-                                   P<int32_t>(p->expB), P<int32_t>(p->bmap), &p->qstart, &p->qsteps);
     if (ctx->claim_order == SPAMM_ORDER_LONGEST_FIRST)
       p->uorder = unit_order_longest(ctx, P<int64_t>(p->qstart), p->bs == 128 ? p->T.ngroups : p->T.nquads);
   }
-  CK(cudaEventRecord(ev.e[3], ctx->stream));
+  CK(cudaEventRecord(ev.e[5], ctx->stream));
   sync_and_check(ctx);
+  if (p->T.ngroups > 0) tree_set_counts(sk.get(), counts);
+  p->cskel = sk->lv;
+  p->cdcount = sk->dcount;
   p->ms_truncate = elapsed_ms(ev.e[0], ev.e[1]);
-  p->ms_tasks = elapsed_ms(ev.e[1], ev.e[2]);
-  p->ms_prep = elapsed_ms(ev.e[2], ev.e[3]);
+  p->ms_tasks = elapsed_ms(ev.e[1], ev.e[2]) + elapsed_ms(ev.e[3], ev.e[4]);
+  p->ms_prep = elapsed_ms(ev.e[2], ev.e[3]) + elapsed_ms(ev.e[4], ev.e[5]);
   p->launches = (int64_t)(g_kernel_launches - launches0);
   ctx->live_handles++;
   return p.release();
@@ -456,6 +470,7 @@ PlanOut make_output(spamm_ctx ctx, const spamm_plan_s& p) {
   o.C.reset(new_mat(ctx, p.n, bs));
   spamm_mat Cm = o.C.get();
   Cm->lv = p.cskel;
+  Cm->dcount = p.cdcount;
   Cm->nleaves = p.T.ngroups;
   Cm->pool = alloc_n<double>(ctx, p.T.ngroups * e);
   Cm->slot = alloc_n<int64_t>(ctx, p.T.ngroups);
@@ -549,19 +564,21 @@ std::vector<spamm_mat> execute_plans(spamm_ctx ctx, const std::vector<spamm_plan
   CK(cudaMemcpyAsync(P<PlanDev>(dplans), host.data(), np * sizeof(PlanDev), cudaMemcpyHostToDevice, ctx->stream));
   CK(cudaMemcpyAsync(P<int64_t>(dub), ubegin.data(), (np + 1) * sizeof(int64_t), cudaMemcpyHostToDevice,
                      ctx->stream));
-  std::vector<NormBatchLevel> nlv;
-  BufP ntab = norm_batch_tables(ctx, outp, &nlv);
+  NormBatch norms;
+  BufP ntab = norm_tables(ctx, outp, &norms);
   BatchDev batch{P<PlanDev>(dplans), P<int64_t>(dub), (int)np, ubegin[np]};
 
   auto sequence = [&](unsigned evflags) {
     CK(cudaEventRecordWithFlags(ev.e[0], ctx->stream, evflags));
     launch_gemm(ctx, prec, bs, batch);
     CK(cudaEventRecordWithFlags(ev.e[1], ctx->stream, evflags));
-    if (prec != SPAMM_PREC_FP64)
-      for (int64_t r = 0; r < np; ++r)
-        tc_finish(ctx, prec, P<double>(outp[r]->pool), outp[r]->nleaves, bs, P<double>(outp[r]->lv[outp[r]->L].sq));
-    for (int64_t r = 0; r < np; ++r) fill_iota_i64(ctx, P<int64_t>(outp[r]->slot), outp[r]->nleaves);
-    propagate_norms_batch(ctx, nlv);
+    for (int64_t r = 0; r < np; ++r)
+      if (prec != SPAMM_PREC_FP64)
+        tc_finish(ctx, prec, P<double>(outp[r]->pool), outp[r]->nleaves, bs, P<double>(outp[r]->lv[outp[r]->L].sq),
+                  P<int64_t>(outp[r]->slot));
+      else
+        fill_iota_i64(ctx, P<int64_t>(outp[r]->slot), outp[r]->nleaves);
+    propagate_norms(ctx, norms);
     CK(cudaEventRecordWithFlags(ev.e[2], ctx->stream, evflags));
   };
   if (ctx->exec_graph) {
@@ -806,11 +823,13 @@ spamm_status spamm_job_finish(spamm_ctx ctx, spamm_job job, spamm_mat* C, spamm_
     Events ev;
     CK(cudaEventRecord(ev.e[0], ctx->stream));
     if (job->plan->prec != SPAMM_PREC_FP64)
-      tc_finish(ctx, job->plan->prec, P<double>(Cm->pool), Cm->nleaves, job->plan->bs, P<double>(Cm->lv[Cm->L].sq));
-    fill_iota_i64(ctx, P<int64_t>(Cm->slot), Cm->nleaves);
-    std::vector<NormBatchLevel> nlv;
-    BufP ntab = norm_batch_tables(ctx, {Cm}, &nlv);
-    propagate_norms_batch(ctx, nlv);
+      tc_finish(ctx, job->plan->prec, P<double>(Cm->pool), Cm->nleaves, job->plan->bs, P<double>(Cm->lv[Cm->L].sq),
+                P<int64_t>(Cm->slot));
+    else
+      fill_iota_i64(ctx, P<int64_t>(Cm->slot), Cm->nleaves);
+    NormBatch norms;
+    BufP ntab = norm_tables(ctx, {Cm}, &norms);
+    propagate_norms(ctx, norms);
     CK(cudaEventRecord(ev.e[1], ctx->stream));
     sync_and_check(ctx);
     if (stats) {
@@ -909,13 +928,15 @@ spamm_status spamm_kept_tasks(spamm_ctx ctx, spamm_mat A, spamm_mat B, double ta
   return guarded(ctx, [&] {
     check_pair(A, B, tau, mode);
     spamm_mat At = nullptr, Bt = nullptr;
-    run_truncation(A, B, tau, mode, &At, &Bt);
+    run_truncation(A, B, tau, mode, &At, &Bt, ctx);
     std::unique_ptr<spamm_mat_s> ownA(At != A ? At : nullptr), ownB((Bt != B && Bt != At) ? Bt : nullptr);
-    TaskList T = build_tasks(At, Bt, tau, mode != SPAMM_MODE_TRUNCATE);
+    TaskList T;
+    std::shared_ptr<TaskBuild> tb = task_begin(At, Bt, tau, mode != SPAMM_MODE_TRUNCATE, ctx, &T);
     *count = T.ntasks;
     if (T.ntasks > cap) fail(SPAMM_E_CAPACITY, "ikj_out holds fewer triples than the kept set");
     if (T.ntasks == 0) return;
     need(ikj_out != nullptr, "ikj_out must be non-NULL");
+    task_finish(ctx, tb.get(), &T, nullptr, nullptr, nullptr);
     BufP d = alloc_n<int32_t>(ctx, 3 * T.ntasks);
     tasks_to_ikj(At, T, P<int32_t>(d));
     CK(cudaMemcpyAsync(ikj_out, P<int32_t>(d), 3 * T.ntasks * sizeof(int32_t), cudaMemcpyDeviceToHost, ctx->stream));

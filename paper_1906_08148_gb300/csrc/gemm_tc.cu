@@ -712,7 +712,7 @@ constexpr int64_t kFinishLeavesPerBlock = 8;
 
 template <bool TWO>
 __global__ void __launch_bounds__(256) tc_finish_kernel(double* __restrict__ pool, int64_t m, int bs,
-                                                        double* __restrict__ sq) {
+                                                        double* __restrict__ sq, int64_t* __restrict__ slot) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int64_t e = (int64_t)bs * bs;
   const int pairs = bs * bs / 2;
@@ -740,18 +740,21 @@ __global__ void __launch_bounds__(256) tc_finish_kernel(double* __restrict__ poo
     }
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
-    if (lane == 0) sq[q] = s;
+    if (lane == 0) {
+      sq[q] = s;
+      slot[q] = q;
+    }
   }
 }
 
-void tc_finish(spamm_ctx ctx, spamm_prec prec, double* pool, int64_t nleaves, int bs, double* sq) {
+void tc_finish(spamm_ctx ctx, spamm_prec prec, double* pool, int64_t nleaves, int bs, double* sq, int64_t* slot) {
   if (nleaves <= 0) return;
   const int64_t nblk = (nleaves + kFinishLeavesPerBlock - 1) / kFinishLeavesPerBlock;
   const unsigned grid = (unsigned)(nblk < (1ll << 30) ? nblk : (1ll << 30));
   if (prec == SPAMM_PREC_FP16_SCALED)
-    tc_finish_kernel<false><<<grid, 256, 0, ctx->stream>>>(pool, nleaves, bs, sq);
+    tc_finish_kernel<false><<<grid, 256, 0, ctx->stream>>>(pool, nleaves, bs, sq, slot);
   else
-    tc_finish_kernel<true><<<grid, 256, 0, ctx->stream>>>(pool, nleaves, bs, sq);
+    tc_finish_kernel<true><<<grid, 256, 0, ctx->stream>>>(pool, nleaves, bs, sq, slot);
   CK_LAUNCH("tc_finish_kernel");
 }
 

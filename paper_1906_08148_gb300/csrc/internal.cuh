@@ -24,15 +24,18 @@ extern thread_local unsigned long long g_kernel_launches;
 #define CK_LAUNCH(what) \
   (++::spamm::g_kernel_launches, ::spamm::check_cuda(cudaGetLastError(), what, __FILE__, __LINE__))
 
-// Device buffer owned through the context allocator.
+// Device buffer owned through the context allocator, or a part of one (`owner` keeps
+// the whole alive).
 struct Buf {
   spamm_ctx ctx = nullptr;
   void* p = nullptr;
   size_t bytes = 0;
+  std::shared_ptr<Buf> owner;
   ~Buf();
 };
 using BufP = std::shared_ptr<Buf>;
 BufP alloc_bytes(spamm_ctx ctx, size_t bytes);
+BufP sub_buf(const BufP& whole, size_t at, size_t bytes);
 template <class T>
 BufP alloc_n(spamm_ctx ctx, int64_t count) {
   return alloc_bytes(ctx, (size_t)(count > 0 ? count : 0) * sizeof(T));
@@ -130,33 +133,53 @@ struct spamm_mat_s {
   spamm::BufP slot;  // int64 per leaf: payload slot of leaf m (leaves in Morton order)
   int symmetric = 0;  // the matrix equals its transpose (set by the generator or the caller)
   std::vector<spamm::Level> lv;  // levels 0..L
+  spamm::BufP dcount;            // uint64 [L + 1]: nodes per level, as `count` of the levels (null: no leaves)
+  bool pending = false;          // the counts are bounds: the device's have not been taken over yet
 };
 
 namespace spamm {
 // ---- quadtree store (store.cu) ----
 spamm_mat new_mat(spamm_ctx ctx, int64_t n, int bs);
-void build_tree(spamm_mat m);  // levels L-1..0 from m->lv[L]
-// build_tree in parts: the structure (codes, child links; synchronises per
-// level for the counts), then norm buffers, then the norms (no host sync, so
-// it can be captured in a CUDA graph).  The addition order is build_tree's.
-void build_skeleton(spamm_mat m);
-void alloc_level_norms(spamm_mat m);
-void propagate_norms(spamm_mat m);
-// propagate_norms of several matrices at once: one launch per height above the
-// leaves.  norm_batch_tables uploads the per-height segment tables (norm
-// buffers must already exist); propagate_norms_batch launches (no host sync).
-struct NormBatchLevel {
-  const void* seg = nullptr;       // device segment table of this height
-  const int64_t* begin = nullptr;  // device: first parent of each segment
-  int first = 0, nseg = 0;
-  int64_t total = 0;
+// ---- quadtree structure (tree.cu) ----
+// A matrix's leaves and levels from candidates sorted by code: candidate q (code
+// code[q], or q if null; slot slot[q], or q) is a leaf iff keep[q], or, without
+// `keep`, iff it passes the block rule of threshold tau.
+struct TreeReq {
+  spamm_mat m;
+  int64_t n;
+  const uint32_t* code;
+  const double* sq;
+  const int64_t* slot;
+  const uint8_t* keep;
+  double tau;
 };
-BufP norm_batch_tables(spamm_ctx ctx, const std::vector<spamm_mat>& ms, std::vector<NormBatchLevel>* levels);
-void propagate_norms_batch(spamm_ctx ctx, const std::vector<NormBatchLevel>& levels);
+// Enqueues the building of k <= 2 trees.  The levels' counts are upper bounds and
+// nleaves is unset until the device counts are taken over (tree_resolve, or
+// tree_counts_async, a wait, tree_set_counts).
+void tree_from_candidates(spamm_ctx ctx, TreeReq* req, int k);
+void tree_resolve(spamm_ctx ctx, spamm_mat m);
+void tree_counts_async(spamm_ctx ctx, spamm_mat m, uint64_t* host);  // host: L + 1 pinned words
+void tree_set_counts(spamm_mat m, const uint64_t* host);
+// The levels above given leaf codes (count exact), without norms; counts as above.
+void tree_skeleton(spamm_ctx ctx, spamm_mat m);
+void alloc_level_norms(spamm_mat m);
+// The parents' norms of several matrices whose structure and leaf norms exist:
+// norm_tables uploads the tables (norm buffers must already exist),
+// propagate_norms launches (no host sync, so it can be captured in a CUDA graph).
+struct NormBatch {
+  const void* tab = nullptr;
+  int ntrees = 0;
+  int wide = 0;        // heights with a launch of their own
+  int64_t widest = 0;  // nodes of the largest of them
+};
+BufP norm_tables(spamm_ctx ctx, const std::vector<spamm_mat>& ms, NormBatch* nb);
+void propagate_norms(spamm_ctx ctx, const NormBatch& nb);
 // Leaf set from candidate leaves: keep[q] selects rows of (code, sq, slot) already sorted by code.
 void set_leaves_compacted(spamm_mat m, int64_t ncand, const uint32_t* code, const double* sq, const int64_t* slot,
                           const uint8_t* keep);
 spamm_mat truncate_block(spamm_mat in, double tau, spamm_ctx on = nullptr);  // work on `on` (default: in's context)
+// Both operands of a multiply (B may be A), enqueued only: counts not taken over yet.
+void truncate_pair(spamm_ctx ctx, spamm_mat A, spamm_mat B, double tau, spamm_mat* At, spamm_mat* Bt);
 spamm_mat truncate_element(spamm_mat in, double tau);
 spamm_mat truncate_error_controlled(spamm_mat in, double tau, spamm_ctx on = nullptr);
 void leaf_sqnorms(spamm_ctx ctx, const double* pool, const int64_t* slot, int64_t nleaves, int bs, double* sq,
@@ -181,8 +204,20 @@ struct TaskList {
   int64_t n_candidates[SPAMM_MAX_LEVELS] = {};
   int64_t n_kept_level[SPAMM_MAX_LEVELS] = {};
   int64_t n_borderline = 0;
+  int64_t nsteps = 0;  // steps of all quads
 };
-TaskList build_tasks(spamm_mat A, spamm_mat B, double tau, int test_norms, spamm_ctx on = nullptr);
+// The list in two parts, so that the operand terms (whose scales go into the quad
+// steps) are prepared in between.  task_begin descends and counts: T's sizes and
+// statistics, and the node counts of A and B where they were pending; it waits
+// once.  task_finish writes the list, and with `exps` the quad steps of 64 x 64
+// leaves (enqueued only).
+struct TaskBuild;
+struct StepExps {
+  const int32_t *expA, *expB;  // the leaves' scale exponents
+  const int32_t* bmap;         // null, or for B's leaf q the leaf whose terms serve as its B operand
+};
+std::shared_ptr<TaskBuild> task_begin(spamm_mat A, spamm_mat B, double tau, int test_norms, spamm_ctx ctx, TaskList* T);
+void task_finish(spamm_ctx ctx, TaskBuild* tb, TaskList* T, const StepExps* exps, BufP* qstart, BufP* qsteps);
 
 // ---- batched leaf products (gemm_fp64.cu, gemm_tc.cu) ----
 // One k step of a quad of output leaves (2I + h, 2J + c) in the tensor-core
@@ -249,22 +284,14 @@ BufP unit_order_longest(spamm_ctx ctx, const int64_t* start, int64_t n);
 // The tensor-core forms' persistent quad kernel (gemm_tc.cu).
 void gemm_tc_batch(spamm_ctx ctx, spamm_prec prec, const BatchDev& b);
 // Kernel (d) of the tensor-core forms: the GEMM's two-float output slots to
-// FP64 in place, and each leaf's squared norm (kernel (a)'s order).
-void tc_finish(spamm_ctx ctx, spamm_prec prec, double* pool, int64_t nleaves, int bs, double* sq);
+// FP64 in place, each leaf's squared norm (kernel (a)'s order) and its payload slot.
+void tc_finish(spamm_ctx ctx, spamm_prec prec, double* pool, int64_t nleaves, int bs, double* sq, int64_t* slot);
 // 64 x 64 operand tiles per leaf of the tensor forms (bs 64: 1, bs 128: 4).
 inline int tc_tiles_per_leaf(int bs) { return (bs / 64) * (bs / 64); }
 // Operand terms of a leaf set for a tensor form (role 0: used as A, 1: as B),
 // and each tile's power-of-two scale exponent.
 void prep_terms(spamm_mat M, spamm_prec prec, int role, BufP* terms, BufP* expo, spamm_ctx on = nullptr);
-// Step list of every quad of T for the tensor-core kernel; returns the step count.
-// codeA: Morton codes of A's leaves (the k of a task is the column of its A
-// leaf); expA/expB: the leaves' scale exponents (null: no scaling).
-// bmap (may be null): for B's leaf q, the index of the leaf whose terms serve
-// as its B operand (a symmetric matrix times itself uses A's terms of the
-// transposed leaf); the step list then refers to that index.
-int64_t build_quad_steps(spamm_ctx ctx, const TaskList& T, const uint32_t* codeA, const int32_t* expA,
-                         const int32_t* expB, const int32_t* bmap, BufP* qstart, BufP* qsteps);
-// The same for 128 x 128 leaves: one unit per output leaf, two K-half steps
+// The step list of 128 x 128 leaves for the tensor-core kernel: one unit per output leaf, two K-half steps
 // per kept product (T.gstart doubled), on the tile-split operand terms.
 int64_t build_leaf128_steps(spamm_ctx ctx, const TaskList& T, const int32_t* expA, const int32_t* expB,
                             const int32_t* bmap, BufP* qstart, BufP* qsteps);

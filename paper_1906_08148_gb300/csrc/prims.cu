@@ -22,7 +22,7 @@ void check_cuda(cudaError_t e, const char* what, const char* file, int line) {
 }
 
 Buf::~Buf() {
-  if (!p) return;
+  if (!p || owner) return;
   if (ctx->ufree)
     ctx->ufree(p, ctx->user);
   else
@@ -61,6 +61,15 @@ BufP alloc_bytes(spamm_ctx ctx, size_t bytes) {
   return b;
 }
 
+BufP sub_buf(const BufP& whole, size_t at, size_t bytes) {
+  auto b = std::make_shared<Buf>();
+  b->ctx = whole->ctx;
+  b->owner = whole;
+  b->bytes = bytes;
+  b->p = bytes ? static_cast<uint8_t*>(whole->p) + at : nullptr;
+  return b;
+}
+
 template <class T>
 T read_scalar(spamm_ctx ctx, const T* d) {
   CK(cudaMemcpyAsync(ctx->h_pinned, d, sizeof(T), cudaMemcpyDeviceToHost, ctx->stream));
@@ -76,10 +85,13 @@ template int read_scalar<int>(spamm_ctx, const int*);
 
 void clear_device_error(spamm_ctx ctx) { CK(cudaMemsetAsync(ctx->d_err, 0, sizeof(int), ctx->stream)); }
 
+// One wait for the work and the error word (read into the last word of the pinned page).
 void sync_and_check(spamm_ctx ctx) {
+  int* word = reinterpret_cast<int*>(static_cast<uint8_t*>(ctx->h_pinned) + 4096) - 1;
+  CK(cudaMemcpyAsync(word, ctx->d_err, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
   CK(cudaStreamSynchronize(ctx->stream));
   CK(cudaGetLastError());
-  int err = read_scalar<int>(ctx, ctx->d_err);
+  const int err = *word;
   if (!err) return;
   clear_device_error(ctx);
   if (err & DEV_ERR_TIMEOUT) fail(SPAMM_E_TIMEOUT, "a bounded device-side wait ran out");

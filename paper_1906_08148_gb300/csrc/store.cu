@@ -16,7 +16,6 @@ namespace spamm {
 
 constexpr int kThreads = 256;
 
-void fill_iota_u32(spamm_ctx ctx, uint32_t* p, int64_t n);
 void fill_iota_i64(spamm_ctx ctx, int64_t* p, int64_t n);
 void and_u8(spamm_ctx ctx, uint8_t* a, const uint8_t* b, int64_t n);
 
@@ -97,25 +96,6 @@ void leaf_sqnorms(spamm_ctx ctx, const double* pool, const int64_t* slot, int64_
   CK_LAUNCH("leaf_sqnorm_kernel");
 }
 
-// ------------------------------------------------------------ compaction
-__global__ void keep_to_u64_kernel(const uint8_t* __restrict__ keep, int64_t n, uint64_t* __restrict__ out) {
-  for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < n; q += (int64_t)gridDim.x * blockDim.x)
-    out[q] = keep[q] ? 1u : 0u;
-}
-
-__global__ void compact_leaves_kernel(int64_t n, const uint8_t* __restrict__ keep, const uint64_t* __restrict__ pos,
-                                      const uint32_t* __restrict__ code, const double* __restrict__ sq,
-                                      const int64_t* __restrict__ slot, uint32_t* __restrict__ ocode,
-                                      double* __restrict__ osq, int64_t* __restrict__ oslot) {
-  for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < n; q += (int64_t)gridDim.x * blockDim.x) {
-    if (!keep[q]) continue;
-    int64_t p = (int64_t)pos[q];
-    ocode[p] = code[q];
-    osq[p] = sq[q];
-    oslot[p] = slot ? slot[q] : q;
-  }
-}
-
 spamm_mat new_mat(spamm_ctx ctx, int64_t n, int bs) {
   spamm_mat m = new spamm_mat_s();
   m->ctx = ctx;
@@ -128,217 +108,26 @@ spamm_mat new_mat(spamm_ctx ctx, int64_t n, int bs) {
 
 void set_leaves_compacted(spamm_mat m, int64_t ncand, const uint32_t* code, const double* sq, const int64_t* slot,
                           const uint8_t* keep) {
-  spamm_ctx ctx = m->ctx;
-  Level& leaf = m->lv[m->L];
   if (ncand <= 0) {
     m->nleaves = 0;
-    leaf.count = 0;
-    build_tree(m);
     return;
   }
-  BufP flags = alloc_n<uint64_t>(ctx, ncand), pos = alloc_n<uint64_t>(ctx, ncand), tot = alloc_n<uint64_t>(ctx, 1);
-  keep_to_u64_kernel<<<grid_for(ctx, ncand, kThreads), kThreads, 0, ctx->stream>>>(keep, ncand, P<uint64_t>(flags));
-  CK_LAUNCH("keep_to_u64_kernel");
-  scan_exclusive_u64(ctx, P<uint64_t>(flags), P<uint64_t>(pos), ncand, P<uint64_t>(tot));
-  int64_t cnt = (int64_t)read_scalar<uint64_t>(ctx, P<uint64_t>(tot));
-  leaf.count = cnt;
-  m->nleaves = cnt;
-  leaf.code = alloc_n<uint32_t>(ctx, cnt);
-  leaf.sq = alloc_n<double>(ctx, cnt);
-  m->slot = alloc_n<int64_t>(ctx, cnt);
-  if (cnt > 0) {
-    compact_leaves_kernel<<<grid_for(ctx, ncand, kThreads), kThreads, 0, ctx->stream>>>(
-        ncand, keep, P<uint64_t>(pos), code, sq, slot, P<uint32_t>(leaf.code), P<double>(leaf.sq),
-        P<int64_t>(m->slot));
-    CK_LAUNCH("compact_leaves_kernel");
-  }
-  build_tree(m);
-}
-
-// ----------------------------------------------------- parents (Section 2)
-// ||A^t||_F^2 = sum of the four children's squared norms, added in the fixed
-// order (0,0), (0,1), (1,0), (1,1); children are found from the sorted codes
-// of the level below (parent code = child code >> 2).
-// The level below holds *dn nodes (the arrays have room for ncap); flags past
-// *dn are 0 so that a scan over the capacity gives the parent count.
-__global__ void parent_flags_kernel(const uint32_t* __restrict__ code, int64_t ncap, const uint64_t* __restrict__ dn,
-                                    uint64_t* __restrict__ flags) {
-  const int64_t n = (int64_t)*dn;
-  for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < ncap; q += (int64_t)gridDim.x * blockDim.x)
-    flags[q] = q < n && (q == 0 || (code[q] >> 2) != (code[q - 1] >> 2)) ? 1u : 0u;
-}
-
-__global__ void parent_link_kernel(const uint32_t* __restrict__ code, const uint64_t* __restrict__ dn,
-                                   const uint64_t* __restrict__ flags, const uint64_t* __restrict__ excl,
-                                   uint32_t* __restrict__ pcode, int4* __restrict__ pchild) {
-  const int64_t n = (int64_t)*dn;
-  for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < n; q += (int64_t)gridDim.x * blockDim.x) {
-    int64_t p = (int64_t)(excl[q] + flags[q]) - 1;
-    uint32_t c = code[q];
-    if (flags[q]) pcode[p] = c >> 2;
-    reinterpret_cast<int*>(pchild + p)[c & 3u] = (int)q;
-  }
-}
-
-__global__ void parent_sum_kernel(int64_t np, const int4* __restrict__ child, const double* __restrict__ csq,
-                                  double* __restrict__ psq) {
-  for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < np; p += (int64_t)gridDim.x * blockDim.x) {
-    int4 ch = child[p];
-    double s = 0.0;
-    if (ch.x >= 0) s += csq[ch.x];
-    if (ch.y >= 0) s += csq[ch.y];
-    if (ch.z >= 0) s += csq[ch.z];
-    if (ch.w >= 0) s += csq[ch.w];
-    psq[p] = s;
-  }
-}
-
-// Node counts stay on the device while the levels are built (each level's
-// arrays sized by an upper bound: no more parents than children, and no more
-// than the level's grid); one read-back at the end gives the exact counts.
-void build_skeleton(spamm_mat m) {
-  spamm_ctx ctx = m->ctx;
-  const int L = m->L;
-  if (L == 0) return;
-  BufP dcnt = alloc_n<uint64_t>(ctx, L + 1);
-  uint64_t* d = P<uint64_t>(dcnt);
-  const uint64_t nleaf = (uint64_t)m->lv[L].count;
-  CK(cudaMemcpyAsync(d + L, &nleaf, sizeof(uint64_t), cudaMemcpyHostToDevice, ctx->stream));
-  std::vector<BufP> keep;  // scan buffers live until the counts are read
-  int64_t ncap = m->lv[L].count;
-  int top = L;  // lowest level index built
-  for (int t = L; t >= 1 && ncap > 0; --t) {
-    Level& ch = m->lv[t];
-    Level& pa = m->lv[t - 1];
-    const int64_t grid_nodes = (int64_t)1 << (2 * (t - 1));
-    const int64_t pcap = ncap < grid_nodes ? ncap : grid_nodes;
-    BufP flags = alloc_n<uint64_t>(ctx, ncap), excl = alloc_n<uint64_t>(ctx, ncap);
-    parent_flags_kernel<<<grid_for(ctx, ncap, kThreads), kThreads, 0, ctx->stream>>>(P<uint32_t>(ch.code), ncap,
-                                                                                    d + t, P<uint64_t>(flags));
-    CK_LAUNCH("parent_flags_kernel");
-    scan_exclusive_u64(ctx, P<uint64_t>(flags), P<uint64_t>(excl), ncap, d + t - 1);
-    pa.code = alloc_n<uint32_t>(ctx, pcap);
-    pa.sq.reset();
-    pa.child = alloc_n<int4>(ctx, pcap);
-    CK(cudaMemsetAsync(P<int4>(pa.child), 0xFF, pcap * sizeof(int4), ctx->stream));
-    parent_link_kernel<<<grid_for(ctx, ncap, kThreads), kThreads, 0, ctx->stream>>>(
-        P<uint32_t>(ch.code), d + t, P<uint64_t>(flags), P<uint64_t>(excl), P<uint32_t>(pa.code), P<int4>(pa.child));
-    CK_LAUNCH("parent_link_kernel");
-    keep.push_back(flags);
-    keep.push_back(excl);
-    ncap = pcap;
-    top = t - 1;
-  }
-  std::vector<uint64_t> h(L + 1, 0);
-  CK(cudaMemcpyAsync(h.data(), d, (L + 1) * sizeof(uint64_t), cudaMemcpyDeviceToHost, ctx->stream));
-  CK(cudaStreamSynchronize(ctx->stream));
-  for (int t = 0; t < L; ++t) {
-    Level& pa = m->lv[t];
-    pa.count = t >= top ? (int64_t)h[t] : 0;
-    if (pa.count == 0) {
-      pa.code.reset();
-      pa.sq.reset();
-      pa.child.reset();
-    }
-  }
+  TreeReq r{m, ncand, code, sq, slot, keep, 0.0};
+  tree_from_candidates(m->ctx, &r, 1);
+  tree_resolve(m->ctx, m);
 }
 
 void alloc_level_norms(spamm_mat m) {
-  for (int t = 0; t < m->L; ++t)
-    if (m->lv[t].count > 0) m->lv[t].sq = alloc_n<double>(m->ctx, m->lv[t].count);
-}
-
-void propagate_norms(spamm_mat m) {
-  spamm_ctx ctx = m->ctx;
-  for (int t = m->L; t >= 1; --t) {
-    const Level& ch = m->lv[t];
-    const Level& pa = m->lv[t - 1];
-    if (pa.count == 0) continue;
-    parent_sum_kernel<<<grid_for(ctx, pa.count, kThreads), kThreads, 0, ctx->stream>>>(
-        pa.count, P<int4>(pa.child), P<double>(ch.sq), P<double>(pa.sq));
-    CK_LAUNCH("parent_sum_kernel");
+  auto up = [](size_t b) { return (b + 255) & ~(size_t)255; };
+  size_t bytes = 0;
+  for (int t = 0; t < m->L; ++t) bytes += up(m->lv[t].count * sizeof(double));
+  if (bytes == 0) return;
+  BufP arena = alloc_bytes(m->ctx, bytes);
+  size_t at = 0;
+  for (int t = 0; t < m->L; ++t) {
+    m->lv[t].sq = sub_buf(arena, at, m->lv[t].count * sizeof(double));
+    at += up(m->lv[t].count * sizeof(double));
   }
-}
-
-// Parent norms of several matrices, one launch per height above the leaves:
-// segment q of height h is one matrix's level L - h.
-struct NormSeg {
-  const int4* child;
-  const double* csq;
-  double* psq;
-};
-__global__ void parent_sum_batch_kernel(const NormSeg* __restrict__ seg, const int64_t* __restrict__ begin, int nseg,
-                                        int64_t total) {
-  for (int64_t u = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; u < total; u += (int64_t)gridDim.x * blockDim.x) {
-    int lo = 0, hi = nseg - 1;
-    while (lo < hi) {
-      const int mid = (lo + hi + 1) >> 1;
-      if (begin[mid] <= u)
-        lo = mid;
-      else
-        hi = mid - 1;
-    }
-    const NormSeg sg = seg[lo];
-    const int64_t p = u - begin[lo];
-    const int4 ch = sg.child[p];
-    double s = 0.0;
-    if (ch.x >= 0) s += sg.csq[ch.x];
-    if (ch.y >= 0) s += sg.csq[ch.y];
-    if (ch.z >= 0) s += sg.csq[ch.z];
-    if (ch.w >= 0) s += sg.csq[ch.w];
-    sg.psq[p] = s;
-  }
-}
-
-BufP norm_batch_tables(spamm_ctx ctx, const std::vector<spamm_mat>& ms, std::vector<NormBatchLevel>* levels) {
-  int H = 0;
-  for (spamm_mat m : ms) H = m->L > H ? m->L : H;
-  std::vector<NormSeg> segs;
-  std::vector<int64_t> begins;
-  levels->clear();
-  for (int h = 1; h <= H; ++h) {
-    NormBatchLevel lv;
-    lv.first = (int)segs.size();
-    int64_t tot = 0;
-    for (spamm_mat m : ms) {
-      if (m->L < h) continue;
-      const Level& pa = m->lv[m->L - h];
-      if (pa.count == 0) continue;
-      segs.push_back({P<int4>(pa.child), P<double>(m->lv[m->L - h + 1].sq), P<double>(pa.sq)});
-      begins.push_back(tot);
-      tot += pa.count;
-    }
-    lv.nseg = (int)segs.size() - lv.first;
-    lv.total = tot;
-    levels->push_back(lv);
-  }
-  // pageable sources: each copy has read them by the time it returns
-  const size_t sb = segs.size() * sizeof(NormSeg), bb = begins.size() * sizeof(int64_t);
-  BufP tab = alloc_bytes(ctx, sb + bb + 16);
-  if (!segs.empty()) {
-    CK(cudaMemcpyAsync(tab->p, segs.data(), sb, cudaMemcpyHostToDevice, ctx->stream));
-    CK(cudaMemcpyAsync(static_cast<uint8_t*>(tab->p) + sb, begins.data(), bb, cudaMemcpyHostToDevice, ctx->stream));
-  }
-  for (NormBatchLevel& lv : *levels) {
-    lv.seg = static_cast<const void*>(static_cast<const NormSeg*>(tab->p) + lv.first);
-    lv.begin = reinterpret_cast<const int64_t*>(static_cast<const uint8_t*>(tab->p) + sb) + lv.first;
-  }
-  return tab;
-}
-
-void propagate_norms_batch(spamm_ctx ctx, const std::vector<NormBatchLevel>& levels) {
-  for (const NormBatchLevel& lv : levels) {
-    if (lv.total == 0) continue;
-    parent_sum_batch_kernel<<<grid_for(ctx, lv.total, kThreads), kThreads, 0, ctx->stream>>>(
-        static_cast<const NormSeg*>(lv.seg), lv.begin, lv.nseg, lv.total);
-    CK_LAUNCH("parent_sum_batch_kernel");
-  }
-}
-
-void build_tree(spamm_mat m) {
-  build_skeleton(m);
-  alloc_level_norms(m);
-  propagate_norms(m);
 }
 
 // ----------------------------------------------------------- truncation
@@ -348,21 +137,37 @@ __global__ void block_keep_kernel(const double* __restrict__ sq, int64_t n, doub
     keep[q] = !(sqrt(sq[q]) < tau);
 }
 
-spamm_mat truncate_block(spamm_mat in, double tau, spamm_ctx on) {
-  spamm_ctx ctx = on ? on : in->ctx;
+// A view of `in` without leaves of its own yet.
+static spamm_mat view_of(spamm_ctx ctx, spamm_mat in) {
   spamm_mat out = new_mat(ctx, in->n, in->bs);
   out->symmetric = in->symmetric;
   out->pool = in->pool;
-  const int64_t n = in->nleaves;
-  BufP keep = alloc_n<uint8_t>(ctx, n);
-  if (n > 0) {
-    block_keep_kernel<<<grid_for(ctx, n, kThreads), kThreads, 0, ctx->stream>>>(P<double>(in->lv[in->L].sq), n, tau,
-                                                                               P<uint8_t>(keep));
-    CK_LAUNCH("block_keep_kernel");
-  }
-  set_leaves_compacted(out, n, P<uint32_t>(in->lv[in->L].code), P<double>(in->lv[in->L].sq), P<int64_t>(in->slot),
-                       P<uint8_t>(keep));
   return out;
+}
+static TreeReq block_request(spamm_mat out, spamm_mat in, double tau) {
+  return {out, in->nleaves, P<uint32_t>(in->lv[in->L].code), P<double>(in->lv[in->L].sq), P<int64_t>(in->slot), nullptr,
+          tau};
+}
+
+spamm_mat truncate_block(spamm_mat in, double tau, spamm_ctx on) {
+  spamm_ctx ctx = on ? on : in->ctx;
+  spamm_mat out = view_of(ctx, in);
+  if (in->nleaves > 0) {
+    TreeReq r = block_request(out, in, tau);
+    tree_from_candidates(ctx, &r, 1);
+    tree_resolve(ctx, out);
+  }
+  return out;
+}
+
+void truncate_pair(spamm_ctx ctx, spamm_mat A, spamm_mat B, double tau, spamm_mat* At, spamm_mat* Bt) {
+  TreeReq r[2];
+  int k = 0;
+  *At = view_of(ctx, A);
+  *Bt = A == B ? *At : view_of(ctx, B);
+  if (A->nleaves > 0) r[k++] = block_request(*At, A, tau);
+  if (A != B && B->nleaves > 0) r[k++] = block_request(*Bt, B, tau);
+  if (k) tree_from_candidates(ctx, r, k);
 }
 
 // Error-controlled rule: drop the smallest leaves (ascending squared norm,
@@ -627,15 +432,13 @@ static spamm_mat build_from_elements(spamm_ctx ctx, int64_t n, int bs, Elem elem
   spamm_mat m = new_mat(ctx, n, bs);
   const int64_t nb = (n + bs - 1) / bs;
   const int64_t ncand = (int64_t)1 << (2 * m->L);
-  BufP sq = alloc_n<double>(ctx, ncand), keep = alloc_n<uint8_t>(ctx, ncand), code = alloc_n<uint32_t>(ctx, ncand);
+  BufP sq = alloc_n<double>(ctx, ncand), keep = alloc_n<uint8_t>(ctx, ncand);
   candidate_stats_kernel<<<grid_for(ctx, ncand, kThreads / 32), kThreads, 0, ctx->stream>>>(
       elem, ncand, bs, nb, tau, (int)rule, P<double>(sq), P<uint8_t>(keep), ctx->d_err);
   CK_LAUNCH("candidate_stats_kernel");
   sync_and_check(ctx);
   // the candidates' codes are their indices 0 .. 4^L - 1
-  uint32_t* c32 = P<uint32_t>(code);
-  fill_iota_u32(ctx, c32, ncand);
-  set_leaves_compacted(m, ncand, c32, P<double>(sq), nullptr, P<uint8_t>(keep));
+  set_leaves_compacted(m, ncand, nullptr, P<double>(sq), nullptr, P<uint8_t>(keep));
   // payload for the kept leaves, slot = leaf index
   const int64_t e = (int64_t)bs * bs;
   m->pool = alloc_n<double>(ctx, m->nleaves * e);
@@ -648,18 +451,9 @@ static spamm_mat build_from_elements(spamm_ctx ctx, int64_t n, int bs, Elem elem
   return m;
 }
 
-__global__ void iota_u32_kernel(uint32_t* p, int64_t n) {
-  for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < n; q += (int64_t)gridDim.x * blockDim.x)
-    p[q] = (uint32_t)q;
-}
 __global__ void iota_i64_kernel(int64_t* p, int64_t n) {
   for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < n; q += (int64_t)gridDim.x * blockDim.x)
     p[q] = q;
-}
-void fill_iota_u32(spamm_ctx ctx, uint32_t* p, int64_t n) {
-  if (n <= 0) return;
-  iota_u32_kernel<<<grid_for(ctx, n, kThreads), kThreads, 0, ctx->stream>>>(p, n);
-  CK_LAUNCH("iota_u32_kernel");
 }
 void fill_iota_i64(spamm_ctx ctx, int64_t* p, int64_t n) {
   if (n <= 0) return;

@@ -1,0 +1,499 @@
+// tree.cu -- quadtree structure: the leaf set kept from sorted candidates
+// (truncation, builders), the levels above it and their squared norms.
+//
+// Every level is in Morton order, so each step works on runs: the kept leaves
+// are a compaction of the candidates, and the parents of a level are its runs of
+// equal code >> 2, a parent's children being consecutive nodes.  A step is a
+// prefix count over flags; the thread that sees the first child of a run also
+// sees the others (at most three nodes further on), so it writes the parent's
+// code, child links and squared norm at once.
+//
+// Two forms.  Up to kTopNodes items one block of 1024 threads takes all steps
+// of a tree in one launch (a level of a few thousand nodes is a few microseconds
+// of latency for one block, about what a launch takes, and the host launches once
+// instead of five times per level): truncating both operands of a 4096-row lattice
+// (some 4000 leaves of 64 x 64 each, seven levels) takes 32 us instead of 360.  Larger
+// levels take two launches each, a count per tile of 2048 and the placing, where every
+// tile adds up the counts before it, until the level is small enough for the rest.
+// Node counts stay on the device; the host reads them once (tree_resolve).
+#include <cmath>
+#include <cstring>
+
+#include "internal.cuh"
+
+namespace spamm {
+
+namespace {
+
+constexpr int kTopThreads = 1024;
+constexpr int kTopPer = 4;  // items per thread and tile of the one-block form
+constexpr int64_t kTopNodes = 32768;
+constexpr int kTileThreads = 256;
+constexpr int kTilePer = 8;
+constexpr int64_t kTile = kTileThreads * kTilePer;
+// Up to this many tiles every tile adds up the counts before it itself (at most
+// four loads per thread); more are scanned first.
+constexpr int64_t kTilesSummed = 1024;
+
+// One tree to build.  rule 0: the leaf level is given (code, *dn nodes); 1: leaf
+// q is kept iff keep[q]; 2: iff !(sq[q] < smin).  Levels t0 - 1 .. 0 are built.
+struct TreeDev {
+  int64_t n = 0;                   // candidates
+  const uint32_t* code = nullptr;  // null: candidate q has code q
+  const double* sq = nullptr;
+  const int64_t* slot = nullptr;   // null: candidate q has slot q
+  const uint8_t* keep = nullptr;
+  double smin = 0.0;
+  int rule = 0;
+  int L = 0, t0 = 0;
+  uint64_t* count = nullptr;  // nodes per level
+  uint32_t* ocode[SPAMM_MAX_LEVELS] = {};
+  double* osq[SPAMM_MAX_LEVELS] = {};  // null: no norms
+  int4* ochild[SPAMM_MAX_LEVELS] = {};
+  int64_t* oslot = nullptr;
+};
+struct TreePair {
+  TreeDev t[2];
+};
+
+__device__ __forceinline__ bool kept(const TreeDev& T, int64_t q) {
+  return T.rule == 1 ? T.keep[q] != 0 : !(T.sq[q] < T.smin);
+}
+__device__ __forceinline__ void place_leaf(const TreeDev& T, int64_t q, int64_t p) {
+  T.ocode[T.L][p] = T.code ? T.code[q] : (uint32_t)q;
+  T.osq[T.L][p] = T.sq[q];
+  T.oslot[p] = T.slot ? T.slot[q] : q;
+}
+// Node q of a level of n nodes starts a parent.
+__device__ __forceinline__ bool first_child(const uint32_t* code, int64_t q) {
+  return q == 0 || (code[q] >> 2) != (code[q - 1] >> 2);
+}
+// Parent p (on level t - 1) whose first child is node q of level t (n nodes).
+// ||A^t||_F^2 = sum of the children's squared norms, added in the fixed order
+// (0,0), (0,1), (1,0), (1,1) (Section 2).
+__device__ __forceinline__ void place_parent(const TreeDev& T, int t, int64_t n, int64_t q, int64_t p) {
+  const uint32_t* code = T.ocode[t];
+  const uint32_t up = code[q] >> 2;
+  int ch[4] = {-1, -1, -1, -1};
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+    if (q + i < n) {
+      const uint32_t c = code[q + i];
+      if ((c >> 2) == up) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+          if ((c & 3u) == (uint32_t)k) ch[k] = (int)(q + i);
+      }
+    }
+  T.ocode[t - 1][p] = up;
+  T.ochild[t - 1][p] = make_int4(ch[0], ch[1], ch[2], ch[3]);
+  if (T.osq[t - 1]) {
+    const double* csq = T.osq[t];
+    double s = 0.0;
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+      if (ch[k] >= 0) s += csq[ch[k]];
+    T.osq[t - 1][p] = s;
+  }
+}
+
+// Exclusive prefix of v over the block's threads, the sum in *total.
+template <int THREADS>
+__device__ __forceinline__ uint32_t block_prefix(uint32_t v, uint32_t* total) {
+  __shared__ uint32_t ws[THREADS / 32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  uint32_t x = v;
+#pragma unroll
+  for (int off = 1; off < 32; off <<= 1) {
+    const uint32_t y = __shfl_up_sync(0xffffffffu, x, off);
+    if (lane >= off) x += y;
+  }
+  if (lane == 31) ws[warp] = x;
+  __syncthreads();
+  if (warp == 0) {
+    uint32_t w = lane < THREADS / 32 ? ws[lane] : 0;
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+      const uint32_t y = __shfl_up_sync(0xffffffffu, w, off);
+      if (lane >= off) w += y;
+    }
+    if (lane < THREADS / 32) ws[lane] = w;
+  }
+  __syncthreads();
+  const uint32_t before = warp ? ws[warp - 1] : 0;
+  *total = ws[THREADS / 32 - 1];
+  __syncthreads();
+  return before + x - v;
+}
+
+// Positions of the flagged items of [0, n), in order, by one block; returns their number.
+template <class Flag, class Place>
+__device__ __forceinline__ int64_t block_compact(int64_t n, Flag flag, Place place) {
+  int64_t base = 0;
+  for (int64_t b0 = 0; b0 < n; b0 += kTopThreads * kTopPer) {
+    const int64_t q0 = b0 + (int64_t)threadIdx.x * kTopPer;
+    unsigned f = 0;
+#pragma unroll
+    for (int i = 0; i < kTopPer; ++i)
+      if (q0 + i < n && flag(q0 + i)) f |= 1u << i;
+    uint32_t total;
+    int64_t p = base + block_prefix<kTopThreads>((uint32_t)__popc(f), &total);
+#pragma unroll
+    for (int i = 0; i < kTopPer; ++i)
+      if (f >> i & 1u) place(q0 + i, p++);
+    base += total;
+  }
+  return base;
+}
+
+// One block per tree: the leaves (rules 1, 2), then the levels t0 - 1 .. 0.
+__global__ void __launch_bounds__(kTopThreads) tree_top_kernel(const __grid_constant__ TreePair P) {
+  const TreeDev& T = P.t[blockIdx.x];
+  int64_t n;
+  if (T.rule != 0) {
+    n = block_compact(T.n, [&](int64_t q) { return kept(T, q); }, [&](int64_t q, int64_t p) { place_leaf(T, q, p); });
+    if (threadIdx.x == 0) T.count[T.L] = (uint64_t)n;
+    __syncthreads();
+  } else {
+    n = (int64_t)T.count[T.t0];
+  }
+  for (int t = T.t0; t >= 1; --t) {
+    const uint32_t* code = T.ocode[t];
+    n = block_compact(n, [&](int64_t q) { return first_child(code, q); },
+                      [&, nt = n](int64_t q, int64_t p) { place_parent(T, t, nt, q, p); });
+    if (threadIdx.x == 0) T.count[t - 1] = (uint64_t)n;
+    __syncthreads();
+  }
+}
+
+// The tiled form of one step: t = L + 1 the candidates' compaction, else the
+// parents of level t (whose node count is on the device).
+__device__ __forceinline__ unsigned tile_flags(const TreeDev& T, int t, int64_t n, int64_t q0) {
+  unsigned f = 0;
+#pragma unroll
+  for (int i = 0; i < kTilePer; ++i)
+    if (q0 + i < n && (t > T.L ? kept(T, q0 + i) : first_child(T.ocode[t], q0 + i))) f |= 1u << i;
+  return f;
+}
+
+__global__ void __launch_bounds__(kTileThreads)
+    tile_count_kernel(const __grid_constant__ TreeDev T, int t, uint64_t* __restrict__ tiles) {
+  const int64_t n = t > T.L ? T.n : (int64_t)T.count[t];
+  const unsigned f = tile_flags(T, t, n, (int64_t)blockIdx.x * kTile + (int64_t)threadIdx.x * kTilePer);
+  uint32_t total;
+  block_prefix<kTileThreads>((uint32_t)__popc(f), &total);
+  if (threadIdx.x == 0) tiles[blockIdx.x] = total;
+}
+
+// Sum of tiles[0 .. upto) by the whole block.
+__device__ __forceinline__ int64_t tiles_before(const uint64_t* __restrict__ tiles, int64_t upto) {
+  __shared__ unsigned long long s_sum;
+  if (threadIdx.x == 0) s_sum = 0;
+  __syncthreads();
+  unsigned long long v = 0;
+  for (int64_t i = threadIdx.x; i < upto; i += blockDim.x) v += tiles[i];
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+  if ((threadIdx.x & 31) == 0 && v) atomicAdd(&s_sum, v);
+  __syncthreads();
+  return (int64_t)s_sum;
+}
+
+__global__ void tile_total_kernel(const uint64_t* __restrict__ tiles, int64_t ntiles, uint64_t* __restrict__ out) {
+  const int64_t s = tiles_before(tiles, ntiles);
+  if (threadIdx.x == 0) *out = (uint64_t)s;
+}
+
+__global__ void __launch_bounds__(kTileThreads)
+    tile_place_kernel(const __grid_constant__ TreeDev T, int t, const uint64_t* __restrict__ tiles, int64_t ntiles) {
+  const int64_t n = t > T.L ? T.n : (int64_t)T.count[t];
+  const int64_t q0 = (int64_t)blockIdx.x * kTile + (int64_t)threadIdx.x * kTilePer;
+  const int64_t base = ntiles > kTilesSummed ? (int64_t)tiles[blockIdx.x] : tiles_before(tiles, blockIdx.x);
+  const unsigned f = tile_flags(T, t, n, q0);
+  uint32_t total;
+  int64_t p = base + block_prefix<kTileThreads>((uint32_t)__popc(f), &total);
+#pragma unroll
+  for (int i = 0; i < kTilePer; ++i)
+    if (f >> i & 1u) {
+      if (t > T.L)
+        place_leaf(T, q0 + i, p++);
+      else
+        place_parent(T, t, n, q0 + i, p++);
+    }
+  if (blockIdx.x == ntiles - 1 && threadIdx.x == 0) T.count[t - 1] = (uint64_t)(base + total);
+}
+
+// Smallest squared norm a leaf may have without being dropped: the least double s
+// with sqrt(s) >= tau (the rounded square root is monotone, so the block rule's
+// test !(sqrt(s) < tau) equals !(s < smin), without a square root per leaf).
+double least_kept(double tau) {
+  uint64_t lo = 0, hi = 0x7FF0000000000000ull;  // sqrt(inf) >= tau
+  while (lo < hi) {
+    const uint64_t mid = lo + (hi - lo) / 2;
+    double s;
+    memcpy(&s, &mid, sizeof s);
+    if (std::sqrt(s) >= tau)
+      hi = mid;
+    else
+      lo = mid + 1;
+  }
+  double s;
+  memcpy(&s, &lo, sizeof s);
+  return s;
+}
+
+int64_t level_cap(int64_t nleaves, int t) {
+  const int64_t grid = (int64_t)1 << (2 * t);
+  return nleaves < grid ? nleaves : grid;
+}
+
+// Storage of the levels t < L (codes, child links, norms unless `structure`),
+// and of the leaf level and slots if `leaves`, for at most n leaves, in one block.
+void alloc_levels(spamm_ctx ctx, spamm_mat m, int64_t n, bool leaves, bool structure) {
+  const int L = m->L;
+  auto up = [](size_t b) { return (b + 255) & ~(size_t)255; };
+  size_t bytes = up((L + 1) * sizeof(uint64_t));
+  for (int t = 0; t < L; ++t) {
+    const int64_t c = level_cap(n, t);
+    bytes += up(c * sizeof(uint32_t)) + up(c * sizeof(int4)) + (structure ? 0 : up(c * sizeof(double)));
+  }
+  if (leaves) bytes += up(n * sizeof(uint32_t)) + up(n * sizeof(double)) + up(n * sizeof(int64_t));
+  BufP arena = alloc_bytes(ctx, bytes);
+  size_t at = 0;
+  auto take = [&](size_t b) {
+    BufP v = sub_buf(arena, at, b);
+    at += up(b);
+    return v;
+  };
+  m->dcount = take((L + 1) * sizeof(uint64_t));
+  for (int t = 0; t < L; ++t) {
+    const int64_t c = level_cap(n, t);
+    m->lv[t].count = c;
+    m->lv[t].code = take(c * sizeof(uint32_t));
+    m->lv[t].child = take(c * sizeof(int4));
+    m->lv[t].sq = structure ? BufP() : take(c * sizeof(double));
+  }
+  if (leaves) {
+    m->lv[L].count = n;
+    m->lv[L].code = take(n * sizeof(uint32_t));
+    m->lv[L].sq = take(n * sizeof(double));
+    m->slot = take(n * sizeof(int64_t));
+  }
+}
+
+void point_at(TreeDev* T, spamm_mat m) {
+  T->L = m->L;
+  T->count = P<uint64_t>(m->dcount);
+  for (int t = 0; t <= m->L; ++t) {
+    T->ocode[t] = P<uint32_t>(m->lv[t].code);
+    T->osq[t] = P<double>(m->lv[t].sq);
+    T->ochild[t] = t < m->L ? P<int4>(m->lv[t].child) : nullptr;
+  }
+  T->oslot = P<int64_t>(m->slot);
+}
+
+// One step in tiles over at most n items.
+void tiled_step(spamm_ctx ctx, const TreeDev& T, int t, int64_t n, uint64_t* tiles) {
+  const int64_t ntiles = (n + kTile - 1) / kTile;
+  if (t <= T.L) {  // the candidates' tiles were counted before the leaf level was allocated
+    tile_count_kernel<<<(unsigned)ntiles, kTileThreads, 0, ctx->stream>>>(T, t, tiles);
+    CK_LAUNCH("tile_count_kernel");
+    if (ntiles > kTilesSummed) scan_exclusive_u64(ctx, tiles, tiles, ntiles, nullptr);
+  }
+  tile_place_kernel<<<(unsigned)ntiles, kTileThreads, 0, ctx->stream>>>(T, t, tiles, ntiles);
+  CK_LAUNCH("tile_place_kernel");
+}
+
+// The levels above level t0 (at most n nodes there), large ones in tiles; T.t0
+// is left at the level the one-block form starts from.
+void tiled_levels(spamm_ctx ctx, TreeDev* T, int64_t n) {
+  int t = T->L;
+  int64_t cap = n;
+  if (cap > kTopNodes) {
+    BufP tiles = alloc_n<uint64_t>(ctx, (cap + kTile - 1) / kTile);
+    for (; t >= 1 && cap > kTopNodes; --t, cap = level_cap(n, t)) tiled_step(ctx, *T, t, cap, P<uint64_t>(tiles));
+  }
+  T->t0 = t;
+}
+
+}  // namespace
+
+void tree_from_candidates(spamm_ctx ctx, TreeReq* req, int k) {
+  if (k > 2) fail(SPAMM_E_CUDA, "at most two trees are built at once");
+  TreePair pair;
+  BufP tiles[2];
+  bool wide[2] = {false, false};
+  uint64_t* host = static_cast<uint64_t*>(ctx->h_pinned);
+  for (int i = 0; i < k; ++i) {
+    TreeReq& r = req[i];
+    TreeDev& T = pair.t[i];
+    T.n = r.n;
+    T.code = r.code;
+    T.sq = r.sq;
+    T.slot = r.slot;
+    T.keep = r.keep;
+    T.rule = r.keep ? 1 : 2;
+    T.smin = r.keep ? 0.0 : least_kept(r.tau);
+    T.L = r.m->L;
+    T.t0 = T.L;
+    wide[i] = r.n > kTopNodes;
+    if (wide[i]) {
+      // the exact leaf count first: the leaf level may be much smaller than its candidates
+      const int64_t ntiles = (r.n + kTile - 1) / kTile;
+      tiles[i] = alloc_n<uint64_t>(ctx, ntiles);
+      BufP total = alloc_n<uint64_t>(ctx, 1);
+      tile_count_kernel<<<(unsigned)ntiles, kTileThreads, 0, ctx->stream>>>(T, T.L + 1, P<uint64_t>(tiles[i]));
+      CK_LAUNCH("tile_count_kernel");
+      if (ntiles > kTilesSummed) {
+        scan_exclusive_u64(ctx, P<uint64_t>(tiles[i]), P<uint64_t>(tiles[i]), ntiles, P<uint64_t>(total));
+      } else {
+        tile_total_kernel<<<1, 1024, 0, ctx->stream>>>(P<uint64_t>(tiles[i]), ntiles, P<uint64_t>(total));
+        CK_LAUNCH("tile_total_kernel");
+      }
+      CK(cudaMemcpyAsync(host + i, P<uint64_t>(total), sizeof(uint64_t), cudaMemcpyDeviceToHost, ctx->stream));
+    } else {
+      alloc_levels(ctx, r.m, r.n, true, false);
+      point_at(&T, r.m);
+    }
+  }
+  if (wide[0] || wide[1]) CK(cudaStreamSynchronize(ctx->stream));
+  for (int i = 0; i < k; ++i) {
+    if (!wide[i]) continue;
+    TreeDev& T = pair.t[i];
+    const int64_t n = (int64_t)host[i];
+    alloc_levels(ctx, req[i].m, n, true, false);
+    point_at(&T, req[i].m);
+    tiled_step(ctx, T, T.L + 1, T.n, P<uint64_t>(tiles[i]));
+    T.rule = 0;  // the one-block form starts above the leaves
+    tiled_levels(ctx, &T, n);
+  }
+  tree_top_kernel<<<k, kTopThreads, 0, ctx->stream>>>(pair);
+  CK_LAUNCH("tree_top_kernel");
+  for (int i = 0; i < k; ++i) req[i].m->pending = true;
+}
+
+void tree_skeleton(spamm_ctx ctx, spamm_mat m) {
+  const int64_t n = m->lv[m->L].count;
+  alloc_levels(ctx, m, n, false, true);
+  CK(cudaMemcpyAsync(P<uint64_t>(m->dcount) + m->L, &n, sizeof(uint64_t), cudaMemcpyHostToDevice, ctx->stream));
+  TreePair pair;
+  TreeDev& T = pair.t[0];
+  point_at(&T, m);
+  tiled_levels(ctx, &T, n);
+  tree_top_kernel<<<1, kTopThreads, 0, ctx->stream>>>(pair);
+  CK_LAUNCH("tree_top_kernel");
+  m->pending = true;
+}
+
+void tree_counts_async(spamm_ctx ctx, spamm_mat m, uint64_t* host) {
+  CK(cudaMemcpyAsync(host, P<uint64_t>(m->dcount), (m->L + 1) * sizeof(uint64_t), cudaMemcpyDeviceToHost, ctx->stream));
+}
+
+void tree_set_counts(spamm_mat m, const uint64_t* host) {
+  for (int t = 0; t <= m->L; ++t) {
+    m->lv[t].count = (int64_t)host[t];
+    if (host[t] == 0) {
+      m->lv[t].code.reset();
+      m->lv[t].child.reset();
+      if (t < m->L) m->lv[t].sq.reset();
+    }
+  }
+  m->nleaves = (int64_t)host[m->L];
+  m->pending = false;
+}
+
+void tree_resolve(spamm_ctx ctx, spamm_mat m) {
+  uint64_t* host = static_cast<uint64_t*>(ctx->h_pinned);
+  tree_counts_async(ctx, m, host);
+  CK(cudaStreamSynchronize(ctx->stream));
+  tree_set_counts(m, host);
+}
+
+// ------------------------------------------------------ norms of given trees
+// The parents' squared norms of an output whose structure was built at plan
+// time, from its leaves' norms up, for every tree of a batch: levels of more than
+// kTopNodes nodes one launch each (all trees), the rest by one block per tree in
+// one launch.  The additions are place_parent's.
+struct NormTree {
+  int32_t L;
+  int32_t pad;
+  int64_t count[SPAMM_MAX_LEVELS];
+  const int4* child[SPAMM_MAX_LEVELS];
+  double* sq[SPAMM_MAX_LEVELS];
+};
+
+__device__ __forceinline__ void node_norm(const NormTree& T, int t, int64_t p) {
+  const int4 ch = T.child[t][p];
+  const double* csq = T.sq[t + 1];
+  double s = 0.0;
+  if (ch.x >= 0) s += csq[ch.x];
+  if (ch.y >= 0) s += csq[ch.y];
+  if (ch.z >= 0) s += csq[ch.z];
+  if (ch.w >= 0) s += csq[ch.w];
+  T.sq[t][p] = s;
+}
+
+// Height h above the leaves of every tree that has more than kTopNodes nodes there.
+__global__ void norms_wide_kernel(const NormTree* __restrict__ tab, int ntrees, int h) {
+  for (int r = blockIdx.y; r < ntrees; r += gridDim.y) {
+    const NormTree& T = tab[r];
+    const int t = T.L - h;
+    if (t < 0 || T.count[t] <= kTopNodes) continue;
+    for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < T.count[t];
+         p += (int64_t)gridDim.x * blockDim.x)
+      node_norm(T, t, p);
+  }
+}
+
+__global__ void __launch_bounds__(kTopThreads) norms_top_kernel(const NormTree* __restrict__ tab) {
+  const NormTree& T = tab[blockIdx.x];
+  for (int t = T.L - 1; t >= 0; --t) {
+    if (T.count[t] > kTopNodes) continue;
+    for (int64_t p = threadIdx.x; p < T.count[t]; p += kTopThreads) node_norm(T, t, p);
+    __syncthreads();
+  }
+}
+
+BufP norm_tables(spamm_ctx ctx, const std::vector<spamm_mat>& ms, NormBatch* nb) {
+  std::vector<NormTree> tab(ms.size());
+  nb->ntrees = (int)ms.size();
+  nb->wide = 0;
+  nb->widest = 0;
+  for (size_t r = 0; r < ms.size(); ++r) {
+    spamm_mat m = ms[r];
+    NormTree& T = tab[r];
+    memset(&T, 0, sizeof T);
+    T.L = m->L;
+    for (int t = 0; t <= m->L; ++t) {
+      T.count[t] = m->lv[t].count;
+      T.child[t] = t < m->L ? P<int4>(m->lv[t].child) : nullptr;
+      T.sq[t] = P<double>(m->lv[t].sq);
+      if (t < m->L && T.count[t] > kTopNodes) {
+        nb->wide = nb->wide > m->L - t ? nb->wide : m->L - t;
+        nb->widest = nb->widest > T.count[t] ? nb->widest : T.count[t];
+      }
+    }
+  }
+  // a pageable source: the copy has read it by the time it returns
+  BufP d = alloc_n<NormTree>(ctx, (int64_t)tab.size());
+  CK(cudaMemcpyAsync(d->p, tab.data(), tab.size() * sizeof(NormTree), cudaMemcpyHostToDevice, ctx->stream));
+  nb->tab = d->p;
+  return d;
+}
+
+void propagate_norms(spamm_ctx ctx, const NormBatch& nb) {
+  const NormTree* tab = static_cast<const NormTree*>(nb.tab);
+  if (nb.ntrees == 0) return;
+  int64_t g = (nb.widest + 255) / 256;
+  const int64_t cap = (int64_t)ctx->num_sms * 8;
+  if (g > cap) g = cap;
+  for (int h = 1; h <= nb.wide; ++h) {
+    norms_wide_kernel<<<dim3((unsigned)g, (unsigned)(nb.ntrees < 1024 ? nb.ntrees : 1024)), 256, 0, ctx->stream>>>(
+        tab, nb.ntrees, h);
+    CK_LAUNCH("norms_wide_kernel");
+  }
+  norms_top_kernel<<<(unsigned)nb.ntrees, kTopThreads, 0, ctx->stream>>>(tab);
+  CK_LAUNCH("norms_top_kernel");
+}
+
+}  // namespace spamm
