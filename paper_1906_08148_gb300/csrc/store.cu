@@ -182,15 +182,15 @@ __global__ void sq_sort_keys_kernel(const double* __restrict__ sq, int64_t n, ui
   }
 }
 
-__global__ void sorted_sq_kernel(const uint64_t* __restrict__ keys, int64_t n, double* __restrict__ v) {
-  for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < n; q += (int64_t)gridDim.x * blockDim.x)
-    v[q] = __longlong_as_double((long long)keys[q]);
-}
-
+// Number of running sums within the budget.
 __global__ void within_budget_kernel(const double* __restrict__ csum, int64_t n, double budget,
-                                     uint64_t* __restrict__ flag) {
+                                     unsigned long long* __restrict__ count) {
+  unsigned long long c = 0;
   for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < n; q += (int64_t)gridDim.x * blockDim.x)
-    flag[q] = csum[q] <= budget ? 1u : 0u;
+    c += csum[q] <= budget ? 1u : 0u;
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) c += __shfl_xor_sync(0xffffffffu, c, off);
+  if ((threadIdx.x & 31) == 0 && c) atomicAdd(count, c);
 }
 
 // The first *ndrop leaves of the sorted order are dropped (a prefix, even if
@@ -210,20 +210,18 @@ spamm_mat truncate_error_controlled(spamm_mat in, double tau, spamm_ctx on) {
   const int64_t n = in->nleaves;
   BufP keep = alloc_n<uint8_t>(ctx, n);
   if (n > 0) {
-    BufP keys = alloc_n<uint64_t>(ctx, n), idx = alloc_n<int64_t>(ctx, n), v = alloc_n<double>(ctx, n);
-    BufP csum = alloc_n<double>(ctx, n), flag = alloc_n<uint64_t>(ctx, n), pos = alloc_n<uint64_t>(ctx, n);
+    BufP keys = alloc_n<uint64_t>(ctx, n), idx = alloc_n<int64_t>(ctx, n), csum = alloc_n<double>(ctx, n);
     BufP ndrop = alloc_n<uint64_t>(ctx, 1);
+    CK(cudaMemsetAsync(P<uint64_t>(ndrop), 0, sizeof(uint64_t), ctx->stream));
     const unsigned g = grid_for(ctx, n, kThreads);
     sq_sort_keys_kernel<<<g, kThreads, 0, ctx->stream>>>(P<double>(in->lv[in->L].sq), n, P<uint64_t>(keys),
                                                           P<int64_t>(idx));
     CK_LAUNCH("sq_sort_keys_kernel");
     radix_sort_pairs(ctx, P<uint64_t>(keys), P<int64_t>(idx), n, 64);  // stable: ties keep Morton order
-    sorted_sq_kernel<<<g, kThreads, 0, ctx->stream>>>(P<uint64_t>(keys), n, P<double>(v));
-    CK_LAUNCH("sorted_sq_kernel");
-    scan_inclusive_f64(ctx, P<double>(v), P<double>(csum), n);
-    within_budget_kernel<<<g, kThreads, 0, ctx->stream>>>(P<double>(csum), n, tau * tau, P<uint64_t>(flag));
+    scan_inclusive_f64(ctx, P<double>(keys), P<double>(csum), n);  // the sorted keys are the squared norms' bits
+    within_budget_kernel<<<g, kThreads, 0, ctx->stream>>>(P<double>(csum), n, tau * tau,
+                                                          P<unsigned long long>(ndrop));
     CK_LAUNCH("within_budget_kernel");
-    scan_exclusive_u64(ctx, P<uint64_t>(flag), P<uint64_t>(pos), n, P<uint64_t>(ndrop));
     drop_prefix_kernel<<<g, kThreads, 0, ctx->stream>>>(P<int64_t>(idx), n, P<uint64_t>(ndrop), P<uint8_t>(keep));
     CK_LAUNCH("drop_prefix_kernel");
   }
