@@ -2,7 +2,10 @@
 // beside the multiply (Section 4.4 lists addition and rescaling among the
 // leaf library's operations; density-matrix purification, Section 1, is the
 // application): alpha X + beta Y, the identity, and the trace.
+#include <cmath>
+
 #include "internal.cuh"
+#include "leafpass.cuh"
 
 namespace spamm {
 
@@ -64,22 +67,57 @@ __global__ void add_place_kernel(const uint32_t* __restrict__ xc, int64_t nx, co
 }
 
 // out = alpha x + beta y element by element, an absent side taken as 0:
-// fl(fl(alpha x) + fl(beta y)).  One block per output leaf.
-__global__ void add_payload_kernel(int64_t nout, int64_t e, double alpha, const double* __restrict__ xpool,
-                                   const int64_t* __restrict__ xslot, const int64_t* __restrict__ oxi, double beta,
-                                   const double* __restrict__ ypool, const int64_t* __restrict__ yslot,
-                                   const int64_t* __restrict__ oyi, double* __restrict__ out) {
-  for (int64_t q = blockIdx.x; q < nout; q += gridDim.x) {
+// fl(fl(alpha x) + fl(beta y)), with the leaf's norm (leafpass.cuh).  Written out that is
+// three FP64 instructions beside the norm's, which at two per clock and SM take longer
+// than the memory traffic (24 B per element).  A factor +-2^k, k >= 0, multiplies
+// exactly unless the product overflows, so one FMA rounds like the two operations
+// (an overflow, which those turn into an infinity, is found from the exponent);
+// +-1 is a sign.  The chain's 2 X - X^2 is one FMA per element.
+// FORM 0: both products rounded; 1: alpha x exact; 2: beta y exact.  UNIT: the other
+// side's factor is +-1.
+template <int FORM, bool UNIT>
+struct AddOp {
+  double alpha, beta;
+  const double *xpool, *ypool;
+  const int64_t *xslot, *oxi, *yslot, *oyi;
+  uint32_t emax_exact;  // largest biased exponent the exact factor does not overflow
+  const double2 *xs, *ys;
+  uint32_t eseen;
+  struct Raw {
+    double2 x, y;
+  };
+  __device__ __forceinline__ void begin(int64_t q, int64_t e) {
     const int64_t xi = oxi[q], yi = oyi[q];
-    const double* xs = xi >= 0 ? xpool + xslot[xi] * e : nullptr;
-    const double* ys = yi >= 0 ? ypool + yslot[yi] * e : nullptr;
-    double* d = out + q * e;
-    for (int64_t i = threadIdx.x; i < e; i += blockDim.x) {
-      const double a = xs ? __dmul_rn(alpha, xs[i]) : 0.0;
-      const double b = ys ? __dmul_rn(beta, ys[i]) : 0.0;
-      d[i] = __dadd_rn(a, b);
-    }
+    xs = xi >= 0 ? reinterpret_cast<const double2*>(xpool + xslot[xi] * e) : nullptr;
+    ys = yi >= 0 ? reinterpret_cast<const double2*>(ypool + yslot[yi] * e) : nullptr;
+    eseen = 0;
   }
+  __device__ __forceinline__ Raw read(int i) const {
+    return {xs ? __ldg(xs + i) : make_double2(0.0, 0.0), ys ? __ldg(ys + i) : make_double2(0.0, 0.0)};
+  }
+  // the factor's product of the side that is rounded first
+  __device__ __forceinline__ double times(double f, double v) const {
+    if (UNIT) return f < 0.0 ? -v : v;
+    return __dmul_rn(f, v);
+  }
+  __device__ __forceinline__ double one(double x, double y) {
+    if (FORM == 0) return __dadd_rn(xs ? times(alpha, x) : 0.0, ys ? __dmul_rn(beta, y) : 0.0);
+    const double f = FORM == 1 ? alpha : beta, v = FORM == 1 ? x : y;
+    eseen = max(eseen, (uint32_t)__double2hiint(v) & 0x7ff00000u);
+    const double other = FORM == 1 ? (ys ? times(beta, y) : 0.0) : (xs ? times(alpha, x) : 0.0);
+    if (!(FORM == 1 ? xs : ys)) return __dadd_rn(0.0, other);  // absent: +0, whatever the factor's sign
+    return __fma_rn(f, v, other);
+  }
+  __device__ __forceinline__ double2 value(const Raw& r) { return make_double2(one(r.x.x, r.y.x), one(r.x.y, r.y.y)); }
+  __device__ __forceinline__ bool overflowed() const { return FORM != 0 && (eseen >> 20) > emax_exact; }
+};
+
+// |f| = 2^k, 0 <= k <= 1023
+bool power_of_two(double f, int* k) {
+  int e = 0;
+  const double m = std::frexp(std::fabs(f), &e);
+  *k = e - 1;
+  return m == 0.5 && e >= 1;
 }
 
 // Identity leaves (i, i): ones on the diagonal rows that lie inside the matrix.
@@ -132,11 +170,26 @@ spamm_mat add_scaled(double alpha, spamm_mat X, double beta, spamm_mat Y, spamm_
     add_place_kernel<<<grid_of(ctx, nx + ny, 256), 256, 0, ctx->stream>>>(
         xc, nx, yc, ny, P<uint64_t>(ynew), P<uint64_t>(ypos), P<uint32_t>(code), P<int64_t>(oxi), P<int64_t>(oyi));
     CK_LAUNCH("add_place_kernel");
-    add_payload_kernel<<<grid_of(ctx, nout, 1), 256, 0, ctx->stream>>>(
-        nout, e, alpha, P<double>(X->pool), P<int64_t>(X->slot), P<int64_t>(oxi), beta, P<double>(Y->pool),
-        P<int64_t>(Y->slot), P<int64_t>(oyi), P<double>(out->pool));
-    CK_LAUNCH("add_payload_kernel");
-    leaf_sqnorms(ctx, P<double>(out->pool), nullptr, nout, X->bs, P<double>(sq), P<uint8_t>(nz), 1);
+    int k = 0;
+    auto pass = [&](auto op) {
+      op.alpha = alpha;
+      op.beta = beta;
+      op.xpool = P<double>(X->pool);
+      op.ypool = P<double>(Y->pool);
+      op.xslot = P<int64_t>(X->slot);
+      op.yslot = P<int64_t>(Y->slot);
+      op.oxi = P<int64_t>(oxi);
+      op.oyi = P<int64_t>(oyi);
+      op.emax_exact = (uint32_t)(2046 - k);
+      leaf_pass(ctx, op, nout, X->bs, P<double>(out->pool), P<double>(sq), P<uint8_t>(nz), 1);
+    };
+    const bool ua = std::fabs(alpha) == 1.0, ub = std::fabs(beta) == 1.0;
+    if (power_of_two(alpha, &k))
+      ub ? pass(AddOp<1, true>()) : pass(AddOp<1, false>());
+    else if (power_of_two(beta, &k))
+      ua ? pass(AddOp<2, true>()) : pass(AddOp<2, false>());
+    else
+      pass(AddOp<0, false>());
   }
   // a leaf whose sum is exactly zero is null (stored iff it has a non-zero element)
   set_leaves_compacted(out.get(), nout, P<uint32_t>(code), P<double>(sq), nullptr, P<uint8_t>(nz));

@@ -11,6 +11,7 @@
 
 #include "../../synth/decaygen.h"
 #include "internal.cuh"
+#include "leafpass.cuh"
 
 namespace spamm {
 
@@ -231,19 +232,6 @@ spamm_mat truncate_error_controlled(spamm_mat in, double tau, spamm_ctx on) {
 }
 
 // Element rule (Theorem 1): a -> 0 iff |a| < tau, into a fresh pool.
-__global__ void element_trunc_copy_kernel(const double* __restrict__ src, const int64_t* __restrict__ slot, int64_t n,
-                                          int bs, double tau, double* __restrict__ dst) {
-  const int64_t e = (int64_t)bs * bs;
-  for (int64_t q = blockIdx.x; q < n; q += gridDim.x) {
-    const double* s = src + slot[q] * e;
-    double* d = dst + q * e;
-    for (int64_t i = threadIdx.x; i < e; i += blockDim.x) {
-      double v = s[i];
-      d[i] = fabs(v) < tau ? 0.0 : v;
-    }
-  }
-}
-
 spamm_mat truncate_element(spamm_mat in, double tau) {
   spamm_ctx ctx = in->ctx;
   const int64_t n = in->nleaves, e = (int64_t)in->bs * in->bs;
@@ -252,10 +240,8 @@ spamm_mat truncate_element(spamm_mat in, double tau) {
   out->pool = alloc_n<double>(ctx, n * e);
   BufP sq = alloc_n<double>(ctx, n), nz = alloc_n<uint8_t>(ctx, n);
   if (n > 0) {
-    element_trunc_copy_kernel<<<grid_for(ctx, n, 1), kThreads, 0, ctx->stream>>>(
-        P<double>(in->pool), P<int64_t>(in->slot), n, in->bs, tau, P<double>(out->pool));
-    CK_LAUNCH("element_trunc_copy_kernel");
-    leaf_sqnorms(ctx, P<double>(out->pool), nullptr, n, in->bs, P<double>(sq), P<uint8_t>(nz), 0);
+    leaf_pass(ctx, CopyOp{P<double>(in->pool), P<int64_t>(in->slot), tau, nullptr}, n, in->bs, P<double>(out->pool),
+              P<double>(sq), P<uint8_t>(nz), 0);
   }
   set_leaves_compacted(out, n, P<uint32_t>(in->lv[in->L].code), P<double>(sq), nullptr, P<uint8_t>(nz));
   return out;
@@ -297,13 +283,15 @@ __global__ void zero_below_kernel(double* __restrict__ a, int64_t n, double tau)
     if (fabs(a[q]) < tau) a[q] = 0.0;
 }
 
-// Leaves given as a pool of `nblocks` payloads already on the device in input order.
-static spamm_mat finish_from_pool(spamm_ctx ctx, int64_t n, int bs, BufP pool, int64_t nblocks, const int32_t* d_bi,
-                                  const int32_t* d_bj, double tau, spamm_trunc_rule rule) {
+// Leaves given as `nblocks` payloads on the device in input order: at `payload`, to be
+// copied into the pool, or (null) in the pool already.
+static spamm_mat finish_from_pool(spamm_ctx ctx, int64_t n, int bs, BufP pool, const double* payload, int64_t nblocks,
+                                  const int32_t* d_bi, const int32_t* d_bj, double tau, spamm_trunc_rule rule) {
   spamm_mat m = new_mat(ctx, n, bs);
   m->pool = pool;
   const int64_t e = (int64_t)bs * bs;
-  if (rule == SPAMM_TRUNC_ELEMENT && tau > 0.0 && nblocks > 0) {
+  const bool element = rule == SPAMM_TRUNC_ELEMENT && tau > 0.0;
+  if (element && nblocks > 0 && !payload) {
     zero_below_kernel<<<grid_for(ctx, nblocks * e, kThreads), kThreads, 0, ctx->stream>>>(P<double>(pool),
                                                                                          nblocks * e, tau);
     CK_LAUNCH("zero_below_kernel");
@@ -313,7 +301,11 @@ static spamm_mat finish_from_pool(spamm_ctx ctx, int64_t n, int bs, BufP pool, i
   BufP code = alloc_n<uint32_t>(ctx, nblocks), ssq = alloc_n<double>(ctx, nblocks);
   BufP slot = alloc_n<int64_t>(ctx, nblocks), keep = alloc_n<uint8_t>(ctx, nblocks);
   if (nblocks > 0) {
-    leaf_sqnorms(ctx, P<double>(pool), nullptr, nblocks, bs, P<double>(sq), P<uint8_t>(nz), 1);
+    if (payload)
+      leaf_pass(ctx, CopyOp{payload, nullptr, element ? tau : 0.0, nullptr}, nblocks, bs, P<double>(pool), P<double>(sq),
+                P<uint8_t>(nz), 1);
+    else
+      leaf_sqnorms(ctx, P<double>(pool), nullptr, nblocks, bs, P<double>(sq), P<uint8_t>(nz), 1);
     const int64_t nb = (n + bs - 1) / bs;
     block_codes_kernel<<<grid_for(ctx, nblocks, kThreads), kThreads, 0, ctx->stream>>>(
         d_bi, d_bj, nblocks, nb, P<uint64_t>(keys), P<int64_t>(vals), ctx->d_err);
@@ -334,14 +326,24 @@ spamm_mat build_from_blocks(spamm_ctx ctx, int64_t n, int bs, int64_t nblocks, c
                             const double* payload, int on_device, double tau, spamm_trunc_rule rule) {
   const int64_t e = (int64_t)bs * bs;
   BufP pool = alloc_n<double>(ctx, nblocks * e);
-  BufP dbi = alloc_n<int32_t>(ctx, nblocks), dbj = alloc_n<int32_t>(ctx, nblocks);
+  BufP dbi, dbj;
+  if (!on_device) {
+    dbi = alloc_n<int32_t>(ctx, nblocks);
+    dbj = alloc_n<int32_t>(ctx, nblocks);
+  }
+  // leaves on the device are copied and their norms taken in one pass (which reads
+  // 16-byte pairs; a payload that starts between them is copied first)
+  const bool pass = on_device && (reinterpret_cast<uintptr_t>(payload) & 15) == 0;
   cudaMemcpyKind kind = on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
   if (nblocks > 0) {
-    CK(cudaMemcpyAsync(P<double>(pool), payload, nblocks * e * sizeof(double), kind, ctx->stream));
-    CK(cudaMemcpyAsync(P<int32_t>(dbi), bi, nblocks * sizeof(int32_t), kind, ctx->stream));
-    CK(cudaMemcpyAsync(P<int32_t>(dbj), bj, nblocks * sizeof(int32_t), kind, ctx->stream));
+    if (!pass) CK(cudaMemcpyAsync(P<double>(pool), payload, nblocks * e * sizeof(double), kind, ctx->stream));
+    if (!on_device) {
+      CK(cudaMemcpyAsync(P<int32_t>(dbi), bi, nblocks * sizeof(int32_t), kind, ctx->stream));
+      CK(cudaMemcpyAsync(P<int32_t>(dbj), bj, nblocks * sizeof(int32_t), kind, ctx->stream));
+    }
   }
-  return finish_from_pool(ctx, n, bs, pool, nblocks, P<int32_t>(dbi), P<int32_t>(dbj), tau, rule);
+  return finish_from_pool(ctx, n, bs, pool, pass ? payload : nullptr, nblocks, on_device ? bi : P<int32_t>(dbi),
+                          on_device ? bj : P<int32_t>(dbj), tau, rule);
 }
 
 // Candidate leaves in Morton order over the 2^L x 2^L grid, those inside
