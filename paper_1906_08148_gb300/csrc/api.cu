@@ -17,7 +17,6 @@ spamm_mat build_from_coo(spamm_ctx, int64_t, int64_t, const int64_t*, const int6
 void export_dense(spamm_mat, double*, int64_t, int);
 void export_blocks(spamm_mat, int32_t*, int32_t*, double*, double*, int);
 void tasks_to_ikj(spamm_mat A, const TaskList& T, int32_t* d_out);
-void fill_iota_i64(spamm_ctx ctx, int64_t* p, int64_t n);
 void gather_leaves(spamm_mat m, int64_t nq, const int32_t* bi, const int32_t* bj, double* out, int32_t* found,
                    int on_device);
 }  // namespace spamm
@@ -452,13 +451,11 @@ void fill_stats(const spamm_plan_s& p, spamm_stats* st) {
   st->ms_prep = p.ms_prep;
 }
 
-// The output of one plan (its leaves, slots, norms and quadtree levels, the
-// FP64 sub-tile partial norms) and the device view of the plan over all its
-// work units: output leaves (or their 64 x 64 sub-tiles) for the FP64 kernel,
+// The output of one plan (its leaves, slots, norms and quadtree levels) and the
+// device view of the plan over all its work units: output leaves (or their 64 x 64 sub-tiles) for the FP64 kernel,
 // quads of output leaves for the tensor-core kernel.
 struct PlanOut {
   std::unique_ptr<spamm_mat_s> C;
-  BufP part;
   PlanDev dev{};
   int64_t units = 0;
 };
@@ -490,13 +487,8 @@ PlanOut make_output(spamm_ctx ctx, const spamm_plan_s& p) {
   d.qstart = P<int64_t>(p.qstart);
   d.qsteps = P<QuadStep>(p.qsteps);
   d.cpool = P<double>(Cm->pool);
-  d.csq = P<double>(Cm->lv[Cm->L].sq);
   d.uorder = P<int64_t>(p.uorder);
   const int64_t per_leaf = p.prec == SPAMM_PREC_FP64 ? fp64_units_per_leaf(bs) : 1;
-  if (per_leaf > 1) {
-    o.part = alloc_n<double>(ctx, p.T.ngroups * per_leaf);
-    d.csq_part = P<double>(o.part);
-  }
   d.tc_bs = bs;
   o.units = p.T.ngroups == 0 ? 0
             : p.prec == SPAMM_PREC_FP64 ? p.T.ngroups * per_leaf
@@ -518,8 +510,6 @@ PlanDev slice_view(const spamm_plan_s& p, const PlanDev& d, int64_t first) {
     } else {
       v.gstart += leaf0;
       v.cpool += leaf0 * (int64_t)p.bs * p.bs;
-      v.csq += leaf0;
-      if (v.csq_part) v.csq_part += leaf0 * fp64_units_per_leaf(p.bs);
     }
   } else if (v.uorder) {
     v.uorder += first;  // units in claiming order; steps and outputs indexed by the unit itself
@@ -534,6 +524,15 @@ void launch_gemm(spamm_ctx ctx, spamm_prec prec, int bs, const BatchDev& batch) 
     gemm_fp64_batch(ctx, bs, batch);
   else
     gemm_tc_batch(ctx, prec, batch);
+}
+
+// Kernel (d): an output's leaf norms and slots (tensor forms: and its elements).
+void finish_leaves(spamm_ctx ctx, spamm_prec prec, spamm_mat C) {
+  double* sq = P<double>(C->lv[C->L].sq);
+  if (prec != SPAMM_PREC_FP64)
+    tc_finish(ctx, prec, P<double>(C->pool), C->nleaves, C->bs, sq, P<int64_t>(C->slot));
+  else
+    leaf_sqnorms(ctx, P<double>(C->pool), nullptr, C->nleaves, C->bs, sq, nullptr, 0, P<int64_t>(C->slot));
 }
 
 // One persistent launch over all plans, then every output's parent norms (one
@@ -572,12 +571,7 @@ std::vector<spamm_mat> execute_plans(spamm_ctx ctx, const std::vector<spamm_plan
     CK(cudaEventRecordWithFlags(ev.e[0], ctx->stream, evflags));
     launch_gemm(ctx, prec, bs, batch);
     CK(cudaEventRecordWithFlags(ev.e[1], ctx->stream, evflags));
-    for (int64_t r = 0; r < np; ++r)
-      if (prec != SPAMM_PREC_FP64)
-        tc_finish(ctx, prec, P<double>(outp[r]->pool), outp[r]->nleaves, bs, P<double>(outp[r]->lv[outp[r]->L].sq),
-                  P<int64_t>(outp[r]->slot));
-      else
-        fill_iota_i64(ctx, P<int64_t>(outp[r]->slot), outp[r]->nleaves);
+    for (int64_t r = 0; r < np; ++r) finish_leaves(ctx, prec, outp[r]);
     propagate_norms(ctx, norms);
     CK(cudaEventRecordWithFlags(ev.e[2], ctx->stream, evflags));
   };
@@ -660,10 +654,9 @@ spamm_status spamm_plan_info(spamm_plan p, int64_t* n_kept, int64_t* n_c_leaves,
   if (n_c_leaves) *n_c_leaves = p->T.ngroups;
   if (plan_bytes) *plan_bytes = (int64_t)held_bytes(*p);
   if (exec_bytes) {
-    // output payload, slot and squared norm per leaf, the FP64 sub-tile partial
-    // norms, the parents' norms (at most a third of the leaves), the batch tables
-    const int64_t parts = p->prec == SPAMM_PREC_FP64 && fp64_units_per_leaf(p->bs) > 1 ? fp64_units_per_leaf(p->bs) : 0;
-    *exec_bytes = p->T.ngroups * ((int64_t)p->bs * p->bs * 8 + 8 + 8 + 8 * parts) + (p->T.ngroups / 3 + 1) * 8 + 4096;
+    // output payload, slot and squared norm per leaf, the parents' norms (at
+    // most a third of the leaves), the batch tables
+    *exec_bytes = p->T.ngroups * ((int64_t)p->bs * p->bs * 8 + 8 + 8) + (p->T.ngroups / 3 + 1) * 8 + 4096;
   }
   return SPAMM_OK;
 }
@@ -822,11 +815,7 @@ spamm_status spamm_job_finish(spamm_ctx ctx, spamm_job job, spamm_mat* C, spamm_
     spamm_mat Cm = job->out.C.get();
     Events ev;
     CK(cudaEventRecord(ev.e[0], ctx->stream));
-    if (job->plan->prec != SPAMM_PREC_FP64)
-      tc_finish(ctx, job->plan->prec, P<double>(Cm->pool), Cm->nleaves, job->plan->bs, P<double>(Cm->lv[Cm->L].sq),
-                P<int64_t>(Cm->slot));
-    else
-      fill_iota_i64(ctx, P<int64_t>(Cm->slot), Cm->nleaves);
+    finish_leaves(ctx, job->plan->prec, Cm);
     NormBatch norms;
     BufP ntab = norm_tables(ctx, {Cm}, &norms);
     propagate_norms(ctx, norms);
@@ -838,7 +827,6 @@ spamm_status spamm_job_finish(spamm_ctx ctx, spamm_job job, spamm_mat* C, spamm_
       stats->ms_cnorm = elapsed_ms(ev.e[0], ev.e[1]);
       stats->n_launches = job->launches;
     }
-    job->out.part.reset();
     *C = registered(job->out.C.release());
   });
 }

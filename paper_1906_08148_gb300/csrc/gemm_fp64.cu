@@ -1,25 +1,30 @@
-// gemm_fp64.cu -- kernel (c), FP64 form, with the C-leaf norms of kernel (d)
-// fused into its epilogue.
+// gemm_fp64.cu -- kernel (c), FP64 form.
 //
 // C_ij = sum over the kept k (ascending) of A_ik B_kj (Algorithm 1, "C = AB"
 // at the lowest level, run batched over the task list as Section 4.4
-// describes).  A work unit is one output leaf, or for 128 x 128 and 256 x 256
-// leaves one 64 x 64 sub-tile of an output leaf (4 or 16 per leaf: a leaf
-// product of that size takes milliseconds on one SM, so whole leaves would
-// leave most SMs idle on small problems).  The units of every plan in a batch
-// form one work list; persistent CTAs claim them from an atomic counter (the
-// large leaves in order of decreasing kept-product count, so the last claims
-// are short).  Every output element is computed by one CTA, so there are no
-// atomics on C and the k order is fixed (results do not depend on the schedule
-// or on the batch); a sub-tile writes its partial squared norm, and a second
-// launch adds a leaf's partials in sub-tile order.  Operand panels are staged
-// in shared memory by 1-D TMA bulk copies issued by one warp, double-buffered
-// on mbarriers; the product is register-tiled DFMA (FP64 has no tcgen05 kind;
-// DFMA measures faster than the FP64 mma.sync path on this part).  A 32 x 32
-// leaf is staged whole (one copy per operand); a 64 x 64 output tile in
-// K-panels of KP = 32 (A's panel as 64 row segments of 256 bytes, B's as 32
-// rows: one copy for 64 x 64 leaves, 32 segments of 512 bytes for larger
-// ones), so three CTAs share an SM (64 KB of shared memory each).
+// describes).  A work unit is a TILE x TILE sub-tile of an output leaf.  The units
+// of every plan in a batch form one work list; persistent CTAs claim them from an
+// atomic counter (the large leaves in order of decreasing kept-product count, so
+// the last claims are short).  Every output element is computed by one CTA, so
+// there are no atomics on C and the k order is fixed: results do not depend on the
+// schedule, the tile or the batch.  The leaf norms (kernel (d)) are kernel (a) on
+// the finished leaves, in a launch of their own, so they do not depend on the
+// tile either (one FMA per element against bs per element and product here).
+//
+// Bound by the FP64 pipe (two FMAs per clock and SM): a 64 x 64 x 64 product takes an
+// SM 63 us, so what is lost is lost at the end, when some SMs still work on their
+// last units.  Tiles are 64 x 64 (32 x 32 leaves whole) where a launch holds many units
+// per SM, and a quarter of that where it does not (launch_fp64): 1744 leaves of 32 x 32
+// (26,440 products, 1.38 ms at the pipe's rate) 1.54 -> 1.44 ms; 100 leaves (932 products)
+// 94 -> 78 us.
+//
+// Operand panels are staged in shared memory by 1-D TMA bulk copies issued by one
+// warp, double-buffered on mbarriers; the product is register-tiled DFMA (FP64 has
+// no tcgen05 kind; DFMA measures faster than the FP64 mma.sync path on this part).
+// A 32 x 32 leaf is staged whole (one copy per operand); other tiles in K-panels of
+// KP = 32 (A's panel as row segments of 256 bytes, B's as 32 row segments, one copy
+// where they are contiguous), so three CTAs of 64 x 64 tiles share an SM (64 KB of
+// shared memory each).
 #include "internal.cuh"
 #include "ptx.cuh"
 
@@ -33,7 +38,7 @@ constexpr int64_t kUnitKeyMax = (int64_t)1 << 17;
 
 template <int BS, int KP, int TILE>
 __global__ void __launch_bounds__(kGemmThreads)
-    gemm_fp64_kernel(BatchDev batch, unsigned long long* __restrict__ work, int* __restrict__ err) {
+    gemm_fp64_kernel(BatchDev batch, int nq, unsigned long long* __restrict__ work, int* __restrict__ err) {
   constexpr int LEAF = BS * BS;
   constexpr int NP = BS / KP;                    // K-panels per leaf product
   constexpr int NQ = (BS / TILE) * (BS / TILE);  // work units (sub-tiles) per output leaf
@@ -47,7 +52,6 @@ __global__ void __launch_bounds__(kGemmThreads)
   __shared__ __align__(8) uint64_t bar[2];
   __shared__ int64_t s_u;
   __shared__ int s_abort;
-  __shared__ double s_red[kGemmThreads / 32];
 
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int tr = tid >> 4, tc = tid & 15;
@@ -60,17 +64,18 @@ __global__ void __launch_bounds__(kGemmThreads)
   __syncthreads();
   uint32_t phase[2] = {0u, 0u};
   uint32_t inflight = 0;  // bit s: stage s has a copy that nobody waited for
+  const int64_t nunits = batch.nunits / nq * NQ;  // the batch counts nq units per leaf
 
   for (;;) {
     if (tid == 0) s_u = (int64_t)atomicAdd(work, 1ull);
     __syncthreads();
     const int64_t u = s_u;
-    if (u >= batch.nunits || s_abort) break;
-    const int r = plan_of(batch.ubegin, batch.nplans, u);
+    if (u >= nunits || s_abort) break;
+    const int64_t leaf = u / NQ;
+    const int sub = (int)(u - leaf * NQ);
+    const int r = plan_of(batch.ubegin, batch.nplans, leaf * nq);
     const PlanDev& pl = batch.plans[r];
-    const int64_t lu = u - batch.ubegin[r];
-    const int64_t li = lu / NQ;  // leaf position in claiming order
-    const int sub = (int)(lu - li * NQ);
+    const int64_t li = leaf - batch.ubegin[r] / nq;  // leaf position in claiming order
     const int64_t g = pl.uorder ? pl.uorder[li] : li;
     const int64_t r0 = (int64_t)(sub / (BS / TILE)) * TILE, c0 = (int64_t)(sub % (BS / TILE)) * TILE;
     const int64_t q0 = pl.gstart[g], q1 = pl.gstart[g + 1];
@@ -138,28 +143,11 @@ __global__ void __launch_bounds__(kGemmThreads)
     }
     if (nsteps <= 0) inflight &= ~1u;
     if (s_abort) break;
-    // epilogue: write the output tile and its squared Frobenius norm (kernel (d))
     double* C = pl.cpool + g * LEAF + r0 * BS + c0;
-    double s2 = 0.0;
 #pragma unroll
     for (int i = 0; i < TM; ++i)
 #pragma unroll
-      for (int j = 0; j < TM; ++j) {
-        C[(tr + 16 * i) * BS + tc + 16 * j] = acc[i][j];
-        s2 = __fma_rn(acc[i][j], acc[i][j], s2);
-      }
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) s2 += __shfl_xor_sync(0xffffffffu, s2, off);
-    if (lane == 0) s_red[warp] = s2;
-    __syncthreads();
-    if (tid == 0) {
-      double t = 0.0;
-      for (int w = 0; w < kGemmThreads / 32; ++w) t += s_red[w];
-      if constexpr (NQ == 1)
-        pl.csq[g] = t;
-      else
-        pl.csq_part[g * NQ + sub] = t;
-    }
+      for (int j = 0; j < TM; ++j) C[(tr + 16 * i) * BS + tc + 16 * j] = acc[i][j];
   }
   // leave no bulk copy in flight into this CTA's shared memory
   if (tid == 0) {
@@ -169,27 +157,9 @@ __global__ void __launch_bounds__(kGemmThreads)
   __syncthreads();
 }
 
-// Squared norm of each output leaf from its sub-tiles' partials, added in
-// sub-tile order; one thread per leaf over every plan of the batch.
-__global__ void leaf_norm_from_parts_kernel(BatchDev batch, int nq) {
-  const int64_t nleaves = batch.nunits / nq;
-  for (int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; x < nleaves;
-       x += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t u = x * nq;
-    const int r = plan_of(batch.ubegin, batch.nplans, u);
-    const PlanDev& pl = batch.plans[r];
-    const int64_t li = (u - batch.ubegin[r]) / nq;  // leaf position in claiming order
-    const int64_t g = pl.uorder ? pl.uorder[li] : li;
-    double t = 0.0;
-    for (int k = 0; k < nq; ++k) t += pl.csq_part[g * nq + k];
-    pl.csq[g] = t;
-  }
-}
-
-template <int BS>
-static void launch_fp64(spamm_ctx ctx, const BatchDev& b) {
-  constexpr int KP = BS <= 32 ? BS : 32;
-  constexpr int TILE = BS <= 64 ? BS : 64;
+template <int BS, int TILE>
+static void launch_tile(spamm_ctx ctx, const BatchDev& b) {
+  constexpr int KP = 32;
   auto kern = gemm_fp64_kernel<BS, KP, TILE>;
   const size_t smem = 4 * (size_t)TILE * KP * sizeof(double);
   CK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
@@ -197,19 +167,30 @@ static void launch_fp64(spamm_ctx ctx, const BatchDev& b) {
   CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kGemmThreads, smem));
   if (per_sm < 1) per_sm = 1;
   const int sms = ctx->gemm_sm_limit > 0 ? ctx->gemm_sm_limit : ctx->num_sms;
+  const int nq = fp64_units_per_leaf(BS);
+  const int64_t units = b.nunits / nq * ((BS / TILE) * (BS / TILE));
   int64_t grid = (int64_t)sms * per_sm;
-  if (grid > b.nunits) grid = b.nunits;
+  if (grid > units) grid = units;
   unsigned long long* work = ctx->d_scratch + 8;
   CK(cudaMemsetAsync(work, 0, sizeof(unsigned long long), ctx->stream));
-  kern<<<(unsigned)grid, kGemmThreads, smem, ctx->stream>>>(b, work, ctx->d_err);
+  kern<<<(unsigned)grid, kGemmThreads, smem, ctx->stream>>>(b, nq, work, ctx->d_err);
   CK_LAUNCH("gemm_fp64_kernel");
-  constexpr int NQ = (BS / TILE) * (BS / TILE);
-  if constexpr (NQ > 1) {
-    int64_t g2 = (b.nunits / NQ + 255) / 256;
-    if (g2 > 4 * (int64_t)ctx->num_sms) g2 = 4 * (int64_t)ctx->num_sms;
-    leaf_norm_from_parts_kernel<<<(unsigned)g2, 256, 0, ctx->stream>>>(b, NQ);
-    CK_LAUNCH("leaf_norm_from_parts_kernel");
-  }
+}
+
+// 64 x 64 tiles (whole 32 x 32 leaves) for at least kUnitsPerSm of them per SM, else
+// quarters: with u equal units per SM the last ones leave SMs idle for about 1 / u of
+// the time, and a tile of a quarter reads its operands twice as often from L2, which
+// costs a per cent or two of the FP64 time (1271 leaves of 128 x 128, 33 tiles of 64 x 64
+// per SM: 20.5 ms, 99.3 % of the pipe).
+constexpr int64_t kUnitsPerSm = 24;
+template <int BS>
+static void launch_fp64(spamm_ctx ctx, const BatchDev& b) {
+  constexpr int TILE = BS <= 64 ? BS : 64;
+  const int sms = ctx->gemm_sm_limit > 0 ? ctx->gemm_sm_limit : ctx->num_sms;
+  if (b.nunits >= kUnitsPerSm * sms)
+    launch_tile<BS, TILE>(ctx, b);
+  else
+    launch_tile<BS, TILE / 2>(ctx, b);
 }
 
 int fp64_units_per_leaf(int bs) { return bs <= 64 ? 1 : (bs / 64) * (bs / 64); }

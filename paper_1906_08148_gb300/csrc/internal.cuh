@@ -182,8 +182,9 @@ spamm_mat truncate_block(spamm_mat in, double tau, spamm_ctx on = nullptr);  // 
 void truncate_pair(spamm_ctx ctx, spamm_mat A, spamm_mat B, double tau, spamm_mat* At, spamm_mat* Bt);
 spamm_mat truncate_element(spamm_mat in, double tau);
 spamm_mat truncate_error_controlled(spamm_mat in, double tau, spamm_ctx on = nullptr);
+// Kernel (a); with `slot_out` also the slots 0 .. nleaves - 1 of leaves stored in order.
 void leaf_sqnorms(spamm_ctx ctx, const double* pool, const int64_t* slot, int64_t nleaves, int bs, double* sq,
-                  uint8_t* nonzero, int check_finite);
+                  uint8_t* nonzero, int check_finite, int64_t* slot_out = nullptr);
 double error_fro(spamm_mat X, spamm_mat Y);
 double device_sum(spamm_ctx ctx, const double* in, int64_t n);  // deterministic reduction, synchronises
 
@@ -233,7 +234,7 @@ static_assert(sizeof(QuadStep) == 32, "QuadStep is two 16-byte words");
 // its work units (output leaves, or quads of output leaves for the
 // tensor-core kernel) are numbered consecutively across plans: plan r owns
 // units [ubegin[r], ubegin[r+1]).  Output leaf g of plan r is the sum over its
-// tasks of A[ta] B[tb], written to cpool + g*bs*bs with its squared norm in csq[g].
+// tasks of A[ta] B[tb], written to cpool + g*bs*bs.
 struct PlanDev {
   const int64_t* gstart;
   const int32_t* ta;
@@ -248,9 +249,7 @@ struct PlanDev {
   const int64_t* qstart;    // tensor forms: steps of quad Q are qsteps[qstart[Q] .. qstart[Q+1])
   const QuadStep* qsteps;
   double* cpool;
-  double* csq;
   const int64_t* uorder;  // unit (FP64: output leaf; tensor forms: quad or 128-leaf) at each claiming position, or null for identity
-  double* csq_part;       // FP64 form, leaves split into sub-tile units: partial squared norms [leaf][sub-tile]
   int32_t tc_bs;          // tensor forms: 64 (units are quads of output leaves) or 128 (units are output leaves)
   int64_t ufirst;         // tensor forms without uorder: unit number of this view's unit 0 (sliced execution)
 };
@@ -273,7 +272,7 @@ __device__ __forceinline__ int plan_of(const int64_t* __restrict__ ubegin, int n
   return lo;
 }
 void gemm_fp64_batch(spamm_ctx ctx, int bs, const BatchDev& b);
-// Work units per output leaf of the FP64 kernel (sub-tiles of 64 x 64 for larger leaves).
+// Work units per output leaf that FP64 plans and jobs are counted in (sub-tiles of 64 x 64 for larger leaves).
 int fp64_units_per_leaf(int bs);
 // Output leaves ordered by their number of kept products, largest first
 // (stable), for the FP64 kernel's unit claiming; an empty buffer when the

@@ -72,7 +72,7 @@ __device__ __forceinline__ void warp_leaf_sumsq(Get get, int bs, int lane, doubl
 constexpr int64_t kNormLeavesPerBlock = 8;
 __global__ void leaf_sqnorm_kernel(const double* __restrict__ pool, const int64_t* __restrict__ slot, int64_t m,
                                    int bs, double* __restrict__ sq, uint8_t* __restrict__ nonzero, int check_finite,
-                                   int* err) {
+                                   int* err, int64_t* __restrict__ slot_out) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwb = blockDim.x >> 5;
   const int64_t e = (int64_t)bs * bs;
   for (int64_t q = (int64_t)blockIdx.x * kNormLeavesPerBlock + warp; q < m; q += (int64_t)gridDim.x * nwb) {
@@ -83,17 +83,18 @@ __global__ void leaf_sqnorm_kernel(const double* __restrict__ pool, const int64_
     if (lane == 0) {
       sq[q] = s;
       if (nonzero) nonzero[q] = nz;
+      if (slot_out) slot_out[q] = q;
       if (bad && check_finite) atomicOr(err, DEV_ERR_NONFINITE);
     }
   }
 }
 
 void leaf_sqnorms(spamm_ctx ctx, const double* pool, const int64_t* slot, int64_t nleaves, int bs, double* sq,
-                  uint8_t* nonzero, int check_finite) {
+                  uint8_t* nonzero, int check_finite, int64_t* slot_out) {
   if (nleaves <= 0) return;
   const int64_t nblk = (nleaves + kNormLeavesPerBlock - 1) / kNormLeavesPerBlock;
   leaf_sqnorm_kernel<<<(unsigned)(nblk < (1ll << 30) ? nblk : (1ll << 30)), kThreads, 0, ctx->stream>>>(
-      pool, slot, nleaves, bs, sq, nonzero, check_finite, ctx->d_err);
+      pool, slot, nleaves, bs, sq, nonzero, check_finite, ctx->d_err, slot_out);
   CK_LAUNCH("leaf_sqnorm_kernel");
 }
 
