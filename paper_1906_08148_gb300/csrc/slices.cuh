@@ -49,8 +49,9 @@ SLICE_HD int slice_line_exp(int emax_line_biased, int f) { return emax_line_bias
 // exponent is emax_line (>= x's own).  x is rounded to the last digit's unit
 // (half away from zero), then split into balanced base-512 digits from the
 // last one up, so the leading digit takes what is left (|d_0| <= 256).
+// This form works on the whole 9 S bit integer in 64 bits.
 template <int S>
-SLICE_HD void slice_digits(uint64_t b, int emax_line, int32_t* d) {
+SLICE_HD void slice_digits_wide(uint64_t b, int emax_line, int32_t* d) {
   static_assert(S >= 1 && S <= 6, "the shift below needs 9 S <= 54");
   const int E = slice_biased_exp(b);
   int64_t M = 0;
@@ -69,6 +70,46 @@ SLICE_HD void slice_digits(uint64_t b, int emax_line, int32_t* d) {
     M = (M - t) >> 9;  // exact: M - t is a multiple of 512 (arithmetic shift of a two's-complement multiple)
   }
   d[0] = (int32_t)M;
+}
+
+// The balanced digit of x: its low nine bits as a number in [-256, 255].
+SLICE_HD int32_t slice_low_digit(int32_t x) { return ((x + 256) & 511) - 256; }
+
+// The same digits for S = 3 and 4, mostly in 32 bits: the split passes are bound by
+// integer instructions, and a 64-bit one is two or three.  The rounded magnitude has
+// 27 or 36 bits (the leading one included); for S = 4 its two's complement is cut into
+// the low 18 bits, which hold two digits and a carry, and the rest, which holds the
+// other two.  (m + half) >> sh is ((m >> (sh - 1)) + 1) >> 1, as sh >= 1 here.
+template <int S>
+SLICE_HD void slice_digits(uint64_t b, int emax_line, int32_t* d) {
+  if (S != 3 && S != 4) {
+    slice_digits_wide<S>(b, emax_line, d);
+    return;
+  }
+  const uint32_t hi = (uint32_t)(b >> 32);
+  const int E = (int)((hi >> 20) & 0x7FFu);
+  const int sh = 53 + emax_line - E - 9 * S;  // one less than the shift: 17 .. for S = 4, 26 .. for S = 3
+  const uint64_t m = ((uint64_t)((hi & 0xFFFFFu) | 0x100000u) << 32) | (uint32_t)b;
+  // beyond 53 the rounded value is 0 (m < 2^53), as for a zero or subnormal x
+  uint64_t mag = (E != 0 && sh <= 53) ? ((m >> sh) + 1) >> 1 : 0;
+  const bool neg = (int32_t)hi < 0;
+  if (S == 3) {
+    int32_t M = neg ? -(int32_t)mag : (int32_t)mag;
+    d[2] = slice_low_digit(M);
+    M = (M - d[2]) >> 9;
+    d[1] = slice_low_digit(M);
+    d[0] = (M - d[1]) >> 9;
+  } else {
+    if (neg) mag = 0 - mag;
+    const int32_t lo = (int32_t)((uint32_t)mag & 0x3FFFFu);  // 0 .. 2^18 - 1
+    int32_t top = (int32_t)(mag >> 18);                      // the rest, signed (|.| <= 2^18)
+    d[S - 1] = slice_low_digit(lo);
+    const int32_t l1 = (lo - d[S - 1]) >> 9;  // 0 .. 512
+    d[2] = slice_low_digit(l1);
+    top += (l1 - d[2]) >> 9;  // 0 or 1
+    d[1] = slice_low_digit(top);
+    d[0] = (top - d[1]) >> 9;
+  }
 }
 
 SLICE_HD uint32_t slice_f32_bits(float x) {
@@ -102,4 +143,19 @@ SLICE_HD uint16_t slice_bf16_bits(int32_t d, int p) {
   const float f = slice_f32_from_bits(0x4B400000u + (uint32_t)d) - 12582912.0f;
   const float v = f * slice_f32_from_bits((uint32_t)(p + 127) << 23);
   return (uint16_t)(slice_f32_bits(v) >> 16);
+}
+
+// 2^p for slice_bf16_x2, 0 for a dropped digit.
+SLICE_HD float slice_unit(int p) { return p < -126 ? 0.0f : slice_f32_from_bits((uint32_t)(p + 127) << 23); }
+
+// Two digits of one unit as BF16 values, d0 in the low half (a dropped digit may
+// come out as a zero of either sign).
+SLICE_HD uint32_t slice_bf16_x2(int32_t d0, int32_t d1, float unit) {
+  const uint32_t v0 = slice_f32_bits((slice_f32_from_bits(0x4B400000u + (uint32_t)d0) - 12582912.0f) * unit);
+  const uint32_t v1 = slice_f32_bits((slice_f32_from_bits(0x4B400000u + (uint32_t)d1) - 12582912.0f) * unit);
+#if defined(__CUDA_ARCH__)
+  return __byte_perm(v0, v1, 0x7632);
+#else
+  return (v0 >> 16) | (v1 & 0xFFFF0000u);
+#endif
 }
