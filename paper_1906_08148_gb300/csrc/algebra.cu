@@ -2,6 +2,7 @@
 // beside the multiply (Section 4.4 lists addition and rescaling among the
 // leaf library's operations; density-matrix purification, Section 1, is the
 // application): alpha X + beta Y, the identity, and the trace.
+#include <climits>
 #include <cmath>
 
 #include "internal.cuh"
@@ -81,6 +82,7 @@ struct AddOp {
   const double *xpool, *ypool;
   const int64_t *xslot, *oxi, *yslot, *oyi;
   uint32_t emax_exact;  // largest biased exponent the exact factor does not overflow
+  int flip;             // UNIT: sign bit of the other side's factor
   const double2 *xs, *ys;
   uint32_t eseen;
   struct Raw {
@@ -97,7 +99,7 @@ struct AddOp {
   }
   // the factor's product of the side that is rounded first
   __device__ __forceinline__ double times(double f, double v) const {
-    if (UNIT) return f < 0.0 ? -v : v;
+    if (UNIT) return __hiloint2double(__double2hiint(v) ^ flip, __double2loint(v));
     return __dmul_rn(f, v);
   }
   __device__ __forceinline__ double one(double x, double y) {
@@ -105,7 +107,10 @@ struct AddOp {
     const double f = FORM == 1 ? alpha : beta, v = FORM == 1 ? x : y;
     eseen = max(eseen, (uint32_t)__double2hiint(v) & 0x7ff00000u);
     const double other = FORM == 1 ? (ys ? times(beta, y) : 0.0) : (xs ? times(alpha, x) : 0.0);
-    if (!(FORM == 1 ? xs : ys)) return __dadd_rn(0.0, other);  // absent: +0, whatever the factor's sign
+    // an absent side is +0, whatever its factor's sign: +0 + other, which only turns -0
+    // into +0 (in the integer pipe: an addition here would be executed beside the FMA)
+    if (!(FORM == 1 ? xs : ys))
+      return __double2hiint(other) == INT_MIN && __double2loint(other) == 0 ? 0.0 : other;
     return __fma_rn(f, v, other);
   }
   __device__ __forceinline__ double2 value(const Raw& r) { return make_double2(one(r.x.x, r.y.x), one(r.x.y, r.y.y)); }
@@ -170,7 +175,7 @@ spamm_mat add_scaled(double alpha, spamm_mat X, double beta, spamm_mat Y, spamm_
     add_place_kernel<<<grid_of(ctx, nx + ny, 256), 256, 0, ctx->stream>>>(
         xc, nx, yc, ny, P<uint64_t>(ynew), P<uint64_t>(ypos), P<uint32_t>(code), P<int64_t>(oxi), P<int64_t>(oyi));
     CK_LAUNCH("add_place_kernel");
-    int k = 0;
+    int k = 0, flip = 0;
     auto pass = [&](auto op) {
       op.alpha = alpha;
       op.beta = beta;
@@ -181,15 +186,19 @@ spamm_mat add_scaled(double alpha, spamm_mat X, double beta, spamm_mat Y, spamm_
       op.oxi = P<int64_t>(oxi);
       op.oyi = P<int64_t>(oyi);
       op.emax_exact = (uint32_t)(2046 - k);
+      op.flip = flip;
       leaf_pass(ctx, op, nout, X->bs, P<double>(out->pool), P<double>(sq), P<uint8_t>(nz), 1);
     };
     const bool ua = std::fabs(alpha) == 1.0, ub = std::fabs(beta) == 1.0;
-    if (power_of_two(alpha, &k))
+    if (power_of_two(alpha, &k)) {
+      flip = std::signbit(beta) ? INT_MIN : 0;
       ub ? pass(AddOp<1, true>()) : pass(AddOp<1, false>());
-    else if (power_of_two(beta, &k))
+    } else if (power_of_two(beta, &k)) {
+      flip = std::signbit(alpha) ? INT_MIN : 0;
       ua ? pass(AddOp<2, true>()) : pass(AddOp<2, false>());
-    else
+    } else {
       pass(AddOp<0, false>());
+    }
   }
   // a leaf whose sum is exactly zero is null (stored iff it has a non-zero element)
   set_leaves_compacted(out.get(), nout, P<uint32_t>(code), P<double>(sq), nullptr, P<uint8_t>(nz));
