@@ -159,7 +159,8 @@ typedef struct {
   double ms_prep;        /* device time of the tensor-form operand terms and quad step list (0 for FP64) */
   int64_t n_steps;       /* leaf-GEMM steps: FP64 = n_kept; tensor forms = k steps of output quads */
   double executed_flops; /* flops the leaf-GEMM kernel executes: FP64 = kept_flops; tensor forms =
-                            n_steps x every term product over a 128 x 128 x 64 tile */
+                            n_steps x every term product over a 128 x 128 x 64 tile (BF16 splits: half
+                            of it for a step whose kept products lie in one output leaf column) */
   int64_t terms_shared;  /* tensor forms: 1 if A and B were one symmetric matrix and one set of
                             operand terms served both roles (see spamm_set_symmetric), else 0 */
 } spamm_stats;

@@ -444,7 +444,10 @@ void fill_stats(const spamm_plan_s& p, spamm_stats* st) {
   st->bs = p.bs;
   st->kept_flops = 2.0 * (double)p.bs * p.bs * p.bs * (double)p.T.ntasks;
   st->n_steps = p.prec == SPAMM_PREC_FP64 ? p.T.ntasks : p.nsteps;
-  st->executed_flops = p.prec == SPAMM_PREC_FP64 ? st->kept_flops : (double)p.nsteps * quad_step_flops(p.prec);
+  // the split forms run a step whose kept products lie in one output column at half width
+  const double half = p.bs == 64 && p.prec != SPAMM_PREC_FP16_SCALED ? 0.5 * (double)p.T.nhalf : 0.0;
+  st->executed_flops =
+      p.prec == SPAMM_PREC_FP64 ? st->kept_flops : ((double)p.nsteps - half) * quad_step_flops(p.prec);
   st->terms_shared = p.bmap ? 1 : 0;
   st->ms_truncate = p.ms_truncate;
   st->ms_tasks = p.ms_tasks;

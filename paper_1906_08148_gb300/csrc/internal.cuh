@@ -206,6 +206,7 @@ struct TaskList {
   int64_t n_kept_level[SPAMM_MAX_LEVELS] = {};
   int64_t n_borderline = 0;
   int64_t nsteps = 0;  // steps of all quads
+  int64_t nhalf = 0;   // of those, steps whose kept products lie in one output column
 };
 // The list in two parts, so that the operand terms (whose scales go into the quad
 // steps) are prepared in between.  task_begin descends and counts: T's sizes and

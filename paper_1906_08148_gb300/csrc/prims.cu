@@ -256,8 +256,8 @@ void scan_inclusive_f64(spamm_ctx ctx, const double* in, double* out, int64_t n)
 // warps, tiles and digits gives every item its place.  Up to kSortSmall items one
 // block takes all passes in one launch (16 rounds a pass); more take three launches
 // a pass: digit counts per tile, their prefix per digit, placing.  2,000,000 pairs by 32
-// bits: 0.25 ms where eight 4-bit passes, each a scan over all blocks and digits,
-// took 0.87; 10,000 pairs by 64 bits one launch instead of 64.
+// bits: 0.23 ms where eight 4-bit passes, each a scan over all blocks and digits,
+// took 0.85; 10,000 pairs by 64 bits one launch instead of 64.
 constexpr int kDigits = 256;
 constexpr int kSortThreads = 256;
 constexpr int kSortRounds = 16;                       // rounds of 32 items per warp

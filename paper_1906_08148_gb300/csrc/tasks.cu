@@ -15,17 +15,17 @@
 //   count  (warp per group) evaluate the 8 children of every pair, store an 8-bit
 //          kept mask per pair and per child output node c = 2ci + cj the number
 //          of kept pairs, packed as (count | nonempty << 36); the sums of
-//          each tile of 64 groups, and by the last block the level's totals.
+//          each tile of groups, and by the last block the level's totals.
 //   write  (block per tile) offsets from the tiles before and a prefix sum over
 //          the tile, then (warp per group) every lane takes one pair, per child
 //          group two warp ballots (k-child 0 and 1) place the kept pairs; within
 //          a child group pairs stay in parent order with k = 2K, 2K+1, so the
 //          children are again sorted by k.
-// The first steps (at most five, as long as a leaf step remains: up to 4096
+// The first steps (at most four, as long as a leaf step remains: up to 512
 // pairs each) run in one launch of one block that keeps the pairs in shared
 // memory; the records of every level's nodes are made by one launch before.  So
-// the list of a 4096-row lattice with 64-leaves, output structure included, takes five
-// launches and 0.135 ms instead of 54 and 0.33.
+// the list of a 4096-row lattice with 64-leaves, output structure included, takes seven
+// launches and 0.10 ms instead of 54 and 0.33.
 // Because a parent's squared norm is a floating-point sum of non-negative
 // children, the test is monotone down the tree and the pruned descent keeps
 // exactly the leaf pairs that pass the leaf-level test.
@@ -175,9 +175,10 @@ __device__ __forceinline__ unsigned child_mask(const NodeRec& ra, const NodeRec&
 
 // Sizes and statistics of one level, on the device.  pairs, groups: entered on this
 // level; cand, border: child pairs formed and borderline cases when it was made;
-// steps: quad steps (of the leaf level's quads, in the entry of the leaf level).
+// steps: quad steps (of the leaf level's quads, in the entry of the leaf level), half:
+// those of them whose kept pairs lie in one column of the quad.
 struct LevelInfo {
-  unsigned long long pairs, groups, cand, border, steps;
+  unsigned long long pairs, groups, cand, border, steps, half;
 };
 
 // One level step's view.
@@ -200,22 +201,31 @@ struct StepDev {
   int32_t* quad;         // leaf step: the four children of each group
 };
 
-constexpr int kTileGroups = 64;
+// Groups per tile: eight (one per warp of a block) while there are few tiles, so that
+// a level of a thousand groups still spreads over the SMs (16 blocks and 28 us with 64
+// groups per tile, n = 4096 lattice), else 64, as every tile adds up the tiles before it.
+constexpr int kFewGroups = 8, kManyGroups = 64;
+static int tile_groups(int64_t groups) { return groups <= (1 << 14) ? kFewGroups : kManyGroups; }
 
 // Number of quad steps in a pair's mask: its two child k-indices, each a step if
 // any of the four child groups keeps it.
 __device__ __forceinline__ unsigned mask_steps(unsigned m) { return ((m & 0x55u) != 0) + ((m & 0xAAu) != 0); }
+// Those of them whose kept child groups lie in one column (children 0, 2 or 1, 3).
+__device__ __forceinline__ unsigned mask_half_steps(unsigned m) {
+  return (((m & 0x11u) != 0) != ((m & 0x44u) != 0)) + (((m & 0x22u) != 0) != ((m & 0x88u) != 0));
+}
 
 template <bool LEAF>
 __global__ void __launch_bounds__(kWarpsPerBlock * 32)
-    task_count_kernel(const __grid_constant__ StepDev S, TauScreen sc, double tau, int test) {
-  __shared__ unsigned long long s_tile, s_cand, s_border;
+    task_count_kernel(const __grid_constant__ StepDev S, int tg, TauScreen sc, double tau, int test) {
+  __shared__ unsigned long long s_tile, s_cand, s_border, s_half;
   __shared__ unsigned s_steps, s_last;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int64_t G = (int64_t)S.in->groups;
-  const int64_t ntiles = (G + kTileGroups - 1) / kTileGroups;
+  const int64_t ntiles = (G + tg - 1) / tg;
   long long cand = 0, border = 0;
-  if (threadIdx.x == 0) s_cand = s_border = 0;
+  unsigned half = 0;
+  if (threadIdx.x == 0) s_cand = s_border = s_half = 0;
   for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
     if (threadIdx.x == 0) {
       s_tile = 0;
@@ -224,7 +234,7 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32)
     __syncthreads();
     uint64_t sum = 0;
     unsigned steps = 0;
-    for (int64_t g = tile * kTileGroups + warp; g < min(G, (tile + 1) * kTileGroups); g += kWarpsPerBlock) {
+    for (int64_t g = tile * tg + warp; g < min(G, (tile + 1) * tg); g += kWarpsPerBlock) {
       const int64_t q0 = S.gstart[g], q1 = S.gstart[g + 1];
       uint64_t cnt01 = 0, cnt23 = 0;  // kept pairs of the four children, two per word
       for (int64_t q = q0 + lane; q < q1; q += 32) {
@@ -234,7 +244,10 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32)
         S.mask[q] = (uint8_t)m;
         cnt01 += (uint64_t)__popc(m & 3u) | ((uint64_t)__popc((m >> 2) & 3u) << 32);
         cnt23 += (uint64_t)__popc((m >> 4) & 3u) | ((uint64_t)__popc((m >> 6) & 3u) << 32);
-        if (LEAF) steps += mask_steps(m);
+        if (LEAF) {
+          steps += mask_steps(m);
+          half += mask_half_steps(m);
+        }
       }
 #pragma unroll
       for (int off = 16; off > 0; off >>= 1) {
@@ -267,17 +280,20 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32)
   for (int off = 16; off > 0; off >>= 1) {
     cand += __shfl_xor_sync(0xffffffffu, cand, off);
     border += __shfl_xor_sync(0xffffffffu, border, off);
+    if (LEAF) half += __shfl_xor_sync(0xffffffffu, half, off);
   }
   __syncthreads();
   if (lane == 0) {
     if (cand) atomicAdd(&s_cand, (unsigned long long)cand);
     if (border) atomicAdd(&s_border, (unsigned long long)border);
+    if (half) atomicAdd(&s_half, (unsigned long long)half);
   }
   __syncthreads();
   // one atomic per block; the block that is last to finish adds up the tiles
   if (threadIdx.x == 0) {
     if (s_cand) atomicAdd(&S.out->cand, s_cand);
     if (s_border) atomicAdd(&S.out->border, s_border);
+    if (s_half) atomicAdd(&S.out->half, s_half);
     __threadfence();
     s_last = atomicAdd(S.ticket, 1u) == gridDim.x - 1;
     s_tile = 0;
@@ -340,14 +356,14 @@ __device__ __forceinline__ uint64_t block_prefix_u64(uint64_t v, uint64_t* total
 
 template <bool LEAF>
 __global__ void __launch_bounds__(kWarpsPerBlock * 32)
-    task_write_kernel(const __grid_constant__ StepDev S, const __grid_constant__ StepsDev Q) {
-  static_assert(kTileGroups * 4 == kWarpsPerBlock * 32, "one thread per child group of a tile");
-  __shared__ uint64_t s_off[kTileGroups * 4];
+    task_write_kernel(const __grid_constant__ StepDev S, int tg, const __grid_constant__ StepsDev Q) {
+  static_assert(kManyGroups * 4 == kWarpsPerBlock * 32, "at most one child group of a tile per thread");
+  __shared__ uint64_t s_off[kManyGroups * 4];
   __shared__ unsigned long long s_base, s_sbase;
-  __shared__ unsigned s_step[kTileGroups];
+  __shared__ unsigned s_step[kManyGroups];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int64_t G = (int64_t)S.in->groups;
-  const int64_t ntiles = (G + kTileGroups - 1) / kTileGroups;
+  const int64_t ntiles = (G + tg - 1) / tg;
   const bool want_steps = LEAF && Q.steps != nullptr;
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     S.gstart2[S.out->groups] = (int64_t)S.out->pairs;
@@ -370,8 +386,8 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32)
       if (v) atomicAdd(&s_base, v);
       if (w) atomicAdd(&s_sbase, w);
     }
-    const int64_t g0 = tile * kTileGroups;
-    const int64_t ge = min(G, g0 + kTileGroups);
+    const int64_t g0 = tile * tg;
+    const int64_t ge = min(G, g0 + tg);
     if (want_steps) {  // steps of each group of the tile
       for (int64_t g = g0 + warp; g < ge; g += kWarpsPerBlock) {
         unsigned n = 0;
@@ -473,10 +489,12 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32)
   }
 }
 
-// The first `steps` level steps (at most five: 8^4 pairs, 4^4 groups at the last)
-// by one block, from the root pair; the last one's pairs and groups go to memory.
-constexpr int kTopSteps = 5;
-constexpr int kTopPairs = 4096, kTopGroups = 256;
+// The first `steps` level steps (at most four: 8^3 pairs, 4^3 groups at the last)
+// by one block, from the root pair; the last one's pairs and groups go to memory.  (A
+// fifth step of up to 4096 pairs takes one SM 25 us, two tiled launches 15.)
+constexpr int kTopSteps = 4;
+constexpr int kTopThreads = 512;
+constexpr int kTopPairs = 512, kTopGroups = 64;
 struct TopDev {
   const uint64_t *nrootA, *nrootB;
   const NodeRec *recA[kTopSteps], *recB[kTopSteps];
@@ -496,10 +514,9 @@ struct TopShared {
   unsigned cand, border;
 };
 
-__global__ void __launch_bounds__(1024)
+__global__ void __launch_bounds__(kTopThreads)
     task_top_kernel(const __grid_constant__ TopDev T, int steps, TauScreen sc, double tau, int test) {
-  extern __shared__ __align__(16) unsigned char top_smem[];
-  TopShared& s = *reinterpret_cast<TopShared*>(top_smem);
+  __shared__ TopShared s;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   int Q = *T.nrootA > 0 && *T.nrootB > 0 ? 1 : 0, G = Q;  // the root pair is entered
   if (threadIdx.x == 0) {
@@ -516,7 +533,7 @@ __global__ void __launch_bounds__(1024)
     __syncthreads();
     // the children of every pair
     long long cand = 0, border = 0;
-    for (int q = threadIdx.x; q < Q; q += 1024) {
+    for (int q = threadIdx.x; q < Q; q += kTopThreads) {
       const int32_t ia = s.ta[cur][q], ib = s.tb[cur][q];
       s.mask[q] = (uint8_t)child_mask(T.recA[t][ia], T.recB[t][ib], T.normA[t] + ia, T.normB[t] + ib, sc, tau, test,
                                       false, &cand, &border);
@@ -529,7 +546,7 @@ __global__ void __launch_bounds__(1024)
     if (lane == 0 && cand) atomicAdd(&s.cand, (unsigned)cand);
     __syncthreads();
     // kept pairs of every child group
-    for (int g = warp; g < G; g += 32) {
+    for (int g = warp; g < G; g += kTopThreads / 32) {
       unsigned c01 = 0, c23 = 0;
       for (int q = (int)s.gstart[cur][g] + lane; q < (int)s.gstart[cur][g + 1]; q += 32) {
         const unsigned m = s.mask[q];
@@ -554,17 +571,17 @@ __global__ void __launch_bounds__(1024)
     if (lane == 31) s.ws[warp] = x;
     __syncthreads();
     if (warp == 0) {
-      uint32_t w = s.ws[lane];
+      uint32_t w = lane < kTopThreads / 32 ? s.ws[lane] : 0;
 #pragma unroll
       for (int o = 1; o < 32; o <<= 1) {
         const uint32_t y = __shfl_up_sync(0xffffffffu, w, o);
         if (lane >= o) w += y;
       }
-      s.ws[lane] = w;
+      if (lane < kTopThreads / 32) s.ws[lane] = w;
     }
     __syncthreads();
     const uint32_t off = x - v + (warp ? s.ws[warp - 1] : 0u);
-    const uint32_t total = s.ws[31];
+    const uint32_t total = s.ws[kTopThreads / 32 - 1];
     const int Q2 = (int)(total & 0xfffffu), G2 = (int)(total >> 20);
     if (i < 4 * G) {
       s.off[i] = off & 0xfffffu;
@@ -592,7 +609,7 @@ __global__ void __launch_bounds__(1024)
     __syncthreads();
     int32_t* ta2 = out ? T.ta : s.ta[nxt];
     int32_t* tb2 = out ? T.tb : s.tb[nxt];
-    for (int g = warp; g < G; g += 32) {
+    for (int g = warp; g < G; g += kTopThreads / 32) {
       int base[4];
 #pragma unroll
       for (int k = 0; k < 4; ++k) base[k] = (int)s.off[4 * g + k];
@@ -638,7 +655,7 @@ __global__ void root_test_kernel(const uint64_t* nA, const double* sqA, const ui
   const bool both = *nA > 0 && *nB > 0;
   const double prod = both ? __dmul_rn(sqrt(sqA[0]), sqrt(sqB[0])) : 0.0;
   const bool keep = both && (!test || prod >= tau);
-  lv[0].pairs = lv[0].groups = lv[0].steps = keep ? 1 : 0;
+  lv[0].pairs = lv[0].groups = lv[0].steps = lv[0].half = keep ? 1 : 0;
   lv[0].border = both && test && fabs(prod - tau) <= 1e-12 * tau ? 1 : 0;
 }
 __global__ void root_list_kernel(uint32_t* gcode, int64_t* gstart, int32_t* ta, int32_t* tb, int32_t* quads, StepsDev Q) {
@@ -667,8 +684,8 @@ static unsigned warps_grid(spamm_ctx ctx, int64_t items) {
   if (g > cap) g = cap;
   return (unsigned)(g < 1 ? 1 : g);
 }
-static unsigned tiles_grid(spamm_ctx ctx, int64_t groups) {
-  const int64_t g = (groups + kTileGroups - 1) / kTileGroups, cap = (int64_t)ctx->num_sms * 64;
+static unsigned tiles_grid(spamm_ctx ctx, int64_t groups, int tg) {
+  const int64_t g = (groups + tg - 1) / tg, cap = (int64_t)ctx->num_sms * 64;
   return (unsigned)(g < 1 ? 1 : (g > cap ? cap : g));
 }
 
@@ -683,7 +700,7 @@ constexpr int64_t kGroupsNoSync = 1ll << 20;
 struct TaskBuild {
   spamm_mat A = nullptr, B = nullptr;
   StepDev leaf{};         // the leaf step, counted
-  int64_t gcap = 0;       // its groups (at most)
+  int tg = kManyGroups;   // its groups per tile
   std::vector<BufP> keep; // its buffers
   LevelInfo* lv = nullptr;
 };
@@ -719,6 +736,7 @@ std::shared_ptr<TaskBuild> task_begin(spamm_mat A, spamm_mat B, double tau, int 
     T->ntasks = (int64_t)hl[L].pairs;
     T->nquads = L > 0 ? (int64_t)hl[L - 1].groups : T->ngroups;
     T->nsteps = (int64_t)hl[L].steps;
+    T->nhalf = (int64_t)hl[L].half;
   };
   if (!A->dcount || !B->dcount) {  // an operand without leaves
     finish_counts(nullptr);
@@ -807,9 +825,7 @@ std::shared_ptr<TaskBuild> task_begin(spamm_mat A, spamm_mat B, double tau, int 
     T0.tb = dtb;
     T0.gcode = dgc;
     T0.gstart = dgs;
-    const int smem = (int)sizeof(TopShared);
-    CK(cudaFuncSetAttribute(task_top_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    task_top_kernel<<<1, 1024, smem, ctx->stream>>>(T0, top, screen, tau, test_norms);
+    task_top_kernel<<<1, kTopThreads, 0, ctx->stream>>>(T0, top, screen, tau, test_norms);
     CK_LAUNCH("task_top_kernel");
     if (top == 0) {
       const int64_t h[2] = {0, 1};
@@ -819,7 +835,8 @@ std::shared_ptr<TaskBuild> task_begin(spamm_mat A, spamm_mat B, double tau, int 
   }
   for (int t = top; t < L; ++t) {
     const bool leaf = t + 1 == L;
-    const int64_t ntiles = (G + kTileGroups - 1) / kTileGroups;
+    const int tg = tile_groups(G);
+    const int64_t ntiles = (G + tg - 1) / tg;
     auto up = [](size_t b) { return (b + 255) & ~(size_t)255; };
     const size_t mb = up(Q), pb = up(4 * G * sizeof(uint64_t)), tbts = up(ntiles * sizeof(uint64_t));
     BufP work = alloc_bytes(ctx, mb + pb + tbts + ntiles * sizeof(uint32_t));
@@ -841,13 +858,15 @@ std::shared_ptr<TaskBuild> task_begin(spamm_mat A, spamm_mat B, double tau, int 
     S.tile_steps = reinterpret_cast<uint32_t*>(w + mb + pb + tbts);
     S.ticket = tickets + t;
     if (leaf)
-      task_count_kernel<true><<<tiles_grid(ctx, G), kWarpsPerBlock * 32, 0, ctx->stream>>>(S, screen, tau, test_norms);
+      task_count_kernel<true><<<tiles_grid(ctx, G, tg), kWarpsPerBlock * 32, 0, ctx->stream>>>(S, tg, screen, tau,
+                                                                                              test_norms);
     else
-      task_count_kernel<false><<<tiles_grid(ctx, G), kWarpsPerBlock * 32, 0, ctx->stream>>>(S, screen, tau, test_norms);
+      task_count_kernel<false><<<tiles_grid(ctx, G, tg), kWarpsPerBlock * 32, 0, ctx->stream>>>(S, tg, screen, tau,
+                                                                                               test_norms);
     CK_LAUNCH("task_count_kernel");
     if (leaf) {
       tb->leaf = S;
-      tb->gcap = G;
+      tb->tg = tg;
       tb->keep.push_back(ta);
       tb->keep.push_back(gc);
       tb->keep.push_back(work);
@@ -867,7 +886,7 @@ std::shared_ptr<TaskBuild> task_begin(spamm_mat A, spamm_mat B, double tau, int 
     S.tb2 = S.ta2 + Q2;
     S.gstart2 = static_cast<int64_t*>(gc2->p);
     S.gcode2 = reinterpret_cast<uint32_t*>(S.gstart2 + G2 + 1);
-    task_write_kernel<false><<<tiles_grid(ctx, G), kWarpsPerBlock * 32, 0, ctx->stream>>>(S, StepsDev{});
+    task_write_kernel<false><<<tiles_grid(ctx, G, tg), kWarpsPerBlock * 32, 0, ctx->stream>>>(S, tg, StepsDev{});
     CK_LAUNCH("task_write_kernel");
     ta = ta2;
     gc = gc2;
@@ -916,7 +935,7 @@ void task_finish(spamm_ctx ctx, TaskBuild* tb, TaskList* T, const StepExps* exps
   S.gcode2 = P<uint32_t>(T->gcode);
   S.gstart2 = P<int64_t>(T->gstart);
   S.quad = P<int32_t>(T->quads);
-  task_write_kernel<true><<<tiles_grid(ctx, T->nquads), kWarpsPerBlock * 32, 0, ctx->stream>>>(S, Q);
+  task_write_kernel<true><<<tiles_grid(ctx, T->nquads, tb->tg), kWarpsPerBlock * 32, 0, ctx->stream>>>(S, tb->tg, Q);
   CK_LAUNCH("task_write_kernel");
 }
 
