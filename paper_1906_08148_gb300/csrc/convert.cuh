@@ -33,3 +33,30 @@ CONV_HD uint64_t f32_to_f64_bits(uint32_t b) {
   const int sh = conv_clz32(m) - 8;  // moves the leading bit to position 23
   return sign | ((uint64_t)(897 - sh) << 52) | ((uint64_t)((m << sh) & 0x7fffffu) << 29);
 }
+
+// Whether f32_pair_sum_bits covers hi + lo: the larger is normal, the other zero or
+// normal and less than 2^29 times smaller, so the sum has at most 53 bits.
+CONV_HD bool f32_pair_sum_covers(uint32_t hi, uint32_t lo) {
+  const uint32_t mh = hi & 0x7fffffffu, ml = lo & 0x7fffffffu;
+  const uint32_t a = mh > ml ? mh : ml, b = mh > ml ? ml : mh;
+  return a - 0x00800000u < 0x7f000000u && (b == 0u || (b >= 0x00800000u && (a >> 23) - (b >> 23) <= 28u));
+}
+
+// hi + lo as binary64 bits, exactly, with integer operations: mantissas on the
+// smaller exponent's grid, one 64-bit addition, the leading bit moved to place.
+CONV_HD uint64_t f32_pair_sum_bits(uint32_t hi, uint32_t lo) {
+  const uint32_t mh = hi & 0x7fffffffu, ml = lo & 0x7fffffffu;
+  const uint32_t a = mh > ml ? mh : ml, b = mh > ml ? ml : mh;
+  const uint32_t sign = (mh > ml ? hi : lo) & 0x80000000u;  // equal magnitudes: 0 or twice, both of lo's sign
+  const uint32_t ea = a >> 23;
+  const uint32_t d = b ? ea - (b >> 23) : 0u;
+  const uint64_t big = (uint64_t)((a & 0x7fffffu) | 0x800000u) << d;
+  const uint32_t small = b ? (b & 0x7fffffu) | 0x800000u : 0u;
+  const uint64_t m = (int32_t)(hi ^ lo) < 0 ? big - small : big + small;
+  if (m == 0) return 0;  // exact cancellation: +0
+  const uint32_t top = (uint32_t)(m >> 32);
+  const int lz = top ? conv_clz32(top) : 32 + conv_clz32((uint32_t)m);
+  // leading bit 63 - lz of m counts 2^(63 - lz + ea - d - 150)
+  const uint32_t e = 63u - (uint32_t)lz + ea - d - 150u + 1023u;
+  return ((uint64_t)sign << 32) + ((uint64_t)(e - 1u) << 52) + (m << (lz - 11));
+}
