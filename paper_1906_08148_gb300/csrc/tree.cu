@@ -6,14 +6,15 @@
 // equal code >> 2, a parent's children being consecutive nodes.  A step is a
 // prefix count over flags; the thread that sees the first child of a run also
 // sees the others (at most three nodes further on), so it writes the parent's
-// code, child links and squared norm at once.
+// code and child links at once; the squared norms follow over the parents (an FP64
+// addition keeps a quarter SM's pipe for 64 cycles whether one lane needs it or 32).
 //
 // Two forms.  Up to kTopNodes items one block of 1024 threads takes all steps
 // of a tree in one launch (a level of a few thousand nodes is a few microseconds
 // of latency for one block, about what a launch takes, and the host launches once
 // instead of five times per level): truncating both operands of a 4096-row lattice
 // (some 4000 leaves of 64 x 64 each, seven levels) takes 32 us instead of 360.  Larger
-// levels take two launches each, a count per tile of 2048 and the placing, where every
+// levels take two launches each, a count per tile of 1024 and the placing, where every
 // tile adds up the counts before it, until the level is small enough for the rest.
 // Node counts stay on the device; the host reads them once (tree_resolve).
 #include <cmath>
@@ -27,9 +28,10 @@ namespace {
 
 constexpr int kTopThreads = 1024;
 constexpr int kTopPer = 4;  // items per thread and tile of the one-block form
-constexpr int64_t kTopNodes = 32768;
+constexpr int64_t kTopNodes = 4096;
+constexpr int64_t kBoundNodes = 32768;  // up to here the leaf level is allocated for every candidate
 constexpr int kTileThreads = 256;
-constexpr int kTilePer = 8;
+constexpr int kTilePer = 4;
 constexpr int64_t kTile = kTileThreads * kTilePer;
 // Up to this many tiles every tile adds up the counts before it itself (at most
 // four loads per thread); more are scanned first.
@@ -69,8 +71,6 @@ __device__ __forceinline__ bool first_child(const uint32_t* code, int64_t q) {
   return q == 0 || (code[q] >> 2) != (code[q - 1] >> 2);
 }
 // Parent p (on level t - 1) whose first child is node q of level t (n nodes).
-// ||A^t||_F^2 = sum of the children's squared norms, added in the fixed order
-// (0,0), (0,1), (1,0), (1,1) (Section 2).
 __device__ __forceinline__ void place_parent(const TreeDev& T, int t, int64_t n, int64_t q, int64_t p) {
   const uint32_t* code = T.ocode[t];
   const uint32_t up = code[q] >> 2;
@@ -87,13 +87,22 @@ __device__ __forceinline__ void place_parent(const TreeDev& T, int t, int64_t n,
     }
   T.ocode[t - 1][p] = up;
   T.ochild[t - 1][p] = make_int4(ch[0], ch[1], ch[2], ch[3]);
-  if (T.osq[t - 1]) {
-    const double* csq = T.osq[t];
+}
+// ||A^t||_F^2 = sum of the children's squared norms, added in the fixed order
+// (0,0), (0,1), (1,0), (1,1) (Section 2): parents p0 .. p1 - 1 of level t - 1, by the block.
+__device__ __forceinline__ void sum_parents(const TreeDev& T, int t, int64_t p0, int64_t p1) {
+  double* out = T.osq[t - 1];
+  if (!out) return;
+  const int4* child = T.ochild[t - 1];
+  const double* csq = T.osq[t];
+  for (int64_t p = p0 + threadIdx.x; p < p1; p += blockDim.x) {
+    const int4 ch = child[p];
     double s = 0.0;
-#pragma unroll
-    for (int k = 0; k < 4; ++k)
-      if (ch[k] >= 0) s += csq[ch[k]];
-    T.osq[t - 1][p] = s;
+    if (ch.x >= 0) s += csq[ch.x];
+    if (ch.y >= 0) s += csq[ch.y];
+    if (ch.z >= 0) s += csq[ch.z];
+    if (ch.w >= 0) s += csq[ch.w];
+    out[p] = s;
   }
 }
 
@@ -163,6 +172,8 @@ __global__ void __launch_bounds__(kTopThreads) tree_top_kernel(const __grid_cons
                       [&, nt = n](int64_t q, int64_t p) { place_parent(T, t, nt, q, p); });
     if (threadIdx.x == 0) T.count[t - 1] = (uint64_t)n;
     __syncthreads();
+    sum_parents(T, t, 0, n);
+    __syncthreads();
   }
 }
 
@@ -220,6 +231,10 @@ __global__ void __launch_bounds__(kTileThreads)
       else
         place_parent(T, t, n, q0 + i, p++);
     }
+  if (t <= T.L) {
+    __syncthreads();
+    sum_parents(T, t, base, base + total);
+  }
   if (blockIdx.x == ntiles - 1 && threadIdx.x == 0) T.count[t - 1] = (uint64_t)(base + total);
 }
 
@@ -322,7 +337,7 @@ void tree_from_candidates(spamm_ctx ctx, TreeReq* req, int k) {
   if (k > 2) fail(SPAMM_E_CUDA, "at most two trees are built at once");
   TreePair pair;
   BufP tiles[2];
-  bool wide[2] = {false, false};
+  bool wide[2] = {false, false}, exact[2] = {false, false};
   uint64_t* host = static_cast<uint64_t*>(ctx->h_pinned);
   for (int i = 0; i < k; ++i) {
     TreeReq& r = req[i];
@@ -337,32 +352,37 @@ void tree_from_candidates(spamm_ctx ctx, TreeReq* req, int k) {
     T.L = r.m->L;
     T.t0 = T.L;
     wide[i] = r.n > kTopNodes;
-    if (wide[i]) {
-      // the exact leaf count first: the leaf level may be much smaller than its candidates
-      const int64_t ntiles = (r.n + kTile - 1) / kTile;
-      tiles[i] = alloc_n<uint64_t>(ctx, ntiles);
-      BufP total = alloc_n<uint64_t>(ctx, 1);
-      tile_count_kernel<<<(unsigned)ntiles, kTileThreads, 0, ctx->stream>>>(T, T.L + 1, P<uint64_t>(tiles[i]));
-      CK_LAUNCH("tile_count_kernel");
-      if (ntiles > kTilesSummed) {
-        scan_exclusive_u64(ctx, P<uint64_t>(tiles[i]), P<uint64_t>(tiles[i]), ntiles, P<uint64_t>(total));
-      } else {
-        tile_total_kernel<<<1, 1024, 0, ctx->stream>>>(P<uint64_t>(tiles[i]), ntiles, P<uint64_t>(total));
-        CK_LAUNCH("tile_total_kernel");
-      }
-      CK(cudaMemcpyAsync(host + i, P<uint64_t>(total), sizeof(uint64_t), cudaMemcpyDeviceToHost, ctx->stream));
-    } else {
+    exact[i] = r.n > kBoundNodes;
+    if (!exact[i]) {
       alloc_levels(ctx, r.m, r.n, true, false);
       point_at(&T, r.m);
     }
+    if (wide[i]) {
+      const int64_t ntiles = (r.n + kTile - 1) / kTile;
+      tiles[i] = alloc_n<uint64_t>(ctx, ntiles);
+      tile_count_kernel<<<(unsigned)ntiles, kTileThreads, 0, ctx->stream>>>(T, T.L + 1, P<uint64_t>(tiles[i]));
+      CK_LAUNCH("tile_count_kernel");
+      // of many candidates the exact leaf count first: the leaf level may be much smaller
+      BufP total = exact[i] ? alloc_n<uint64_t>(ctx, 1) : BufP();
+      if (ntiles > kTilesSummed) {
+        scan_exclusive_u64(ctx, P<uint64_t>(tiles[i]), P<uint64_t>(tiles[i]), ntiles, P<uint64_t>(total));
+      } else if (exact[i]) {
+        tile_total_kernel<<<1, 1024, 0, ctx->stream>>>(P<uint64_t>(tiles[i]), ntiles, P<uint64_t>(total));
+        CK_LAUNCH("tile_total_kernel");
+      }
+      if (exact[i])
+        CK(cudaMemcpyAsync(host + i, P<uint64_t>(total), sizeof(uint64_t), cudaMemcpyDeviceToHost, ctx->stream));
+    }
   }
-  if (wide[0] || wide[1]) CK(cudaStreamSynchronize(ctx->stream));
+  if (exact[0] || exact[1]) CK(cudaStreamSynchronize(ctx->stream));
   for (int i = 0; i < k; ++i) {
     if (!wide[i]) continue;
     TreeDev& T = pair.t[i];
-    const int64_t n = (int64_t)host[i];
-    alloc_levels(ctx, req[i].m, n, true, false);
-    point_at(&T, req[i].m);
+    const int64_t n = exact[i] ? (int64_t)host[i] : T.n;
+    if (exact[i]) {
+      alloc_levels(ctx, req[i].m, n, true, false);
+      point_at(&T, req[i].m);
+    }
     tiled_step(ctx, T, T.L + 1, T.n, P<uint64_t>(tiles[i]));
     T.rule = 0;  // the one-block form starts above the leaves
     tiled_levels(ctx, &T, n);
