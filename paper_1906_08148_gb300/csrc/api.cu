@@ -85,17 +85,6 @@ double elapsed_ms(cudaEvent_t a, cudaEvent_t b) {
   return (double)ms;
 }
 
-struct Events {
-  cudaEvent_t e[6] = {};
-  Events() {
-    for (auto& x : e) CK(cudaEventCreate(&x));
-  }
-  ~Events() {
-    for (auto& x : e)
-      if (x) cudaEventDestroy(x);
-  }
-};
-
 }  // namespace
 
 extern "C" {
@@ -119,6 +108,7 @@ spamm_status spamm_create(int device, void* cuda_stream, spamm_ctx* out) {
     CK(cudaMalloc(&ctx->d_scratch, 64 * sizeof(unsigned long long)));
     CK(cudaMemset(ctx->d_scratch, 0, 64 * sizeof(unsigned long long)));
     CK(cudaMallocHost(&ctx->h_pinned, 4096));
+    for (cudaEvent_t& e : ctx->events) CK(cudaEventCreate(&e));
     // keep freed stream-ordered memory in the pool instead of returning it
     cudaMemPool_t pool;
     CK(cudaDeviceGetDefaultMemPool(&pool, device));
@@ -129,6 +119,8 @@ spamm_status spamm_create(int device, void* cuda_stream, spamm_ctx* out) {
     if (ctx->d_err) cudaFree(ctx->d_err);
     if (ctx->d_scratch) cudaFree(ctx->d_scratch);
     if (ctx->h_pinned) cudaFreeHost(ctx->h_pinned);
+    for (cudaEvent_t e : ctx->events)
+      if (e) cudaEventDestroy(e);
     delete ctx;
     return st;
   }
@@ -144,6 +136,7 @@ spamm_status spamm_destroy(spamm_ctx ctx) {
   cudaFree(ctx->d_err);
   cudaFree(ctx->d_scratch);
   cudaFreeHost(ctx->h_pinned);
+  for (cudaEvent_t e : ctx->events) cudaEventDestroy(e);
   if (ctx->graph_exec) cudaGraphExecDestroy(ctx->graph_exec);
   if (ctx->capture_stream) cudaStreamDestroy(ctx->capture_stream);
   delete ctx;
@@ -349,10 +342,28 @@ void check_form(spamm_prec prec, int bs) {
     fail(SPAMM_E_UNSUPPORTED, "tensor-core precision forms are built for bs = 64 and 128");
 }
 
+// After the wait that follows make_plan: its phases' times and the output's node
+// counts (until then the counts are upper bounds).
+void settle_plan(spamm_plan_s* p) {
+  const cudaEvent_t* ev = p->ctx->events;
+  if (p->T.ngroups > 0) {
+    spamm_mat_s sk;
+    sk.L = p->L;
+    sk.lv = p->cskel;
+    tree_set_counts(&sk, static_cast<const uint64_t*>(p->ctx->h_pinned));
+    p->cskel = sk.lv;
+  }
+  p->ms_truncate = elapsed_ms(ev[0], ev[1]);
+  p->ms_tasks = elapsed_ms(ev[1], ev[2]) + elapsed_ms(ev[3], ev[4]);
+  p->ms_prep = elapsed_ms(ev[2], ev[3]) + elapsed_ms(ev[4], ev[5]);
+}
+
+// Waits once, for the sizes of the task list; what follows is enqueued, and
+// settle_plan takes the rest over after the caller's wait.
 spamm_plan make_plan(spamm_ctx ctx, spamm_mat A, spamm_mat B, double tau, spamm_mode mode, spamm_prec prec) {
   check_pair(A, B, tau, mode);
   check_form(prec, A->bs);
-  Events ev;
+  const cudaEvent_t* ev = ctx->events;
   const unsigned long long launches0 = g_kernel_launches;
   std::unique_ptr<spamm_plan_s> p(new spamm_plan_s());
   p->ctx = ctx;
@@ -360,15 +371,15 @@ spamm_plan make_plan(spamm_ctx ctx, spamm_mat A, spamm_mat B, double tau, spamm_
   p->bs = A->bs;
   p->L = A->L;
   p->prec = prec;
-  CK(cudaEventRecord(ev.e[0], ctx->stream));
+  CK(cudaEventRecord(ev[0], ctx->stream));
   spamm_mat At = nullptr, Bt = nullptr;
   run_truncation(A, B, tau, mode, &At, &Bt, ctx);
   std::unique_ptr<spamm_mat_s> ownA(At != A ? At : nullptr), ownB((Bt != B && Bt != At) ? Bt : nullptr);
-  CK(cudaEventRecord(ev.e[1], ctx->stream));
+  CK(cudaEventRecord(ev[1], ctx->stream));
   std::shared_ptr<TaskBuild> tb = task_begin(At, Bt, tau, mode != SPAMM_MODE_TRUNCATE, ctx, &p->T);
   p->na = At->nleaves;
   p->nb = Bt->nleaves;
-  CK(cudaEventRecord(ev.e[2], ctx->stream));
+  CK(cudaEventRecord(ev[2], ctx->stream));
   const bool tensor = prec != SPAMM_PREC_FP64;
   if (tensor) {
     prep_terms(At, prec, 0, &p->termsA, &p->expA, ctx);
@@ -384,7 +395,7 @@ spamm_plan make_plan(spamm_ctx ctx, spamm_mat A, spamm_mat B, double tau, spamm_
       prep_terms(Bt, prec, 1, &p->termsB, &p->expB, ctx);
     }
   }
-  CK(cudaEventRecord(ev.e[3], ctx->stream));
+  CK(cudaEventRecord(ev[3], ctx->stream));
   {
     const StepExps exps{P<int32_t>(p->expA), P<int32_t>(p->expB), P<int32_t>(p->bmap)};
     const bool quads = tensor && p->bs == 64;
@@ -400,7 +411,7 @@ spamm_plan make_plan(spamm_ctx ctx, spamm_mat A, spamm_mat B, double tau, spamm_
     tree_skeleton(ctx, sk.get());
     tree_counts_async(ctx, sk.get(), counts);
   }
-  CK(cudaEventRecord(ev.e[4], ctx->stream));
+  CK(cudaEventRecord(ev[4], ctx->stream));
   if (!tensor) {
     p->poolA = At->pool;
     p->slotA = At->slot;
@@ -416,16 +427,10 @@ spamm_plan make_plan(spamm_ctx ctx, spamm_mat A, spamm_mat B, double tau, spamm_
     if (ctx->claim_order == SPAMM_ORDER_LONGEST_FIRST)
       p->uorder = unit_order_longest(ctx, P<int64_t>(p->qstart), p->bs == 128 ? p->T.ngroups : p->T.nquads);
   }
-  CK(cudaEventRecord(ev.e[5], ctx->stream));
-  sync_and_check(ctx);
-  if (p->T.ngroups > 0) tree_set_counts(sk.get(), counts);
+  CK(cudaEventRecord(ev[5], ctx->stream));
   p->cskel = sk->lv;
   p->cdcount = sk->dcount;
-  p->ms_truncate = elapsed_ms(ev.e[0], ev.e[1]);
-  p->ms_tasks = elapsed_ms(ev.e[1], ev.e[2]) + elapsed_ms(ev.e[3], ev.e[4]);
-  p->ms_prep = elapsed_ms(ev.e[2], ev.e[3]) + elapsed_ms(ev.e[4], ev.e[5]);
   p->launches = (int64_t)(g_kernel_launches - launches0);
-  ctx->live_handles++;
   return p.release();
 }
 
@@ -473,9 +478,7 @@ PlanOut make_output(spamm_ctx ctx, const spamm_plan_s& p) {
   Cm->dcount = p.cdcount;
   Cm->nleaves = p.T.ngroups;
   Cm->pool = alloc_n<double>(ctx, p.T.ngroups * e);
-  Cm->slot = alloc_n<int64_t>(ctx, p.T.ngroups);
-  Cm->lv[Cm->L].sq = alloc_n<double>(ctx, p.T.ngroups);
-  alloc_level_norms(Cm);
+  alloc_norms(Cm);
   PlanDev& d = o.dev;
   d.gstart = P<int64_t>(p.T.gstart);
   d.ta = P<int32_t>(p.T.ta);
@@ -538,10 +541,31 @@ void finish_leaves(spamm_ctx ctx, spamm_prec prec, spamm_mat C) {
     leaf_sqnorms(ctx, P<double>(C->pool), nullptr, C->nleaves, C->bs, sq, nullptr, 0, P<int64_t>(C->slot));
 }
 
-// One persistent launch over all plans, then every output's parent norms (one
-// launch per level for the whole batch).  Buffers are allocated and the plan
-// table uploaded first, so the launch sequence has no host synchronisation;
-// with ctx->exec_graph it is captured and run as one CUDA graph.
+// The tables of a launch in one upload: the plans' views, the first unit of each (units
+// numbered consecutively), and the norm tables of `norm_mats`.
+template <class View, class Units>
+BatchDev upload_batch(spamm_ctx ctx, int64_t np, View view, Units units, const std::vector<spamm_mat>& norm_mats,
+                      NormBatch* norms, BufP* tables) {
+  const size_t pb = np * sizeof(PlanDev), ub = (np + 1) * sizeof(int64_t), nb = norm_table_bytes(norm_mats.size());
+  std::vector<uint8_t> host(pb + ub + nb);
+  *tables = alloc_bytes(ctx, host.size());
+  uint8_t* dev = static_cast<uint8_t*>((*tables)->p);
+  PlanDev* hp = reinterpret_cast<PlanDev*>(host.data());
+  int64_t* hu = reinterpret_cast<int64_t*>(host.data() + pb);
+  hu[0] = 0;
+  for (int64_t r = 0; r < np; ++r) {
+    hp[r] = view(r);
+    hu[r + 1] = hu[r] + units(r);
+  }
+  if (norms) norm_tables(norm_mats, host.data() + pb + ub, dev + pb + ub, norms);
+  // a pageable source: the copy has read it by the time it returns
+  CK(cudaMemcpyAsync(dev, host.data(), host.size(), cudaMemcpyHostToDevice, ctx->stream));
+  return BatchDev{reinterpret_cast<const PlanDev*>(dev), reinterpret_cast<const int64_t*>(dev + pb), (int)np, hu[np]};
+}
+
+// One persistent launch over all plans, then every output's norms.  Buffers are
+// allocated and the tables uploaded first, so the launch sequence has no host
+// synchronisation; with ctx->exec_graph it is captured and run as one CUDA graph.
 std::vector<spamm_mat> execute_plans(spamm_ctx ctx, const std::vector<spamm_plan>& plans, double* ms_gemm,
                                      double* ms_cnorm, int64_t* launches) {
   const int64_t np = (int64_t)plans.size();
@@ -550,33 +574,26 @@ std::vector<spamm_mat> execute_plans(spamm_ctx ctx, const std::vector<spamm_plan
   for (spamm_plan p : plans)
     if (p->ctx->device != ctx->device || p->prec != prec || p->bs != bs)
       fail(SPAMM_E_INVALID_ARG, "a batch needs one device, one precision form and one leaf size");
-  Events ev;
+  const cudaEvent_t* ev = ctx->events + 6;
   const unsigned long long launches0 = g_kernel_launches;
   std::vector<PlanOut> pout;
   std::vector<spamm_mat> outp;
-  std::vector<PlanDev> host(np);
-  std::vector<int64_t> ubegin(np + 1, 0);
   for (int64_t r = 0; r < np; ++r) {
     pout.push_back(make_output(ctx, *plans[r]));
     outp.push_back(pout.back().C.get());
-    host[r] = pout.back().dev;
-    ubegin[r + 1] = ubegin[r] + pout.back().units;
   }
-  BufP dplans = alloc_n<PlanDev>(ctx, np), dub = alloc_n<int64_t>(ctx, np + 1);
-  CK(cudaMemcpyAsync(P<PlanDev>(dplans), host.data(), np * sizeof(PlanDev), cudaMemcpyHostToDevice, ctx->stream));
-  CK(cudaMemcpyAsync(P<int64_t>(dub), ubegin.data(), (np + 1) * sizeof(int64_t), cudaMemcpyHostToDevice,
-                     ctx->stream));
   NormBatch norms;
-  BufP ntab = norm_tables(ctx, outp, &norms);
-  BatchDev batch{P<PlanDev>(dplans), P<int64_t>(dub), (int)np, ubegin[np]};
+  BufP tables;
+  const BatchDev batch = upload_batch(
+      ctx, np, [&](int64_t r) { return pout[r].dev; }, [&](int64_t r) { return pout[r].units; }, outp, &norms, &tables);
 
   auto sequence = [&](unsigned evflags) {
-    CK(cudaEventRecordWithFlags(ev.e[0], ctx->stream, evflags));
+    CK(cudaEventRecordWithFlags(ev[0], ctx->stream, evflags));
     launch_gemm(ctx, prec, bs, batch);
-    CK(cudaEventRecordWithFlags(ev.e[1], ctx->stream, evflags));
+    CK(cudaEventRecordWithFlags(ev[1], ctx->stream, evflags));
     for (int64_t r = 0; r < np; ++r) finish_leaves(ctx, prec, outp[r]);
     propagate_norms(ctx, norms);
-    CK(cudaEventRecordWithFlags(ev.e[2], ctx->stream, evflags));
+    CK(cudaEventRecordWithFlags(ev[2], ctx->stream, evflags));
   };
   if (ctx->exec_graph) {
     // capture on the context's capture stream (the legacy stream cannot be captured), run on its stream
@@ -631,8 +648,8 @@ std::vector<spamm_mat> execute_plans(spamm_ctx ctx, const std::vector<spamm_plan
     sequence(cudaEventRecordDefault);
   }
   sync_and_check(ctx);
-  *ms_gemm = elapsed_ms(ev.e[0], ev.e[1]);
-  *ms_cnorm = elapsed_ms(ev.e[1], ev.e[2]);
+  *ms_gemm = elapsed_ms(ev[0], ev[1]);
+  *ms_cnorm = elapsed_ms(ev[1], ev[2]);
   *launches = (int64_t)(g_kernel_launches - launches0);
   std::vector<spamm_mat> res;
   for (auto& o : pout) res.push_back(o.C.release());
@@ -647,7 +664,13 @@ spamm_status spamm_plan_create(spamm_ctx ctx, spamm_mat A, spamm_mat B, double t
                                spamm_plan* out) {
   if (!ctx || !A || !B || !out) return SPAMM_E_INVALID_ARG;
   *out = nullptr;
-  return guarded(ctx, [&] { *out = make_plan(ctx, A, B, tau, mode, prec); });
+  return guarded(ctx, [&] {
+    std::unique_ptr<spamm_plan_s> p(make_plan(ctx, A, B, tau, mode, prec));
+    sync_and_check(ctx);
+    settle_plan(p.get());
+    ctx->live_handles++;
+    *out = p.release();
+  });
 }
 
 spamm_status spamm_plan_info(spamm_plan p, int64_t* n_kept, int64_t* n_c_leaves, int64_t* plan_bytes,
@@ -784,18 +807,16 @@ spamm_status spamm_run(spamm_ctx ctx, int64_t njobs, const spamm_job* jobs, cons
     double ms = 0.0;
     if (!host.empty()) {
       const int64_t np = (int64_t)host.size();
-      BufP dplans = alloc_n<PlanDev>(ctx, np), dub = alloc_n<int64_t>(ctx, np + 1);
-      CK(cudaMemcpyAsync(P<PlanDev>(dplans), host.data(), np * sizeof(PlanDev), cudaMemcpyHostToDevice,
-                         ctx->stream));
-      CK(cudaMemcpyAsync(P<int64_t>(dub), ubegin.data(), (np + 1) * sizeof(int64_t), cudaMemcpyHostToDevice,
-                         ctx->stream));
-      BatchDev batch{P<PlanDev>(dplans), P<int64_t>(dub), (int)np, ubegin.back()};
-      Events ev;
-      CK(cudaEventRecord(ev.e[0], ctx->stream));
+      BufP tables;
+      const BatchDev batch = upload_batch(
+          ctx, np, [&](int64_t r) { return host[r]; }, [&](int64_t r) { return ubegin[r + 1] - ubegin[r]; }, {}, nullptr,
+          &tables);
+      const cudaEvent_t* ev = ctx->events + 6;
+      CK(cudaEventRecord(ev[0], ctx->stream));
       launch_gemm(ctx, prec, bs, batch);
-      CK(cudaEventRecord(ev.e[1], ctx->stream));
+      CK(cudaEventRecord(ev[1], ctx->stream));
       sync_and_check(ctx);
-      ms = elapsed_ms(ev.e[0], ev.e[1]);
+      ms = elapsed_ms(ev[0], ev[1]);
     }
     for (int64_t r = 0; r < njobs; ++r) {
       jobs[r]->done += take[r];
@@ -816,18 +837,22 @@ spamm_status spamm_job_finish(spamm_ctx ctx, spamm_job job, spamm_mat* C, spamm_
     if (job->done != job->out.units) fail(SPAMM_E_BUSY, "the job has units that have not run");
     if (!job->out.C) fail(SPAMM_E_INVALID_ARG, "the job was already finished");
     spamm_mat Cm = job->out.C.get();
-    Events ev;
-    CK(cudaEventRecord(ev.e[0], ctx->stream));
-    finish_leaves(ctx, job->plan->prec, Cm);
+    const cudaEvent_t* ev = ctx->events + 6;
     NormBatch norms;
-    BufP ntab = norm_tables(ctx, {Cm}, &norms);
+    const size_t nb = norm_table_bytes(1);
+    BufP tab = alloc_bytes(ctx, nb);
+    std::vector<uint8_t> host(nb);
+    norm_tables({Cm}, host.data(), tab->p, &norms);
+    CK(cudaMemcpyAsync(tab->p, host.data(), nb, cudaMemcpyHostToDevice, ctx->stream));
+    CK(cudaEventRecord(ev[0], ctx->stream));
+    finish_leaves(ctx, job->plan->prec, Cm);
     propagate_norms(ctx, norms);
-    CK(cudaEventRecord(ev.e[1], ctx->stream));
+    CK(cudaEventRecord(ev[1], ctx->stream));
     sync_and_check(ctx);
     if (stats) {
       fill_stats(*job->plan, stats);
       stats->ms_gemm = job->ms_gemm;
-      stats->ms_cnorm = elapsed_ms(ev.e[0], ev.e[1]);
+      stats->ms_cnorm = elapsed_ms(ev[0], ev[1]);
       stats->n_launches = job->launches;
     }
     *C = registered(job->out.C.release());
@@ -898,11 +923,14 @@ spamm_status spamm_multiply(spamm_ctx ctx, spamm_mat A, spamm_mat B, double tau,
   if (!ctx || !A || !B || !C) return SPAMM_E_INVALID_ARG;
   *C = nullptr;
   return guarded(ctx, [&] {
+    // the plan is internal to this call: its last kernels and the execution's run on
+    // without a wait between them
     std::unique_ptr<spamm_plan_s> p(make_plan(ctx, A, B, tau, mode, prec));
-    ctx->live_handles--;  // the plan is internal to this call
     double ms_gemm = 0, ms_cnorm = 0;
     int64_t launches = 0;
     std::vector<spamm_mat> out = execute_plans(ctx, {p.get()}, &ms_gemm, &ms_cnorm, &launches);
+    settle_plan(p.get());
+    if (p->T.ngroups > 0) tree_set_counts(out[0], static_cast<const uint64_t*>(ctx->h_pinned));
     if (stats) {
       fill_stats(*p, stats);
       stats->ms_gemm = ms_gemm;

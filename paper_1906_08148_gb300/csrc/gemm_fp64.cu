@@ -162,10 +162,15 @@ static void launch_tile(spamm_ctx ctx, const BatchDev& b) {
   constexpr int KP = 32;
   auto kern = gemm_fp64_kernel<BS, KP, TILE>;
   const size_t smem = 4 * (size_t)TILE * KP * sizeof(double);
-  CK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  int per_sm = 0;
-  CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kGemmThreads, smem));
-  if (per_sm < 1) per_sm = 1;
+  // looked up once per context (two kernels per leaf size)
+  constexpr int id = (BS == 32 ? 0 : BS == 64 ? 2 : 4) + (TILE == (BS <= 64 ? BS : 64) ? 1 : 0);
+  int& per_sm = ctx->fp64_ctas[BS == 256 ? id + 2 : id];
+  if (per_sm == 0) {
+    CK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    int n = 0;
+    CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kern, kGemmThreads, smem));
+    per_sm = n < 1 ? 1 : n;
+  }
   const int sms = ctx->gemm_sm_limit > 0 ? ctx->gemm_sm_limit : ctx->num_sms;
   const int nq = fp64_units_per_leaf(BS);
   const int64_t units = b.nunits / nq * ((BS / TILE) * (BS / TILE));

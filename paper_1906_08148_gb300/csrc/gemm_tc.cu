@@ -694,11 +694,15 @@ static void launch_quads(spamm_ctx ctx, const BatchDev& b) {
   const size_t smem = QuadLayout<PREC>::SMEM;
   // the register split in the kernel assumes exactly kLaunchRegs per thread at
   // launch: with fewer, the epilogue's increase could never be granted
-  cudaFuncAttributes attr;
-  CK(cudaFuncGetAttributes(&attr, gemm_quad_kernel<PREC>));
-  if (attr.numRegs != (int)kLaunchRegs || attr.maxThreadsPerBlock < kQuadThreads)
-    fail(SPAMM_E_CUDA, "tensor-core kernel built with an unexpected register count; refusing to launch");
-  CK(cudaFuncSetAttribute(gemm_quad_kernel<PREC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  // (checked once per context)
+  if (!(ctx->tc_ready >> PREC & 1)) {
+    cudaFuncAttributes attr;
+    CK(cudaFuncGetAttributes(&attr, gemm_quad_kernel<PREC>));
+    if (attr.numRegs != (int)kLaunchRegs || attr.maxThreadsPerBlock < kQuadThreads)
+      fail(SPAMM_E_CUDA, "tensor-core kernel built with an unexpected register count; refusing to launch");
+    CK(cudaFuncSetAttribute(gemm_quad_kernel<PREC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    ctx->tc_ready |= 1 << PREC;
+  }
   unsigned long long* work = ctx->d_scratch + 9;  // quad claim counter
   CK(cudaMemsetAsync(work, 0, sizeof(unsigned long long), ctx->stream));
   gemm_quad_kernel<PREC><<<gemm_grid(ctx, b.nunits), kQuadThreads, smem, ctx->stream>>>(b, work, ctx->d_err);

@@ -121,6 +121,11 @@ struct spamm_ctx_s {
   cudaGraphExec_t graph_exec = nullptr;      // the last execute graph, updated in place for the next batch
   int64_t graph_instantiations = 0, graph_updates = 0;
   int live_handles = 0;
+  // timing events of the calls on this context (a context is used by one thread at a
+  // time): plan 0 .. 5, execution 6 .. 8
+  cudaEvent_t events[9] = {};
+  int fp64_ctas[8] = {};  // CTAs per SM of the FP64 leaf products' kernels (0: not set up yet)
+  int tc_ready = 0;       // bit per tensor form: kernel checked and its shared memory set
 };
 
 struct spamm_mat_s {
@@ -162,17 +167,20 @@ void tree_counts_async(spamm_ctx ctx, spamm_mat m, uint64_t* host);  // host: L 
 void tree_set_counts(spamm_mat m, const uint64_t* host);
 // The levels above given leaf codes (count exact), without norms; counts as above.
 void tree_skeleton(spamm_ctx ctx, spamm_mat m);
-void alloc_level_norms(spamm_mat m);
+// Squared norms of every level and the leaves' slots, for the levels' counts.
+void alloc_norms(spamm_mat m);
 // The parents' norms of several matrices whose structure and leaf norms exist:
-// norm_tables uploads the tables (norm buffers must already exist),
-// propagate_norms launches (no host sync, so it can be captured in a CUDA graph).
+// norm_tables fills the table (norm_table_bytes; norm buffers must already exist) for
+// a copy at `device`, propagate_norms launches (no host sync, so it can be captured in
+// a CUDA graph).
 struct NormBatch {
   const void* tab = nullptr;
   int ntrees = 0;
   int wide = 0;        // heights with a launch of their own
   int64_t widest = 0;  // nodes of the largest of them
 };
-BufP norm_tables(spamm_ctx ctx, const std::vector<spamm_mat>& ms, NormBatch* nb);
+size_t norm_table_bytes(size_t ntrees);
+void norm_tables(const std::vector<spamm_mat>& ms, void* host, const void* device, NormBatch* nb);
 void propagate_norms(spamm_ctx ctx, const NormBatch& nb);
 // Leaf set from candidate leaves: keep[q] selects rows of (code, sq, slot) already sorted by code.
 void set_leaves_compacted(spamm_mat m, int64_t ncand, const uint32_t* code, const double* sq, const int64_t* slot,

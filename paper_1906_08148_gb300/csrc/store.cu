@@ -119,17 +119,18 @@ void set_leaves_compacted(spamm_mat m, int64_t ncand, const uint32_t* code, cons
   tree_resolve(m->ctx, m);
 }
 
-void alloc_level_norms(spamm_mat m) {
+void alloc_norms(spamm_mat m) {
   auto up = [](size_t b) { return (b + 255) & ~(size_t)255; };
-  size_t bytes = 0;
-  for (int t = 0; t < m->L; ++t) bytes += up(m->lv[t].count * sizeof(double));
-  if (bytes == 0) return;
+  const int64_t n = m->lv[m->L].count;
+  size_t bytes = up(n * sizeof(int64_t));
+  for (const Level& lv : m->lv) bytes += up(lv.count * sizeof(double));
   BufP arena = alloc_bytes(m->ctx, bytes);
   size_t at = 0;
-  for (int t = 0; t < m->L; ++t) {
-    m->lv[t].sq = sub_buf(arena, at, m->lv[t].count * sizeof(double));
-    at += up(m->lv[t].count * sizeof(double));
+  for (Level& lv : m->lv) {
+    lv.sq = sub_buf(arena, at, lv.count * sizeof(double));
+    at += up(lv.count * sizeof(double));
   }
+  m->slot = sub_buf(arena, at, n * sizeof(int64_t));
 }
 
 // ----------------------------------------------------------- truncation

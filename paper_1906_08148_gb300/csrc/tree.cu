@@ -435,9 +435,8 @@ void tree_resolve(spamm_ctx ctx, spamm_mat m) {
 // kTopNodes nodes one launch each (all trees), the rest by one block per tree in
 // one launch.  The additions are place_parent's.
 struct NormTree {
-  int32_t L;
-  int32_t pad;
-  int64_t count[SPAMM_MAX_LEVELS];
+  int64_t L;
+  const uint64_t* count;  // nodes per level, on the device
   const int4* child[SPAMM_MAX_LEVELS];
   double* sq[SPAMM_MAX_LEVELS];
 };
@@ -457,25 +456,30 @@ __device__ __forceinline__ void node_norm(const NormTree& T, int t, int64_t p) {
 __global__ void norms_wide_kernel(const NormTree* __restrict__ tab, int ntrees, int h) {
   for (int r = blockIdx.y; r < ntrees; r += gridDim.y) {
     const NormTree& T = tab[r];
-    const int t = T.L - h;
-    if (t < 0 || T.count[t] <= kTopNodes) continue;
-    for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < T.count[t];
-         p += (int64_t)gridDim.x * blockDim.x)
+    const int t = (int)T.L - h;
+    const int64_t n = t >= 0 && T.count ? (int64_t)T.count[t] : 0;
+    if (n <= kTopNodes) continue;
+    for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < n; p += (int64_t)gridDim.x * blockDim.x)
       node_norm(T, t, p);
   }
 }
 
 __global__ void __launch_bounds__(kTopThreads) norms_top_kernel(const NormTree* __restrict__ tab) {
   const NormTree& T = tab[blockIdx.x];
-  for (int t = T.L - 1; t >= 0; --t) {
-    if (T.count[t] > kTopNodes) continue;
-    for (int64_t p = threadIdx.x; p < T.count[t]; p += kTopThreads) node_norm(T, t, p);
+  if (!T.count) return;  // no leaves
+  for (int t = (int)T.L - 1; t >= 0; --t) {
+    const int64_t n = (int64_t)T.count[t];
+    if (n > kTopNodes) continue;
+    for (int64_t p = threadIdx.x; p < n; p += kTopThreads) node_norm(T, t, p);
     __syncthreads();
   }
 }
 
-BufP norm_tables(spamm_ctx ctx, const std::vector<spamm_mat>& ms, NormBatch* nb) {
-  std::vector<NormTree> tab(ms.size());
+size_t norm_table_bytes(size_t ntrees) { return ntrees * sizeof(NormTree); }
+
+void norm_tables(const std::vector<spamm_mat>& ms, void* host, const void* device, NormBatch* nb) {
+  NormTree* tab = static_cast<NormTree*>(host);
+  nb->tab = device;
   nb->ntrees = (int)ms.size();
   nb->wide = 0;
   nb->widest = 0;
@@ -484,21 +488,16 @@ BufP norm_tables(spamm_ctx ctx, const std::vector<spamm_mat>& ms, NormBatch* nb)
     NormTree& T = tab[r];
     memset(&T, 0, sizeof T);
     T.L = m->L;
+    T.count = P<uint64_t>(m->dcount);
     for (int t = 0; t <= m->L; ++t) {
-      T.count[t] = m->lv[t].count;
       T.child[t] = t < m->L ? P<int4>(m->lv[t].child) : nullptr;
       T.sq[t] = P<double>(m->lv[t].sq);
-      if (t < m->L && T.count[t] > kTopNodes) {
+      if (t < m->L && m->lv[t].count > kTopNodes) {  // exact, or an upper bound
         nb->wide = nb->wide > m->L - t ? nb->wide : m->L - t;
-        nb->widest = nb->widest > T.count[t] ? nb->widest : T.count[t];
+        nb->widest = nb->widest > m->lv[t].count ? nb->widest : m->lv[t].count;
       }
     }
   }
-  // a pageable source: the copy has read it by the time it returns
-  BufP d = alloc_n<NormTree>(ctx, (int64_t)tab.size());
-  CK(cudaMemcpyAsync(d->p, tab.data(), tab.size() * sizeof(NormTree), cudaMemcpyHostToDevice, ctx->stream));
-  nb->tab = d->p;
-  return d;
 }
 
 void propagate_norms(spamm_ctx ctx, const NormBatch& nb) {
