@@ -254,16 +254,17 @@ void scan_inclusive_f64(spamm_ctx ctx, const double* in, double* out, int64_t n)
 // places after the warp's earlier ones, counted per warp and digit in shared
 // memory; the warps of a block own consecutive runs of items, so a prefix over
 // warps, tiles and digits gives every item its place.  Up to kSortSmall items one
-// block takes all passes in one launch (16 rounds a pass); more take three launches
+// block takes all passes in one launch (four rounds a pass); more take three launches
 // a pass: digit counts per tile, their prefix per digit, placing.  2,000,000 pairs by 32
 // bits: 0.23 ms where eight 4-bit passes, each a scan over all blocks and digits,
 // took 0.85; 10,000 pairs by 64 bits one launch instead of 64.
 constexpr int kDigits = 256;
 constexpr int kSortThreads = 256;
-constexpr int kSortRounds = 16;                       // rounds of 32 items per warp
+constexpr int kSortRounds = 8;                        // rounds of 32 items per warp
 constexpr int kSortTile = kSortThreads * kSortRounds;  // items per block
 constexpr int kSmallThreads = 1024;
-constexpr int64_t kSortSmall = kSmallThreads * kSortRounds;
+constexpr int64_t kSortSmall = 4096;
+static_assert(kSortSmall <= kSmallThreads * kSortRounds, "the one-block sort holds its items in registers");
 
 // Ranks the warp's items (digit d[r] of round r, valid where bit r of `in`) within its
 // counters cnt[256], which it leaves at the warp's digit counts.

@@ -177,12 +177,54 @@ void truncate_pair(spamm_ctx ctx, spamm_mat A, spamm_mat B, double tau, spamm_ma
 // ties in Morton order) as long as the sum of their squared norms, added in
 // that order, stays <= tau^2, so ||A - A~||_F <= tau.  The squared norms are
 // non-negative doubles, so their bit patterns sort like their values.
-__global__ void sq_sort_keys_kernel(const double* __restrict__ sq, int64_t n, uint64_t* __restrict__ keys,
-                                    int64_t* __restrict__ idx) {
-  for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < n; q += (int64_t)gridDim.x * blockDim.x) {
-    keys[q] = (uint64_t)__double_as_longlong(sq[q]);
-    idx[q] = q;
+//
+// Only a leaf whose own squared norm is within the budget can be dropped (a running
+// sum is at least its last term), so the others are left out of the sort and of the
+// sums: the candidates come first in the sorted order, and the running sums over them
+// are the same numbers without what follows.
+constexpr int kSelectPer = 4;
+constexpr int64_t kSelectTile = kThreads * kSelectPer;
+
+// Candidates per tile; with `tiles` scanned (place = true) their keys and indexes, in
+// leaf order.
+__global__ void __launch_bounds__(kThreads)
+    select_small_kernel(const double* __restrict__ sq, int64_t n, double budget, uint64_t* __restrict__ tiles, bool place,
+                        uint64_t* __restrict__ keys, int64_t* __restrict__ idx) {
+  __shared__ unsigned ws[kThreads / 32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int64_t q0 = (int64_t)blockIdx.x * kSelectTile + (int64_t)threadIdx.x * kSelectPer;
+  double v[kSelectPer];
+  unsigned c = 0;
+#pragma unroll
+  for (int i = 0; i < kSelectPer; ++i) {
+    v[i] = q0 + i < n ? sq[q0 + i] : budget + 1.0;
+    c += (q0 + i < n) && v[i] <= budget;
   }
+  unsigned x = c;
+#pragma unroll
+  for (int off = 1; off < 32; off <<= 1) {
+    const unsigned y = __shfl_up_sync(0xffffffffu, x, off);
+    if (lane >= off) x += y;
+  }
+  if (lane == 31) ws[warp] = x;
+  __syncthreads();
+  unsigned before = 0, all = 0;
+#pragma unroll
+  for (int w = 0; w < kThreads / 32; ++w) {
+    if (w < warp) before += ws[w];
+    all += ws[w];
+  }
+  if (!place) {
+    if (threadIdx.x == 0) tiles[blockIdx.x] = all;
+    return;
+  }
+  int64_t p = (int64_t)tiles[blockIdx.x] + before + x - c;
+#pragma unroll
+  for (int i = 0; i < kSelectPer; ++i)
+    if (q0 + i < n && v[i] <= budget) {
+      keys[p] = (uint64_t)__double_as_longlong(v[i]);
+      idx[p++] = q0 + i;
+    }
 }
 
 // Number of running sums within the budget.
@@ -196,13 +238,13 @@ __global__ void within_budget_kernel(const double* __restrict__ csum, int64_t n,
   if ((threadIdx.x & 31) == 0 && c) atomicAdd(count, c);
 }
 
-// The first *ndrop leaves of the sorted order are dropped (a prefix, even if
+// The first *ndrop of the sorted candidates are dropped (a prefix, even if
 // rounding made the running sums non-monotone by an ulp).
 __global__ void drop_prefix_kernel(const int64_t* __restrict__ idx, int64_t n, const uint64_t* __restrict__ ndrop,
                                    uint8_t* __restrict__ keep) {
-  const int64_t k = (int64_t)*ndrop;
-  for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < n; q += (int64_t)gridDim.x * blockDim.x)
-    keep[idx[q]] = q >= k;
+  const int64_t k = min((int64_t)*ndrop, n);
+  for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < k; q += (int64_t)gridDim.x * blockDim.x)
+    keep[idx[q]] = 0;
 }
 
 spamm_mat truncate_error_controlled(spamm_mat in, double tau, spamm_ctx on) {
@@ -213,20 +255,31 @@ spamm_mat truncate_error_controlled(spamm_mat in, double tau, spamm_ctx on) {
   const int64_t n = in->nleaves;
   BufP keep = alloc_n<uint8_t>(ctx, n);
   if (n > 0) {
-    BufP keys = alloc_n<uint64_t>(ctx, n), idx = alloc_n<int64_t>(ctx, n), csum = alloc_n<double>(ctx, n);
-    BufP ndrop = alloc_n<uint64_t>(ctx, 1);
-    CK(cudaMemsetAsync(P<uint64_t>(ndrop), 0, sizeof(uint64_t), ctx->stream));
-    const unsigned g = grid_for(ctx, n, kThreads);
-    sq_sort_keys_kernel<<<g, kThreads, 0, ctx->stream>>>(P<double>(in->lv[in->L].sq), n, P<uint64_t>(keys),
-                                                          P<int64_t>(idx));
-    CK_LAUNCH("sq_sort_keys_kernel");
-    radix_sort_pairs(ctx, P<uint64_t>(keys), P<int64_t>(idx), n, 64);  // stable: ties keep Morton order
-    scan_inclusive_f64(ctx, P<double>(keys), P<double>(csum), n);  // the sorted keys are the squared norms' bits
-    within_budget_kernel<<<g, kThreads, 0, ctx->stream>>>(P<double>(csum), n, tau * tau,
-                                                          P<unsigned long long>(ndrop));
-    CK_LAUNCH("within_budget_kernel");
-    drop_prefix_kernel<<<g, kThreads, 0, ctx->stream>>>(P<int64_t>(idx), n, P<uint64_t>(ndrop), P<uint8_t>(keep));
-    CK_LAUNCH("drop_prefix_kernel");
+    const double budget = tau * tau;
+    const double* sq = P<double>(in->lv[in->L].sq);
+    CK(cudaMemsetAsync(P<uint8_t>(keep), 1, n, ctx->stream));
+    const int64_t ntiles = (n + kSelectTile - 1) / kSelectTile;
+    BufP tiles = alloc_n<uint64_t>(ctx, ntiles + 1);
+    select_small_kernel<<<(unsigned)ntiles, kThreads, 0, ctx->stream>>>(sq, n, budget, P<uint64_t>(tiles), false, nullptr,
+                                                                        nullptr);
+    CK_LAUNCH("select_small_kernel");
+    scan_exclusive_u64(ctx, P<uint64_t>(tiles), P<uint64_t>(tiles), ntiles, P<uint64_t>(tiles) + ntiles);
+    const int64_t c = (int64_t)read_scalar<uint64_t>(ctx, P<uint64_t>(tiles) + ntiles);
+    if (c > 0) {
+      BufP keys = alloc_n<uint64_t>(ctx, c), idx = alloc_n<int64_t>(ctx, c), csum = alloc_n<double>(ctx, c);
+      BufP ndrop = alloc_n<uint64_t>(ctx, 1);
+      CK(cudaMemsetAsync(P<uint64_t>(ndrop), 0, sizeof(uint64_t), ctx->stream));
+      select_small_kernel<<<(unsigned)ntiles, kThreads, 0, ctx->stream>>>(sq, n, budget, P<uint64_t>(tiles), true,
+                                                                          P<uint64_t>(keys), P<int64_t>(idx));
+      CK_LAUNCH("select_small_kernel");
+      const unsigned g = grid_for(ctx, c, kThreads);
+      radix_sort_pairs(ctx, P<uint64_t>(keys), P<int64_t>(idx), c, 64);  // stable: ties keep Morton order
+      scan_inclusive_f64(ctx, P<double>(keys), P<double>(csum), c);  // the sorted keys are the squared norms' bits
+      within_budget_kernel<<<g, kThreads, 0, ctx->stream>>>(P<double>(csum), c, budget, P<unsigned long long>(ndrop));
+      CK_LAUNCH("within_budget_kernel");
+      drop_prefix_kernel<<<g, kThreads, 0, ctx->stream>>>(P<int64_t>(idx), c, P<uint64_t>(ndrop), P<uint8_t>(keep));
+      CK_LAUNCH("drop_prefix_kernel");
+    }
   }
   set_leaves_compacted(out, n, P<uint32_t>(in->lv[in->L].code), P<double>(in->lv[in->L].sq), P<int64_t>(in->slot),
                        P<uint8_t>(keep));

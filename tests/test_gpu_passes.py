@@ -98,7 +98,7 @@ def test_device_leaves_equal_host_leaves(S, ctx, rule, tau, offset):
 
 
 # one round of one warp, one item more, the largest one-block sort, one more, several tiles
-@pytest.mark.parametrize("nnz", [1, 32, 33, 1024, 4097, 16384, 16385, 50000])
+@pytest.mark.parametrize("nnz", [1, 32, 33, 1024, 4096, 4097, 16384, 16385, 50000])
 def test_coo_sums_duplicates_in_input_order(S, ctx, nnz):
     rng = np.random.default_rng(nnz)
     n, bs = 5000, 32
