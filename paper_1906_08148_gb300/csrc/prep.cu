@@ -6,6 +6,7 @@
 
 #include "fbits.cuh"
 #include "internal.cuh"
+#include "ptx.cuh"
 #include "slices.cuh"
 #include "tcforms.cuh"
 
@@ -13,14 +14,7 @@ namespace spamm {
 
 // Thread <-> element mapping shared by both kernels: one CTA of 512 threads
 // per 64 x 64 tile of a leaf; a thread owns one 16-byte chunk of the K-major
-// term tiles (8 consecutive k of one tile row) and loads its 8 FP64 elements
-// first.  A tile is loaded, measured (line and tile maxima), split and written with
-// a barrier between, so other CTAs have to fill the gaps: one chunk per thread keeps
-// the registers at 64, 1024 threads per SM, where two chunks in 256 threads (124
-// registers, 512 threads) left the memory idle half of the time.  Both operands of the
-// n = 16384 lattice as 3 slices (4.2 GB moved) 1.10 -> 0.87 ms, of n = 65536 as 4 slices
-// (32.8 GB) 9.5 -> 7.8 ms, with the 32-bit digits of slices.cuh; FP16, whose packed
-// conversions made up for its second barrier, unchanged.
+// term tiles (8 consecutive k of one tile row), 8 FP64 elements.
 // role 0 (A): tile row = leaf row t >> 3, k = leaf columns 8 (t & 7) ..
 // role 1 (B): tile row = leaf column t & 63, k = leaf rows 8 (t >> 6) ..,
 // so the lanes of a warp read consecutive doubles of each leaf row.
@@ -31,20 +25,20 @@ struct ChunkMap {
     row = role == 0 ? t >> 3 : (t & 63);
     c8 = role == 0 ? (t & 7) : t >> 6;
   }
-  // src: the tile's first element; ld: the leaf's row length
-  __device__ void load(const unsigned long long* src, int ld, int role, unsigned long long (&v)[8]) const {
+  // src: the tile's first element (shared or global memory); ld: its row length
+  __device__ __forceinline__ void load(const unsigned long long* src, int ld, int role, unsigned long long (&v)[8]) const {
     if (role == 0) {
       // 8 consecutive doubles of one row: four 16-byte loads
       const ulonglong2* p = reinterpret_cast<const ulonglong2*>(src + row * ld + 8 * c8);
 #pragma unroll
       for (int e = 0; e < 4; ++e) {
-        const ulonglong2 w = __ldg(p + e);
+        const ulonglong2 w = p[e];
         v[2 * e] = w.x;
         v[2 * e + 1] = w.y;
       }
     } else {
 #pragma unroll
-      for (int e = 0; e < 8; ++e) v[e] = __ldg(src + (8 * c8 + e) * ld + row);
+      for (int e = 0; e < 8; ++e) v[e] = src[(8 * c8 + e) * ld + row];
     }
   }
 };
@@ -62,121 +56,194 @@ __device__ __forceinline__ const double* tile_src(const double* leaf, int bs, in
   return role == 0 ? leaf + (int64_t)(64 * r2) * bs + 64 * kh : leaf + (int64_t)(64 * kh) * bs + 64 * r2;
 }
 
-// ------------------------------------------------------- BF16 slices (error-free split)
-// Per leaf: the largest biased exponent of every line (A: row, B: column) and
-// of the leaf, the leaf's scale exponent f (stored in expo[m]), then every
-// element's S digits (slices.cuh) as BF16 values d_s 2^(e - 8 - 9 s).  The
-// slices are assembled in shared memory and leave as one contiguous block.
-template <int S, int KPARTS>
-__global__ void __launch_bounds__(kPrepThreads, 2)
-    prep_slices_kernel(const double* __restrict__ pool, const int64_t* __restrict__ slot, int64_t nleaves, int bs,
-                       int role, uint8_t* __restrict__ out, int32_t* __restrict__ expo) {
-  constexpr uint32_t LEAF = (uint32_t)S * kTerm;
-  __shared__ uint4 stile[LEAF / 16];
-  __shared__ int s_line[8][64];  // role 1: per-column maxima of each eighth of the leaf rows
-  __shared__ int s_warp[kPrepThreads / 32];
+// A CTA takes tiles blockIdx.x, blockIdx.x + gridDim.x, ...  A tile is measured, split
+// and written with a barrier between, and while it was loaded into registers first
+// the memory was idle half of the time.  STAGED (64 x 64 leaves: a tile is one run
+// of memory): bulk copies bring the doubles into two buffers of shared memory, two
+// tiles ahead.  The finished terms leave as one bulk copy.  Two CTAs per SM.
+// Both operands, n = 65536 as 4 slices (32.8 GB moved) 7.8 -> 6.5 ms, n = 16384 as 3
+// slices (4.2 GB) 0.87 -> 0.70.  The quarters of a 128 x 128 leaf are 64 runs of 512
+// bytes each, for which the staged form is the slower one (n = 20000 FP16, 5.3 GB: 1.50
+// ms, 1.17 with loads into registers).
+struct TileStream {
+  static constexpr uint32_t kBytes = 64 * 64 * sizeof(double);
+  const double* pool;
+  const int64_t* slot;
+  int64_t total;  // tiles
+  int bs, role;
+  uint8_t* in;    // two tiles
+  uint64_t* full;
+
+  __device__ __forceinline__ const double* source(int64_t m) const {
+    const int tiles = (bs / 64) * (bs / 64);
+    const int64_t leaf = m / tiles;
+    return tile_src(pool + slot[leaf] * (int64_t)bs * bs, bs, role, (int)(m - leaf * tiles));
+  }
+  // STAGED, by one thread: tile m into buffer b (nothing past the last tile)
+  __device__ __forceinline__ void fetch(int64_t m, int b) const {
+    if (m >= total) return;
+    const double* src = source(m);
+    fence_proxy_async_smem();
+    mbar_arrive_expect_tx(&full[b], kBytes);
+    bulk_g2s(in + (uint32_t)b * kBytes, src, kBytes, &full[b]);
+  }
+  // the last two fetches of a CTA that gave up have landed
+  __device__ __forceinline__ void drain(int64_t m, uint32_t it) const {
+    for (int i = 0; i < 2; ++i)
+      if (m + (int64_t)i * gridDim.x < total) mbar_wait_bounded(&full[(it + i) & 1], ((it + i) >> 1) & 1u);
+  }
+};
+
+// Form: measure(v) gives a thread's words for the line and tile maxima (the first
+// combined by max, the second by or), shift the tile's scale exponent from them, split
+// the thread's chunk of every term.
+template <class Form, bool STAGED>
+__global__ void __launch_bounds__(kPrepThreads, STAGED || Form::kLines ? 2 : 3)
+    prep_kernel(const double* __restrict__ pool, const int64_t* __restrict__ slot, int64_t nleaves, int bs, int role,
+                uint8_t* __restrict__ out, int32_t* __restrict__ expo, int* __restrict__ err) {
+  constexpr uint32_t LEAF = Form::kLeaf;
+  extern __shared__ __align__(128) uint8_t prep_smem[];
+  uint8_t* stile = prep_smem + (STAGED ? 2 * TileStream::kBytes : 0);  // the finished terms
+  __shared__ __align__(8) uint64_t full[2];
+  __shared__ uint32_t s_line[8][64];
+  __shared__ uint2 s_warp[kPrepThreads / 32];
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
   const ChunkMap cm(t, role);
-  const int tiles = (bs / 64) * (bs / 64);
-  for (int64_t m = blockIdx.x; m < nleaves * tiles; m += gridDim.x) {
-    const int64_t leaf = m / tiles;
-    const unsigned long long* src = reinterpret_cast<const unsigned long long*>(
-        tile_src(pool + slot[leaf] * (int64_t)bs * bs, bs, role, (int)(m - leaf * tiles)));
+  const TileStream ts{pool, slot, nleaves * (bs / 64) * (bs / 64), bs, role, prep_smem, full};
+  int64_t m = blockIdx.x;
+  if (STAGED) {
+    if (t == 0) {
+      mbar_init(&full[0], 1);
+      mbar_init(&full[1], 1);
+      fence_mbar_init();
+    }
+    __syncthreads();
+    if (t == 0) {
+      ts.fetch(m, 0);
+      ts.fetch(m + gridDim.x, 1);
+    }
+  }
+  bool failed = false;
+  uint32_t it = 0;
+  for (; m < ts.total; m += gridDim.x, ++it) {
+    const int b = (int)(it & 1);
+    bool ok = true;
     unsigned long long v[8];
-    cm.load(src, bs, role, v);
-    // largest biased exponent of this thread's line
-    int em = 0;
-#pragma unroll
-    for (int e = 0; e < 8; ++e) em = max(em, slice_biased_exp(v[e]));
-    if (role == 0) {
-      // a row's 8 chunks are held by 8 consecutive lanes
-#pragma unroll
-      for (int off = 1; off < 8; off <<= 1) em = max(em, __shfl_xor_sync(0xffffffffu, em, off));
+    if (STAGED) {
+      ok = mbar_wait_bounded(&full[b], (it >> 1) & 1u);
+      cm.load(reinterpret_cast<const unsigned long long*>(prep_smem + (uint32_t)b * TileStream::kBytes), 64, role, v);
     } else {
-      // a column's 8 chunks are held by the threads t & 63 == column of 8 warp pairs
-      s_line[t >> 6][t & 63] = em;
-      __syncthreads();
-#pragma unroll
-      for (int h = 0; h < 8; ++h) em = max(em, s_line[h][t & 63]);
+      cm.load(reinterpret_cast<const unsigned long long*>(ts.source(m)), bs, role, v);
     }
-    const int lm = __reduce_max_sync(0xffffffffu, em);
-    if (lane == 0) s_warp[warp] = lm;
-    __syncthreads();
-    const int leaf_max = __reduce_max_sync(0xffffffffu, s_warp[lane & (kPrepThreads / 32 - 1)]);
-    const int f = slice_leaf_shift(leaf_max);
+    // the largest of this thread's line (A: row, B: column), then of the tile
+    uint2 top = Form::measure(v);
+    if (Form::kLines) {
+      if (role == 0) {
+        // a row's 8 chunks are held by 8 consecutive lanes
+#pragma unroll
+        for (int off = 1; off < 8; off <<= 1) top.x = max(top.x, __shfl_xor_sync(0xffffffffu, top.x, off));
+      } else {
+        // a column's 8 chunks are held by the threads t & 63 == column of 8 warp pairs
+        s_line[t >> 6][t & 63] = top.x;
+        __syncthreads();
+#pragma unroll
+        for (int h = 0; h < 8; ++h) top.x = max(top.x, s_line[h][t & 63]);
+      }
+    }
+    const uint32_t line = top.x;
+    const uint32_t wx = __reduce_max_sync(0xffffffffu, top.x), wy = __reduce_or_sync(0xffffffffu, top.y);
+    if (lane == 0) s_warp[warp] = make_uint2(wx, wy);
+    if (t == 0) bulk_wait_read();  // the last tile's terms have left stile
+    failed = __syncthreads_or(!ok);
+    if (failed) break;
+    if (STAGED && t == 0) ts.fetch(m + 2 * (int64_t)gridDim.x, b);  // every thread holds its elements in registers
+    const uint2 w = s_warp[lane & (kPrepThreads / 32 - 1)];
+    const int f = Form::shift(__reduce_max_sync(0xffffffffu, w.x), __reduce_or_sync(0xffffffffu, w.y));
     if (t == 0) expo[m] = f;
-    const int e = slice_line_exp(em, f);
-    float unit[S];
-#pragma unroll
-    for (int s = 0; s < S; ++s) unit[s] = slice_unit(e - 8 - 9 * s);
-    uint32_t term[S][4];
-#pragma unroll
-    for (int q = 0; q < 8; q += 2) {
-      int32_t d0[S], d1[S];
-      slice_digits<S>(v[q], em, d0);
-      slice_digits<S>(v[q + 1], em, d1);
-#pragma unroll
-      for (int s = 0; s < S; ++s) term[s][q / 2] = slice_bf16_x2(d0[s], d1[s], unit[s]);
-    }
-#pragma unroll
-    for (int s = 0; s < S; ++s) {
-      const uint32_t off = term_offset<KPARTS>(S, s, cm.row, 8 * cm.c8);
-      stile[off >> 4] = make_uint4(term[s][0], term[s][1], term[s][2], term[s][3]);
-    }
+    Form::split(v, (int)line, f, [&](int s, uint4 chunk) {
+      *reinterpret_cast<uint4*>(stile + term_offset<Form::kParts>(Form::kTerms, s, cm.row, 8 * cm.c8)) = chunk;
+    });
+    fence_proxy_async_smem();
     __syncthreads();
-    // the leaf's slices leave in order: consecutive threads, consecutive 16-byte chunks
-    uint4* d4 = reinterpret_cast<uint4*>(out + m * (int64_t)LEAF);
-#pragma unroll
-    for (int i = 0; i < (int)(LEAF / 16) / kPrepThreads; ++i) d4[t + i * kPrepThreads] = stile[t + i * kPrepThreads];
-    __syncthreads();  // stile, s_line and s_warp are reused by the next leaf
+    if (t == 0) bulk_s2g(out + m * (int64_t)LEAF, stile, LEAF);
+  }
+  if (t == 0) {
+    bulk_wait_all();
+    if (failed) {
+      atomicOr(err, DEV_ERR_TIMEOUT);
+      ts.drain(m, it);
+    }
   }
 }
 
+// ------------------------------------------------------- BF16 slices (error-free split)
+// Per tile: the largest biased exponent of every line (A: row, B: column) and
+// of the tile, the tile's scale exponent f (stored in expo[m]), then every
+// element's S digits (slices.cuh) as BF16 values d_s 2^(e - 8 - 9 s).
+template <int PREC>
+struct SliceForm {
+  static constexpr int kTerms = FormCfg<PREC>::TERMS, kParts = FormCfg<PREC>::KPARTS;
+  static constexpr uint32_t kLeaf = leaf_bytes<PREC>();
+  static constexpr bool kLines = true;
+  __device__ static __forceinline__ uint2 measure(const unsigned long long (&v)[8]) {
+    int em = 0;
+#pragma unroll
+    for (int e = 0; e < 8; ++e) em = max(em, slice_biased_exp(v[e]));
+    return make_uint2((uint32_t)em, 0u);
+  }
+  __device__ static __forceinline__ int shift(uint32_t emax, uint32_t) { return slice_leaf_shift((int)emax); }
+  template <class Put>
+  __device__ static __forceinline__ void split(const unsigned long long (&v)[8], int em, int f, Put put) {
+    const int e = slice_line_exp(em, f);
+    uint32_t term[kTerms][4];
+    float unit[kTerms];
+#pragma unroll
+    for (int s = 0; s < kTerms; ++s) unit[s] = slice_unit(e - 8 - 9 * s);
+#pragma unroll
+    for (int q = 0; q < 8; q += 2) {
+      int32_t d0[kTerms], d1[kTerms];
+      slice_digits<kTerms>(v[q], em, d0);
+      slice_digits<kTerms>(v[q + 1], em, d1);
+#pragma unroll
+      for (int s = 0; s < kTerms; ++s) term[s][q / 2] = slice_bf16_x2(d0[s], d1[s], unit[s]);
+    }
+#pragma unroll
+    for (int s = 0; s < kTerms; ++s) put(s, make_uint4(term[s][0], term[s][1], term[s][2], term[s][3]));
+  }
+};
+
 // ------------------------------------------------------------ FP16 terms
 // Each element is rounded once to FP32 on its bits (fbits.cuh) with the
-// per-leaf scale 2^e folded in, max|a 2^e| in [2^14, 2^15), then split in
+// per-tile scale 2^e folded in, max|a 2^e| in [2^14, 2^15), then split in
 // FP32: h0 = f16(a 2^e), h1 = f16(a 2^e - h0) (the residual is exact in FP32).
-__global__ void __launch_bounds__(kPrepThreads, 2)
-    prep_fp16_kernel(const double* __restrict__ pool, const int64_t* __restrict__ slot, int64_t nleaves, int bs, int role,
-                     uint8_t* __restrict__ out, int32_t* __restrict__ expo) {
-  constexpr int TERMS = FormCfg<SPAMM_PREC_FP16_SCALED>::TERMS;
-  constexpr uint32_t LEAF = leaf_bytes<SPAMM_PREC_FP16_SCALED>();
-  __shared__ uint2 smax[kPrepThreads / 32];
-  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-  const ChunkMap cm(t, role);
-  const int tiles = (bs / 64) * (bs / 64);
-  for (int64_t m = blockIdx.x; m < nleaves * tiles; m += gridDim.x) {
-    const int64_t leaf = m / tiles;
-    const unsigned long long* src = reinterpret_cast<const unsigned long long*>(
-        tile_src(pool + slot[leaf] * (int64_t)bs * bs, bs, role, (int)(m - leaf * tiles)));
-    unsigned long long v[8];
-    cm.load(src, bs, role, v);
-    // largest |a| of the tile: |x| of doubles orders like their bits without the sign,
-    // and the scale depends on the high word of the largest alone, but for an all-zero tile
+// |x| of doubles orders like their bits without the sign, and the scale depends on the
+// high word of the largest alone, but for an all-zero tile.
+struct Fp16Form {
+  static constexpr int PREC = SPAMM_PREC_FP16_SCALED;
+  static constexpr int kTerms = FormCfg<PREC>::TERMS, kParts = FormCfg<PREC>::KPARTS;
+  static constexpr uint32_t kLeaf = leaf_bytes<PREC>();
+  static constexpr bool kLines = false;
+  __device__ static __forceinline__ uint2 measure(const unsigned long long (&v)[8]) {
     uint32_t mh = 0, any = 0;
 #pragma unroll
     for (int e = 0; e < 8; ++e) {
       mh = max(mh, (uint32_t)(v[e] >> 32) & 0x7FFFFFFFu);
       any |= (uint32_t)v[e];
     }
-    mh = __reduce_max_sync(0xffffffffu, mh);
-    any = __any_sync(0xffffffffu, any != 0);
-    if (lane == 0) smax[warp] = make_uint2(mh, any);
-    __syncthreads();
-    const uint2 w = smax[lane & (kPrepThreads / 32 - 1)];
-    mh = __reduce_max_sync(0xffffffffu, w.x);
-    any = __any_sync(0xffffffffu, w.y != 0);
-    const unsigned long long mx = ((unsigned long long)mh << 32) | any;
-    const int shift = fp16_leaf_shift(mx);
-    if (t == 0) expo[m] = shift;
-    uint8_t* dst = out + m * (int64_t)LEAF;
-    uint32_t term[TERMS][4];
+    return make_uint2(mh, any);
+  }
+  __device__ static __forceinline__ int shift(uint32_t mh, uint32_t any) {
+    return fp16_leaf_shift(((uint64_t)mh << 32) | (any != 0));
+  }
+  template <class Put>
+  __device__ static __forceinline__ void split(const unsigned long long (&v)[8], int, int shift, Put put) {
+    uint32_t term[kTerms][4];
 #pragma unroll
     for (int e = 0; e < 8; e += 2) {
       float2 a = make_float2(__uint_as_float(fbits_from_double_rn(v[e], shift)),
                              __uint_as_float(fbits_from_double_rn(v[e + 1], shift)));
 #pragma unroll
-      for (int s = 0; s < TERMS; ++s) {  // two at a time: one packed conversion each way
+      for (int s = 0; s < kTerms; ++s) {  // two at a time: one packed conversion each way
         const __half2 h = __float22half2_rn(a);
         term[s][e / 2] = *reinterpret_cast<const uint32_t*>(&h);
         const float2 g = __half22float2(h);
@@ -185,12 +252,9 @@ __global__ void __launch_bounds__(kPrepThreads, 2)
       }
     }
 #pragma unroll
-    for (int s = 0; s < TERMS; ++s)
-      *reinterpret_cast<uint4*>(dst + term_offset<FormCfg<SPAMM_PREC_FP16_SCALED>::KPARTS>(TERMS, s, cm.row, 8 * cm.c8)) =
-          make_uint4(term[s][0], term[s][1], term[s][2], term[s][3]);
-    __syncthreads();  // smax is reused by the next leaf
+    for (int s = 0; s < kTerms; ++s) put(s, make_uint4(term[s][0], term[s][1], term[s][2], term[s][3]));
   }
-}
+};
 
 static uint32_t form_leaf_bytes(spamm_prec prec) {
   switch (prec) {
@@ -204,26 +268,33 @@ void prep_terms(spamm_mat M, spamm_prec prec, int role, BufP* terms, BufP* expo,
   spamm_ctx ctx = on ? on : M->ctx;
   const int bs = M->bs;
   if (bs != 64 && bs != 128) fail(SPAMM_E_UNSUPPORTED, "tensor-core precision forms are built for bs = 64 and 128");
-  const int64_t ntiles = M->nleaves * tc_tiles_per_leaf(bs), cap = (int64_t)ctx->num_sms * 8;
-  const unsigned grid = (unsigned)(ntiles < cap ? (ntiles > 0 ? ntiles : 1) : cap);
+  const int64_t ntiles = M->nleaves * tc_tiles_per_leaf(bs);
   *terms = alloc_n<uint8_t>(ctx, ntiles * (int64_t)form_leaf_bytes(prec));
   *expo = alloc_n<int32_t>(ctx, ntiles);
   if (M->nleaves == 0) return;
-  const double* pool = P<double>(M->pool);
-  const int64_t* slot = P<int64_t>(M->slot);
-  if (prec == SPAMM_PREC_BF16_SPLIT) {
-    prep_slices_kernel<3, FormCfg<SPAMM_PREC_BF16_SPLIT>::KPARTS><<<grid, kPrepThreads, 0, ctx->stream>>>(pool, slot, M->nleaves, bs, role,
-                                                                P<uint8_t>(*terms), P<int32_t>(*expo));
-    CK_LAUNCH("prep_slices_kernel<3>");
-  } else if (prec == SPAMM_PREC_BF16_SPLIT4) {
-    prep_slices_kernel<4, FormCfg<SPAMM_PREC_BF16_SPLIT4>::KPARTS><<<grid, kPrepThreads, 0, ctx->stream>>>(pool, slot, M->nleaves, bs, role,
-                                                               P<uint8_t>(*terms), P<int32_t>(*expo));
-    CK_LAUNCH("prep_slices_kernel<4>");
-  } else {
-    prep_fp16_kernel<<<grid, kPrepThreads, 0, ctx->stream>>>(pool, slot, M->nleaves, bs, role, P<uint8_t>(*terms),
-                                                    P<int32_t>(*expo));
-    CK_LAUNCH("prep_fp16_kernel");
-  }
+  const int64_t cap = (int64_t)ctx->num_sms * (bs == 64 ? 2 : 3);
+  const unsigned grid = (unsigned)(ntiles < cap ? ntiles : cap);
+  const bool staged = bs == 64;
+  const int smem = (int)((staged ? 2 * TileStream::kBytes : 0) + form_leaf_bytes(prec));
+  auto launch = [&](auto kern) {
+    CK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    kern<<<grid, kPrepThreads, smem, ctx->stream>>>(P<double>(M->pool), P<int64_t>(M->slot), M->nleaves, bs, role,
+                                                    P<uint8_t>(*terms), P<int32_t>(*expo), ctx->d_err);
+    CK_LAUNCH("prep_kernel");
+  };
+  auto form = [&](auto f) {
+    using Form = decltype(f);
+    if (staged)
+      launch(prep_kernel<Form, true>);
+    else
+      launch(prep_kernel<Form, false>);
+  };
+  if (prec == SPAMM_PREC_BF16_SPLIT)
+    form(SliceForm<SPAMM_PREC_BF16_SPLIT>());
+  else if (prec == SPAMM_PREC_BF16_SPLIT4)
+    form(SliceForm<SPAMM_PREC_BF16_SPLIT4>());
+  else
+    form(Fp16Form());
 }
 
 }  // namespace spamm
