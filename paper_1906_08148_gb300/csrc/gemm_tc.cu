@@ -68,9 +68,9 @@
 // between them is a look at a barrier in shared memory that takes some 250 cycles
 // beside the operand reads.  Measured on the 3-D lattices (GEMM only, CUDA events),
 // with the waits taken out of each role's way as the comments below say: 4 slices,
-// n = 65536, tau = 1e-6, 115.6 -> 94.4 ms (1666 TFLOP/s executed, near the chip's
-// power-limited rate); 3 slices, n = 16384, 8.19 -> 6.67 ms; FP16 with 128-leaves,
-// n = 20000, tau = 1e-4, 7.67 -> 5.78 ms.  With single parts left out the first takes
+// n = 65536, tau = 1e-6, 115.6 -> 93 ms (1.6 PFLOP/s executed, near the chip's
+// power-limited rate); 3 slices, n = 16384, 8.19 -> 6.37 ms; FP16 with 128-leaves,
+// n = 20000, tau = 1e-4, 7.67 -> 5.80 ms.  With single parts left out the first takes
 // 68 ms (MMAs alone), 51 (copies alone), 80 (without epilogue), 85 (without copies).
 #include "convert.cuh"
 #include "internal.cuh"
@@ -165,15 +165,15 @@ static_assert(kQuadBufs == 4, "acc_slot rotates four slots");
 // 8 KB of operands in the 64 cycles it computes, all that shared memory delivers
 // (128 B per clock), beside the copies into the next stage; where consecutive
 // MMAs use the same A piece, the first keeps it in the buffer (fill) and the
-// others read only B.  The sums in an accumulator that is not exact depend on
-// the order, so it is chosen per form:
-//   4 slices  the products of index sum 2 and 3 share one accumulator; A's terms
-//             from the last to the first in the first K-part and back in the last,
-//             each against every B term it meets: 16 reads of A instead of 40,
-//             and the exact accumulators are in use for the shortest time;
-//   3 slices  index sums 2 and 1 share one accumulator, the smaller products first,
-//             each product whole; the exact (0, 0) rides on the last product's A;
-//   FP16      one accumulator, h1 g0, h0 g1, h0 g0, each product whole.
+// others read only B.  The sum in an accumulator that is not exact depends on the
+// order, so that is fixed: the smaller products (the larger index sum) first, each
+// product whole, A's last term first.  (4 slices with each A term against all its B
+// terms, 16 reads of A instead of 32, is as fast and 7e-4 further off.)  The exact
+// products go wherever their accumulators are in use for the shortest time, as the
+// four slots are what the next step waits for: last in the first K-part, where they
+// ride on the A of the smallest index sum that shares an accumulator, and first in
+// the last one.  At the end of the last part instead they cost the 4-slice form 104 ms
+// for 93 (n = 65536), the 3-slice form 6.63 for 6.37 (n = 16384).
 struct MmaOrder {
   int n = 0;
   uint8_t i[48] = {}, j[48] = {}, ks[48] = {}, collect[48] = {};
@@ -189,25 +189,18 @@ template <int PREC>
 __host__ __device__ constexpr MmaOrder mma_order(bool last_part) {
   constexpr int T = FormCfg<PREC>::TERMS, KS = 4 / FormCfg<PREC>::KPARTS;
   MmaOrder o;
-  if (T == 4) {
-    for (int ii = 0; ii < T; ++ii) {
-      const int i = last_part ? ii : T - 1 - ii, m = T - i;
+  if (last_part && T > 2)  // the exact products
+    for (int i = 0; i < T - 2; ++i)
       for (int ks = 0; ks < KS; ++ks)
-        for (int jj = 0; jj < m; ++jj)
-          o.add(i, last_part ? jj : m - 1 - jj, ks,
-                m == 1 ? kCollectNone : jj == 0 ? kCollectFill : jj == m - 1 ? kCollectLast : kCollectUse);
-    }
-    return o;
-  }
-  for (int g = T - 1; g >= 0; --g)
-    for (int i = g; i >= 0; --i) {
-      if (T == 3 && g == 0) continue;
+        for (int j = 0; j < T - 2 - i; ++j)
+          o.add(i, j, ks, i == T - 3 ? kCollectNone : j == 0 ? kCollectFill : kCollectLast);
+  for (int g = T - 1; g >= (T > 2 ? T - 2 : 0); --g)
+    for (int i = g; i >= 0; --i)
       for (int ks = 0; ks < KS; ++ks) {
-        const bool share = T == 3 && g == 1 && i == 0;  // A term 0 also for the exact product
-        o.add(i, g - i, ks, share ? kCollectFill : kCollectNone);
-        if (share) o.add(0, 0, ks, kCollectLast);
+        const int exact = !last_part && g == T - 2 && i < g ? g - i : 0;  // exact products that ride on this A
+        o.add(i, g - i, ks, exact ? kCollectFill : kCollectNone);
+        for (int j = exact - 1; j >= 0; --j) o.add(i, j, ks, j == 0 ? kCollectLast : kCollectUse);
       }
-    }
   return o;
 }
 
