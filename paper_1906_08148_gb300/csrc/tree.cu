@@ -155,25 +155,140 @@ __device__ __forceinline__ int64_t block_compact(int64_t n, Flag flag, Place pla
   return base;
 }
 
-// One block per tree: the leaves (rules 1, 2), then the levels t0 - 1 .. 0.
-__global__ void __launch_bounds__(kTopThreads) tree_top_kernel(const __grid_constant__ TreePair P) {
-  const TreeDev& T = P.t[blockIdx.x];
-  int64_t n;
-  if (T.rule != 0) {
-    n = block_compact(T.n, [&](int64_t q) { return kept(T, q); }, [&](int64_t q, int64_t p) { place_leaf(T, q, p); });
-    if (threadIdx.x == 0) T.count[T.L] = (uint64_t)n;
-    __syncthreads();
-  } else {
-    n = (int64_t)T.count[T.t0];
+// The structure above level t0 in one pass over its nodes.  Node i starts a node on
+// every level from first_level on, so its position on level t is the number of nodes up
+// to i with first_level <= t: one ballot per 32 nodes and level, and a prefix over the
+// warps' counts, for all levels at once.
+__device__ __forceinline__ int first_level(uint32_t code, uint32_t prev, int64_t i, int t0) {
+  return i == 0 ? 0 : t0 - (31 - __clz((int)((code ^ prev) | 1u))) / 2;
+}
+// What node i (code; its predecessor's prev; first_level s) writes on the levels below
+// t0: its entries in the child links (before[t]: nodes of level t that start in earlier
+// groups of 32), the empty entries since its predecessor's, and its ancestors' codes.
+// Called by whole warps, lanes without a node with s = kNoNode.
+constexpr int kNoNode = 255;
+template <class Before>
+__device__ __forceinline__ void place_levels(const TreeDev& T, int64_t i, uint32_t code, uint32_t prev, int s, bool last,
+                                             Before before) {
+  const unsigned upto = 0xFFFFFFFFu >> (31 - (threadIdx.x & 31));  // this lane and those before
+  int64_t below = i;  // the node's position one level further down
+  for (int t = T.t0 - 1; t >= 0; --t) {
+    const unsigned b = __ballot_sync(0xffffffffu, s <= t);
+    const int64_t p = before(t) + __popc(b & upto) - 1;
+    const int shift = 2 * (T.t0 - t - 1);
+    const int digit = (int)(code >> shift & 3u), digit0 = (int)(prev >> shift & 3u);
+    if (s <= t + 1) {
+      int* ch = reinterpret_cast<int*>(T.ochild[t] + p);
+      for (int k = s <= t ? 0 : digit0 + 1; k < digit; ++k) ch[k] = -1;
+      ch[digit] = (int)below;
+      if (s <= t) {
+        if (i > 0)
+          for (int k = digit0 + 1; k < 4; ++k) ch[k - 4] = -1;  // the last parent's
+        T.ocode[t][p] = code >> shift >> 2;
+        below = p;
+      }
+    }
+    if (last)
+      for (int k = digit + 1; k < 4; ++k) reinterpret_cast<int*>(T.ochild[t] + p)[k] = -1;
   }
-  for (int t = T.t0; t >= 1; --t) {
-    const uint32_t* code = T.ocode[t];
-    n = block_compact(n, [&](int64_t q) { return first_child(code, q); },
-                      [&, nt = n](int64_t q, int64_t p) { place_parent(T, t, nt, q, p); });
-    if (threadIdx.x == 0) T.count[t - 1] = (uint64_t)n;
+}
+// Sum of a node's children's squared norms in the fixed order.
+__device__ __forceinline__ double child_sum(const int4& ch, const double* csq) {
+  double s = ch.x >= 0 ? csq[ch.x] : 0.0;
+  if (ch.y >= 0) s += csq[ch.y];
+  if (ch.z >= 0) s += csq[ch.z];
+  if (ch.w >= 0) s += csq[ch.w];
+  return s;
+}
+
+// One block per tree: the leaves (rules 1, 2), then the levels t0 - 1 .. 0, at most
+// kTopNodes nodes each.  The norms go level by level through shared memory, in place
+// (a parent's position is never above its children's), the next child links on the
+// way meanwhile.  All levels' structure in one pass instead of a flag, prefix and
+// placing pass per level: a tree of 1,500 leaves and six levels TREEFIG us.
+__global__ void __launch_bounds__(kTopThreads) tree_top_kernel(const __grid_constant__ TreePair P) {
+  constexpr int kGroups = (int)kTopNodes / 32;
+  __shared__ union {
+    uint32_t code[kTopNodes];
+    double sq[kTopNodes];
+  } s_node;
+  __shared__ uint32_t s_before[SPAMM_MAX_LEVELS][kGroups];
+  __shared__ int s_n[SPAMM_MAX_LEVELS];
+  const TreeDev& T = P.t[blockIdx.x];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, t0 = T.t0;
+  int n;
+  if (T.rule != 0) {
+    n = (int)block_compact(T.n, [&](int64_t q) { return kept(T, q); }, [&](int64_t q, int64_t p) {
+      place_leaf(T, q, p);
+      s_node.code[p] = T.code ? T.code[q] : (uint32_t)q;
+    });
+    if (threadIdx.x == 0) T.count[T.L] = (uint64_t)n;
+  } else {
+    n = (int)T.count[t0];
+    for (int i = threadIdx.x; i < n; i += kTopThreads) s_node.code[i] = T.ocode[t0][i];
+  }
+  __syncthreads();
+  auto node = [&](int i, uint32_t* code, uint32_t* prev) {
+    *code = i < n ? s_node.code[i] : 0;
+    *prev = i > 0 && i < n ? s_node.code[i - 1] : 0;
+    return i < n ? first_level(*code, *prev, i, t0) : kNoNode;
+  };
+  for (int g = warp; g < kGroups; g += kTopThreads / 32) {
+    uint32_t code, prev;
+    const int s = node(32 * g + lane, &code, &prev);
+    for (int t = 0; t < t0; ++t) {
+      const unsigned b = __ballot_sync(0xffffffffu, s <= t);
+      if (lane == 0) s_before[t][g] = (uint32_t)__popc(b);
+    }
+  }
+  __syncthreads();
+  if (warp < t0) {
+    constexpr int kPer = kGroups / 32;
+    uint32_t v[kPer], sum = 0;
+#pragma unroll
+    for (int k = 0; k < kPer; ++k) {
+      v[k] = sum;
+      sum += s_before[warp][kPer * lane + k];
+    }
+    uint32_t x = sum;
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+      const uint32_t y = __shfl_up_sync(0xffffffffu, x, off);
+      if (lane >= off) x += y;
+    }
+#pragma unroll
+    for (int k = 0; k < kPer; ++k) s_before[warp][kPer * lane + k] = x - sum + v[k];
+    if (lane == 31) {
+      s_n[warp] = (int)x;
+      T.count[warp] = x;
+    }
+  }
+  __syncthreads();
+  for (int g = warp; 32 * g < n; g += kTopThreads / 32) {
+    uint32_t code, prev;
+    const int i = 32 * g + lane, s = node(i, &code, &prev);
+    place_levels(T, i, code, prev, s, i == n - 1, [&](int t) { return (int64_t)s_before[t][g]; });
+  }
+  __syncthreads();
+  if (t0 == 0 || !T.osq[t0 - 1]) return;
+  constexpr int kPer = (int)kTopNodes / kTopThreads;
+  const int tid = threadIdx.x;
+  int4 ch = tid < s_n[t0 - 1] ? T.ochild[t0 - 1][tid] : make_int4(-1, -1, -1, -1);
+  const double* csq = T.osq[t0];
+  for (int t = t0 - 1; t >= 0; --t) {
+    const int nt = s_n[t];
+    const int4 next = t > 0 && tid < s_n[t - 1] ? T.ochild[t - 1][tid] : make_int4(-1, -1, -1, -1);
+    double v[kPer];
+#pragma unroll
+    for (int k = 0; k < kPer; ++k)
+      if (tid + k * kTopThreads < nt) v[k] = child_sum(k == 0 ? ch : T.ochild[t][tid + k * kTopThreads], csq);
+    if (t < t0 - 1) __syncthreads();  // every child's norm has been read
+#pragma unroll
+    for (int k = 0; k < kPer; ++k)
+      if (tid + k * kTopThreads < nt) T.osq[t][tid + k * kTopThreads] = s_node.sq[tid + k * kTopThreads] = v[k];
     __syncthreads();
-    sum_parents(T, t, 0, n);
-    __syncthreads();
+    ch = next;
+    csq = s_node.sq;
   }
 }
 
