@@ -1,21 +1,19 @@
 // tree.cu -- quadtree structure: the leaf set kept from sorted candidates
 // (truncation, builders), the levels above it and their squared norms.
 //
-// Every level is in Morton order, so each step works on runs: the kept leaves
-// are a compaction of the candidates, and the parents of a level are its runs of
-// equal code >> 2, a parent's children being consecutive nodes.  A step is a
-// prefix count over flags; the thread that sees the first child of a run also
-// sees the others (at most three nodes further on), so it writes the parent's
-// code and child links at once; the squared norms follow over the parents (an FP64
-// addition keeps a quarter SM's pipe for 64 cycles whether one lane needs it or 32).
+// Every level is in Morton order: the kept leaves are a compaction of the
+// candidates, and the parents of a level are its runs of equal code >> 2, a parent's
+// children being consecutive nodes.  The squared norms follow over the parents (an
+// FP64 addition keeps a quarter SM's pipe for 64 cycles whether one lane needs it or 32).
 //
-// Two forms.  Up to kTopNodes items one block of 1024 threads takes all steps
-// of a tree in one launch (a level of a few thousand nodes is a few microseconds
-// of latency for one block, about what a launch takes, and the host launches once
-// instead of five times per level): truncating both operands of a 4096-row lattice
-// (some 4000 leaves of 64 x 64 each, seven levels) takes 32 us instead of 360.  Larger
-// levels take two launches each, a count per tile of 1024 and the placing, where every
-// tile adds up the counts before it, until the level is small enough for the rest.
+// Two forms.  Up to kTopNodes items one block of 1024 threads takes a whole tree in
+// one launch, all levels' structure in one pass: truncating both operands of a 4096-row
+// lattice (some 4000 leaves of 64 x 64 each, seven levels) is 12.5 us of kernel, where
+// five launches per level took 360.  Larger levels take two launches each, a count per
+// tile of 1024 and the placing, where every tile adds up the counts before it, until
+// the level is small enough for the rest; there the thread that sees the first child of
+// a run also sees the others (at most three nodes further on), so it writes the
+// parent's code and child links at once.
 // Node counts stay on the device; the host reads them once (tree_resolve).
 #include <cmath>
 #include <cstring>
@@ -27,7 +25,6 @@ namespace spamm {
 namespace {
 
 constexpr int kTopThreads = 1024;
-constexpr int kTopPer = 4;  // items per thread and tile of the one-block form
 constexpr int64_t kTopNodes = 4096;
 constexpr int64_t kBoundNodes = 32768;  // up to here the leaf level is allocated for every candidate
 constexpr int kTileThreads = 256;
@@ -58,8 +55,13 @@ struct TreePair {
   TreeDev t[2];
 };
 
+// !(sq < smin) for squared norms (no negative values: they order like their bits, NaN
+// last), without an FP64 comparison.
+__device__ __forceinline__ bool kept_norm(double sq, double smin) {
+  return (uint64_t)__double_as_longlong(sq) >= (uint64_t)__double_as_longlong(smin);
+}
 __device__ __forceinline__ bool kept(const TreeDev& T, int64_t q) {
-  return T.rule == 1 ? T.keep[q] != 0 : !(T.sq[q] < T.smin);
+  return T.rule == 1 ? T.keep[q] != 0 : kept_norm(T.sq[q], T.smin);
 }
 __device__ __forceinline__ void place_leaf(const TreeDev& T, int64_t q, int64_t p) {
   T.ocode[T.L][p] = T.code ? T.code[q] : (uint32_t)q;
@@ -89,21 +91,20 @@ __device__ __forceinline__ void place_parent(const TreeDev& T, int t, int64_t n,
   T.ochild[t - 1][p] = make_int4(ch[0], ch[1], ch[2], ch[3]);
 }
 // ||A^t||_F^2 = sum of the children's squared norms, added in the fixed order
-// (0,0), (0,1), (1,0), (1,1) (Section 2): parents p0 .. p1 - 1 of level t - 1, by the block.
+// (0,0), (0,1), (1,0), (1,1) (Section 2).
+__device__ __forceinline__ double child_sum(const int4& ch, const double* csq) {
+  double s = ch.x >= 0 ? csq[ch.x] : 0.0;
+  if (ch.y >= 0) s += csq[ch.y];
+  if (ch.z >= 0) s += csq[ch.z];
+  if (ch.w >= 0) s += csq[ch.w];
+  return s;
+}
+
+// Parents p0 .. p1 - 1 of level t - 1, by the block.
 __device__ __forceinline__ void sum_parents(const TreeDev& T, int t, int64_t p0, int64_t p1) {
   double* out = T.osq[t - 1];
   if (!out) return;
-  const int4* child = T.ochild[t - 1];
-  const double* csq = T.osq[t];
-  for (int64_t p = p0 + threadIdx.x; p < p1; p += blockDim.x) {
-    const int4 ch = child[p];
-    double s = 0.0;
-    if (ch.x >= 0) s += csq[ch.x];
-    if (ch.y >= 0) s += csq[ch.y];
-    if (ch.z >= 0) s += csq[ch.z];
-    if (ch.w >= 0) s += csq[ch.w];
-    out[p] = s;
-  }
+  for (int64_t p = p0 + threadIdx.x; p < p1; p += blockDim.x) out[p] = child_sum(T.ochild[t - 1][p], T.osq[t]);
 }
 
 // Exclusive prefix of v over the block's threads, the sum in *total.
@@ -135,26 +136,6 @@ __device__ __forceinline__ uint32_t block_prefix(uint32_t v, uint32_t* total) {
   return before + x - v;
 }
 
-// Positions of the flagged items of [0, n), in order, by one block; returns their number.
-template <class Flag, class Place>
-__device__ __forceinline__ int64_t block_compact(int64_t n, Flag flag, Place place) {
-  int64_t base = 0;
-  for (int64_t b0 = 0; b0 < n; b0 += kTopThreads * kTopPer) {
-    const int64_t q0 = b0 + (int64_t)threadIdx.x * kTopPer;
-    unsigned f = 0;
-#pragma unroll
-    for (int i = 0; i < kTopPer; ++i)
-      if (q0 + i < n && flag(q0 + i)) f |= 1u << i;
-    uint32_t total;
-    int64_t p = base + block_prefix<kTopThreads>((uint32_t)__popc(f), &total);
-#pragma unroll
-    for (int i = 0; i < kTopPer; ++i)
-      if (f >> i & 1u) place(q0 + i, p++);
-    base += total;
-  }
-  return base;
-}
-
 // The structure above level t0 in one pass over its nodes.  Node i starts a node on
 // every level from first_level on, so its position on level t is the number of nodes up
 // to i with first_level <= t: one ballot per 32 nodes and level, and a prefix over the
@@ -162,52 +143,94 @@ __device__ __forceinline__ int64_t block_compact(int64_t n, Flag flag, Place pla
 __device__ __forceinline__ int first_level(uint32_t code, uint32_t prev, int64_t i, int t0) {
   return i == 0 ? 0 : t0 - (31 - __clz((int)((code ^ prev) | 1u))) / 2;
 }
-// What node i (code; its predecessor's prev; first_level s) writes on the levels below
-// t0: its entries in the child links (before[t]: nodes of level t that start in earlier
-// groups of 32), the empty entries since its predecessor's, and its ancestors' codes.
-// Called by whole warps, lanes without a node with s = kNoNode.
+// What node i (code; first_level s) writes on the levels below t0, whose child links
+// are empty (-1): its own and its ancestors' places in the links, its ancestors' codes.
+// before(t): nodes of level t that start in earlier groups of 32.  Called by whole
+// warps, lanes without a node with s = kNoNode; no level below the first on which no
+// lane starts a node has anything to write (of 32 leaves of a filled tree three levels).
 constexpr int kNoNode = 255;
 template <class Before>
-__device__ __forceinline__ void place_levels(const TreeDev& T, int64_t i, uint32_t code, uint32_t prev, int s, bool last,
-                                             Before before) {
+__device__ __forceinline__ void place_levels(const TreeDev& T, int i, uint32_t code, int s, Before before) {
   const unsigned upto = 0xFFFFFFFFu >> (31 - (threadIdx.x & 31));  // this lane and those before
-  int64_t below = i;  // the node's position one level further down
+  int below = i;  // the node's position one level further down
   for (int t = T.t0 - 1; t >= 0; --t) {
     const unsigned b = __ballot_sync(0xffffffffu, s <= t);
-    const int64_t p = before(t) + __popc(b & upto) - 1;
-    const int shift = 2 * (T.t0 - t - 1);
-    const int digit = (int)(code >> shift & 3u), digit0 = (int)(prev >> shift & 3u);
+    const int p = before(t) + __popc(b & upto) - 1;
     if (s <= t + 1) {
-      int* ch = reinterpret_cast<int*>(T.ochild[t] + p);
-      for (int k = s <= t ? 0 : digit0 + 1; k < digit; ++k) ch[k] = -1;
-      ch[digit] = (int)below;
-      if (s <= t) {
-        if (i > 0)
-          for (int k = digit0 + 1; k < 4; ++k) ch[k - 4] = -1;  // the last parent's
-        T.ocode[t][p] = code >> shift >> 2;
-        below = p;
-      }
+      reinterpret_cast<int*>(T.ochild[t] + p)[code & 3u] = below;
+      code >>= 2;
+      below = p;
+      if (s <= t) T.ocode[t][p] = code;
     }
-    if (last)
-      for (int k = digit + 1; k < 4; ++k) reinterpret_cast<int*>(T.ochild[t] + p)[k] = -1;
+    if (b == 0) break;
   }
 }
-// Sum of a node's children's squared norms in the fixed order.
-__device__ __forceinline__ double child_sum(const int4& ch, const double* csq) {
-  double s = ch.x >= 0 ? csq[ch.x] : 0.0;
-  if (ch.y >= 0) s += csq[ch.y];
-  if (ch.z >= 0) s += csq[ch.z];
-  if (ch.w >= 0) s += csq[ch.w];
-  return s;
+// Squared norms of the levels `top` .. 0 (count[t] <= kTopNodes nodes) by one block, from
+// those of level top + 1: level by level through `s` in place (a parent's position is
+// never above its children's).  Four levels' links are on their way ahead, each in
+// registers of its own (a copy would wait for its load).  A level of few nodes takes
+// some 950 cycles, nearly all of them its three dependent FP64 additions.
+template <class Child, class Sq>
+__device__ __forceinline__ void block_norms(int top, const int* count, Child child, Sq sq, double* s) {
+  constexpr int kAhead = 4, kPer = (int)kTopNodes / kTopThreads;
+  const int tid = threadIdx.x;
+  int4 ch[kAhead];
+  auto links = [&](int t) { return t >= 0 && tid < count[t] ? child(t)[tid] : make_int4(-1, -1, -1, -1); };
+#pragma unroll
+  for (int j = 0; j < kAhead; ++j) ch[j] = links(top - j);
+  const double* csq = sq(top + 1);
+  for (int t0 = top; t0 >= 0; t0 -= kAhead)
+#pragma unroll
+    for (int j = 0; j < kAhead; ++j) {
+      const int t = t0 - j;
+      if (t < 0) break;
+      const int nt = count[t];
+      double v[kPer];
+#pragma unroll
+      for (int k = 0; k < kPer; ++k)
+        if (tid + k * kTopThreads < nt) v[k] = child_sum(k == 0 ? ch[j] : child(t)[tid + k * kTopThreads], csq);
+      ch[j] = links(t - kAhead);
+      if (t < top) __syncthreads();  // every child's norm has been read
+      double* out = sq(t);
+#pragma unroll
+      for (int k = 0; k < kPer; ++k)
+        if (tid + k * kTopThreads < nt) out[tid + k * kTopThreads] = s[tid + k * kTopThreads] = v[k];
+      __syncthreads();
+      csq = s;
+    }
+}
+
+// Exclusive prefixes of the rows v[r][0 .. kGroups) of shared memory, warp r row r < rows;
+// the rows' sums in total[r].
+constexpr int kGroups = (int)kTopNodes / 32;
+__device__ __forceinline__ void group_prefixes(uint32_t (*v)[kGroups], int rows, int* total) {
+  constexpr int kPer = kGroups / 32;
+  const int lane = threadIdx.x & 31, r = threadIdx.x >> 5;
+  if (r >= rows) return;
+  uint32_t e[kPer], sum = 0;
+#pragma unroll
+  for (int k = 0; k < kPer; ++k) {
+    e[k] = sum;
+    sum += v[r][kPer * lane + k];
+  }
+  uint32_t x = sum;
+#pragma unroll
+  for (int off = 1; off < 32; off <<= 1) {
+    const uint32_t y = __shfl_up_sync(0xffffffffu, x, off);
+    if (lane >= off) x += y;
+  }
+#pragma unroll
+  for (int k = 0; k < kPer; ++k) v[r][kPer * lane + k] = x - sum + e[k];
+  if (lane == 31) total[r] = (int)x;
 }
 
 // One block per tree: the leaves (rules 1, 2), then the levels t0 - 1 .. 0, at most
-// kTopNodes nodes each.  The norms go level by level through shared memory, in place
-// (a parent's position is never above its children's), the next child links on the
-// way meanwhile.  All levels' structure in one pass instead of a flag, prefix and
-// placing pass per level: a tree of 1,500 leaves and six levels TREEFIG us.
+// kTopNodes nodes each.  One block lives on latency: every thread's loads of a phase
+// are in flight together, and groups of 32 nodes keep a warp's accesses together.  All
+// levels' structure in one pass, instead of a flag, prefix and placing pass per level:
+// truncating both 4,088-leaf operands of a 4096-row lattice 20.8 -> 12.5 us.
 __global__ void __launch_bounds__(kTopThreads) tree_top_kernel(const __grid_constant__ TreePair P) {
-  constexpr int kGroups = (int)kTopNodes / 32;
+  constexpr int kWarps = kTopThreads / 32, kPer = kGroups / kWarps;  // groups per warp
   __shared__ union {
     uint32_t code[kTopNodes];
     double sq[kTopNodes];
@@ -215,81 +238,85 @@ __global__ void __launch_bounds__(kTopThreads) tree_top_kernel(const __grid_cons
   __shared__ uint32_t s_before[SPAMM_MAX_LEVELS][kGroups];
   __shared__ int s_n[SPAMM_MAX_LEVELS];
   const TreeDev& T = P.t[blockIdx.x];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, t0 = T.t0;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, t0 = T.t0;
+  const unsigned earlier = (1u << lane) - 1u;
   int n;
   if (T.rule != 0) {
-    n = (int)block_compact(T.n, [&](int64_t q) { return kept(T, q); }, [&](int64_t q, int64_t p) {
-      place_leaf(T, q, p);
-      s_node.code[p] = T.code ? T.code[q] : (uint32_t)q;
+    const int cand = (int)T.n;
+    double sq[kPer] = {};
+    int64_t slot[kPer];
+    uint32_t code[kPer];
+    unsigned keep[kPer];
+    auto each = [&](auto f) {
+#pragma unroll
+      for (int k = 0; k < kPer; ++k) f(k, 32 * (warp + k * kWarps) + lane);
+    };
+    each([&](int k, int q) {
+      slot[k] = q;
+      code[k] = (uint32_t)q;
+      keep[k] = 1;
+      if (q < cand) sq[k] = T.sq[q];
     });
-    if (threadIdx.x == 0) T.count[T.L] = (uint64_t)n;
-  } else {
-    n = (int)T.count[t0];
-    for (int i = threadIdx.x; i < n; i += kTopThreads) s_node.code[i] = T.ocode[t0][i];
-  }
-  __syncthreads();
-  auto node = [&](int i, uint32_t* code, uint32_t* prev) {
-    *code = i < n ? s_node.code[i] : 0;
-    *prev = i > 0 && i < n ? s_node.code[i - 1] : 0;
-    return i < n ? first_level(*code, *prev, i, t0) : kNoNode;
-  };
-  for (int g = warp; g < kGroups; g += kTopThreads / 32) {
-    uint32_t code, prev;
-    const int s = node(32 * g + lane, &code, &prev);
-    for (int t = 0; t < t0; ++t) {
-      const unsigned b = __ballot_sync(0xffffffffu, s <= t);
-      if (lane == 0) s_before[t][g] = (uint32_t)__popc(b);
-    }
-  }
-  __syncthreads();
-  if (warp < t0) {
-    constexpr int kPer = kGroups / 32;
-    uint32_t v[kPer], sum = 0;
+    if (T.code) each([&](int k, int q) { if (q < cand) code[k] = T.code[q]; });
+    if (T.slot) each([&](int k, int q) { if (q < cand) slot[k] = T.slot[q]; });
+    if (T.rule == 1) each([&](int k, int q) { if (q < cand) keep[k] = T.keep[q]; });
+    if (T.rule == 2) each([&](int k, int) { keep[k] = kept_norm(sq[k], T.smin); });
+    each([&](int k, int q) { keep[k] = q < cand && keep[k]; });
 #pragma unroll
     for (int k = 0; k < kPer; ++k) {
-      v[k] = sum;
-      sum += s_before[warp][kPer * lane + k];
+      keep[k] = __ballot_sync(0xffffffffu, keep[k] != 0);
+      if (lane == 0) s_before[0][warp + k * kWarps] = (uint32_t)__popc(keep[k]);
     }
-    uint32_t x = sum;
+    __syncthreads();
+    group_prefixes(s_before, 1, s_n);
+    __syncthreads();
 #pragma unroll
-    for (int off = 1; off < 32; off <<= 1) {
-      const uint32_t y = __shfl_up_sync(0xffffffffu, x, off);
-      if (lane >= off) x += y;
-    }
+    for (int k = 0; k < kPer; ++k)
+      if (keep[k] >> lane & 1u) {
+        const int p = (int)s_before[0][warp + k * kWarps] + __popc(keep[k] & earlier);
+        s_node.code[p] = T.ocode[T.L][p] = code[k];
+        T.osq[T.L][p] = sq[k];
+        T.oslot[p] = slot[k];
+      }
+    n = s_n[0];
+    if (tid == 0) T.count[T.L] = (uint64_t)n;
+  } else {
+    n = (int)T.count[t0];
 #pragma unroll
-    for (int k = 0; k < kPer; ++k) s_before[warp][kPer * lane + k] = x - sum + v[k];
-    if (lane == 31) {
-      s_n[warp] = (int)x;
-      T.count[warp] = x;
-    }
+    for (int k = 0; k < kPer; ++k)
+      if (tid + k * kTopThreads < n) s_node.code[tid + k * kTopThreads] = T.ocode[t0][tid + k * kTopThreads];
   }
   __syncthreads();
-  for (int g = warp; 32 * g < n; g += kTopThreads / 32) {
-    uint32_t code, prev;
-    const int i = 32 * g + lane, s = node(i, &code, &prev);
-    place_levels(T, i, code, prev, s, i == n - 1, [&](int t) { return (int64_t)s_before[t][g]; });
+  uint32_t code[kPer];
+  int first[kPer];
+#pragma unroll
+  for (int k = 0; k < kPer; ++k) {
+    const int g = warp + k * kWarps, i = 32 * g + lane;
+    code[k] = i < n ? s_node.code[i] : 0;
+    first[k] = i < n ? first_level(code[k], i > 0 ? s_node.code[i - 1] : 0, i, t0) : kNoNode;
+    uint32_t c = 0;  // lane t: the group's nodes of level t
+    for (int t = t0 - 1; t >= 0; --t) {
+      const unsigned b = __ballot_sync(0xffffffffu, first[k] <= t);
+      if (b == 0) break;
+      if (lane == t) c = (uint32_t)__popc(b);
+    }
+    if (lane < t0) s_before[lane][g] = c;
+  }
+  __syncthreads();
+  group_prefixes(s_before, t0, s_n);
+  __syncthreads();
+  if (tid < t0) T.count[tid] = (uint64_t)s_n[tid];
+  for (int t = 0; t < t0; ++t)
+    for (int p = tid; p < s_n[t]; p += kTopThreads) T.ochild[t][p] = make_int4(-1, -1, -1, -1);
+  __syncthreads();
+#pragma unroll
+  for (int k = 0; k < kPer; ++k) {
+    const int g = warp + k * kWarps;
+    place_levels(T, 32 * g + lane, code[k], first[k], [&](int t) { return (int)s_before[t][g]; });
   }
   __syncthreads();
   if (t0 == 0 || !T.osq[t0 - 1]) return;
-  constexpr int kPer = (int)kTopNodes / kTopThreads;
-  const int tid = threadIdx.x;
-  int4 ch = tid < s_n[t0 - 1] ? T.ochild[t0 - 1][tid] : make_int4(-1, -1, -1, -1);
-  const double* csq = T.osq[t0];
-  for (int t = t0 - 1; t >= 0; --t) {
-    const int nt = s_n[t];
-    const int4 next = t > 0 && tid < s_n[t - 1] ? T.ochild[t - 1][tid] : make_int4(-1, -1, -1, -1);
-    double v[kPer];
-#pragma unroll
-    for (int k = 0; k < kPer; ++k)
-      if (tid + k * kTopThreads < nt) v[k] = child_sum(k == 0 ? ch : T.ochild[t][tid + k * kTopThreads], csq);
-    if (t < t0 - 1) __syncthreads();  // every child's norm has been read
-#pragma unroll
-    for (int k = 0; k < kPer; ++k)
-      if (tid + k * kTopThreads < nt) T.osq[t][tid + k * kTopThreads] = s_node.sq[tid + k * kTopThreads] = v[k];
-    __syncthreads();
-    ch = next;
-    csq = s_node.sq;
-  }
+  block_norms(t0 - 1, s_n, [&](int t) { return T.ochild[t]; }, [&](int t) { return T.osq[t]; }, s_node.sq);
 }
 
 // The tiled form of one step: t = L + 1 the candidates' compaction, else the
@@ -558,13 +585,7 @@ struct NormTree {
 
 __device__ __forceinline__ void node_norm(const NormTree& T, int t, int64_t p) {
   const int4 ch = T.child[t][p];
-  const double* csq = T.sq[t + 1];
-  double s = 0.0;
-  if (ch.x >= 0) s += csq[ch.x];
-  if (ch.y >= 0) s += csq[ch.y];
-  if (ch.z >= 0) s += csq[ch.z];
-  if (ch.w >= 0) s += csq[ch.w];
-  T.sq[t][p] = s;
+  T.sq[t][p] = child_sum(ch, T.sq[t + 1]);
 }
 
 // Height h above the leaves of every tree that has more than kTopNodes nodes there.
@@ -580,14 +601,22 @@ __global__ void norms_wide_kernel(const NormTree* __restrict__ tab, int ntrees, 
 }
 
 __global__ void __launch_bounds__(kTopThreads) norms_top_kernel(const NormTree* __restrict__ tab) {
+  __shared__ double s_sq[kTopNodes];
+  __shared__ const int4* s_child[SPAMM_MAX_LEVELS];
+  __shared__ double* s_out[SPAMM_MAX_LEVELS];
+  __shared__ int s_n[SPAMM_MAX_LEVELS];
   const NormTree& T = tab[blockIdx.x];
+  const int t = threadIdx.x;
   if (!T.count) return;  // no leaves
-  for (int t = (int)T.L - 1; t >= 0; --t) {
-    const int64_t n = (int64_t)T.count[t];
-    if (n > kTopNodes) continue;
-    for (int64_t p = threadIdx.x; p < n; p += kTopThreads) node_norm(T, t, p);
-    __syncthreads();
+  if (t <= T.L) {
+    s_child[t] = T.child[t];
+    s_out[t] = T.sq[t];
+    s_n[t] = (int)T.count[t];
   }
+  __syncthreads();
+  int top = (int)T.L - 1;
+  while (top >= 0 && s_n[top] > kTopNodes) --top;
+  if (top >= 0) block_norms(top, s_n, [&](int l) { return s_child[l]; }, [&](int l) { return s_out[l]; }, s_sq);
 }
 
 size_t norm_table_bytes(size_t ntrees) { return ntrees * sizeof(NormTree); }
