@@ -491,12 +491,17 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32)
 
 // The first `steps` level steps (at most four: 8^3 pairs, 4^3 groups at the last)
 // by one block, from the root pair; the last one's pairs and groups go to memory.  (A
-// fifth step of up to 4096 pairs takes one SM 25 us, two tiled launches 15.)
+// fifth step of up to 4096 pairs takes one SM 25 us, two tiled launches 15.)  One block
+// lives on latency: the node records of all its levels are fetched at once, one warp
+// takes the prefix of a step, and 32 warps share the groups.  Four steps 13 us
+// (15.2 with a record's fetch in every step, a prefix over the block and 16 warps).
 constexpr int kTopSteps = 4;
-constexpr int kTopThreads = 512;
+constexpr int kTopThreads = 1024;
 constexpr int kTopPairs = 512, kTopGroups = 64;
+constexpr int kTopNodes = 1 + 4 + 16 + 64;  // on the levels the steps start from
+__device__ __forceinline__ int top_node(int t) { return ((1 << 2 * t) - 1) / 3; }  // level t's first of them
 struct TopDev {
-  const uint64_t *nrootA, *nrootB;
+  const uint64_t *countA, *countB;  // nodes per level
   const NodeRec *recA[kTopSteps], *recB[kTopSteps];
   const double4 *normA[kTopSteps], *normB[kTopSteps];
   LevelInfo* lv;  // level t's entry at lv[t]
@@ -507,10 +512,11 @@ struct TopDev {
 struct TopShared {
   int32_t ta[2][kTopPairs], tb[2][kTopPairs];
   uint8_t mask[kTopPairs];
-  uint32_t cnt[4 * kTopGroups], off[4 * kTopGroups];
+  NodeRec recA[kTopNodes], recB[kTopNodes];
+  uint32_t cnt[4 * kTopGroups], off[4 * kTopGroups];  // off: prefix of cnt | (cnt > 0) << 20
   uint32_t gcode[2][kTopGroups];
   uint32_t gstart[2][kTopGroups + 1];
-  uint32_t ws[32];
+  uint32_t total;
   unsigned cand, border;
 };
 
@@ -518,7 +524,18 @@ __global__ void __launch_bounds__(kTopThreads)
     task_top_kernel(const __grid_constant__ TopDev T, int steps, TauScreen sc, double tau, int test) {
   __shared__ TopShared s;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  int Q = *T.nrootA > 0 && *T.nrootB > 0 ? 1 : 0, G = Q;  // the root pair is entered
+  int Q = *T.countA > 0 && *T.countB > 0 ? 1 : 0, G = Q;  // the root pair is entered
+  {
+    const int i = (int)threadIdx.x & 127;
+    const int t = i < 1 ? 0 : i < 5 ? 1 : i < 21 ? 2 : 3, m = i - top_node(t);
+    if (i < kTopNodes && t < steps) {
+      if (threadIdx.x < 128) {
+        if (m < (int64_t)T.countA[t]) s.recA[i] = T.recA[t][m];
+      } else if (threadIdx.x < 256) {
+        if (m < (int64_t)T.countB[t]) s.recB[i] = T.recB[t][m];
+      }
+    }
+  }
   if (threadIdx.x == 0) {
     s.ta[0][0] = s.tb[0][0] = 0;
     s.gcode[0][0] = 0;
@@ -529,13 +546,14 @@ __global__ void __launch_bounds__(kTopThreads)
   for (int t = 0; t < steps; ++t) {
     const int cur = t & 1, nxt = cur ^ 1;
     const bool out = t + 1 == steps;
+    const NodeRec *recA = s.recA + top_node(t), *recB = s.recB + top_node(t);
     if (threadIdx.x == 0) s.cand = s.border = 0;
     __syncthreads();
     // the children of every pair
     long long cand = 0, border = 0;
     for (int q = threadIdx.x; q < Q; q += kTopThreads) {
       const int32_t ia = s.ta[cur][q], ib = s.tb[cur][q];
-      s.mask[q] = (uint8_t)child_mask(T.recA[t][ia], T.recB[t][ib], T.normA[t] + ia, T.normB[t] + ib, sc, tau, test,
+      s.mask[q] = (uint8_t)child_mask(recA[ia], recB[ib], T.normA[t] + ia, T.normB[t] + ib, sc, tau, test,
                                       false, &cand, &border);
     }
     cand += __shfl_xor_sync(0xffffffffu, cand, 16);
@@ -559,33 +577,33 @@ __global__ void __launch_bounds__(kTopThreads)
     }
     __syncthreads();
     // offsets (low 20 bits) and indexes among the non-empty ones
-    const int i = threadIdx.x;
-    const uint32_t c = i < 4 * G ? s.cnt[i] : 0;
-    const uint32_t v = c | ((uint32_t)(c > 0) << 20);
-    uint32_t x = v;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
-      if (lane >= o) x += y;
-    }
-    if (lane == 31) s.ws[warp] = x;
-    __syncthreads();
     if (warp == 0) {
-      uint32_t w = lane < kTopThreads / 32 ? s.ws[lane] : 0;
+      constexpr int kPer = 4 * kTopGroups / 32;
+      uint32_t v[kPer], sum = 0;
+#pragma unroll
+      for (int k = 0; k < kPer; ++k) {
+        const int i = kPer * lane + k;
+        const uint32_t c = i < 4 * G ? s.cnt[i] : 0;
+        v[k] = sum;
+        sum += c | ((uint32_t)(c > 0) << 20);
+      }
+      uint32_t x = sum;
 #pragma unroll
       for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t y = __shfl_up_sync(0xffffffffu, w, o);
-        if (lane >= o) w += y;
+        const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
       }
-      if (lane < kTopThreads / 32) s.ws[lane] = w;
+#pragma unroll
+      for (int k = 0; k < kPer; ++k) s.off[kPer * lane + k] = x - sum + v[k];
+      if (lane == 31) s.total = x;
     }
     __syncthreads();
-    const uint32_t off = x - v + (warp ? s.ws[warp - 1] : 0u);
-    const uint32_t total = s.ws[kTopThreads / 32 - 1];
+    const uint32_t total = s.total;
     const int Q2 = (int)(total & 0xfffffu), G2 = (int)(total >> 20);
+    const int i = threadIdx.x;
     if (i < 4 * G) {
-      s.off[i] = off & 0xfffffu;
-      if (c) {
+      const uint32_t off = s.off[i];
+      if (s.cnt[i]) {
         const uint32_t gid = off >> 20, code = 4u * s.gcode[cur][i >> 2] + (uint32_t)(i & 3);
         if (out) {
           T.gcode[gid] = code;
@@ -606,21 +624,20 @@ __global__ void __launch_bounds__(kTopThreads)
       lv.groups = (unsigned long long)G2;
       lv.cand = s.cand;
     }
-    __syncthreads();
     int32_t* ta2 = out ? T.ta : s.ta[nxt];
     int32_t* tb2 = out ? T.tb : s.tb[nxt];
     for (int g = warp; g < G; g += kTopThreads / 32) {
       int base[4];
 #pragma unroll
-      for (int k = 0; k < 4; ++k) base[k] = (int)s.off[4 * g + k];
+      for (int k = 0; k < 4; ++k) base[k] = (int)(s.off[4 * g + k] & 0xfffffu);
       const int q1 = (int)s.gstart[cur][g + 1];
       for (int qb = (int)s.gstart[cur][g]; qb < q1; qb += 32) {
         const int q = qb + lane;
         const unsigned m = q < q1 ? s.mask[q] : 0u;
         int4 ca = make_int4(-1, -1, -1, -1), cb = ca;
         if (m) {
-          ca = rec_children(T.recA[t][s.ta[cur][q]]);
-          cb = rec_children(T.recB[t][s.tb[cur][q]]);
+          ca = rec_children(recA[s.ta[cur][q]]);
+          cb = rec_children(recB[s.tb[cur][q]]);
         }
         const unsigned lt = (1u << lane) - 1u;
 #pragma unroll
@@ -812,8 +829,8 @@ std::shared_ptr<TaskBuild> task_begin(spamm_mat A, spamm_mat B, double tau, int 
   }
   {
     TopDev T0{};
-    T0.nrootA = P<uint64_t>(A->dcount);
-    T0.nrootB = P<uint64_t>(B->dcount);
+    T0.countA = P<uint64_t>(A->dcount);
+    T0.countB = P<uint64_t>(B->dcount);
     for (int t = 0; t < top; ++t) {
       T0.recA[t] = recA[t];
       T0.recB[t] = recB[t];
