@@ -407,10 +407,7 @@ spamm_plan make_plan(spamm_ctx ctx, spamm_mat A, spamm_mat B, double tau, spamm_
   sk->lv[sk->L].count = p->T.ngroups;
   sk->lv[sk->L].code = p->T.gcode;
   uint64_t* counts = static_cast<uint64_t*>(ctx->h_pinned);
-  if (p->T.ngroups > 0) {
-    tree_skeleton(ctx, sk.get());
-    tree_counts_async(ctx, sk.get(), counts);
-  }
+  if (p->T.ngroups > 0) tree_skeleton(ctx, sk.get(), counts);
   CK(cudaEventRecord(ev[4], ctx->stream));
   if (!tensor) {
     p->poolA = At->pool;

@@ -159,14 +159,15 @@ struct TreeReq {
   double tau;
 };
 // Enqueues the building of k <= 2 trees.  The levels' counts are upper bounds and
-// nleaves is unset until the device counts are taken over (tree_resolve, or
-// tree_counts_async, a wait, tree_set_counts).
-void tree_from_candidates(spamm_ctx ctx, TreeReq* req, int k);
-void tree_resolve(spamm_ctx ctx, spamm_mat m);
+// nleaves is unset until the device counts are taken over: at once, with a wait, if
+// `resolve`, else later (tree_counts_async, or a kernel that writes them to the host's
+// memory; a wait; tree_set_counts).
+void tree_from_candidates(spamm_ctx ctx, TreeReq* req, int k, bool resolve);
 void tree_counts_async(spamm_ctx ctx, spamm_mat m, uint64_t* host);  // host: L + 1 pinned words
 void tree_set_counts(spamm_mat m, const uint64_t* host);
-// The levels above given leaf codes (count exact), without norms; counts as above.
-void tree_skeleton(spamm_ctx ctx, spamm_mat m);
+// The levels above given leaf codes (count exact), without norms; counts as above, also
+// written to `host` (L + 1 pinned words).
+void tree_skeleton(spamm_ctx ctx, spamm_mat m, uint64_t* host);
 // Squared norms of every level and the leaves' slots, for the levels' counts.
 void alloc_norms(spamm_mat m);
 // The parents' norms of several matrices whose structure and leaf norms exist:

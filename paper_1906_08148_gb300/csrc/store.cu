@@ -115,8 +115,7 @@ void set_leaves_compacted(spamm_mat m, int64_t ncand, const uint32_t* code, cons
     return;
   }
   TreeReq r{m, ncand, code, sq, slot, keep, 0.0};
-  tree_from_candidates(m->ctx, &r, 1);
-  tree_resolve(m->ctx, m);
+  tree_from_candidates(m->ctx, &r, 1, true);
 }
 
 void alloc_norms(spamm_mat m) {
@@ -157,8 +156,7 @@ spamm_mat truncate_block(spamm_mat in, double tau, spamm_ctx on) {
   spamm_mat out = view_of(ctx, in);
   if (in->nleaves > 0) {
     TreeReq r = block_request(out, in, tau);
-    tree_from_candidates(ctx, &r, 1);
-    tree_resolve(ctx, out);
+    tree_from_candidates(ctx, &r, 1, true);
   }
   return out;
 }
@@ -170,7 +168,7 @@ void truncate_pair(spamm_ctx ctx, spamm_mat A, spamm_mat B, double tau, spamm_ma
   *Bt = A == B ? *At : view_of(ctx, B);
   if (A->nleaves > 0) r[k++] = block_request(*At, A, tau);
   if (A != B && B->nleaves > 0) r[k++] = block_request(*Bt, B, tau);
-  if (k) tree_from_candidates(ctx, r, k);
+  if (k) tree_from_candidates(ctx, r, k, false);
 }
 
 // Error-controlled rule: drop the smallest leaves (ascending squared norm,

@@ -93,8 +93,12 @@ struct RecTable {
   RecLevel lv[2 * SPAMM_MAX_LEVELS];  // A's levels, then B's (if B is not A)
 };
 
-// Records of every level of both operands: block row y takes table entry y.
-__global__ void __launch_bounds__(256) node_rec_kernel(const __grid_constant__ RecTable T, int* err) {
+// Records of every level of both operands: block row y takes table entry y.  Clears the
+// `words` words that the steps count in.
+__global__ void __launch_bounds__(256)
+    node_rec_kernel(const __grid_constant__ RecTable T, unsigned* __restrict__ clear, int words, int* err) {
+  if (blockIdx.x == 0 && blockIdx.y == 0)
+    for (int i = threadIdx.x; i < words; i += blockDim.x) clear[i] = 0;
   const RecLevel& R = T.lv[blockIdx.y];
   const int64_t n = (int64_t)*R.n;
   for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < n; q += (int64_t)gridDim.x * blockDim.x) {
@@ -195,6 +199,11 @@ struct StepDev {
   uint64_t* tiles;       // per tile of groups: sum of packed
   uint32_t* tile_steps;  // leaf step: quad steps
   unsigned* ticket;      // blocks that have counted
+  // leaf step: the sizes of all levels and the operands' node counts for the host
+  const uint64_t* info;  // the LevelInfo entries as words
+  const uint64_t *countA, *countB;
+  uint64_t* host;        // pinned memory: levels (LevelInfo + 2 words)
+  int levels;
   int32_t *ta2, *tb2;    // outputs
   uint32_t* gcode2;
   int64_t* gstart2;
@@ -322,6 +331,14 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32)
     S.out->groups = s_tile >> 36;
     S.out->steps = s_cand;
   }
+  if (!LEAF) return;
+  // straight to the host's memory: three copies would take 3 us each
+  __syncthreads();
+  const int words = S.levels * (int)(sizeof(LevelInfo) / sizeof(uint64_t));
+  for (int i = threadIdx.x; i < words + 2 * S.levels; i += blockDim.x)
+    S.host[i] = i < words               ? __ldcg(S.info + i)
+                : i < words + S.levels ? S.countA[i - words]
+                                       : S.countB[i - words - S.levels];
 }
 
 // What the quad steps need beside the pairs (leaf step of the tensor-core forms).
@@ -728,16 +745,17 @@ std::shared_ptr<TaskBuild> task_begin(spamm_mat A, spamm_mat B, double tau, int 
   tb->B = B;
   const int L = A->L;
   uint64_t* host = static_cast<uint64_t*>(ctx->h_pinned);
-  auto finish_counts = [&](LevelInfo* dlv) {
-    // the level sizes and both operands' node counts, one wait
+  auto finish_counts = [&](LevelInfo* dlv, bool written) {
+    // the level sizes and both operands' node counts, one wait (written: by the leaf step's kernel)
     LevelInfo* hl = reinterpret_cast<LevelInfo*>(host);
     uint64_t* ha = reinterpret_cast<uint64_t*>(hl + (L + 1));
     uint64_t* hb = ha + (L + 1);
     static_assert((SPAMM_MAX_LEVELS) * (sizeof(LevelInfo) + 2 * sizeof(uint64_t)) <= 4096, "fits the pinned page");
-    if (dlv) CK(cudaMemcpyAsync(hl, dlv, (L + 1) * sizeof(LevelInfo), cudaMemcpyDeviceToHost, ctx->stream));
+    if (dlv && !written)
+      CK(cudaMemcpyAsync(hl, dlv, (L + 1) * sizeof(LevelInfo), cudaMemcpyDeviceToHost, ctx->stream));
     const bool pa = A->pending, pb = B != A && B->pending;
-    if (pa) tree_counts_async(ctx, A, ha);
-    if (pb) tree_counts_async(ctx, B, hb);
+    if (pa && !written) tree_counts_async(ctx, A, ha);
+    if (pb && !written) tree_counts_async(ctx, B, hb);
     if (dlv || pa || pb) CK(cudaStreamSynchronize(ctx->stream));
     if (pa) tree_set_counts(A, ha);
     if (pb) tree_set_counts(B, hb);
@@ -756,7 +774,7 @@ std::shared_ptr<TaskBuild> task_begin(spamm_mat A, spamm_mat B, double tau, int 
     T->nhalf = (int64_t)hl[L].half;
   };
   if (!A->dcount || !B->dcount) {  // an operand without leaves
-    finish_counts(nullptr);
+    finish_counts(nullptr, false);
     return tb;
   }
   const int nlev = L + 1;
@@ -765,12 +783,13 @@ std::shared_ptr<TaskBuild> task_begin(spamm_mat A, spamm_mat B, double tau, int 
   unsigned* tickets = reinterpret_cast<unsigned*>(lv + nlev);
   tb->keep.push_back(info);
   tb->lv = lv;
-  CK(cudaMemsetAsync(lv, 0, nlev * (sizeof(LevelInfo) + sizeof(unsigned)), ctx->stream));
+  const size_t clear = nlev * (sizeof(LevelInfo) + sizeof(unsigned));
   if (L == 0) {
+    CK(cudaMemsetAsync(lv, 0, clear, ctx->stream));
     root_test_kernel<<<1, 32, 0, ctx->stream>>>(P<uint64_t>(A->dcount), P<double>(A->lv[0].sq), P<uint64_t>(B->dcount),
                                                 P<double>(B->lv[0].sq), tau, test_norms, lv);
     CK_LAUNCH("root_test_kernel");
-    finish_counts(lv);
+    finish_counts(lv, false);
     return tb;
   }
   const TauScreen screen = make_screen(tau);
@@ -810,7 +829,8 @@ std::shared_ptr<TaskBuild> task_begin(spamm_mat A, spamm_mat B, double tau, int 
     int64_t g = (most + 255) / 256;
     const int64_t cap = (int64_t)ctx->num_sms * 8;
     if (g > cap) g = cap;
-    node_rec_kernel<<<dim3((unsigned)g, (unsigned)rows), 256, 0, ctx->stream>>>(tab, ctx->d_err);
+    node_rec_kernel<<<dim3((unsigned)g, (unsigned)rows), 256, 0, ctx->stream>>>(tab, reinterpret_cast<unsigned*>(lv),
+                                                                                  (int)(clear / sizeof(unsigned)), ctx->d_err);
     CK_LAUNCH("node_rec_kernel");
   }
   // the first steps in one block
@@ -874,6 +894,11 @@ std::shared_ptr<TaskBuild> task_begin(spamm_mat A, spamm_mat B, double tau, int 
     S.tiles = reinterpret_cast<uint64_t*>(w + mb + pb);
     S.tile_steps = reinterpret_cast<uint32_t*>(w + mb + pb + tbts);
     S.ticket = tickets + t;
+    S.info = reinterpret_cast<const uint64_t*>(lv);
+    S.countA = P<uint64_t>(A->dcount);
+    S.countB = P<uint64_t>(B->dcount);
+    S.host = host;
+    S.levels = nlev;
     if (leaf)
       task_count_kernel<true><<<tiles_grid(ctx, G, tg), kWarpsPerBlock * 32, 0, ctx->stream>>>(S, tg, screen, tau,
                                                                                               test_norms);
@@ -887,7 +912,7 @@ std::shared_ptr<TaskBuild> task_begin(spamm_mat A, spamm_mat B, double tau, int 
       tb->keep.push_back(ta);
       tb->keep.push_back(gc);
       tb->keep.push_back(work);
-      finish_counts(lv);
+      finish_counts(lv, true);
       break;
     }
     // capacities of the next level: exact after a wait, else the bounds 8 Q and 4 G

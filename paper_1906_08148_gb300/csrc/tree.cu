@@ -34,8 +34,9 @@ constexpr int64_t kTile = kTileThreads * kTilePer;
 // four loads per thread); more are scanned first.
 constexpr int64_t kTilesSummed = 1024;
 
-// One tree to build.  rule 0: the leaf level is given (code, *dn nodes); 1: leaf
-// q is kept iff keep[q]; 2: iff !(sq[q] < smin).  Levels t0 - 1 .. 0 are built.
+// One tree to build.  rule 0: level t0 is there (count[t0] nodes); 1: leaf q is kept iff
+// keep[q]; 2: iff !(sq[q] < smin); 3: the leaf level is there (n nodes).  Levels t0 - 1 .. 0
+// are built.
 struct TreeDev {
   int64_t n = 0;                   // candidates
   const uint32_t* code = nullptr;  // null: candidate q has code q
@@ -46,6 +47,7 @@ struct TreeDev {
   int rule = 0;
   int L = 0, t0 = 0;
   uint64_t* count = nullptr;  // nodes per level
+  uint64_t* host = nullptr;   // the same in pinned memory, for the host (null: not wanted)
   uint32_t* ocode[SPAMM_MAX_LEVELS] = {};
   double* osq[SPAMM_MAX_LEVELS] = {};  // null: no norms
   int4* ochild[SPAMM_MAX_LEVELS] = {};
@@ -241,7 +243,7 @@ __global__ void __launch_bounds__(kTopThreads) tree_top_kernel(const __grid_cons
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, t0 = T.t0;
   const unsigned earlier = (1u << lane) - 1u;
   int n;
-  if (T.rule != 0) {
+  if (T.rule == 1 || T.rule == 2) {
     const int cand = (int)T.n;
     double sq[kPer] = {};
     int64_t slot[kPer];
@@ -281,7 +283,8 @@ __global__ void __launch_bounds__(kTopThreads) tree_top_kernel(const __grid_cons
     n = s_n[0];
     if (tid == 0) T.count[T.L] = (uint64_t)n;
   } else {
-    n = (int)T.count[t0];
+    n = T.rule == 3 && t0 == T.L ? (int)T.n : (int)T.count[t0];
+    if (T.rule == 3 && tid == 0) T.count[T.L] = (uint64_t)T.n;
 #pragma unroll
     for (int k = 0; k < kPer; ++k)
       if (tid + k * kTopThreads < n) s_node.code[tid + k * kTopThreads] = T.ocode[t0][tid + k * kTopThreads];
@@ -306,6 +309,7 @@ __global__ void __launch_bounds__(kTopThreads) tree_top_kernel(const __grid_cons
   group_prefixes(s_before, t0, s_n);
   __syncthreads();
   if (tid < t0) T.count[tid] = (uint64_t)s_n[tid];
+  if (T.host && tid <= T.L) T.host[tid] = tid < t0 ? (uint64_t)s_n[tid] : T.count[tid];
   for (int t = 0; t < t0; ++t)
     for (int p = tid; p < s_n[t]; p += kTopThreads) T.ochild[t][p] = make_int4(-1, -1, -1, -1);
   __syncthreads();
@@ -331,7 +335,7 @@ __device__ __forceinline__ unsigned tile_flags(const TreeDev& T, int t, int64_t 
 
 __global__ void __launch_bounds__(kTileThreads)
     tile_count_kernel(const __grid_constant__ TreeDev T, int t, uint64_t* __restrict__ tiles) {
-  const int64_t n = t > T.L ? T.n : (int64_t)T.count[t];
+  const int64_t n = t > T.L || (t == T.L && T.rule == 3) ? T.n : (int64_t)T.count[t];
   const unsigned f = tile_flags(T, t, n, (int64_t)blockIdx.x * kTile + (int64_t)threadIdx.x * kTilePer);
   uint32_t total;
   block_prefix<kTileThreads>((uint32_t)__popc(f), &total);
@@ -359,7 +363,7 @@ __global__ void tile_total_kernel(const uint64_t* __restrict__ tiles, int64_t nt
 
 __global__ void __launch_bounds__(kTileThreads)
     tile_place_kernel(const __grid_constant__ TreeDev T, int t, const uint64_t* __restrict__ tiles, int64_t ntiles) {
-  const int64_t n = t > T.L ? T.n : (int64_t)T.count[t];
+  const int64_t n = t > T.L || (t == T.L && T.rule == 3) ? T.n : (int64_t)T.count[t];
   const int64_t q0 = (int64_t)blockIdx.x * kTile + (int64_t)threadIdx.x * kTilePer;
   const int64_t base = ntiles > kTilesSummed ? (int64_t)tiles[blockIdx.x] : tiles_before(tiles, blockIdx.x);
   const unsigned f = tile_flags(T, t, n, q0);
@@ -475,7 +479,7 @@ void tiled_levels(spamm_ctx ctx, TreeDev* T, int64_t n) {
 
 }  // namespace
 
-void tree_from_candidates(spamm_ctx ctx, TreeReq* req, int k) {
+void tree_from_candidates(spamm_ctx ctx, TreeReq* req, int k, bool resolve) {
   if (k > 2) fail(SPAMM_E_CUDA, "at most two trees are built at once");
   TreePair pair;
   BufP tiles[2];
@@ -529,18 +533,25 @@ void tree_from_candidates(spamm_ctx ctx, TreeReq* req, int k) {
     T.rule = 0;  // the one-block form starts above the leaves
     tiled_levels(ctx, &T, n);
   }
+  if (resolve)
+    for (int i = 0; i < k; ++i) pair.t[i].host = host + i * SPAMM_MAX_LEVELS;
   tree_top_kernel<<<k, kTopThreads, 0, ctx->stream>>>(pair);
   CK_LAUNCH("tree_top_kernel");
   for (int i = 0; i < k; ++i) req[i].m->pending = true;
+  if (!resolve) return;
+  CK(cudaStreamSynchronize(ctx->stream));
+  for (int i = 0; i < k; ++i) tree_set_counts(req[i].m, host + i * SPAMM_MAX_LEVELS);
 }
 
-void tree_skeleton(spamm_ctx ctx, spamm_mat m) {
+void tree_skeleton(spamm_ctx ctx, spamm_mat m, uint64_t* host) {
   const int64_t n = m->lv[m->L].count;
   alloc_levels(ctx, m, n, false, true);
-  CK(cudaMemcpyAsync(P<uint64_t>(m->dcount) + m->L, &n, sizeof(uint64_t), cudaMemcpyHostToDevice, ctx->stream));
   TreePair pair;
   TreeDev& T = pair.t[0];
   point_at(&T, m);
+  T.n = n;
+  T.rule = 3;
+  T.host = host;
   tiled_levels(ctx, &T, n);
   tree_top_kernel<<<1, kTopThreads, 0, ctx->stream>>>(pair);
   CK_LAUNCH("tree_top_kernel");
@@ -562,13 +573,6 @@ void tree_set_counts(spamm_mat m, const uint64_t* host) {
   }
   m->nleaves = (int64_t)host[m->L];
   m->pending = false;
-}
-
-void tree_resolve(spamm_ctx ctx, spamm_mat m) {
-  uint64_t* host = static_cast<uint64_t*>(ctx->h_pinned);
-  tree_counts_async(ctx, m, host);
-  CK(cudaStreamSynchronize(ctx->stream));
-  tree_set_counts(m, host);
 }
 
 // ------------------------------------------------------ norms of given trees
