@@ -529,22 +529,28 @@ void launch_gemm(spamm_ctx ctx, spamm_prec prec, int bs, const BatchDev& batch) 
     gemm_tc_batch(ctx, prec, batch);
 }
 
-// Kernel (d): an output's leaf norms and slots (tensor forms: and its elements).
-void finish_leaves(spamm_ctx ctx, spamm_prec prec, spamm_mat C) {
-  double* sq = P<double>(C->lv[C->L].sq);
-  if (prec != SPAMM_PREC_FP64)
-    tc_finish(ctx, prec, P<double>(C->pool), C->nleaves, C->bs, sq, P<int64_t>(C->slot));
-  else
-    leaf_sqnorms(ctx, P<double>(C->pool), nullptr, C->nleaves, C->bs, sq, nullptr, 0, P<int64_t>(C->slot));
+// Kernel (d): the outputs' leaf norms and slots (tensor forms: and their elements).
+void finish_leaves(spamm_ctx ctx, spamm_prec prec, const std::vector<spamm_mat>& ms, const OutBatch& out) {
+  if (prec != SPAMM_PREC_FP64) {
+    tc_finish(ctx, prec, out, ms[0]->bs);
+    return;
+  }
+  for (spamm_mat C : ms)
+    leaf_sqnorms(ctx, P<double>(C->pool), nullptr, C->nleaves, C->bs, P<double>(C->lv[C->L].sq), nullptr, 0,
+                 P<int64_t>(C->slot));
 }
+OutLeaves out_leaves(spamm_mat C) { return {P<double>(C->pool), P<double>(C->lv[C->L].sq), P<int64_t>(C->slot)}; }
 
 // The tables of a launch in one upload: the plans' views, the first unit of each (units
-// numbered consecutively), and the norm tables of `norm_mats`.
+// numbered consecutively), the claim counter, and the norm and leaf tables of the
+// outputs that the launch completes.
 template <class View, class Units>
-BatchDev upload_batch(spamm_ctx ctx, int64_t np, View view, Units units, const std::vector<spamm_mat>& norm_mats,
-                      NormBatch* norms, BufP* tables) {
-  const size_t pb = np * sizeof(PlanDev), ub = (np + 1) * sizeof(int64_t), nb = norm_table_bytes(norm_mats.size());
-  std::vector<uint8_t> host(pb + ub + nb);
+BatchDev upload_batch(spamm_ctx ctx, int64_t np, View view, Units units, const std::vector<spamm_mat>& outs,
+                      NormBatch* norms, OutBatch* leaves, BufP* tables) {
+  const size_t no = outs.size(), pb = np * sizeof(PlanDev), ub = (np + 1) * sizeof(int64_t);
+  const size_t at_work = pb + ub, at_norms = at_work + sizeof(unsigned long long);
+  const size_t at_leaves = at_norms + norm_table_bytes(no), at_first = at_leaves + no * sizeof(OutLeaves);
+  std::vector<uint8_t> host(at_first + no * sizeof(int64_t));
   *tables = alloc_bytes(ctx, host.size());
   uint8_t* dev = static_cast<uint8_t*>((*tables)->p);
   PlanDev* hp = reinterpret_cast<PlanDev*>(host.data());
@@ -554,10 +560,24 @@ BatchDev upload_batch(spamm_ctx ctx, int64_t np, View view, Units units, const s
     hp[r] = view(r);
     hu[r + 1] = hu[r] + units(r);
   }
-  if (norms) norm_tables(norm_mats, host.data() + pb + ub, dev + pb + ub, norms);
+  if (no) {
+    norm_tables(outs, host.data() + at_norms, dev + at_norms, norms);
+    OutLeaves* hl = reinterpret_cast<OutLeaves*>(host.data() + at_leaves);
+    int64_t* hf = reinterpret_cast<int64_t*>(host.data() + at_first);
+    leaves->only = out_leaves(outs[0]);
+    leaves->tab = reinterpret_cast<const OutLeaves*>(dev + at_leaves);
+    leaves->first = reinterpret_cast<const int64_t*>(dev + at_first);
+    leaves->n = (int)no;
+    for (size_t r = 0; r < no; ++r) {
+      hl[r] = out_leaves(outs[r]);
+      hf[r] = leaves->total;
+      leaves->total += outs[r]->nleaves;
+    }
+  }
   // a pageable source: the copy has read it by the time it returns
   CK(cudaMemcpyAsync(dev, host.data(), host.size(), cudaMemcpyHostToDevice, ctx->stream));
-  return BatchDev{reinterpret_cast<const PlanDev*>(dev), reinterpret_cast<const int64_t*>(dev + pb), (int)np, hu[np]};
+  return BatchDev{reinterpret_cast<const PlanDev*>(dev), reinterpret_cast<const int64_t*>(dev + pb), (int)np, hu[np],
+                  reinterpret_cast<unsigned long long*>(dev + at_work)};
 }
 
 // One persistent launch over all plans, then every output's norms.  Buffers are
@@ -580,15 +600,17 @@ std::vector<spamm_mat> execute_plans(spamm_ctx ctx, const std::vector<spamm_plan
     outp.push_back(pout.back().C.get());
   }
   NormBatch norms;
+  OutBatch leaves;
   BufP tables;
   const BatchDev batch = upload_batch(
-      ctx, np, [&](int64_t r) { return pout[r].dev; }, [&](int64_t r) { return pout[r].units; }, outp, &norms, &tables);
+      ctx, np, [&](int64_t r) { return pout[r].dev; }, [&](int64_t r) { return pout[r].units; }, outp, &norms, &leaves,
+      &tables);
 
   auto sequence = [&](unsigned evflags) {
     CK(cudaEventRecordWithFlags(ev[0], ctx->stream, evflags));
     launch_gemm(ctx, prec, bs, batch);
     CK(cudaEventRecordWithFlags(ev[1], ctx->stream, evflags));
-    for (int64_t r = 0; r < np; ++r) finish_leaves(ctx, prec, outp[r]);
+    finish_leaves(ctx, prec, outp, leaves);
     propagate_norms(ctx, norms);
     CK(cudaEventRecordWithFlags(ev[2], ctx->stream, evflags));
   };
@@ -807,7 +829,7 @@ spamm_status spamm_run(spamm_ctx ctx, int64_t njobs, const spamm_job* jobs, cons
       BufP tables;
       const BatchDev batch = upload_batch(
           ctx, np, [&](int64_t r) { return host[r]; }, [&](int64_t r) { return ubegin[r + 1] - ubegin[r]; }, {}, nullptr,
-          &tables);
+          nullptr, &tables);
       const cudaEvent_t* ev = ctx->events + 6;
       CK(cudaEventRecord(ev[0], ctx->stream));
       launch_gemm(ctx, prec, bs, batch);
@@ -842,7 +864,11 @@ spamm_status spamm_job_finish(spamm_ctx ctx, spamm_job job, spamm_mat* C, spamm_
     norm_tables({Cm}, host.data(), tab->p, &norms);
     CK(cudaMemcpyAsync(tab->p, host.data(), nb, cudaMemcpyHostToDevice, ctx->stream));
     CK(cudaEventRecord(ev[0], ctx->stream));
-    finish_leaves(ctx, job->plan->prec, Cm);
+    OutBatch leaves;
+    leaves.only = out_leaves(Cm);
+    leaves.n = 1;
+    leaves.total = Cm->nleaves;
+    finish_leaves(ctx, job->plan->prec, {Cm}, leaves);
     propagate_norms(ctx, norms);
     CK(cudaEventRecord(ev[1], ctx->stream));
     sync_and_check(ctx);

@@ -176,9 +176,7 @@ static void launch_tile(spamm_ctx ctx, const BatchDev& b) {
   const int64_t units = b.nunits / nq * ((BS / TILE) * (BS / TILE));
   int64_t grid = (int64_t)sms * per_sm;
   if (grid > units) grid = units;
-  unsigned long long* work = ctx->d_scratch + 8;
-  CK(cudaMemsetAsync(work, 0, sizeof(unsigned long long), ctx->stream));
-  kern<<<(unsigned)grid, kGemmThreads, smem, ctx->stream>>>(b, nq, work, ctx->d_err);
+  kern<<<(unsigned)grid, kGemmThreads, smem, ctx->stream>>>(b, nq, b.work, ctx->d_err);
   CK_LAUNCH("gemm_fp64_kernel");
 }
 

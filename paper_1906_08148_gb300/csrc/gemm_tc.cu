@@ -696,9 +696,7 @@ static void launch_quads(spamm_ctx ctx, const BatchDev& b) {
     CK(cudaFuncSetAttribute(gemm_quad_kernel<PREC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     ctx->tc_ready |= 1 << PREC;
   }
-  unsigned long long* work = ctx->d_scratch + 9;  // quad claim counter
-  CK(cudaMemsetAsync(work, 0, sizeof(unsigned long long), ctx->stream));
-  gemm_quad_kernel<PREC><<<gemm_grid(ctx, b.nunits), kQuadThreads, smem, ctx->stream>>>(b, work, ctx->d_err);
+  gemm_quad_kernel<PREC><<<gemm_grid(ctx, b.nunits), kQuadThreads, smem, ctx->stream>>>(b, b.work, ctx->d_err);
   CK_LAUNCH("gemm_quad_kernel");
 }
 
@@ -719,18 +717,23 @@ static void launch_quads(spamm_ctx ctx, const BatchDev& b) {
 // writes go to where the reads come from, so the compiler keeps their order and a
 // lane would wait for memory at every piece.  4088 leaves (134 MB, FP16 form): 313 ->
 // 45 us, 20023 leaves of 128 x 128 (2.6 GB) 1.50 -> 0.78 ms; with 64 leaves per block a few
-// thousand leaves kept a third of the SMs busy.
+// thousand leaves kept a third of the SMs busy.  All outputs of a batch in one launch:
+// a leaf's chain of additions takes 20 us however few leaves there are, and eight
+// outputs of 250 to 4088 leaves took 272 us one after the other; in one launch their
+// batch takes 2.76 ms instead of 2.88.
 constexpr int64_t kFinishLeavesPerBlock = 8;
 
 template <bool TWO>
-__global__ void __launch_bounds__(256) tc_finish_kernel(double* __restrict__ pool, int64_t m, int bs,
-                                                        double* __restrict__ sq, int64_t* __restrict__ slot) {
+__global__ void __launch_bounds__(256) tc_finish_kernel(const __grid_constant__ OutBatch out, int bs) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int64_t e = (int64_t)bs * bs;
   const int pairs = bs * bs / 2;
-  for (int64_t q = (int64_t)blockIdx.x * kFinishLeavesPerBlock + warp; q < m;
-       q += (int64_t)gridDim.x * kFinishLeavesPerBlock) {
-    uint4* leaf = reinterpret_cast<uint4*>(pool + q * e);
+  for (int64_t u = (int64_t)blockIdx.x * kFinishLeavesPerBlock + warp; u < out.total;
+       u += (int64_t)gridDim.x * kFinishLeavesPerBlock) {
+    const int r = out.n > 1 ? plan_of(out.first, out.n, u) : 0;
+    const OutLeaves C = out.n > 1 ? out.tab[r] : out.only;
+    const int64_t q = out.n > 1 ? u - out.first[r] : u;
+    uint4* leaf = reinterpret_cast<uint4*>(C.pool + q * e);
     double s = 0.0;
     for (int i = lane; i < pairs; i += 32 * 8) {
       uint64_t x[8][2];  // (hi, lo) of elements 2i and 2i + 1, then their values' bits
@@ -779,20 +782,20 @@ __global__ void __launch_bounds__(256) tc_finish_kernel(double* __restrict__ poo
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
     if (lane == 0) {
-      sq[q] = s;
-      slot[q] = q;
+      C.sq[q] = s;
+      C.slot[q] = q;
     }
   }
 }
 
-void tc_finish(spamm_ctx ctx, spamm_prec prec, double* pool, int64_t nleaves, int bs, double* sq, int64_t* slot) {
-  if (nleaves <= 0) return;
-  const int64_t nblk = (nleaves + kFinishLeavesPerBlock - 1) / kFinishLeavesPerBlock;
+void tc_finish(spamm_ctx ctx, spamm_prec prec, const OutBatch& out, int bs) {
+  if (out.total <= 0) return;
+  const int64_t nblk = (out.total + kFinishLeavesPerBlock - 1) / kFinishLeavesPerBlock;
   const unsigned grid = (unsigned)(nblk < (1ll << 30) ? nblk : (1ll << 30));
   if (prec == SPAMM_PREC_FP16_SCALED)
-    tc_finish_kernel<false><<<grid, 256, 0, ctx->stream>>>(pool, nleaves, bs, sq, slot);
+    tc_finish_kernel<false><<<grid, 256, 0, ctx->stream>>>(out, bs);
   else
-    tc_finish_kernel<true><<<grid, 256, 0, ctx->stream>>>(pool, nleaves, bs, sq, slot);
+    tc_finish_kernel<true><<<grid, 256, 0, ctx->stream>>>(out, bs);
   CK_LAUNCH("tc_finish_kernel");
 }
 

@@ -268,6 +268,7 @@ struct BatchDev {
   const int64_t* ubegin;  // nplans + 1 entries
   int nplans;
   int64_t nunits;
+  unsigned long long* work;  // claim counter, zero before the launch
 };
 // Plan owning unit u (the last r with ubegin[r] <= u).
 __device__ __forceinline__ int plan_of(const int64_t* __restrict__ ubegin, int nplans, int64_t u) {
@@ -294,7 +295,21 @@ BufP unit_order_longest(spamm_ctx ctx, const int64_t* start, int64_t n);
 void gemm_tc_batch(spamm_ctx ctx, spamm_prec prec, const BatchDev& b);
 // Kernel (d) of the tensor-core forms: the GEMM's two-float output slots to
 // FP64 in place, each leaf's squared norm (kernel (a)'s order) and its payload slot.
-void tc_finish(spamm_ctx ctx, spamm_prec prec, double* pool, int64_t nleaves, int bs, double* sq, int64_t* slot);
+// The outputs of a batch whose leaves are finished in one launch, leaves numbered
+// consecutively: output r's from first[r] on.
+struct OutLeaves {
+  double* pool;
+  double* sq;
+  int64_t* slot;
+};
+struct OutBatch {
+  OutLeaves only{};                // the output of a batch of one
+  const OutLeaves* tab = nullptr;  // on the device (more than one)
+  const int64_t* first = nullptr;
+  int n = 0;
+  int64_t total = 0;
+};
+void tc_finish(spamm_ctx ctx, spamm_prec prec, const OutBatch& out, int bs);
 // 64 x 64 operand tiles per leaf of the tensor forms (bs 64: 1, bs 128: 4).
 inline int tc_tiles_per_leaf(int bs) { return (bs / 64) * (bs / 64); }
 // Operand terms of a leaf set for a tensor form (role 0: used as A, 1: as B),
