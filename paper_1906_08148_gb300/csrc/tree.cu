@@ -9,16 +9,17 @@
 // Two forms.  Up to kTopNodes items one block of 1024 threads takes a whole tree in
 // one launch, all levels' structure in one pass: truncating both operands of a 4096-row
 // lattice (some 4000 leaves of 64 x 64 each, seven levels) is 12.5 us of kernel, where
-// five launches per level took 360.  Larger levels take two launches each, a count per
-// tile of 1024 and the placing, where every tile adds up the counts before it, until
-// the level is small enough for the rest; there the thread that sees the first child of
-// a run also sees the others (at most three nodes further on), so it writes the
-// parent's code and child links at once.
-// Node counts stay on the device; the host reads them once (tree_resolve).
+// five launches per level took 360; up to kBoundNodes a cluster of eight such blocks.
+// Larger levels take two launches each, a count per tile of 1024 and the placing, where
+// every tile adds up the counts before it, until the level is small enough for the rest;
+// there the thread that sees the first child of a run also sees the others (at most
+// three nodes further on), so it writes the parent's code and child links at once.
+// Node counts stay on the device; the host reads them once.
 #include <cmath>
 #include <cstring>
 
 #include "internal.cuh"
+#include "ptx.cuh"
 
 namespace spamm {
 
@@ -26,7 +27,7 @@ namespace {
 
 constexpr int kTopThreads = 1024;
 constexpr int64_t kTopNodes = 4096;
-constexpr int64_t kBoundNodes = 32768;  // up to here the leaf level is allocated for every candidate
+constexpr int64_t kBoundNodes = 32768;  // a cluster's; up to here the leaf level is allocated for every candidate
 constexpr int kTileThreads = 256;
 constexpr int kTilePer = 4;
 constexpr int64_t kTile = kTileThreads * kTilePer;
@@ -52,6 +53,7 @@ struct TreeDev {
   double* osq[SPAMM_MAX_LEVELS] = {};  // null: no norms
   int4* ochild[SPAMM_MAX_LEVELS] = {};
   int64_t* oslot = nullptr;
+  uint32_t* xchg = nullptr;  // cluster form: a row of counts per block
 };
 struct TreePair {
   TreeDev t[2];
@@ -226,11 +228,17 @@ __device__ __forceinline__ void group_prefixes(uint32_t (*v)[kGroups], int rows,
   if (lane == 31) total[r] = (int)x;
 }
 
-// One block per tree: the leaves (rules 1, 2), then the levels t0 - 1 .. 0, at most
-// kTopNodes nodes each.  One block lives on latency: every thread's loads of a phase
-// are in flight together, and groups of 32 nodes keep a warp's accesses together.  All
-// levels' structure in one pass, instead of a flag, prefix and placing pass per level:
-// truncating both 4,088-leaf operands of a 4096-row lattice 20.8 -> 12.5 us.
+// One block (or a cluster of CTAS blocks, of kTopNodes consecutive nodes each) per tree: the
+// leaves (rules 1, 2), then the levels t0 - 1 .. 0.  A block lives on latency: every
+// thread's loads of a phase are in flight together, and groups of 32 nodes keep a warp's
+// accesses together.  All levels' structure in one pass, instead of a flag, prefix and
+// placing pass per level: truncating both 4,088-leaf operands of a 4096-row lattice 20.8
+// -> 12.5 us.  The blocks of a cluster exchange their counts, of leaves and of all levels,
+// through global memory between cluster barriers and share the norms of the levels of
+// more than kTopNodes nodes: the tree of 12,000 leaves from triplets one launch instead of
+// eleven (the whole building 570 -> 526 us), a purification's three 2.61 -> 2.57 ms.
+constexpr int kXchgRow = SPAMM_MAX_LEVELS + 1;
+template <int CTAS>
 __global__ void __launch_bounds__(kTopThreads) tree_top_kernel(const __grid_constant__ TreePair P) {
   constexpr int kWarps = kTopThreads / 32, kPer = kGroups / kWarps;  // groups per warp
   __shared__ union {
@@ -238,10 +246,29 @@ __global__ void __launch_bounds__(kTopThreads) tree_top_kernel(const __grid_cons
     double sq[kTopNodes];
   } s_node;
   __shared__ uint32_t s_before[SPAMM_MAX_LEVELS][kGroups];
-  __shared__ int s_n[SPAMM_MAX_LEVELS];
-  const TreeDev& T = P.t[blockIdx.x];
+  __shared__ int s_n[SPAMM_MAX_LEVELS], s_base[SPAMM_MAX_LEVELS];
+  const TreeDev& T = P.t[blockIdx.x / CTAS];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, t0 = T.t0;
+  const int cta = (int)blockIdx.x % CTAS, node0 = cta * (int)kTopNodes;
   const unsigned earlier = (1u << lane) - 1u;
+  auto sync_all = [] {
+    if (CTAS > 1)
+      cluster_sync();
+    else
+      __syncthreads();
+  };
+  // v of every block in column `col`: the sum over the earlier blocks, all blocks' in *total
+  auto exchanged = [&](int col, int* total) {
+    int before = 0, all = 0;
+#pragma unroll
+    for (int c = 0; c < CTAS; ++c) {
+      const int v = (int)__ldcg(T.xchg + c * kXchgRow + col);
+      before += c < cta ? v : 0;
+      all += v;
+    }
+    *total = all;
+    return before;
+  };
   int n;
   if (T.rule == 1 || T.rule == 2) {
     const int cand = (int)T.n;
@@ -251,7 +278,7 @@ __global__ void __launch_bounds__(kTopThreads) tree_top_kernel(const __grid_cons
     unsigned keep[kPer];
     auto each = [&](auto f) {
 #pragma unroll
-      for (int k = 0; k < kPer; ++k) f(k, 32 * (warp + k * kWarps) + lane);
+      for (int k = 0; k < kPer; ++k) f(k, node0 + 32 * (warp + k * kWarps) + lane);
     };
     each([&](int k, int q) {
       slot[k] = q;
@@ -272,31 +299,45 @@ __global__ void __launch_bounds__(kTopThreads) tree_top_kernel(const __grid_cons
     __syncthreads();
     group_prefixes(s_before, 1, s_n);
     __syncthreads();
+    int p0 = 0;
+    n = s_n[0];
+    if (CTAS > 1) {
+      if (tid == 0) T.xchg[cta * kXchgRow + SPAMM_MAX_LEVELS] = (uint32_t)n;
+      cluster_sync();
+      p0 = exchanged(SPAMM_MAX_LEVELS, &n);
+    }
 #pragma unroll
     for (int k = 0; k < kPer; ++k)
       if (keep[k] >> lane & 1u) {
-        const int p = (int)s_before[0][warp + k * kWarps] + __popc(keep[k] & earlier);
-        s_node.code[p] = T.ocode[T.L][p] = code[k];
+        const int p = p0 + (int)s_before[0][warp + k * kWarps] + __popc(keep[k] & earlier);
+        if (CTAS == 1) s_node.code[p] = code[k];
+        T.ocode[T.L][p] = code[k];
         T.osq[T.L][p] = sq[k];
         T.oslot[p] = slot[k];
       }
-    n = s_n[0];
-    if (tid == 0) T.count[T.L] = (uint64_t)n;
+    if (cta == 0 && tid == 0) T.count[T.L] = (uint64_t)n;
   } else {
     n = T.rule == 3 && t0 == T.L ? (int)T.n : (int)T.count[t0];
-    if (T.rule == 3 && tid == 0) T.count[T.L] = (uint64_t)T.n;
+    if (T.rule == 3 && cta == 0 && tid == 0) T.count[T.L] = (uint64_t)T.n;
+    if (CTAS == 1)
 #pragma unroll
-    for (int k = 0; k < kPer; ++k)
-      if (tid + k * kTopThreads < n) s_node.code[tid + k * kTopThreads] = T.ocode[t0][tid + k * kTopThreads];
+      for (int k = 0; k < kPer; ++k)
+        if (tid + k * kTopThreads < n) s_node.code[tid + k * kTopThreads] = T.ocode[t0][tid + k * kTopThreads];
   }
-  __syncthreads();
-  uint32_t code[kPer];
+  sync_all();
+  uint32_t code[kPer], prev[kPer];
   int first[kPer];
 #pragma unroll
   for (int k = 0; k < kPer; ++k) {
-    const int g = warp + k * kWarps, i = 32 * g + lane;
-    code[k] = i < n ? s_node.code[i] : 0;
-    first[k] = i < n ? first_level(code[k], i > 0 ? s_node.code[i - 1] : 0, i, t0) : kNoNode;
+    const int i = node0 + 32 * (warp + k * kWarps) + lane;
+    auto at = [&](int j) { return CTAS == 1 ? s_node.code[j] : __ldcg(T.ocode[t0] + j); };
+    code[k] = i < n ? at(i) : 0;
+    prev[k] = i > 0 && i < n ? at(i - 1) : 0;
+  }
+#pragma unroll
+  for (int k = 0; k < kPer; ++k) {
+    const int g = warp + k * kWarps, i = node0 + 32 * g + lane;
+    first[k] = i < n ? first_level(code[k], prev[k], i, t0) : kNoNode;
     uint32_t c = 0;  // lane t: the group's nodes of level t
     for (int t = t0 - 1; t >= 0; --t) {
       const unsigned b = __ballot_sync(0xffffffffu, first[k] <= t);
@@ -308,19 +349,62 @@ __global__ void __launch_bounds__(kTopThreads) tree_top_kernel(const __grid_cons
   __syncthreads();
   group_prefixes(s_before, t0, s_n);
   __syncthreads();
-  if (tid < t0) T.count[tid] = (uint64_t)s_n[tid];
-  if (T.host && tid <= T.L) T.host[tid] = tid < t0 ? (uint64_t)s_n[tid] : T.count[tid];
+  if (CTAS > 1) {
+    if (tid < t0) T.xchg[cta * kXchgRow + tid] = (uint32_t)s_n[tid];
+    cluster_sync();
+    if (tid < t0) s_base[tid] = exchanged(tid, &s_n[tid]);
+    __syncthreads();
+  }
+  if (cta == 0) {
+    if (tid < t0) T.count[tid] = (uint64_t)s_n[tid];
+    if (T.host && tid <= T.L) T.host[tid] = tid < t0 ? (uint64_t)s_n[tid] : T.count[tid];
+  }
   for (int t = 0; t < t0; ++t)
-    for (int p = tid; p < s_n[t]; p += kTopThreads) T.ochild[t][p] = make_int4(-1, -1, -1, -1);
-  __syncthreads();
+    for (int p = cta * kTopThreads + tid; p < s_n[t]; p += CTAS * kTopThreads)
+      T.ochild[t][p] = make_int4(-1, -1, -1, -1);
+  sync_all();
 #pragma unroll
   for (int k = 0; k < kPer; ++k) {
     const int g = warp + k * kWarps;
-    place_levels(T, 32 * g + lane, code[k], first[k], [&](int t) { return (int)s_before[t][g]; });
+    place_levels(T, node0 + 32 * g + lane, code[k], first[k],
+                 [&](int t) { return (CTAS > 1 ? s_base[t] : 0) + (int)s_before[t][g]; });
   }
-  __syncthreads();
+  sync_all();
   if (t0 == 0 || !T.osq[t0 - 1]) return;
-  block_norms(t0 - 1, s_n, [&](int t) { return T.ochild[t]; }, [&](int t) { return T.osq[t]; }, s_node.sq);
+  int top = t0 - 1;
+  if (CTAS > 1) {
+    for (; top >= 0 && s_n[top] > kTopNodes; --top) {
+      for (int p = cta * kTopThreads + tid; p < s_n[top]; p += CTAS * kTopThreads)
+        T.osq[top][p] = child_sum(T.ochild[top][p], T.osq[top + 1]);
+      cluster_sync();
+    }
+    if (cta != 0) return;
+  }
+  block_norms(top, s_n, [&](int t) { return T.ochild[t]; }, [&](int t) { return T.osq[t]; }, s_node.sq);
+}
+
+// The trees of at most kTopNodes nodes each on level t0 (or candidates) one block each, else
+// clusters.
+void launch_top(spamm_ctx ctx, TreePair* pair, int k, int64_t most) {
+  if (most <= kTopNodes) {
+    tree_top_kernel<1><<<k, kTopThreads, 0, ctx->stream>>>(*pair);
+  } else {
+    constexpr int kCtas = (int)(kBoundNodes / kTopNodes);
+    BufP xchg = alloc_n<uint32_t>(ctx, k * kCtas * kXchgRow);
+    for (int i = 0; i < k; ++i) pair->t[i].xchg = P<uint32_t>(xchg) + i * kCtas * kXchgRow;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(k * kCtas);
+    cfg.blockDim = dim3(kTopThreads);
+    cfg.stream = ctx->stream;
+    cudaLaunchAttribute at = {};
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = kCtas;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    CK(cudaLaunchKernelEx(&cfg, tree_top_kernel<kCtas>, *pair));
+  }
+  CK_LAUNCH("tree_top_kernel");
 }
 
 // The tiled form of one step: t = L + 1 the candidates' compaction, else the
@@ -465,16 +549,17 @@ void tiled_step(spamm_ctx ctx, const TreeDev& T, int t, int64_t n, uint64_t* til
   CK_LAUNCH("tile_place_kernel");
 }
 
-// The levels above level t0 (at most n nodes there), large ones in tiles; T.t0
-// is left at the level the one-block form starts from.
-void tiled_levels(spamm_ctx ctx, TreeDev* T, int64_t n) {
+// The levels above the leaves (at most n), large ones in tiles; T.t0 is left at the
+// level that tree_top_kernel starts from, whose nodes are at most the result.
+int64_t tiled_levels(spamm_ctx ctx, TreeDev* T, int64_t n) {
   int t = T->L;
   int64_t cap = n;
-  if (cap > kTopNodes) {
+  if (cap > kBoundNodes) {
     BufP tiles = alloc_n<uint64_t>(ctx, (cap + kTile - 1) / kTile);
-    for (; t >= 1 && cap > kTopNodes; --t, cap = level_cap(n, t)) tiled_step(ctx, *T, t, cap, P<uint64_t>(tiles));
+    for (; t >= 1 && cap > kBoundNodes; --t, cap = level_cap(n, t)) tiled_step(ctx, *T, t, cap, P<uint64_t>(tiles));
   }
   T->t0 = t;
+  return cap;
 }
 
 }  // namespace
@@ -483,7 +568,8 @@ void tree_from_candidates(spamm_ctx ctx, TreeReq* req, int k, bool resolve) {
   if (k > 2) fail(SPAMM_E_CUDA, "at most two trees are built at once");
   TreePair pair;
   BufP tiles[2];
-  bool wide[2] = {false, false}, exact[2] = {false, false};
+  bool wide[2] = {false, false};
+  int64_t most = 0;
   uint64_t* host = static_cast<uint64_t*>(ctx->h_pinned);
   for (int i = 0; i < k; ++i) {
     TreeReq& r = req[i];
@@ -497,46 +583,42 @@ void tree_from_candidates(spamm_ctx ctx, TreeReq* req, int k, bool resolve) {
     T.smin = r.keep ? 0.0 : least_kept(r.tau);
     T.L = r.m->L;
     T.t0 = T.L;
-    wide[i] = r.n > kTopNodes;
-    exact[i] = r.n > kBoundNodes;
-    if (!exact[i]) {
+    wide[i] = r.n > kBoundNodes;
+    if (!wide[i]) {
+      most = r.n > most ? r.n : most;
       alloc_levels(ctx, r.m, r.n, true, false);
       point_at(&T, r.m);
+      continue;
     }
-    if (wide[i]) {
-      const int64_t ntiles = (r.n + kTile - 1) / kTile;
-      tiles[i] = alloc_n<uint64_t>(ctx, ntiles);
-      tile_count_kernel<<<(unsigned)ntiles, kTileThreads, 0, ctx->stream>>>(T, T.L + 1, P<uint64_t>(tiles[i]));
-      CK_LAUNCH("tile_count_kernel");
-      // of many candidates the exact leaf count first: the leaf level may be much smaller
-      BufP total = exact[i] ? alloc_n<uint64_t>(ctx, 1) : BufP();
-      if (ntiles > kTilesSummed) {
-        scan_exclusive_u64(ctx, P<uint64_t>(tiles[i]), P<uint64_t>(tiles[i]), ntiles, P<uint64_t>(total));
-      } else if (exact[i]) {
-        tile_total_kernel<<<1, 1024, 0, ctx->stream>>>(P<uint64_t>(tiles[i]), ntiles, P<uint64_t>(total));
-        CK_LAUNCH("tile_total_kernel");
-      }
-      if (exact[i])
-        CK(cudaMemcpyAsync(host + i, P<uint64_t>(total), sizeof(uint64_t), cudaMemcpyDeviceToHost, ctx->stream));
+    // of many candidates the exact leaf count first: the leaf level may be much smaller
+    const int64_t ntiles = (r.n + kTile - 1) / kTile;
+    tiles[i] = alloc_n<uint64_t>(ctx, ntiles);
+    tile_count_kernel<<<(unsigned)ntiles, kTileThreads, 0, ctx->stream>>>(T, T.L + 1, P<uint64_t>(tiles[i]));
+    CK_LAUNCH("tile_count_kernel");
+    BufP total = alloc_n<uint64_t>(ctx, 1);
+    if (ntiles > kTilesSummed) {
+      scan_exclusive_u64(ctx, P<uint64_t>(tiles[i]), P<uint64_t>(tiles[i]), ntiles, P<uint64_t>(total));
+    } else {
+      tile_total_kernel<<<1, 1024, 0, ctx->stream>>>(P<uint64_t>(tiles[i]), ntiles, P<uint64_t>(total));
+      CK_LAUNCH("tile_total_kernel");
     }
+    CK(cudaMemcpyAsync(host + i, P<uint64_t>(total), sizeof(uint64_t), cudaMemcpyDeviceToHost, ctx->stream));
   }
-  if (exact[0] || exact[1]) CK(cudaStreamSynchronize(ctx->stream));
+  if (wide[0] || wide[1]) CK(cudaStreamSynchronize(ctx->stream));
   for (int i = 0; i < k; ++i) {
     if (!wide[i]) continue;
     TreeDev& T = pair.t[i];
-    const int64_t n = exact[i] ? (int64_t)host[i] : T.n;
-    if (exact[i]) {
-      alloc_levels(ctx, req[i].m, n, true, false);
-      point_at(&T, req[i].m);
-    }
+    const int64_t n = (int64_t)host[i];
+    alloc_levels(ctx, req[i].m, n, true, false);
+    point_at(&T, req[i].m);
     tiled_step(ctx, T, T.L + 1, T.n, P<uint64_t>(tiles[i]));
-    T.rule = 0;  // the one-block form starts above the leaves
-    tiled_levels(ctx, &T, n);
+    T.rule = 0;  // tree_top_kernel starts above the leaves
+    const int64_t cap = tiled_levels(ctx, &T, n);
+    most = cap > most ? cap : most;
   }
   if (resolve)
     for (int i = 0; i < k; ++i) pair.t[i].host = host + i * SPAMM_MAX_LEVELS;
-  tree_top_kernel<<<k, kTopThreads, 0, ctx->stream>>>(pair);
-  CK_LAUNCH("tree_top_kernel");
+  launch_top(ctx, &pair, k, most);
   for (int i = 0; i < k; ++i) req[i].m->pending = true;
   if (!resolve) return;
   CK(cudaStreamSynchronize(ctx->stream));
@@ -552,9 +634,7 @@ void tree_skeleton(spamm_ctx ctx, spamm_mat m, uint64_t* host) {
   T.n = n;
   T.rule = 3;
   T.host = host;
-  tiled_levels(ctx, &T, n);
-  tree_top_kernel<<<1, kTopThreads, 0, ctx->stream>>>(pair);
-  CK_LAUNCH("tree_top_kernel");
+  launch_top(ctx, &pair, 1, tiled_levels(ctx, &T, n));
   m->pending = true;
 }
 
