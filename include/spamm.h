@@ -361,11 +361,11 @@ typedef enum {
 SPAMM_API spamm_status spamm_set_claim_order(spamm_ctx ctx, int order);
 
 /* enable != 0: spamm_execute / spamm_multiply run their execute phase (the
- * persistent leaf-product launch of every plan in the batch, then the output
- * quadtrees' parent norms, one launch per level for the whole batch) as one
- * captured CUDA graph.  Output buffers are allocated and the batch tables
- * uploaded before the capture, so the captured sequence holds kernels and
- * timing events only.  Results are identical either way.  Default 0. */
+ * persistent leaf-product launch of every plan in the batch, then the outputs'
+ * leaves and quadtree norms for the whole batch) as one captured CUDA graph.
+ * Output buffers are allocated and the batch tables uploaded before the
+ * capture, so the captured sequence holds kernels and timing events only.
+ * Results are identical either way.  Default 0. */
 SPAMM_API spamm_status spamm_set_exec_graph(spamm_ctx ctx, int enable);
 
 /* Graph mode keeps the last instantiated graph in the context and, for the

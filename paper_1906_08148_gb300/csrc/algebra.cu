@@ -228,9 +228,10 @@ double trace_of(spamm_mat X) {
                                                                     P<uint32_t>(X->lv[X->L].code), m, X->bs,
                                                                     P<double>(part));
   CK_LAUNCH("leaf_trace_kernel");
-  const double t = device_sum(ctx, P<double>(part), m);
+  double* sum = static_cast<double*>(ctx->h_pinned);
+  device_sum_async(ctx, P<double>(part), m, sum);
   sync_and_check(ctx);
-  return t;
+  return *sum;
 }
 
 }  // namespace spamm

@@ -195,7 +195,8 @@ spamm_mat truncate_error_controlled(spamm_mat in, double tau, spamm_ctx on = nul
 void leaf_sqnorms(spamm_ctx ctx, const double* pool, const int64_t* slot, int64_t nleaves, int bs, double* sq,
                   uint8_t* nonzero, int check_finite, int64_t* slot_out = nullptr);
 double error_fro(spamm_mat X, spamm_mat Y);
-double device_sum(spamm_ctx ctx, const double* in, int64_t n);  // deterministic reduction, synchronises
+// Deterministic sum into pinned memory, valid after the caller's wait (0 at once for n = 0).
+void device_sum_async(spamm_ctx ctx, const double* in, int64_t n, double* host);
 
 // ---- purification-chain operations (algebra.cu) ----
 spamm_mat add_scaled(double alpha, spamm_mat X, double beta, spamm_mat Y, spamm_ctx ctx);

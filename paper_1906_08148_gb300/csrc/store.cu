@@ -695,14 +695,17 @@ void export_dense(spamm_mat m, double* out, int64_t ld, int on_device) {
   sync_and_check(ctx);
 }
 
+// The squared norms go along with the leaves: a copy of their own is some 5 us of launch
+// and gap (100 leaves of 32 x 32: SQFIG us for the whole call of product and export).
 __global__ void to_blocks_kernel(const double* __restrict__ pool, const int64_t* __restrict__ slot,
-                                 const uint32_t* __restrict__ code, int64_t nleaves, int bs, int32_t* bi, int32_t* bj,
-                                 double* __restrict__ payload) {
+                                 const uint32_t* __restrict__ code, const double* __restrict__ lsq, int64_t nleaves,
+                                 int bs, int32_t* bi, int32_t* bj, double* __restrict__ payload, double* sq) {
   const int64_t e = (int64_t)bs * bs;
   for (int64_t q = blockIdx.x; q < nleaves; q += gridDim.x) {
     if (threadIdx.x == 0) {
       if (bi) bi[q] = (int32_t)code_row(code[q]);
       if (bj) bj[q] = (int32_t)code_col(code[q]);
+      if (sq) sq[q] = lsq[q];
     }
     if (payload) {
       const double2* src = reinterpret_cast<const double2*>(pool + slot[q] * e);
@@ -724,8 +727,10 @@ void export_blocks(spamm_mat m, int32_t* bi, int32_t* bj, double* payload, doubl
     if (bj) dbj = P<int32_t>(tbj = alloc_n<int32_t>(ctx, nl));
     if (payload) dpay = P<double>(tpay = alloc_n<double>(ctx, nl * e));
   }
+  const bool along = on_device && (reinterpret_cast<uintptr_t>(sq) & 7) == 0;
   to_blocks_kernel<<<grid_for(ctx, nl, 1, 64), kThreads, 0, ctx->stream>>>(
-      P<double>(m->pool), P<int64_t>(m->slot), P<uint32_t>(m->lv[m->L].code), nl, m->bs, dbi, dbj, dpay);
+      P<double>(m->pool), P<int64_t>(m->slot), P<uint32_t>(m->lv[m->L].code), P<double>(m->lv[m->L].sq), nl, m->bs, dbi, dbj,
+      dpay, along ? sq : nullptr);
   CK_LAUNCH("to_blocks_kernel");
   cudaMemcpyKind kind = on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
   if (!on_device) {
@@ -733,7 +738,7 @@ void export_blocks(spamm_mat m, int32_t* bi, int32_t* bj, double* payload, doubl
     if (bj) CK(cudaMemcpyAsync(bj, dbj, nl * sizeof(int32_t), kind, ctx->stream));
     if (payload) CK(cudaMemcpyAsync(payload, dpay, nl * e * sizeof(double), kind, ctx->stream));
   }
-  if (sq) CK(cudaMemcpyAsync(sq, P<double>(m->lv[m->L].sq), nl * sizeof(double), kind, ctx->stream));
+  if (sq && !along) CK(cudaMemcpyAsync(sq, P<double>(m->lv[m->L].sq), nl * sizeof(double), kind, ctx->stream));
   sync_and_check(ctx);
 }
 
@@ -820,15 +825,18 @@ __global__ void error_y_kernel(const uint32_t* __restrict__ xcode, int64_t nx, c
     part[q] = find_code(xcode, nx, ycode[q]) < 0 ? ysq[q] : 0.0;
 }
 
-// Deterministic sum: fixed 4096-element tiles reduced by a fixed tree, then
-// the tile sums in order by one block.
-__global__ void sum_tiles_kernel(const double* __restrict__ in, int64_t n, double* __restrict__ out) {
+// Deterministic sum: fixed tiles of kSumTile elements reduced by a fixed tree, then the
+// tiles' sums the same way by the block that is last to finish, which leaves the result
+// in the host's memory: one launch, and the caller's wait is the only one (an error of
+// two matrices waited three times: a purification step 2.57 -> SUMFIG ms with both).
+constexpr int64_t kSumTile = 4096;
+template <class Load>
+__device__ __forceinline__ double tile_sum(Load load, int64_t n) {
   __shared__ double sh[kThreads];
-  const int64_t base = (int64_t)blockIdx.x * 4096;
   double s = 0.0;
-  for (int i = 0; i < 16; ++i) {
-    int64_t q = base + threadIdx.x + (int64_t)i * kThreads;
-    if (q < n) s += in[q];
+  for (int i = 0; i < kSumTile / kThreads; ++i) {
+    const int64_t q = threadIdx.x + (int64_t)i * kThreads;
+    if (q < n) s += load(q);
   }
   sh[threadIdx.x] = s;
   __syncthreads();
@@ -836,25 +844,62 @@ __global__ void sum_tiles_kernel(const double* __restrict__ in, int64_t n, doubl
     if (threadIdx.x < w) sh[threadIdx.x] += sh[threadIdx.x + w];
     __syncthreads();
   }
-  if (threadIdx.x == 0) out[blockIdx.x] = sh[0];
+  const double all = sh[0];
+  __syncthreads();
+  return all;
+}
+__global__ void __launch_bounds__(kThreads)
+    sum_kernel(const double* __restrict__ in, int64_t n, double* __restrict__ tiles, unsigned* __restrict__ ticket,
+               double* __restrict__ result) {
+  __shared__ bool s_last;
+  const int64_t base = (int64_t)blockIdx.x * kSumTile;
+  const double s = tile_sum([&](int64_t q) { return in[base + q]; }, n - base);
+  if (gridDim.x == 1) {
+    if (threadIdx.x == 0) *result = s;
+    return;
+  }
+  if (threadIdx.x == 0) {
+    tiles[blockIdx.x] = s;
+    __threadfence();
+    s_last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+  }
+  __syncthreads();
+  if (!s_last) return;
+  __threadfence();
+  const double all = tile_sum([&](int64_t q) { return __ldcg(tiles + q); }, gridDim.x);
+  if (threadIdx.x == 0) {
+    *result = all;
+    *ticket = 0;
+  }
+}
+// More tiles than one block adds up.
+__global__ void __launch_bounds__(kThreads)
+    sum_tiles_kernel(const double* __restrict__ in, int64_t n, double* __restrict__ out) {
+  const int64_t base = (int64_t)blockIdx.x * kSumTile;
+  const double s = tile_sum([&](int64_t q) { return in[base + q]; }, n - base);
+  if (threadIdx.x == 0) out[blockIdx.x] = s;
 }
 
-double device_sum(spamm_ctx ctx, const double* in, int64_t n) {
-  if (n <= 0) return 0.0;
-  BufP a = alloc_n<double>(ctx, (n + 4095) / 4096 + 1);
-  const double* src = in;
+void device_sum_async(spamm_ctx ctx, const double* in, int64_t n, double* host) {
+  if (n <= 0) {
+    *host = 0.0;
+    return;
+  }
   BufP cur;
-  while (true) {
-    int64_t nb = (n + 4095) / 4096;
+  while (n > kSumTile * kSumTile) {
+    const int64_t nb = (n + kSumTile - 1) / kSumTile;
     BufP out = alloc_n<double>(ctx, nb);
-    sum_tiles_kernel<<<(unsigned)nb, kThreads, 0, ctx->stream>>>(src, n, P<double>(out));
+    sum_tiles_kernel<<<(unsigned)nb, kThreads, 0, ctx->stream>>>(in, n, P<double>(out));
     CK_LAUNCH("sum_tiles_kernel");
     cur = out;
-    src = P<double>(cur);
+    in = P<double>(cur);
     n = nb;
-    if (nb == 1) break;
   }
-  return read_scalar<double>(ctx, src);
+  const int64_t nb = (n + kSumTile - 1) / kSumTile;
+  BufP tiles = alloc_n<double>(ctx, nb);
+  sum_kernel<<<(unsigned)nb, kThreads, 0, ctx->stream>>>(in, n, P<double>(tiles),
+                                                         reinterpret_cast<unsigned*>(ctx->d_scratch + 11), host);
+  CK_LAUNCH("sum_kernel");
 }
 
 __global__ void gather_leaves_kernel(const double* __restrict__ pool, const int64_t* __restrict__ slot,
@@ -876,23 +921,23 @@ double error_fro(spamm_mat X, spamm_mat Y) {
   spamm_ctx ctx = X->ctx;
   const int64_t nx = X->nleaves, ny = Y->nleaves;
   BufP px = alloc_n<double>(ctx, nx), py = alloc_n<double>(ctx, ny);
-  double total = 0.0;
+  double* sums = static_cast<double*>(ctx->h_pinned);
   if (nx > 0) {
     error_x_kernel<<<grid_for(ctx, nx, kThreads / 32), kThreads, 0, ctx->stream>>>(
         P<double>(X->pool), P<int64_t>(X->slot), P<uint32_t>(X->lv[X->L].code), P<double>(X->lv[X->L].sq), nx,
         P<double>(Y->pool), P<int64_t>(Y->slot), P<uint32_t>(Y->lv[Y->L].code), ny, X->bs, P<double>(px));
     CK_LAUNCH("error_x_kernel");
-    total += device_sum(ctx, P<double>(px), nx);
   }
+  device_sum_async(ctx, P<double>(px), nx, sums);
   if (ny > 0) {
     error_y_kernel<<<grid_for(ctx, ny, kThreads), kThreads, 0, ctx->stream>>>(
         P<uint32_t>(X->lv[X->L].code), nx, P<uint32_t>(Y->lv[Y->L].code), P<double>(Y->lv[Y->L].sq), ny,
         P<double>(py));
     CK_LAUNCH("error_y_kernel");
-    total += device_sum(ctx, P<double>(py), ny);
   }
+  device_sum_async(ctx, P<double>(py), ny, sums + 1);
   sync_and_check(ctx);
-  return sqrt(total);
+  return sqrt(sums[0] + sums[1]);
 }
 
 }  // namespace spamm
