@@ -475,6 +475,7 @@ PlanOut make_output(spamm_ctx ctx, const spamm_plan_s& p) {
   Cm->dcount = p.cdcount;
   Cm->nleaves = p.T.ngroups;
   Cm->pool = alloc_n<double>(ctx, p.T.ngroups * e);
+  Cm->packed = true;
   alloc_norms(Cm);
   PlanDev& d = o.dev;
   d.gstart = P<int64_t>(p.T.gstart);

@@ -136,6 +136,7 @@ struct spamm_mat_s {
   int64_t nleaves = 0;
   spamm::BufP pool;  // double payload, bs*bs per slot
   spamm::BufP slot;  // int64 per leaf: payload slot of leaf m (leaves in Morton order)
+  bool packed = false;  // leaf m's payload is in slot m (a product's output)
   int symmetric = 0;  // the matrix equals its transpose (set by the generator or the caller)
   std::vector<spamm::Level> lv;  // levels 0..L
   spamm::BufP dcount;            // uint64 [L + 1]: nodes per level, as `count` of the levels (null: no leaves)
