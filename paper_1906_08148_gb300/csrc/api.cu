@@ -382,17 +382,22 @@ spamm_plan make_plan(spamm_ctx ctx, spamm_mat A, spamm_mat B, double tau, spamm_
   CK(cudaEventRecord(ev[2], ctx->stream));
   const bool tensor = prec != SPAMM_PREC_FP64;
   if (tensor) {
-    prep_terms(At, prec, 0, &p->termsA, &p->expA, ctx);
+    const PrepReq both[2] = {{At, 0, &p->termsA, &p->expA}, {Bt, 1, &p->termsB, &p->expB}};
     // X times X with X symmetric: the B operand of leaf (k, j) is the transpose
     // of leaf (j, k), whose A terms are exactly the B terms of (k, j) (rows of
     // (j, k) are columns of (k, j), with the same grid), so one set of terms
     // serves both roles, if every leaf's transpose is present
-    if (Bt == At && At->symmetric && transpose_map(At, &p->bmap, ctx) == 0) {
-      p->termsB = p->termsA;
-      p->expB = p->expA;
+    if (Bt == At && At->symmetric) {
+      prep_terms(ctx, prec, both, 1);
+      if (transpose_map(At, &p->bmap, ctx) == 0) {
+        p->termsB = p->termsA;
+        p->expB = p->expA;
+      } else {
+        p->bmap.reset();
+        prep_terms(ctx, prec, both + 1, 1);
+      }
     } else {
-      p->bmap.reset();
-      prep_terms(Bt, prec, 1, &p->termsB, &p->expB, ctx);
+      prep_terms(ctx, prec, both, 2);
     }
   }
   CK(cudaEventRecord(ev[3], ctx->stream));

@@ -719,7 +719,7 @@ static void launch_quads(spamm_ctx ctx, const BatchDev& b) {
 // 45 us, 20023 leaves of 128 x 128 (2.6 GB) 1.50 -> 0.78 ms; with 64 leaves per block a few
 // thousand leaves kept a third of the SMs busy.  All outputs of a batch in one launch:
 // a leaf's chain of additions takes 20 us however few leaves there are, and eight
-// outputs of 250 to 4088 leaves took 272 us one after the other; in one launch their
+// outputs (n = 1000 .. 5000) took 272 us one after the other; in one launch their
 // batch takes 2.76 ms instead of 2.88.
 constexpr int64_t kFinishLeavesPerBlock = 8;
 

@@ -316,7 +316,13 @@ void tc_finish(spamm_ctx ctx, spamm_prec prec, const OutBatch& out, int bs);
 inline int tc_tiles_per_leaf(int bs) { return (bs / 64) * (bs / 64); }
 // Operand terms of a leaf set for a tensor form (role 0: used as A, 1: as B),
 // and each tile's power-of-two scale exponent.
-void prep_terms(spamm_mat M, spamm_prec prec, int role, BufP* terms, BufP* expo, spamm_ctx on = nullptr);
+struct PrepReq {
+  spamm_mat M;
+  int role;
+  BufP *terms, *expo;
+};
+// k = 1, or 2 with the second a B operand of the same leaf size.
+void prep_terms(spamm_ctx ctx, spamm_prec prec, const PrepReq* req, int k);
 // The step list of 128 x 128 leaves for the tensor-core kernel: one unit per output leaf, two K-half steps
 // per kept product (T.gstart doubled), on the tile-split operand terms.
 int64_t build_leaf128_steps(spamm_ctx ctx, const TaskList& T, const int32_t* expA, const int32_t* expB,

@@ -25,20 +25,21 @@ struct ChunkMap {
     row = role == 0 ? t >> 3 : (t & 63);
     c8 = role == 0 ? (t & 7) : t >> 6;
   }
-  // src: the tile's first element (shared or global memory); ld: its row length
+  // src: the tile's first element (GLOBAL: in global memory, else shared); ld: its row length
+  template <bool GLOBAL>
   __device__ __forceinline__ void load(const unsigned long long* src, int ld, int role, unsigned long long (&v)[8]) const {
     if (role == 0) {
       // 8 consecutive doubles of one row: four 16-byte loads
       const ulonglong2* p = reinterpret_cast<const ulonglong2*>(src + row * ld + 8 * c8);
 #pragma unroll
       for (int e = 0; e < 4; ++e) {
-        const ulonglong2 w = p[e];
+        const ulonglong2 w = GLOBAL ? __ldg(p + e) : p[e];
         v[2 * e] = w.x;
         v[2 * e + 1] = w.y;
       }
     } else {
 #pragma unroll
-      for (int e = 0; e < 8; ++e) v[e] = src[(8 * c8 + e) * ld + row];
+      for (int e = 0; e < 8; ++e) v[e] = GLOBAL ? __ldg(src + (8 * c8 + e) * ld + row) : src[(8 * c8 + e) * ld + row];
     }
   }
 };
@@ -65,27 +66,47 @@ __device__ __forceinline__ const double* tile_src(const double* leaf, int bs, in
 // slices (4.2 GB) 0.87 -> 0.70.  The quarters of a 128 x 128 leaf are 64 runs of 512
 // bytes each, for which the staged form is the slower one (n = 20000 FP16, 5.3 GB: 1.50
 // ms, 1.17 with loads into registers).
-struct TileStream {
-  static constexpr uint32_t kBytes = 64 * 64 * sizeof(double);
+// PAIR: both operands of a product share a launch, where it has few tiles per CTA
+// (kPairTiles) and the latency of the first ones counts: 2 x 3536 tiles 84 -> 80 us, eight
+// products with n = 1000 .. 5000 2.70 -> 2.67 ms.  With 2 x 37,624 tiles it is slower, 0.72 ms
+// for 0.69 (both operands' tables are looked up for every tile).
+struct PrepSide {
   const double* pool;
   const int64_t* slot;
+  uint8_t* out;
+  int32_t* expo;
+  int64_t tiles;
+};
+struct PrepPair {
+  PrepSide side[2];
+  int role0;  // of side 0; side 1 (if it has tiles) is a B operand
+};
+constexpr uint32_t kTileBytes = 64 * 64 * sizeof(double);
+template <bool PAIR>
+struct TileStream {
+  const PrepPair& P;
   int64_t total;  // tiles
-  int bs, role;
+  int bs;
   uint8_t* in;    // two tiles
   uint64_t* full;
 
+  __device__ __forceinline__ bool second(int64_t m) const { return PAIR && m >= P.side[0].tiles; }
   __device__ __forceinline__ const double* source(int64_t m) const {
-    const int tiles = (bs / 64) * (bs / 64);
-    const int64_t leaf = m / tiles;
-    return tile_src(pool + slot[leaf] * (int64_t)bs * bs, bs, role, (int)(m - leaf * tiles));
+    const bool b = second(m);
+    const double* pool = b ? P.side[1].pool : P.side[0].pool;
+    const int64_t* slot = b ? P.side[1].slot : P.side[0].slot;
+    if (b) m -= P.side[0].tiles;
+    const int tiles = (bs / 64) * (bs / 64), shift = bs == 64 ? 0 : 2;
+    const int64_t leaf = m >> shift;  // four tiles in a leaf of 128
+    return tile_src(pool + __ldg(slot + leaf) * (int64_t)bs * bs, bs, b ? 1 : P.role0, (int)(m - leaf * tiles));
   }
   // STAGED, by one thread: tile m into buffer b (nothing past the last tile)
   __device__ __forceinline__ void fetch(int64_t m, int b) const {
     if (m >= total) return;
     const double* src = source(m);
     fence_proxy_async_smem();
-    mbar_arrive_expect_tx(&full[b], kBytes);
-    bulk_g2s(in + (uint32_t)b * kBytes, src, kBytes, &full[b]);
+    mbar_arrive_expect_tx(&full[b], kTileBytes);
+    bulk_g2s(in + (uint32_t)b * kTileBytes, src, kTileBytes, &full[b]);
   }
   // the last two fetches of a CTA that gave up have landed
   __device__ __forceinline__ void drain(int64_t m, uint32_t it) const {
@@ -97,19 +118,18 @@ struct TileStream {
 // Form: measure(v) gives a thread's words for the line and tile maxima (the first
 // combined by max, the second by or), shift the tile's scale exponent from them, split
 // the thread's chunk of every term.
-template <class Form, bool STAGED>
+template <class Form, bool STAGED, bool PAIR>
 __global__ void __launch_bounds__(kPrepThreads, STAGED || Form::kLines ? 2 : 3)
-    prep_kernel(const double* __restrict__ pool, const int64_t* __restrict__ slot, int64_t nleaves, int bs, int role,
-                uint8_t* __restrict__ out, int32_t* __restrict__ expo, int* __restrict__ err) {
+    prep_kernel(const __grid_constant__ PrepPair P, int bs, int* __restrict__ err) {
   constexpr uint32_t LEAF = Form::kLeaf;
   extern __shared__ __align__(128) uint8_t prep_smem[];
-  uint8_t* stile = prep_smem + (STAGED ? 2 * TileStream::kBytes : 0);  // the finished terms
+  uint8_t* stile = prep_smem + (STAGED ? 2 * kTileBytes : 0);  // the finished terms
   __shared__ __align__(8) uint64_t full[2];
   __shared__ uint32_t s_line[8][64];
   __shared__ uint2 s_warp[kPrepThreads / 32];
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-  const ChunkMap cm(t, role);
-  const TileStream ts{pool, slot, nleaves * (bs / 64) * (bs / 64), bs, role, prep_smem, full};
+  const TileStream<PAIR> ts{P, P.side[0].tiles + (PAIR ? P.side[1].tiles : 0), bs, prep_smem, full};
+  const ChunkMap cm0(t, P.role0);
   int64_t m = blockIdx.x;
   if (STAGED) {
     if (t == 0) {
@@ -127,13 +147,16 @@ __global__ void __launch_bounds__(kPrepThreads, STAGED || Form::kLines ? 2 : 3)
   uint32_t it = 0;
   for (; m < ts.total; m += gridDim.x, ++it) {
     const int b = (int)(it & 1);
+    const bool side = ts.second(m);
+    const int role = side ? 1 : P.role0;
+    const ChunkMap cm = PAIR ? ChunkMap(t, role) : cm0;
     bool ok = true;
     unsigned long long v[8];
     if (STAGED) {
       ok = mbar_wait_bounded(&full[b], (it >> 1) & 1u);
-      cm.load(reinterpret_cast<const unsigned long long*>(prep_smem + (uint32_t)b * TileStream::kBytes), 64, role, v);
+      cm.load<false>(reinterpret_cast<const unsigned long long*>(prep_smem + (uint32_t)b * kTileBytes), 64, role, v);
     } else {
-      cm.load(reinterpret_cast<const unsigned long long*>(ts.source(m)), bs, role, v);
+      cm.load<true>(reinterpret_cast<const unsigned long long*>(ts.source(m)), bs, role, v);
     }
     // the largest of this thread's line (A: row, B: column), then of the tile
     uint2 top = Form::measure(v);
@@ -159,13 +182,14 @@ __global__ void __launch_bounds__(kPrepThreads, STAGED || Form::kLines ? 2 : 3)
     if (STAGED && t == 0) ts.fetch(m + 2 * (int64_t)gridDim.x, b);  // every thread holds its elements in registers
     const uint2 w = s_warp[lane & (kPrepThreads / 32 - 1)];
     const int f = Form::shift(__reduce_max_sync(0xffffffffu, w.x), __reduce_or_sync(0xffffffffu, w.y));
-    if (t == 0) expo[m] = f;
+    const int64_t at = side ? m - P.side[0].tiles : m;
+    if (t == 0) (side ? P.side[1].expo : P.side[0].expo)[at] = f;
     Form::split(v, (int)line, f, [&](int s, uint4 chunk) {
       *reinterpret_cast<uint4*>(stile + term_offset<Form::kParts>(Form::kTerms, s, cm.row, 8 * cm.c8)) = chunk;
     });
     fence_proxy_async_smem();
     __syncthreads();
-    if (t == 0) bulk_s2g(out + m * (int64_t)LEAF, stile, LEAF);
+    if (t == 0) bulk_s2g((side ? P.side[1].out : P.side[0].out) + at * (int64_t)LEAF, stile, LEAF);
   }
   if (t == 0) {
     bulk_wait_all();
@@ -264,30 +288,43 @@ static uint32_t form_leaf_bytes(spamm_prec prec) {
   }
 }
 
-void prep_terms(spamm_mat M, spamm_prec prec, int role, BufP* terms, BufP* expo, spamm_ctx on) {
-  spamm_ctx ctx = on ? on : M->ctx;
-  const int bs = M->bs;
+constexpr int64_t kPairTiles = 32;
+void prep_terms(spamm_ctx ctx, spamm_prec prec, const PrepReq* req, int k) {
+  const int bs = req[0].M->bs;
   if (bs != 64 && bs != 128) fail(SPAMM_E_UNSUPPORTED, "tensor-core precision forms are built for bs = 64 and 128");
-  const int64_t ntiles = M->nleaves * tc_tiles_per_leaf(bs);
-  *terms = alloc_n<uint8_t>(ctx, ntiles * (int64_t)form_leaf_bytes(prec));
-  *expo = alloc_n<int32_t>(ctx, ntiles);
-  if (M->nleaves == 0) return;
+  const int64_t tiles0 = req[0].M->nleaves * tc_tiles_per_leaf(bs);
+  if (k == 2 && tiles0 + req[1].M->nleaves * tc_tiles_per_leaf(bs) > kPairTiles * 2 * ctx->num_sms) {
+    prep_terms(ctx, prec, req, 1);
+    prep_terms(ctx, prec, req + 1, 1);
+    return;
+  }
+  PrepPair pair{};
+  int64_t ntiles = 0;
+  for (int i = 0; i < k; ++i) {
+    const PrepReq& r = req[i];
+    const int64_t n = r.M->nleaves * tc_tiles_per_leaf(bs);
+    *r.terms = alloc_n<uint8_t>(ctx, n * (int64_t)form_leaf_bytes(prec));
+    *r.expo = alloc_n<int32_t>(ctx, n);
+    pair.side[i] = {P<double>(r.M->pool), P<int64_t>(r.M->slot), P<uint8_t>(*r.terms), P<int32_t>(*r.expo), n};
+    ntiles += n;
+  }
+  pair.role0 = req[0].role;
+  if (ntiles == 0) return;
   const int64_t cap = (int64_t)ctx->num_sms * (bs == 64 ? 2 : 3);
   const unsigned grid = (unsigned)(ntiles < cap ? ntiles : cap);
   const bool staged = bs == 64;
-  const int smem = (int)((staged ? 2 * TileStream::kBytes : 0) + form_leaf_bytes(prec));
+  const int smem = (int)((staged ? 2 * kTileBytes : 0) + form_leaf_bytes(prec));
   auto launch = [&](auto kern) {
     CK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    kern<<<grid, kPrepThreads, smem, ctx->stream>>>(P<double>(M->pool), P<int64_t>(M->slot), M->nleaves, bs, role,
-                                                    P<uint8_t>(*terms), P<int32_t>(*expo), ctx->d_err);
+    kern<<<grid, kPrepThreads, smem, ctx->stream>>>(pair, bs, ctx->d_err);
     CK_LAUNCH("prep_kernel");
   };
   auto form = [&](auto f) {
     using Form = decltype(f);
     if (staged)
-      launch(prep_kernel<Form, true>);
+      k == 2 ? launch(prep_kernel<Form, true, true>) : launch(prep_kernel<Form, true, false>);
     else
-      launch(prep_kernel<Form, false>);
+      k == 2 ? launch(prep_kernel<Form, false, true>) : launch(prep_kernel<Form, false, false>);
   };
   if (prec == SPAMM_PREC_BF16_SPLIT)
     form(SliceForm<SPAMM_PREC_BF16_SPLIT>());

@@ -36,7 +36,7 @@ def _dense(S, ctx, C, bs, shape):
     return out
 
 
-# 64: two blocks of one tile per multiprocessor; 128: three, four tiles per leaf
+# 64: two blocks per multiprocessor, both operands' tiles in one launch; 128: four tiles per leaf
 @pytest.mark.parametrize("prec", TC)
 @pytest.mark.parametrize("bs,count", [(64, 1), (64, 303), (64, 304), (64, 305), (64, 609), (64, 913), (128, 1),
                                       (128, 113), (128, 114), (128, 115), (128, 229), (128, 343)])
