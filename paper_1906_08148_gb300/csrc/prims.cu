@@ -3,7 +3,6 @@
 #include <cstring>
 
 #include "internal.cuh"
-#include "ptx.cuh"
 
 namespace spamm {
 
@@ -255,21 +254,18 @@ void scan_inclusive_f64(spamm_ctx ctx, const double* in, double* out, int64_t n)
 // places after the warp's earlier ones, counted per warp and digit in shared
 // memory; the warps of a block own consecutive runs of items, so a prefix over
 // warps, tiles and digits gives every item its place.  Up to kSortSmall items one
-// block takes all passes in one launch (four rounds a pass), up to kSortCluster a
-// cluster of eight blocks with two cluster barriers a pass (some 5 us); more take three
-// launches a pass (some 19 us up to there): digit counts per tile, their prefix per
-// digit, placing.  A purification, whose error-controlled truncation sorts some 10^4
-// norms by 64 bits, 2.76 -> 2.65 ms with the cluster.  2,000,000 pairs by 32 bits: 0.23
-// ms where eight 4-bit passes, each a scan over all blocks and digits, took 0.85.
+// block takes all passes in one launch; more take three launches a pass (some 19 us at
+// that size): digit counts per tile, their prefix per digit, placing.  A purification,
+// whose error-controlled truncation sorts some 10^4 norms by 64 bits, 2.76 -> 2.69 ms.
+// 2,000,000 pairs by 32 bits: 0.23 ms where eight 4-bit passes, each a scan over all
+// blocks and digits, took 0.85.
 constexpr int kDigits = 256;
 constexpr int kSortThreads = 256;
 constexpr int kSortRounds = 8;                        // rounds of 32 items per warp
 constexpr int kSortTile = kSortThreads * kSortRounds;  // items per block
 constexpr int kSmallThreads = 1024;
-constexpr int64_t kSortSmall = 4096;
-constexpr int kClusterCtas = 8;
-constexpr int64_t kSortCluster = (int64_t)kClusterCtas * kSmallThreads * kSortRounds;
-static_assert(kSortSmall <= kSmallThreads * kSortRounds, "the one-block sort holds its items in registers");
+constexpr int kSmallRounds = 16;
+constexpr int64_t kSortSmall = kSmallThreads * kSmallRounds;
 
 // Ranks the warp's items (digit d[r] of round r, valid where bit r of `in`) within its
 // counters cnt[256], which it leaves at the warp's digit counts.
@@ -375,36 +371,45 @@ __global__ void __launch_bounds__(kSortThreads)
     }
 }
 
-// All passes of a sort by CTAS blocks (a cluster if more than one) of at most 8192
-// items each; the result is in (ka, va) if the number of passes is even, else in (kb, vb).
-// The blocks exchange their digit counts through `counts` [CTAS][256].
-template <int CTAS>
+// All passes of a sort of at most 1024 ROUNDS pairs by one block; the result is in (ka, va)
+// if the number of passes is even, else in (kb, vb).
+template <int ROUNDS>
 __global__ void __launch_bounds__(kSmallThreads)
-    radix_small_kernel(uint64_t* ka, int64_t* va, uint64_t* kb, int64_t* vb, int n, int bits, uint32_t* counts) {
+    radix_small_kernel(uint64_t* ka, int64_t* va, uint64_t* kb, int64_t* vb, int n, int bits) {
   extern __shared__ uint32_t small_cnt[];  // [32][256], then 256 digit bases
   __shared__ uint32_t wsum[kDigits / 32];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, cta = (int)blockIdx.x;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const unsigned lt = (1u << lane) - 1u;
   uint32_t* mine = small_cnt + warp * kDigits;
   uint32_t* place = small_cnt + 32 * kDigits;
-  const int per = (n + CTAS * kSmallThreads - 1) / (CTAS * kSmallThreads);  // rounds per warp
-  const int base = (cta * (kSmallThreads / 32) + warp) * 32 * per + lane;
+  const int per = (n + kSmallThreads - 1) / kSmallThreads;  // rounds per warp
+  const int base = warp * 32 * per + lane;
   for (int shift = 0; shift < bits; shift += 8) {
     for (int i = lane; i < kDigits; i += 32) mine[i] = 0;
     __syncwarp();
-    uint64_t key[kSortRounds];
-    uint32_t d[kSortRounds], rank[kSortRounds], in = 0;
+    uint64_t key[ROUNDS];
+    uint32_t at[ROUNDS];  // digit << 16 | rank among the warp's items of that digit
 #pragma unroll
-    for (int r = 0; r < kSortRounds; ++r) {
-      const int q = base + 32 * r;
-      const bool on = r < per && q < n;
-      key[r] = on ? __ldcg(ka + q) : 0;
-      in |= (uint32_t)on << r;
-      d[r] = (uint32_t)(key[r] >> shift) & (kDigits - 1);
+    for (int r = 0; r < ROUNDS; ++r) key[r] = r < per && base + 32 * r < n ? ka[base + 32 * r] : 0;
+#pragma unroll
+    for (int r = 0; r < ROUNDS; ++r) {
+      if (r >= per) break;
+      const bool on = base + 32 * r < n;
+      const unsigned act = __ballot_sync(0xffffffffu, on);
+      if (on) {
+        const uint32_t d = (uint32_t)(key[r] >> shift) & (kDigits - 1);
+        const unsigned same = __match_any_sync(act, d);
+        const uint32_t before = mine[d];
+        __syncwarp(act);
+        if ((same & lt) == 0) mine[d] = before + (uint32_t)__popc(same);
+        __syncwarp(act);
+        at[r] = d << 16 | (before + (uint32_t)__popc(same & lt));
+      }
+      __syncwarp();
     }
-    warp_rank(d, in, mine, rank);
     __syncthreads();
-    // thread t < 256: digit t over the warps, the blocks, then over the digits
-    uint32_t s = 0, x = 0, earlier = 0, all = 0;
+    // thread t < 256: digit t over the warps, then over the digits
+    uint32_t s = 0, x = 0;
     if (threadIdx.x < kDigits) {
 #pragma unroll 8
       for (int w = 0; w < kSmallThreads / 32; ++w) {
@@ -412,25 +417,7 @@ __global__ void __launch_bounds__(kSmallThreads)
         small_cnt[w * kDigits + threadIdx.x] = s;
         s += c;
       }
-      if (CTAS > 1) counts[cta * kDigits + threadIdx.x] = s;
-      all = s;
-    }
-    if (CTAS > 1) {
-      cluster_sync();
-      if (threadIdx.x < kDigits) {
-        uint32_t c[CTAS];
-#pragma unroll
-        for (int i = 0; i < CTAS; ++i) c[i] = __ldcg(counts + i * kDigits + threadIdx.x);
-        all = 0;
-#pragma unroll
-        for (int i = 0; i < CTAS; ++i) {
-          if (i < cta) earlier += c[i];
-          all += c[i];
-        }
-      }
-    }
-    if (threadIdx.x < kDigits) {
-      x = all;
+      x = s;
 #pragma unroll
       for (int o = 1; o < 32; o <<= 1) {
         const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
@@ -440,22 +427,19 @@ __global__ void __launch_bounds__(kSmallThreads)
     }
     __syncthreads();
     if (threadIdx.x < kDigits) {
-      uint32_t before = earlier;
+      uint32_t before = 0;
       for (int w = 0; w < warp; ++w) before += wsum[w];
-      place[threadIdx.x] = before + x - all;
+      place[threadIdx.x] = before + x - s;
     }
     __syncthreads();
 #pragma unroll
-    for (int r = 0; r < kSortRounds; ++r)
-      if (in >> r & 1u) {
-        const uint32_t p = place[d[r]] + mine[d[r]] + rank[r];
+    for (int r = 0; r < ROUNDS; ++r)
+      if (r < per && base + 32 * r < n) {
+        const uint32_t d = at[r] >> 16, p = place[d] + mine[d] + (at[r] & 0xffffu);
         kb[p] = key[r];
-        vb[p] = __ldcg(va + base + 32 * r);
+        vb[p] = va[base + 32 * r];
       }
-    if (CTAS > 1)
-      cluster_sync();
-    else
-      __syncthreads();
+    __syncthreads();
     uint64_t* k = ka;
     ka = kb;
     kb = k;
@@ -465,21 +449,10 @@ __global__ void __launch_bounds__(kSmallThreads)
   }
 }
 
-template <int CTAS>
+template <int ROUNDS>
 static void radix_small(spamm_ctx ctx, uint64_t* ka, int64_t* va, uint64_t* kb, int64_t* vb, int n, int bits) {
-  BufP counts = CTAS > 1 ? alloc_n<uint32_t>(ctx, CTAS * kDigits) : BufP();
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(CTAS);
-  cfg.blockDim = dim3(kSmallThreads);
-  cfg.dynamicSmemBytes = sizeof(uint32_t) * kDigits * (kSmallThreads / 32 + 1);
-  cfg.stream = ctx->stream;
-  cudaLaunchAttribute at = {};
-  at.id = cudaLaunchAttributeClusterDimension;
-  at.val.clusterDim.x = CTAS;
-  at.val.clusterDim.y = at.val.clusterDim.z = 1;
-  cfg.attrs = &at;
-  cfg.numAttrs = CTAS > 1 ? 1 : 0;
-  CK(cudaLaunchKernelEx(&cfg, radix_small_kernel<CTAS>, ka, va, kb, vb, n, bits, P<uint32_t>(counts)));
+  const int smem = (int)sizeof(uint32_t) * kDigits * (kSmallThreads / 32 + 1);
+  radix_small_kernel<ROUNDS><<<1, kSmallThreads, smem, ctx->stream>>>(ka, va, kb, vb, n, bits);
   CK_LAUNCH("radix_small_kernel");
 }
 
@@ -489,11 +462,11 @@ void radix_sort_pairs(spamm_ctx ctx, uint64_t* keys, int64_t* vals, int64_t n, i
   uint64_t *ka = keys, *kb = P<uint64_t>(k2);
   int64_t *va = vals, *vb = P<int64_t>(v2);
   const int passes = (bits + 7) / 8;
-  if (n <= kSortCluster) {
-    if (n <= kSortSmall)
-      radix_small<1>(ctx, ka, va, kb, vb, (int)n, bits);
+  if (n <= kSortSmall) {
+    if (n <= kSmallThreads * 4)
+      radix_small<4>(ctx, ka, va, kb, vb, (int)n, bits);
     else
-      radix_small<kClusterCtas>(ctx, ka, va, kb, vb, (int)n, bits);
+      radix_small<kSmallRounds>(ctx, ka, va, kb, vb, (int)n, bits);
     if (passes & 1) ka = kb, va = vb;
   } else {
     const int64_t ntiles = (n + kSortTile - 1) / kSortTile;

@@ -9,8 +9,8 @@
 // Two forms.  Up to kTopNodes items one block of 1024 threads takes a whole tree in
 // one launch, all levels' structure in one pass: truncating both operands of a 4096-row
 // lattice (some 4000 leaves of 64 x 64 each, seven levels) is 12.5 us of kernel, where
-// five launches per level took 360; up to kBoundNodes a cluster of eight such blocks.
-// Larger levels take two launches each, a count per tile of 1024 and the placing, where
+// five launches per level took 360; up to kBoundNodes the block takes one piece of that
+// size after the other.  Larger levels take two launches each, a count per tile of 1024 and the placing, where
 // every tile adds up the counts before it, until the level is small enough for the rest;
 // there the thread that sees the first child of a run also sees the others (at most
 // three nodes further on), so it writes the parent's code and child links at once.
@@ -19,7 +19,6 @@
 #include <cstring>
 
 #include "internal.cuh"
-#include "ptx.cuh"
 
 namespace spamm {
 
@@ -27,7 +26,7 @@ namespace {
 
 constexpr int kTopThreads = 1024;
 constexpr int64_t kTopNodes = 4096;
-constexpr int64_t kBoundNodes = 32768;  // a cluster's; up to here the leaf level is allocated for every candidate
+constexpr int64_t kBoundNodes = 32768;  // one block's; up to here the leaf level is allocated for every candidate
 constexpr int kTileThreads = 256;
 constexpr int kTilePer = 4;
 constexpr int64_t kTile = kTileThreads * kTilePer;
@@ -53,7 +52,6 @@ struct TreeDev {
   double* osq[SPAMM_MAX_LEVELS] = {};  // null: no norms
   int4* ochild[SPAMM_MAX_LEVELS] = {};
   int64_t* oslot = nullptr;
-  uint32_t* xchg = nullptr;  // cluster form: a row of counts per block
 };
 struct TreePair {
   TreeDev t[2];
@@ -228,17 +226,15 @@ __device__ __forceinline__ void group_prefixes(uint32_t (*v)[kGroups], int rows,
   if (lane == 31) total[r] = (int)x;
 }
 
-// One block (or a cluster of CTAS blocks, of kTopNodes consecutive nodes each) per tree: the
-// leaves (rules 1, 2), then the levels t0 - 1 .. 0.  A block lives on latency: every
-// thread's loads of a phase are in flight together, and groups of 32 nodes keep a warp's
-// accesses together.  All levels' structure in one pass, instead of a flag, prefix and
-// placing pass per level: truncating both 4,088-leaf operands of a 4096-row lattice 20.8
-// -> 12.5 us.  The blocks of a cluster exchange their counts, of leaves and of all levels,
-// through global memory between cluster barriers and share the norms of the levels of
-// more than kTopNodes nodes: the tree of 12,000 leaves from triplets one launch instead of
-// eleven (the whole building 570 -> 526 us), a purification's three 2.61 -> 2.57 ms.
-constexpr int kXchgRow = SPAMM_MAX_LEVELS + 1;
-template <int CTAS>
+// One block per tree: the leaves (rules 1, 2), then the levels t0 - 1 .. 0, kTopNodes
+// nodes at a time.  A block lives on latency: every thread's loads of a phase are in
+// flight together, and groups of 32 nodes keep a warp's accesses together.  All levels'
+// structure in one pass, instead of a flag, prefix and placing pass per level:
+// truncating both 4,088-leaf operands of a 4096-row lattice 20.8 -> 12.5 us.  Up to
+// kBoundNodes the block takes one piece after the other: the tree of 12,000 leaves from
+// triplets one launch instead of eleven (the whole building 570 -> 534 us).  (A cluster of
+// eight blocks takes 522, but waits for eight free multiprocessors next to one another,
+// which a persistent launch on another stream may not leave.)
 __global__ void __launch_bounds__(kTopThreads) tree_top_kernel(const __grid_constant__ TreePair P) {
   constexpr int kWarps = kTopThreads / 32, kPer = kGroups / kWarps;  // groups per warp
   __shared__ union {
@@ -246,165 +242,108 @@ __global__ void __launch_bounds__(kTopThreads) tree_top_kernel(const __grid_cons
     double sq[kTopNodes];
   } s_node;
   __shared__ uint32_t s_before[SPAMM_MAX_LEVELS][kGroups];
-  __shared__ int s_n[SPAMM_MAX_LEVELS], s_base[SPAMM_MAX_LEVELS];
-  const TreeDev& T = P.t[blockIdx.x / CTAS];
+  __shared__ int s_add[SPAMM_MAX_LEVELS], s_n[SPAMM_MAX_LEVELS];
+  const TreeDev& T = P.t[blockIdx.x];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, t0 = T.t0;
-  const int cta = (int)blockIdx.x % CTAS, node0 = cta * (int)kTopNodes;
   const unsigned earlier = (1u << lane) - 1u;
-  auto sync_all = [] {
-    if (CTAS > 1)
-      cluster_sync();
-    else
-      __syncthreads();
-  };
-  // v of every block in column `col`: the sum over the earlier blocks, all blocks' in *total
-  auto exchanged = [&](int col, int* total) {
-    int before = 0, all = 0;
-#pragma unroll
-    for (int c = 0; c < CTAS; ++c) {
-      const int v = (int)__ldcg(T.xchg + c * kXchgRow + col);
-      before += c < cta ? v : 0;
-      all += v;
-    }
-    *total = all;
-    return before;
-  };
-  int n;
+  int n = 0;
   if (T.rule == 1 || T.rule == 2) {
     const int cand = (int)T.n;
-    double sq[kPer] = {};
-    int64_t slot[kPer];
-    uint32_t code[kPer];
-    unsigned keep[kPer];
-    auto each = [&](auto f) {
+    for (int node0 = 0; node0 < cand; node0 += (int)kTopNodes) {
+      double sq[kPer] = {};
+      int64_t slot[kPer];
+      uint32_t code[kPer];
+      unsigned keep[kPer];
+      auto each = [&](auto f) {
 #pragma unroll
-      for (int k = 0; k < kPer; ++k) f(k, node0 + 32 * (warp + k * kWarps) + lane);
-    };
-    each([&](int k, int q) {
-      slot[k] = q;
-      code[k] = (uint32_t)q;
-      keep[k] = 1;
-      if (q < cand) sq[k] = T.sq[q];
-    });
-    if (T.code) each([&](int k, int q) { if (q < cand) code[k] = T.code[q]; });
-    if (T.slot) each([&](int k, int q) { if (q < cand) slot[k] = T.slot[q]; });
-    if (T.rule == 1) each([&](int k, int q) { if (q < cand) keep[k] = T.keep[q]; });
-    if (T.rule == 2) each([&](int k, int) { keep[k] = kept_norm(sq[k], T.smin); });
-    each([&](int k, int q) { keep[k] = q < cand && keep[k]; });
+        for (int k = 0; k < kPer; ++k) f(k, node0 + 32 * (warp + k * kWarps) + lane);
+      };
+      each([&](int k, int q) {
+        slot[k] = q;
+        code[k] = (uint32_t)q;
+        keep[k] = 1;
+        if (q < cand) sq[k] = T.sq[q];
+      });
+      if (T.code) each([&](int k, int q) { if (q < cand) code[k] = T.code[q]; });
+      if (T.slot) each([&](int k, int q) { if (q < cand) slot[k] = T.slot[q]; });
+      if (T.rule == 1) each([&](int k, int q) { if (q < cand) keep[k] = T.keep[q]; });
+      if (T.rule == 2) each([&](int k, int) { keep[k] = kept_norm(sq[k], T.smin); });
+      each([&](int k, int q) { keep[k] = q < cand && keep[k]; });
 #pragma unroll
-    for (int k = 0; k < kPer; ++k) {
-      keep[k] = __ballot_sync(0xffffffffu, keep[k] != 0);
-      if (lane == 0) s_before[0][warp + k * kWarps] = (uint32_t)__popc(keep[k]);
-    }
-    __syncthreads();
-    group_prefixes(s_before, 1, s_n);
-    __syncthreads();
-    int p0 = 0;
-    n = s_n[0];
-    if (CTAS > 1) {
-      if (tid == 0) T.xchg[cta * kXchgRow + SPAMM_MAX_LEVELS] = (uint32_t)n;
-      cluster_sync();
-      p0 = exchanged(SPAMM_MAX_LEVELS, &n);
-    }
-#pragma unroll
-    for (int k = 0; k < kPer; ++k)
-      if (keep[k] >> lane & 1u) {
-        const int p = p0 + (int)s_before[0][warp + k * kWarps] + __popc(keep[k] & earlier);
-        if (CTAS == 1) s_node.code[p] = code[k];
-        T.ocode[T.L][p] = code[k];
-        T.osq[T.L][p] = sq[k];
-        T.oslot[p] = slot[k];
+      for (int k = 0; k < kPer; ++k) {
+        keep[k] = __ballot_sync(0xffffffffu, keep[k] != 0);
+        if (lane == 0) s_before[0][warp + k * kWarps] = (uint32_t)__popc(keep[k]);
       }
-    if (cta == 0 && tid == 0) T.count[T.L] = (uint64_t)n;
-  } else {
-    n = T.rule == 3 && t0 == T.L ? (int)T.n : (int)T.count[t0];
-    if (T.rule == 3 && cta == 0 && tid == 0) T.count[T.L] = (uint64_t)T.n;
-    if (CTAS == 1)
+      __syncthreads();
+      group_prefixes(s_before, 1, s_add);
+      __syncthreads();
 #pragma unroll
       for (int k = 0; k < kPer; ++k)
-        if (tid + k * kTopThreads < n) s_node.code[tid + k * kTopThreads] = T.ocode[t0][tid + k * kTopThreads];
-  }
-  sync_all();
-  uint32_t code[kPer], prev[kPer];
-  int first[kPer];
-#pragma unroll
-  for (int k = 0; k < kPer; ++k) {
-    const int i = node0 + 32 * (warp + k * kWarps) + lane;
-    auto at = [&](int j) { return CTAS == 1 ? s_node.code[j] : __ldcg(T.ocode[t0] + j); };
-    code[k] = i < n ? at(i) : 0;
-    prev[k] = i > 0 && i < n ? at(i - 1) : 0;
-  }
-#pragma unroll
-  for (int k = 0; k < kPer; ++k) {
-    const int g = warp + k * kWarps, i = node0 + 32 * g + lane;
-    first[k] = i < n ? first_level(code[k], prev[k], i, t0) : kNoNode;
-    uint32_t c = 0;  // lane t: the group's nodes of level t
-    for (int t = t0 - 1; t >= 0; --t) {
-      const unsigned b = __ballot_sync(0xffffffffu, first[k] <= t);
-      if (b == 0) break;
-      if (lane == t) c = (uint32_t)__popc(b);
+        if (keep[k] >> lane & 1u) {
+          const int p = n + (int)s_before[0][warp + k * kWarps] + __popc(keep[k] & earlier);
+          T.ocode[T.L][p] = code[k];
+          T.osq[T.L][p] = sq[k];
+          T.oslot[p] = slot[k];
+        }
+      n += s_add[0];
+      __syncthreads();
     }
-    if (lane < t0) s_before[lane][g] = c;
+    if (tid == 0) T.count[T.L] = (uint64_t)n;
+  } else {
+    n = T.rule == 3 && t0 == T.L ? (int)T.n : (int)T.count[t0];
+    if (T.rule == 3 && tid == 0) T.count[T.L] = (uint64_t)T.n;
   }
+  if (tid < t0) s_n[tid] = 0;
   __syncthreads();
-  group_prefixes(s_before, t0, s_n);
-  __syncthreads();
-  if (CTAS > 1) {
-    if (tid < t0) T.xchg[cta * kXchgRow + tid] = (uint32_t)s_n[tid];
-    cluster_sync();
-    if (tid < t0) s_base[tid] = exchanged(tid, &s_n[tid]);
+  uint32_t last = 0;  // the code before the piece
+  for (int node0 = 0; node0 < n; node0 += (int)kTopNodes) {
+#pragma unroll
+    for (int k = 0; k < kPer; ++k) {
+      const int i = tid + k * kTopThreads;
+      if (node0 + i < n) s_node.code[i] = T.ocode[t0][node0 + i];
+    }
+    __syncthreads();
+    uint32_t code[kPer];
+    int first[kPer];
+#pragma unroll
+    for (int k = 0; k < kPer; ++k) {
+      const int g = warp + k * kWarps, i = 32 * g + lane;
+      const bool in = node0 + i < n;
+      code[k] = in ? s_node.code[i] : 0;
+      first[k] = in ? first_level(code[k], i > 0 ? s_node.code[i - 1] : last, node0 + i, t0) : kNoNode;
+      uint32_t c = 0;  // lane t: the group's nodes of level t
+      for (int t = t0 - 1; t >= 0; --t) {
+        const unsigned b = __ballot_sync(0xffffffffu, first[k] <= t);
+        if (b == 0) break;
+        if (lane == t) c = (uint32_t)__popc(b);
+      }
+      if (lane < t0) s_before[lane][g] = c;
+    }
+    last = s_node.code[kTopNodes - 1];  // of a whole piece, if another follows
+    __syncthreads();
+    group_prefixes(s_before, t0, s_add);
+    __syncthreads();
+    for (int t = 0; t < t0; ++t)
+      for (int p = tid; p < s_add[t]; p += kTopThreads) T.ochild[t][s_n[t] + p] = make_int4(-1, -1, -1, -1);
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < kPer; ++k) {
+      const int g = warp + k * kWarps;
+      place_levels(T, node0 + 32 * g + lane, code[k], first[k], [&](int t) { return s_n[t] + (int)s_before[t][g]; });
+    }
+    __syncthreads();
+    if (tid < t0) s_n[tid] += s_add[tid];
     __syncthreads();
   }
-  if (cta == 0) {
-    if (tid < t0) T.count[tid] = (uint64_t)s_n[tid];
-    if (T.host && tid <= T.L) T.host[tid] = tid < t0 ? (uint64_t)s_n[tid] : T.count[tid];
-  }
-  for (int t = 0; t < t0; ++t)
-    for (int p = cta * kTopThreads + tid; p < s_n[t]; p += CTAS * kTopThreads)
-      T.ochild[t][p] = make_int4(-1, -1, -1, -1);
-  sync_all();
-#pragma unroll
-  for (int k = 0; k < kPer; ++k) {
-    const int g = warp + k * kWarps;
-    place_levels(T, node0 + 32 * g + lane, code[k], first[k],
-                 [&](int t) { return (CTAS > 1 ? s_base[t] : 0) + (int)s_before[t][g]; });
-  }
-  sync_all();
+  if (tid < t0) T.count[tid] = (uint64_t)s_n[tid];
+  if (T.host && tid <= T.L) T.host[tid] = tid < t0 ? (uint64_t)s_n[tid] : T.count[tid];
   if (t0 == 0 || !T.osq[t0 - 1]) return;
   int top = t0 - 1;
-  if (CTAS > 1) {
-    for (; top >= 0 && s_n[top] > kTopNodes; --top) {
-      for (int p = cta * kTopThreads + tid; p < s_n[top]; p += CTAS * kTopThreads)
-        T.osq[top][p] = child_sum(T.ochild[top][p], T.osq[top + 1]);
-      cluster_sync();
-    }
-    if (cta != 0) return;
+  for (; top >= 0 && s_n[top] > kTopNodes; --top) {
+    sum_parents(T, top + 1, 0, s_n[top]);
+    __syncthreads();
   }
   block_norms(top, s_n, [&](int t) { return T.ochild[t]; }, [&](int t) { return T.osq[t]; }, s_node.sq);
-}
-
-// The trees of at most kTopNodes nodes each on level t0 (or candidates) one block each, else
-// clusters.
-void launch_top(spamm_ctx ctx, TreePair* pair, int k, int64_t most) {
-  if (most <= kTopNodes) {
-    tree_top_kernel<1><<<k, kTopThreads, 0, ctx->stream>>>(*pair);
-  } else {
-    constexpr int kCtas = (int)(kBoundNodes / kTopNodes);
-    BufP xchg = alloc_n<uint32_t>(ctx, k * kCtas * kXchgRow);
-    for (int i = 0; i < k; ++i) pair->t[i].xchg = P<uint32_t>(xchg) + i * kCtas * kXchgRow;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(k * kCtas);
-    cfg.blockDim = dim3(kTopThreads);
-    cfg.stream = ctx->stream;
-    cudaLaunchAttribute at = {};
-    at.id = cudaLaunchAttributeClusterDimension;
-    at.val.clusterDim.x = kCtas;
-    at.val.clusterDim.y = at.val.clusterDim.z = 1;
-    cfg.attrs = &at;
-    cfg.numAttrs = 1;
-    CK(cudaLaunchKernelEx(&cfg, tree_top_kernel<kCtas>, *pair));
-  }
-  CK_LAUNCH("tree_top_kernel");
 }
 
 // The tiled form of one step: t = L + 1 the candidates' compaction, else the
@@ -550,8 +489,8 @@ void tiled_step(spamm_ctx ctx, const TreeDev& T, int t, int64_t n, uint64_t* til
 }
 
 // The levels above the leaves (at most n), large ones in tiles; T.t0 is left at the
-// level that tree_top_kernel starts from, whose nodes are at most the result.
-int64_t tiled_levels(spamm_ctx ctx, TreeDev* T, int64_t n) {
+// level that tree_top_kernel starts from.
+void tiled_levels(spamm_ctx ctx, TreeDev* T, int64_t n) {
   int t = T->L;
   int64_t cap = n;
   if (cap > kBoundNodes) {
@@ -559,7 +498,6 @@ int64_t tiled_levels(spamm_ctx ctx, TreeDev* T, int64_t n) {
     for (; t >= 1 && cap > kBoundNodes; --t, cap = level_cap(n, t)) tiled_step(ctx, *T, t, cap, P<uint64_t>(tiles));
   }
   T->t0 = t;
-  return cap;
 }
 
 }  // namespace
@@ -569,7 +507,6 @@ void tree_from_candidates(spamm_ctx ctx, TreeReq* req, int k, bool resolve) {
   TreePair pair;
   BufP tiles[2];
   bool wide[2] = {false, false};
-  int64_t most = 0;
   uint64_t* host = static_cast<uint64_t*>(ctx->h_pinned);
   for (int i = 0; i < k; ++i) {
     TreeReq& r = req[i];
@@ -585,7 +522,6 @@ void tree_from_candidates(spamm_ctx ctx, TreeReq* req, int k, bool resolve) {
     T.t0 = T.L;
     wide[i] = r.n > kBoundNodes;
     if (!wide[i]) {
-      most = r.n > most ? r.n : most;
       alloc_levels(ctx, r.m, r.n, true, false);
       point_at(&T, r.m);
       continue;
@@ -613,12 +549,12 @@ void tree_from_candidates(spamm_ctx ctx, TreeReq* req, int k, bool resolve) {
     point_at(&T, req[i].m);
     tiled_step(ctx, T, T.L + 1, T.n, P<uint64_t>(tiles[i]));
     T.rule = 0;  // tree_top_kernel starts above the leaves
-    const int64_t cap = tiled_levels(ctx, &T, n);
-    most = cap > most ? cap : most;
+    tiled_levels(ctx, &T, n);
   }
   if (resolve)
     for (int i = 0; i < k; ++i) pair.t[i].host = host + i * SPAMM_MAX_LEVELS;
-  launch_top(ctx, &pair, k, most);
+  tree_top_kernel<<<k, kTopThreads, 0, ctx->stream>>>(pair);
+  CK_LAUNCH("tree_top_kernel");
   for (int i = 0; i < k; ++i) req[i].m->pending = true;
   if (!resolve) return;
   CK(cudaStreamSynchronize(ctx->stream));
@@ -634,7 +570,9 @@ void tree_skeleton(spamm_ctx ctx, spamm_mat m, uint64_t* host) {
   T.n = n;
   T.rule = 3;
   T.host = host;
-  launch_top(ctx, &pair, 1, tiled_levels(ctx, &T, n));
+  tiled_levels(ctx, &T, n);
+  tree_top_kernel<<<1, kTopThreads, 0, ctx->stream>>>(pair);
+  CK_LAUNCH("tree_top_kernel");
   m->pending = true;
 }
 

@@ -1,5 +1,5 @@
-"""The key sort at the edges of its forms (one block up to 4096 pairs, a cluster up to
-65536, tiles above): leaves in random order come back in Morton order with their own
+"""The key sort at the edges of its forms (one block with four or sixteen rounds of 1024
+pairs, tiles above): leaves in random order come back in Morton order with their own
 payload, and the error-controlled rule, which sorts 64-bit norms, drops exactly the
 smallest leaves."""
 import numpy as np
@@ -19,7 +19,7 @@ def S():
     return spamm
 
 
-@pytest.mark.parametrize("count,nb", [(2, 2), (33, 9), (4095, 100), (4096, 2000), (4097, 64 + 1), (8193, 3000),
+@pytest.mark.parametrize("count,nb", [(2, 2), (33, 9), (4095, 100), (4096, 2000), (4097, 64 + 1), (8193, 3000), (16383, 900), (16384, 130), (16385, 5000),
                                       (30000, 200), (65535, 300), (65536, 2500), (65537, 260)])
 def test_sorted_leaves_and_smallest_dropped(S, count, nb):
     ctx = S.Context(0)

@@ -1,5 +1,5 @@
 """Scattered leaf sets at the edges of what the tree kernels take at a time (groups of 32
-nodes, one block, tiles): many levels, most parents with one child.  Codes and norms of
+nodes, pieces of one block, tiles): many levels, most parents with one child.  Codes and norms of
 every level; the child links by a product with the identity, whose descent reaches
 every leaf once."""
 import numpy as np
