@@ -57,8 +57,8 @@ __global__ void __launch_bounds__(kPassThreads)
   }
 }
 
-// Leaf q from src + slot[q] (q without slots), elements below tau zeroed (tau = 0:
-// none; |a| < tau on the two words of the bit patterns, which order like the
+// Leaf q from src + slot[q] (q without slots), elements below tau zeroed (tau = +0:
+// none, and not -0, whose pattern lies above all; |a| < tau on the two words of the bit patterns, which order like the
 // magnitudes: compared as one 64-bit word the compiler takes the FP64 pipe for it,
 // which made the pass 1.6 times as long).
 struct CopyOp {

@@ -293,7 +293,9 @@ spamm_mat truncate_element(spamm_mat in, double tau) {
   out->pool = alloc_n<double>(ctx, n * e);
   BufP sq = alloc_n<double>(ctx, n), nz = alloc_n<uint8_t>(ctx, n);
   if (n > 0) {
-    leaf_pass(ctx, CopyOp{P<double>(in->pool), P<int64_t>(in->slot), tau, nullptr}, n, in->bs, P<double>(out->pool),
+    // tau may be -0.0, which the pass, comparing bit patterns, must not see
+    const double least = tau > 0.0 ? tau : 0.0;
+    leaf_pass(ctx, CopyOp{P<double>(in->pool), P<int64_t>(in->slot), least, nullptr}, n, in->bs, P<double>(out->pool),
               P<double>(sq), P<uint8_t>(nz), 0);
   }
   set_leaves_compacted(out, n, P<uint32_t>(in->lv[in->L].code), P<double>(sq), nullptr, P<uint8_t>(nz));
