@@ -536,14 +536,11 @@ void launch_gemm(spamm_ctx ctx, spamm_prec prec, int bs, const BatchDev& batch) 
 }
 
 // Kernel (d): the outputs' leaf norms and slots (tensor forms: and their elements).
-void finish_leaves(spamm_ctx ctx, spamm_prec prec, const std::vector<spamm_mat>& ms, const OutBatch& out) {
-  if (prec != SPAMM_PREC_FP64) {
-    tc_finish(ctx, prec, out, ms[0]->bs);
-    return;
-  }
-  for (spamm_mat C : ms)
-    leaf_sqnorms(ctx, P<double>(C->pool), nullptr, C->nleaves, C->bs, P<double>(C->lv[C->L].sq), nullptr, 0,
-                 P<int64_t>(C->slot));
+void finish_leaves(spamm_ctx ctx, spamm_prec prec, int bs, const OutBatch& out) {
+  if (prec == SPAMM_PREC_FP64)
+    out_sqnorms(ctx, out, bs);
+  else
+    tc_finish(ctx, prec, out, bs);
 }
 OutLeaves out_leaves(spamm_mat C) { return {P<double>(C->pool), P<double>(C->lv[C->L].sq), P<int64_t>(C->slot)}; }
 
@@ -616,7 +613,7 @@ std::vector<spamm_mat> execute_plans(spamm_ctx ctx, const std::vector<spamm_plan
     CK(cudaEventRecordWithFlags(ev[0], ctx->stream, evflags));
     launch_gemm(ctx, prec, bs, batch);
     CK(cudaEventRecordWithFlags(ev[1], ctx->stream, evflags));
-    finish_leaves(ctx, prec, outp, leaves);
+    finish_leaves(ctx, prec, bs, leaves);
     propagate_norms(ctx, norms);
     CK(cudaEventRecordWithFlags(ev[2], ctx->stream, evflags));
   };
@@ -874,7 +871,7 @@ spamm_status spamm_job_finish(spamm_ctx ctx, spamm_job job, spamm_mat* C, spamm_
     leaves.only = out_leaves(Cm);
     leaves.n = 1;
     leaves.total = Cm->nleaves;
-    finish_leaves(ctx, job->plan->prec, {Cm}, leaves);
+    finish_leaves(ctx, job->plan->prec, Cm->bs, leaves);
     propagate_norms(ctx, norms);
     CK(cudaEventRecord(ev[1], ctx->stream));
     sync_and_check(ctx);

@@ -8,8 +8,8 @@
 // the last claims are short).  Every output element is computed by one CTA, so
 // there are no atomics on C and the k order is fixed: results do not depend on the
 // schedule, the tile or the batch.  The leaf norms (kernel (d)) are kernel (a) on
-// the finished leaves, in a launch of their own, so they do not depend on the
-// tile either (one FMA per element against bs per element and product here).
+// the finished leaves, in one launch for the batch (out_sqnorm_kernel), so they do not
+// depend on the tile either (one FMA per element against bs per element and product here).
 //
 // Bound by the FP64 pipe (two FMAs per clock and SM): a 64 x 64 x 64 product takes an
 // SM 63 us, so what is lost is lost at the end, when some SMs still work on their

@@ -192,9 +192,8 @@ spamm_mat truncate_block(spamm_mat in, double tau, spamm_ctx on = nullptr);  // 
 void truncate_pair(spamm_ctx ctx, spamm_mat A, spamm_mat B, double tau, spamm_mat* At, spamm_mat* Bt);
 spamm_mat truncate_element(spamm_mat in, double tau);
 spamm_mat truncate_error_controlled(spamm_mat in, double tau, spamm_ctx on = nullptr);
-// Kernel (a); with `slot_out` also the slots 0 .. nleaves - 1 of leaves stored in order.
 void leaf_sqnorms(spamm_ctx ctx, const double* pool, const int64_t* slot, int64_t nleaves, int bs, double* sq,
-                  uint8_t* nonzero, int check_finite, int64_t* slot_out = nullptr);
+                  uint8_t* nonzero, int check_finite);
 double error_fro(spamm_mat X, spamm_mat Y);
 // Deterministic sum into pinned memory, valid after the caller's wait (0 at once for n = 0).
 void device_sum_async(spamm_ctx ctx, const double* in, int64_t n, double* host);
@@ -312,6 +311,8 @@ struct OutBatch {
   int64_t total = 0;
 };
 void tc_finish(spamm_ctx ctx, spamm_prec prec, const OutBatch& out, int bs);
+// Kernel (d) of the FP64 form: each leaf's squared norm (kernel (a)'s) and its payload slot (store.cu).
+void out_sqnorms(spamm_ctx ctx, const OutBatch& out, int bs);
 // 64 x 64 operand tiles per leaf of the tensor forms (bs 64: 1, bs 128: 4).
 inline int tc_tiles_per_leaf(int bs) { return (bs / 64) * (bs / 64); }
 // Operand terms of a leaf set for a tensor form (role 0: used as A, 1: as B),

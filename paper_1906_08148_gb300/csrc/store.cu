@@ -72,7 +72,7 @@ __device__ __forceinline__ void warp_leaf_sumsq(Get get, int bs, int lane, doubl
 constexpr int64_t kNormLeavesPerBlock = 8;
 __global__ void leaf_sqnorm_kernel(const double* __restrict__ pool, const int64_t* __restrict__ slot, int64_t m,
                                    int bs, double* __restrict__ sq, uint8_t* __restrict__ nonzero, int check_finite,
-                                   int* err, int64_t* __restrict__ slot_out) {
+                                   int* err) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwb = blockDim.x >> 5;
   const int64_t e = (int64_t)bs * bs;
   for (int64_t q = (int64_t)blockIdx.x * kNormLeavesPerBlock + warp; q < m; q += (int64_t)gridDim.x * nwb) {
@@ -83,19 +83,70 @@ __global__ void leaf_sqnorm_kernel(const double* __restrict__ pool, const int64_
     if (lane == 0) {
       sq[q] = s;
       if (nonzero) nonzero[q] = nz;
-      if (slot_out) slot_out[q] = q;
       if (bad && check_finite) atomicOr(err, DEV_ERR_NONFINITE);
     }
   }
 }
 
 void leaf_sqnorms(spamm_ctx ctx, const double* pool, const int64_t* slot, int64_t nleaves, int bs, double* sq,
-                  uint8_t* nonzero, int check_finite, int64_t* slot_out) {
+                  uint8_t* nonzero, int check_finite) {
   if (nleaves <= 0) return;
   const int64_t nblk = (nleaves + kNormLeavesPerBlock - 1) / kNormLeavesPerBlock;
   leaf_sqnorm_kernel<<<(unsigned)(nblk < (1ll << 30) ? nblk : (1ll << 30)), kThreads, 0, ctx->stream>>>(
-      pool, slot, nleaves, bs, sq, nonzero, check_finite, ctx->d_err, slot_out);
+      pool, slot, nleaves, bs, sq, nonzero, check_finite, ctx->d_err);
   CK_LAUNCH("leaf_sqnorm_kernel");
+}
+
+// Kernel (a) on the outputs of a batch of FP64 products, and their payload slots: one
+// launch for all of them, bound by the FP64 pipe.  A leaf's bs^2 / 32 additions per lane
+// follow one another at 64 cycles each, which takes 1, 4, 17 or 68 us for leaves of 32, 64,
+// 128 or 256, however few there are (a launch per output: eight products of one 256-leaf
+// each 1264 us, in one launch 407).  So a lane's next eight pairs are on their way while
+// it adds the eight before (every leaf has a multiple of 64 x 8 pairs), and a block is one
+// warp, which gives each its own quarter of a pipe: 40 leaves of 256 95 us, 140 with eight
+// warps per block; 60,000 leaves of 32 156 us, 158 with eight.
+__global__ void __launch_bounds__(32) out_sqnorm_kernel(const __grid_constant__ OutBatch out, int bs) {
+  constexpr int U = 8;
+  const int lane = threadIdx.x;
+  const int pairs = bs * bs / 2;
+  for (int64_t u = blockIdx.x; u < out.total; u += gridDim.x) {
+    const int r = out.n > 1 ? plan_of(out.first, out.n, u) : 0;
+    const OutLeaves C = out.n > 1 ? out.tab[r] : out.only;
+    const int64_t q = out.n > 1 ? u - out.first[r] : u;
+    const double2* src = reinterpret_cast<const double2*>(C.pool + q * ((int64_t)bs * bs)) + lane;
+    double2 a[U], b[U];
+    double s = 0.0;
+    auto read = [&](double2(&v)[U], int i) {
+#pragma unroll
+      for (int k = 0; k < U; ++k) v[k] = __ldg(src + i + 32 * k);
+    };
+    auto add = [&](const double2(&v)[U]) {
+#pragma unroll
+      for (int k = 0; k < U; ++k) {
+        s = __fma_rn(v[k].x, v[k].x, s);
+        s = __fma_rn(v[k].y, v[k].y, s);
+      }
+    };
+    read(a, 0);
+    for (int i = 0; i < pairs; i += 64 * U) {
+      read(b, i + 32 * U);
+      add(a);
+      if (i + 64 * U < pairs) read(a, i + 64 * U);
+      add(b);
+    }
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+    if (lane == 0) {
+      C.sq[q] = s;
+      C.slot[q] = q;
+    }
+  }
+}
+
+void out_sqnorms(spamm_ctx ctx, const OutBatch& out, int bs) {
+  if (out.total <= 0) return;
+  out_sqnorm_kernel<<<(unsigned)(out.total < (1ll << 30) ? out.total : (1ll << 30)), 32, 0, ctx->stream>>>(out, bs);
+  CK_LAUNCH("out_sqnorm_kernel");
 }
 
 spamm_mat new_mat(spamm_ctx ctx, int64_t n, int bs) {
