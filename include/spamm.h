@@ -178,8 +178,9 @@ SPAMM_API spamm_status spamm_destroy(spamm_ctx ctx);
 /* Replace the stream all later work of `ctx` runs on. */
 SPAMM_API spamm_status spamm_set_stream(spamm_ctx ctx, void* cuda_stream);
 
-/* Install a device allocator: alloc(bytes, user) returns device memory usable
- * on the context stream in stream order (NULL on failure -> SPAMM_E_OOM);
+/* Install a device allocator: alloc(bytes, user) returns device memory at a
+ * 16-byte boundary (or a larger one), usable on the context stream in stream
+ * order (NULL on failure -> SPAMM_E_OOM);
  * free(ptr, user) returns it.  Pass alloc = free = NULL to go back to
  * cudaMallocAsync.  Must be called while no handle of `ctx` is alive. */
 SPAMM_API spamm_status spamm_set_allocator(spamm_ctx ctx, void* (*alloc)(size_t bytes, void* user),

@@ -646,16 +646,18 @@ __global__ void __launch_bounds__(kQuadThreads, 1)
       // pass (tc_finish_kernel) turns the slots into FP64 and takes the leaf
       // norms, so no FP64 instruction runs here, where it would hold up the
       // draining of the accumulators the next quad's MMAs wait for.  32 bytes
-      // (one sector) per lane and store.
+      // (one sector) per lane and store, 16 where the caller's allocator gave the pool an
+      // address between sectors.
       if (outp) {
         double* out = outp + row * ld;
+        const bool wide = (reinterpret_cast<uintptr_t>(outp) & 31) == 0;  // rows are a multiple of 512 bytes
 #pragma unroll
         for (int q = 0; q < 64; q += 4) {
           if constexpr (NACC == 1)
-            store_32(out + q, __float_as_uint(hi[q]), 0u, __float_as_uint(hi[q + 1]), 0u, __float_as_uint(hi[q + 2]), 0u,
-                     __float_as_uint(hi[q + 3]), 0u);
+            store_32(out + q, wide, __float_as_uint(hi[q]), 0u, __float_as_uint(hi[q + 1]), 0u,
+                     __float_as_uint(hi[q + 2]), 0u, __float_as_uint(hi[q + 3]), 0u);
           else
-            store_32(out + q, (uint32_t)hi2[q / 2], (uint32_t)lo2[q / 2], (uint32_t)(hi2[q / 2] >> 32),
+            store_32(out + q, wide, (uint32_t)hi2[q / 2], (uint32_t)lo2[q / 2], (uint32_t)(hi2[q / 2] >> 32),
                      (uint32_t)(lo2[q / 2] >> 32), (uint32_t)hi2[q / 2 + 1], (uint32_t)lo2[q / 2 + 1],
                      (uint32_t)(hi2[q / 2 + 1] >> 32), (uint32_t)(lo2[q / 2 + 1] >> 32));
         }

@@ -231,12 +231,19 @@ __device__ __forceinline__ uint64_t sub_x2(uint64_t a, uint64_t b) {
   return r;
 }
 
-// 32 bytes (one sector) to global memory; p 32-byte aligned.
-__device__ __forceinline__ void store_32(void* p, uint32_t a, uint32_t b, uint32_t c, uint32_t d, uint32_t e, uint32_t f,
-                                         uint32_t g, uint32_t h) {
-  asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "r"(a), "r"(b), "r"(c), "r"(d),
-               "r"(e), "r"(f), "r"(g), "r"(h)
-               : "memory");
+// 32 bytes to global memory: one sector and one instruction where p is 32-byte aligned
+// (`wide`), else two of 16; p 16-byte aligned.
+__device__ __forceinline__ void store_32(void* p, bool wide, uint32_t a, uint32_t b, uint32_t c, uint32_t d, uint32_t e,
+                                         uint32_t f, uint32_t g, uint32_t h) {
+  if (wide) {
+    asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "r"(a), "r"(b), "r"(c), "r"(d),
+                 "r"(e), "r"(f), "r"(g), "r"(h)
+                 : "memory");
+  } else {
+    uint4* q = reinterpret_cast<uint4*>(p);
+    q[0] = make_uint4(a, b, c, d);
+    q[1] = make_uint4(e, f, g, h);
+  }
 }
 
 // Per-warpgroup register reallocation (all threads of a warpgroup execute
