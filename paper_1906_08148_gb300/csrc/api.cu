@@ -30,6 +30,18 @@ spamm_status set_error(spamm_ctx ctx, spamm_status st, const std::string& msg) {
   return st;
 }
 
+// A failed allocation or CUDA call can end a call with work in flight that reads the
+// operands or the caller's buffers, which are the call's only until it returns, or that
+// writes the context's pinned page: wait for it.  (The other errors come before anything
+// is enqueued or after a wait.)
+spamm_status failed_midway(spamm_ctx ctx, spamm_status st, const std::string& msg) {
+  if (ctx && (st == SPAMM_E_OOM || st == SPAMM_E_CUDA)) {
+    cudaStreamSynchronize(ctx->stream);
+    cudaGetLastError();
+  }
+  return set_error(ctx, st, msg);
+}
+
 template <class F>
 spamm_status guarded(spamm_ctx ctx, F&& f) {
   if (ctx) {
@@ -40,11 +52,11 @@ spamm_status guarded(spamm_ctx ctx, F&& f) {
     f();
     return SPAMM_OK;
   } catch (const Error& e) {
-    return set_error(ctx, e.status, e.msg);
+    return failed_midway(ctx, e.status, e.msg);
   } catch (const std::bad_alloc&) {
-    return set_error(ctx, SPAMM_E_OOM, "host allocation failed");
+    return failed_midway(ctx, SPAMM_E_OOM, "host allocation failed");
   } catch (...) {
-    return set_error(ctx, SPAMM_E_CUDA, "unexpected exception");
+    return failed_midway(ctx, SPAMM_E_CUDA, "unexpected exception");
   }
 }
 

@@ -1,4 +1,5 @@
-"""Allocators of the caller: addresses at 16-byte boundaries, between the 32-byte ones."""
+"""Allocators of the caller: addresses at 16-byte boundaries, between the 32-byte ones, and
+allocations that fail at every point of a call."""
 import ctypes
 
 import numpy as np
@@ -50,3 +51,45 @@ def test_addresses_between_sectors(S, prec, bs, nb):
         got.append([S.spamm_to_blocks(ctx, M) for M in (A, C, D, E)] + [S.spamm_error(ctx, C, D), S.spamm_trace(ctx, C)])
     for x, y in zip(*got):
         assert np.all([np.array_equal(u, v) for u, v in zip(x, y)]) if isinstance(x, tuple) else x == y
+
+
+# operands of another context on another stream: their owner may release them as soon as the call has returned
+@pytest.mark.parametrize("call", ["multiply", "plan", "execute", "add", "truncate"])
+def test_a_failed_call_leaves_nothing_in_flight(S, call):
+    import torch
+    count, limit = [0], [1 << 30]
+
+    def alloc(nbytes, _user):
+        count[0] += 1
+        if count[0] > limit[0]:
+            return None
+        return torch.cuda.caching_allocator_alloc(int(nbytes), 0)
+
+    def free(p, _user):
+        torch.cuda.caching_allocator_delete(p)
+
+    owner, stream = S.Context(0), torch.cuda.Stream()
+    ctx = _context(S, alloc, free, stream)
+    nb, bs = 40, 128
+    rng = np.random.default_rng(1)
+    r, c = np.nonzero(np.ones((nb, nb)))
+    A = S.spamm_from_blocks(owner, nb * bs, bs, r.astype(np.int32), c.astype(np.int32),
+                            rng.uniform(-1, 1, (nb * nb, bs, bs)))
+    mine = S.spamm_from_blocks(ctx, nb * bs, bs, r[:9].astype(np.int32), c[:9].astype(np.int32),
+                               rng.uniform(-1, 1, (9, bs, bs)))
+    plan = S.spamm_plan_create(ctx, A, A, 0.0, "combined", "bf16_split4")
+    run = {"multiply": lambda: S.spamm_multiply(ctx, A, A, 0.0, "combined", "bf16_split4"),
+           "plan": lambda: S.spamm_plan_create(ctx, A, A, 0.0, "combined", "bf16_split4"),
+           "execute": lambda: S.spamm_execute(ctx, [plan, plan]),
+           "add": lambda: S.spamm_add(ctx, 2.0, A, -0.3, A),
+           "truncate": lambda: S.spamm_truncate(ctx, mine, 1.0, "element")}[call]
+    done = None
+    for k in range(200):
+        count[0], limit[0] = 0, k
+        try:
+            done = run()
+            break
+        except S.SpammError as e:
+            assert stream.query()  # nothing of the call is left on its stream
+            assert e.status == S.E_OOM
+    assert done is not None and k > 3
