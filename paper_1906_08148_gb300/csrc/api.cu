@@ -16,7 +16,7 @@ spamm_mat build_from_coo(spamm_ctx, int64_t, int64_t, const int64_t*, const int6
                          spamm_trunc_rule);
 void export_dense(spamm_mat, double*, int64_t, int);
 void export_blocks(spamm_mat, int32_t*, int32_t*, double*, double*, int);
-void tasks_to_ikj(spamm_mat A, const TaskList& T, int32_t* d_out);
+void tasks_to_ikj(spamm_ctx ctx, spamm_mat A, const TaskList& T, int32_t* d_out);
 void gather_leaves(spamm_mat m, int64_t nq, const int32_t* bi, const int32_t* bj, double* out, int32_t* found,
                    int on_device);
 }  // namespace spamm
@@ -995,7 +995,7 @@ spamm_status spamm_kept_tasks(spamm_ctx ctx, spamm_mat A, spamm_mat B, double ta
     need(ikj_out != nullptr, "ikj_out must be non-NULL");
     task_finish(ctx, tb.get(), &T, nullptr, nullptr, nullptr);
     BufP d = alloc_n<int32_t>(ctx, 3 * T.ntasks);
-    tasks_to_ikj(At, T, P<int32_t>(d));
+    tasks_to_ikj(ctx, At, T, P<int32_t>(d));
     CK(cudaMemcpyAsync(ikj_out, P<int32_t>(d), 3 * T.ntasks * sizeof(int32_t), cudaMemcpyDeviceToHost, ctx->stream));
     sync_and_check(ctx);
   });

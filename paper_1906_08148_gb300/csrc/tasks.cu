@@ -997,8 +997,7 @@ __global__ void tasks_to_ikj_kernel(int64_t G, const int64_t* __restrict__ gstar
   }
 }
 
-void tasks_to_ikj(spamm_mat A, const TaskList& T, int32_t* d_out) {
-  spamm_ctx ctx = A->ctx;
+void tasks_to_ikj(spamm_ctx ctx, spamm_mat A, const TaskList& T, int32_t* d_out) {
   if (T.ngroups == 0) return;
   tasks_to_ikj_kernel<<<warps_grid(ctx, T.ngroups), kWarpsPerBlock * 32, 0, ctx->stream>>>(
       T.ngroups, P<int64_t>(T.gstart), P<uint32_t>(T.gcode), P<int32_t>(T.ta), P<uint32_t>(A->lv[A->L].code), d_out);
