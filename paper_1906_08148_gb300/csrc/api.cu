@@ -329,18 +329,25 @@ struct spamm_plan_s {
 
 namespace {
 
+// Device bytes that live as long as the plan: a buffer that is part of a larger one keeps
+// all of it (the slots of a truncated operand its whole tree, the output's levels their
+// block), and shared ones (symmetric operands, parts of one block) count once.  The
+// operands' payload pools are the matrices' own.
 size_t held_bytes(const spamm_plan_s& p) {
-  size_t b = 0;
   std::vector<const Buf*> seen;
-  for (const BufP* x : {&p.T.gcode, &p.T.gstart, &p.T.ta, &p.T.tb, &p.T.quads, &p.qstart, &p.qsteps, &p.slotA,
-                        &p.slotB, &p.termsA, &p.termsB, &p.expA, &p.expB, &p.uorder, &p.bmap}) {
-    if (!*x) continue;
-    bool dup = false;  // shared buffers (symmetric operands) count once
-    for (const Buf* q : seen) dup = dup || q == x->get();
-    if (dup) continue;
-    seen.push_back(x->get());
-    b += (*x)->bytes;
-  }
+  size_t b = 0;
+  auto hold = [&](const BufP& x) {
+    if (!x) return;
+    const Buf* whole = x->owner ? x->owner.get() : x.get();
+    if (std::find(seen.begin(), seen.end(), whole) != seen.end()) return;
+    seen.push_back(whole);
+    b += (whole->bytes + 255) & ~(size_t)255;  // as allocated
+  };
+  for (const BufP* x : {&p.T.gcode, &p.T.gstart, &p.T.ta, &p.T.tb, &p.T.quads, &p.qstart, &p.qsteps, &p.slotA, &p.slotB,
+                        &p.termsA, &p.termsB, &p.expA, &p.expB, &p.uorder, &p.bmap, &p.cdcount})
+    hold(*x);
+  for (const Level& lv : p.cskel)
+    for (const BufP* x : {&lv.code, &lv.child, &lv.sq}) hold(*x);
   return b;
 }
 
