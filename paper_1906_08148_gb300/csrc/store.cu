@@ -432,24 +432,24 @@ spamm_mat build_from_blocks(spamm_ctx ctx, int64_t n, int bs, int64_t nblocks, c
                             const double* payload, int on_device, double tau, spamm_trunc_rule rule) {
   const int64_t e = (int64_t)bs * bs;
   BufP pool = alloc_n<double>(ctx, nblocks * e);
+  // coordinates on the device are read where they are; from an address between 32-bit
+  // words they are copied first, like those of the host
+  auto words = [](const int32_t* p) { return (reinterpret_cast<uintptr_t>(p) & 3) == 0; };
+  const bool place_i = !on_device || !words(bi), place_j = !on_device || !words(bj);
   BufP dbi, dbj;
-  if (!on_device) {
-    dbi = alloc_n<int32_t>(ctx, nblocks);
-    dbj = alloc_n<int32_t>(ctx, nblocks);
-  }
+  if (place_i) dbi = alloc_n<int32_t>(ctx, nblocks);
+  if (place_j) dbj = alloc_n<int32_t>(ctx, nblocks);
   // leaves on the device are copied and their norms taken in one pass (which reads
   // 16-byte pairs; a payload that starts between them is copied first)
   const bool pass = on_device && (reinterpret_cast<uintptr_t>(payload) & 15) == 0;
   cudaMemcpyKind kind = on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
   if (nblocks > 0) {
     if (!pass) CK(cudaMemcpyAsync(P<double>(pool), payload, nblocks * e * sizeof(double), kind, ctx->stream));
-    if (!on_device) {
-      CK(cudaMemcpyAsync(P<int32_t>(dbi), bi, nblocks * sizeof(int32_t), kind, ctx->stream));
-      CK(cudaMemcpyAsync(P<int32_t>(dbj), bj, nblocks * sizeof(int32_t), kind, ctx->stream));
-    }
+    if (place_i) CK(cudaMemcpyAsync(P<int32_t>(dbi), bi, nblocks * sizeof(int32_t), kind, ctx->stream));
+    if (place_j) CK(cudaMemcpyAsync(P<int32_t>(dbj), bj, nblocks * sizeof(int32_t), kind, ctx->stream));
   }
-  return finish_from_pool(ctx, n, bs, pool, pass ? payload : nullptr, nblocks, on_device ? bi : P<int32_t>(dbi),
-                          on_device ? bj : P<int32_t>(dbj), tau, rule);
+  return finish_from_pool(ctx, n, bs, pool, pass ? payload : nullptr, nblocks, place_i ? P<int32_t>(dbi) : bi,
+                          place_j ? P<int32_t>(dbj) : bj, tau, rule);
 }
 
 // Candidate leaves in Morton order over the 2^L x 2^L grid, those inside
