@@ -269,11 +269,11 @@ spamm_status spamm_truncate(spamm_ctx ctx, spamm_mat in, double tau, spamm_trunc
   return guarded(ctx, [&] {
     check_tau(tau);
     check_rule(rule);
-    spamm_mat m = rule == SPAMM_TRUNC_BLOCK_FROB ? truncate_block(in, tau)
-                  : rule == SPAMM_TRUNC_ELEMENT  ? truncate_element(in, tau)
-                                                 : truncate_error_controlled(in, tau);
+    std::unique_ptr<spamm_mat_s> m(rule == SPAMM_TRUNC_BLOCK_FROB ? truncate_block(in, tau)
+                                   : rule == SPAMM_TRUNC_ELEMENT  ? truncate_element(in, tau)
+                                                                  : truncate_error_controlled(in, tau));
     sync_and_check(ctx);
-    *out = registered(m);
+    *out = registered(m.release());
   });
 }
 

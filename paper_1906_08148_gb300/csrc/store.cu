@@ -204,22 +204,23 @@ static TreeReq block_request(spamm_mat out, spamm_mat in, double tau) {
 
 spamm_mat truncate_block(spamm_mat in, double tau, spamm_ctx on) {
   spamm_ctx ctx = on ? on : in->ctx;
-  spamm_mat out = view_of(ctx, in);
+  std::unique_ptr<spamm_mat_s> out(view_of(ctx, in));
   if (in->nleaves > 0) {
-    TreeReq r = block_request(out, in, tau);
+    TreeReq r = block_request(out.get(), in, tau);
     tree_from_candidates(ctx, &r, 1, true);
   }
-  return out;
+  return out.release();
 }
 
 void truncate_pair(spamm_ctx ctx, spamm_mat A, spamm_mat B, double tau, spamm_mat* At, spamm_mat* Bt) {
   TreeReq r[2];
   int k = 0;
-  *At = view_of(ctx, A);
-  *Bt = A == B ? *At : view_of(ctx, B);
-  if (A->nleaves > 0) r[k++] = block_request(*At, A, tau);
-  if (A != B && B->nleaves > 0) r[k++] = block_request(*Bt, B, tau);
+  std::unique_ptr<spamm_mat_s> a(view_of(ctx, A)), b(A == B ? nullptr : view_of(ctx, B));
+  if (A->nleaves > 0) r[k++] = block_request(a.get(), A, tau);
+  if (b && B->nleaves > 0) r[k++] = block_request(b.get(), B, tau);
   if (k) tree_from_candidates(ctx, r, k, false);
+  *At = a.release();
+  *Bt = b ? b.release() : *At;
 }
 
 // Error-controlled rule: drop the smallest leaves (ascending squared norm,
@@ -298,9 +299,7 @@ __global__ void drop_prefix_kernel(const int64_t* __restrict__ idx, int64_t n, c
 
 spamm_mat truncate_error_controlled(spamm_mat in, double tau, spamm_ctx on) {
   spamm_ctx ctx = on ? on : in->ctx;
-  spamm_mat out = new_mat(ctx, in->n, in->bs);
-  out->symmetric = in->symmetric;
-  out->pool = in->pool;
+  std::unique_ptr<spamm_mat_s> out(view_of(ctx, in));
   const int64_t n = in->nleaves;
   BufP keep = alloc_n<uint8_t>(ctx, n);
   if (n > 0) {
@@ -330,16 +329,16 @@ spamm_mat truncate_error_controlled(spamm_mat in, double tau, spamm_ctx on) {
       CK_LAUNCH("drop_prefix_kernel");
     }
   }
-  set_leaves_compacted(out, n, P<uint32_t>(in->lv[in->L].code), P<double>(in->lv[in->L].sq), P<int64_t>(in->slot),
+  set_leaves_compacted(out.get(), n, P<uint32_t>(in->lv[in->L].code), P<double>(in->lv[in->L].sq), P<int64_t>(in->slot),
                        P<uint8_t>(keep));
-  return out;
+  return out.release();
 }
 
 // Element rule (Theorem 1): a -> 0 iff |a| < tau, into a fresh pool.
 spamm_mat truncate_element(spamm_mat in, double tau) {
   spamm_ctx ctx = in->ctx;
   const int64_t n = in->nleaves, e = (int64_t)in->bs * in->bs;
-  spamm_mat out = new_mat(ctx, in->n, in->bs);
+  std::unique_ptr<spamm_mat_s> out(new_mat(ctx, in->n, in->bs));
   out->symmetric = in->symmetric;
   out->pool = alloc_n<double>(ctx, n * e);
   BufP sq = alloc_n<double>(ctx, n), nz = alloc_n<uint8_t>(ctx, n);
@@ -349,8 +348,8 @@ spamm_mat truncate_element(spamm_mat in, double tau) {
     leaf_pass(ctx, CopyOp{P<double>(in->pool), P<int64_t>(in->slot), least, nullptr}, n, in->bs, P<double>(out->pool),
               P<double>(sq), P<uint8_t>(nz), 0);
   }
-  set_leaves_compacted(out, n, P<uint32_t>(in->lv[in->L].code), P<double>(sq), nullptr, P<uint8_t>(nz));
-  return out;
+  set_leaves_compacted(out.get(), n, P<uint32_t>(in->lv[in->L].code), P<double>(sq), nullptr, P<uint8_t>(nz));
+  return out.release();
 }
 
 // --------------------------------------------------------------- builders
@@ -393,7 +392,7 @@ __global__ void zero_below_kernel(double* __restrict__ a, int64_t n, double tau)
 // copied into the pool, or (null) in the pool already.
 static spamm_mat finish_from_pool(spamm_ctx ctx, int64_t n, int bs, BufP pool, const double* payload, int64_t nblocks,
                                   const int32_t* d_bi, const int32_t* d_bj, double tau, spamm_trunc_rule rule) {
-  spamm_mat m = new_mat(ctx, n, bs);
+  std::unique_ptr<spamm_mat_s> m(new_mat(ctx, n, bs));
   m->pool = pool;
   const int64_t e = (int64_t)bs * bs;
   const bool element = rule == SPAMM_TRUNC_ELEMENT && tau > 0.0;
@@ -424,8 +423,8 @@ static spamm_mat finish_from_pool(spamm_ctx ctx, int64_t n, int bs, BufP pool, c
     CK_LAUNCH("gather_sorted_kernel");
     sync_and_check(ctx);
   }
-  set_leaves_compacted(m, nblocks, P<uint32_t>(code), P<double>(ssq), P<int64_t>(slot), P<uint8_t>(keep));
-  return m;
+  set_leaves_compacted(m.get(), nblocks, P<uint32_t>(code), P<double>(ssq), P<int64_t>(slot), P<uint8_t>(keep));
+  return m.release();
 }
 
 spamm_mat build_from_blocks(spamm_ctx ctx, int64_t n, int bs, int64_t nblocks, const int32_t* bi, const int32_t* bj,
@@ -534,8 +533,8 @@ struct GenElem {
 };
 
 template <class Elem>
-static spamm_mat build_from_elements(spamm_ctx ctx, int64_t n, int bs, Elem elem, double tau, spamm_trunc_rule rule) {
-  spamm_mat m = new_mat(ctx, n, bs);
+static std::unique_ptr<spamm_mat_s> build_from_elements(spamm_ctx ctx, int64_t n, int bs, Elem elem, double tau, spamm_trunc_rule rule) {
+  std::unique_ptr<spamm_mat_s> m(new_mat(ctx, n, bs));
   const int64_t nb = (n + bs - 1) / bs;
   const int64_t ncand = (int64_t)1 << (2 * m->L);
   BufP sq = alloc_n<double>(ctx, ncand), keep = alloc_n<uint8_t>(ctx, ncand);
@@ -544,7 +543,7 @@ static spamm_mat build_from_elements(spamm_ctx ctx, int64_t n, int bs, Elem elem
   CK_LAUNCH("candidate_stats_kernel");
   sync_and_check(ctx);
   // the candidates' codes are their indices 0 .. 4^L - 1
-  set_leaves_compacted(m, ncand, nullptr, P<double>(sq), nullptr, P<uint8_t>(keep));
+  set_leaves_compacted(m.get(), ncand, nullptr, P<double>(sq), nullptr, P<uint8_t>(keep));
   // payload for the kept leaves, slot = leaf index
   const int64_t e = (int64_t)bs * bs;
   m->pool = alloc_n<double>(ctx, m->nleaves * e);
@@ -580,9 +579,9 @@ spamm_mat build_from_dense(spamm_ctx ctx, int64_t n, const double* a, int64_t ld
     dlda = n;
   }
   DenseElem el{da, dlda, n, bs};
-  spamm_mat m = build_from_elements(ctx, n, bs, el, tau, rule);
+  std::unique_ptr<spamm_mat_s> m = build_from_elements(ctx, n, bs, el, tau, rule);
   sync_and_check(ctx);  // the temporary copy must outlive the fill
-  return m;
+  return m.release();
 }
 
 spamm_mat build_generated(spamm_ctx ctx, const spamm_gen_params* gp, int bs, double tau, spamm_trunc_rule rule) {
@@ -595,9 +594,9 @@ spamm_mat build_generated(spamm_ctx ctx, const spamm_gen_params* gp, int bs, dou
   el.p.cutoff = gp->cutoff;
   el.p.seed = gp->seed;
   el.bs = bs;
-  spamm_mat m = build_from_elements(ctx, gp->n, bs, el, tau, rule);
+  std::unique_ptr<spamm_mat_s> m = build_from_elements(ctx, gp->n, bs, el, tau, rule);
   m->symmetric = 1;  // u_ij and the decay law are symmetric in (i, j)
-  return m;
+  return m.release();
 }
 
 // COO: sort (leaf code, in-leaf offset) keys stably, sum runs of equal keys
@@ -643,7 +642,7 @@ __global__ void coo_scatter_kernel(const uint64_t* __restrict__ keys, const int6
 
 spamm_mat build_from_coo(spamm_ctx ctx, int64_t n, int64_t nnz, const int64_t* row, const int64_t* col,
                          const double* val, int on_device, int bs, double tau, spamm_trunc_rule rule) {
-  spamm_mat m = new_mat(ctx, n, bs);
+  std::unique_ptr<spamm_mat_s> m(new_mat(ctx, n, bs));
   int lbs = 0;
   while ((1 << lbs) < bs) ++lbs;
   const int64_t e = (int64_t)bs * bs;
@@ -662,8 +661,8 @@ spamm_mat build_from_coo(spamm_ctx ctx, int64_t n, int64_t nnz, const int64_t* r
     v = P<double>(dval);
   }
   if (nnz == 0) {
-    set_leaves_compacted(m, 0, nullptr, nullptr, nullptr, nullptr);
-    return m;
+    set_leaves_compacted(m.get(), 0, nullptr, nullptr, nullptr, nullptr);
+    return m.release();
   }
   BufP keys = alloc_n<uint64_t>(ctx, nnz), vals = alloc_n<int64_t>(ctx, nnz);
   coo_keys_kernel<<<grid_for(ctx, nnz, kThreads), kThreads, 0, ctx->stream>>>(
@@ -697,8 +696,8 @@ spamm_mat build_from_coo(spamm_ctx ctx, int64_t n, int64_t nnz, const int64_t* r
     and_u8(ctx, P<uint8_t>(nz), P<uint8_t>(keep2), nl);
   }
   m->pool = pool;
-  set_leaves_compacted(m, nl, P<uint32_t>(code), P<double>(sq), nullptr, P<uint8_t>(nz));
-  return m;
+  set_leaves_compacted(m.get(), nl, P<uint32_t>(code), P<double>(sq), nullptr, P<uint8_t>(nz));
+  return m.release();
 }
 
 __global__ void and_u8_kernel(uint8_t* a, const uint8_t* b, int64_t n) {

@@ -93,3 +93,67 @@ def test_a_failed_call_leaves_nothing_in_flight(S, call):
             assert stream.query()  # nothing of the call is left on its stream
             assert e.status == S.E_OOM
     assert done is not None and k > 3
+
+
+def test_failed_calls_give_everything_back(S):
+    """Every builder, truncation and product, with each of its allocations failing in turn, and inputs refused for
+    what they hold: what the allocator handed out during the call has come back."""
+    import torch
+    import synth
+    count, limit, live = [0], [1 << 30], set()
+
+    def alloc(nbytes, _user):
+        count[0] += 1
+        if count[0] > limit[0]:
+            return None
+        p = torch.cuda.caching_allocator_alloc(int(nbytes), 0)
+        live.add(p)
+        return p
+
+    def free(p, _user):
+        live.remove(p)
+        torch.cuda.caching_allocator_delete(p)
+
+    ctx = _context(S, alloc, free)
+    n, bs = 640, 64
+    A, B = _operands(S, ctx, 10, bs)
+    r, c, pay, _ = S.spamm_to_blocks(ctx, A)
+    dense = S.spamm_to_dense(ctx, A)
+    i, j = (x[:500] for x in np.nonzero(dense))
+    bad = pay.copy()
+    bad[3, 5, 7] = np.nan
+    bad_dense = dense.copy()
+    bad_dense[9, 9] = np.inf
+    gen = synth.DecayParams(n=n, kind=synth.KIND_1D, alpha=0.5, seed=3)
+    calls = [lambda: S.spamm_from_blocks(ctx, n, bs, r, c, pay, 1e-3, "error"),
+             lambda: S.spamm_from_dense(ctx, dense, bs),
+             lambda: S.spamm_from_coo(ctx, n, i, j, dense[i, j], bs, 1e-6, "block"),
+             lambda: S.spamm_generate(ctx, gen, bs),
+             lambda: S.spamm_identity(ctx, n, bs),
+             lambda: S.spamm_add(ctx, 2.0, A, -1.0, B),
+             lambda: S.spamm_kept_tasks(ctx, A, B, 1e-3, "combined")]
+    calls += [lambda rule=rule: S.spamm_truncate(ctx, A, 0.1, rule) for rule in S.RULES]
+    calls += [lambda prec=prec: S.spamm_multiply(ctx, A, B, 1e-3, "combined", prec) for prec in S.PRECS]
+    refused = [lambda: S.spamm_from_blocks(ctx, n, bs, r, c, bad), lambda: S.spamm_from_dense(ctx, bad_dense, bs),
+               lambda: S.spamm_from_blocks(ctx, n, bs, np.append(r, r[0]), np.append(c, c[0]), pay[[*range(len(r)), 0]]),
+               lambda: S.spamm_from_blocks(ctx, n, bs, r + 1, c, pay),
+               lambda: S.spamm_from_coo(ctx, n, i, j, np.full(len(i), np.nan), bs),
+               lambda: S.spamm_add(ctx, 1e200, S.spamm_add(ctx, 1e200, A, 0.0, B), 1.0, B)]
+    before = set(live)
+    for call in calls:
+        for k in range(300):
+            count[0], limit[0] = 0, k
+            try:
+                call()
+                break
+            except S.SpammError as e:
+                assert e.status == S.E_OOM
+                assert live == before
+        assert k > 0 and live == before  # the result has been released
+    limit[0] = 1 << 30
+    for call in refused:
+        with pytest.raises(S.SpammError) as e:
+            call()
+        assert e.value.status in (S.E_NONFINITE, S.E_INVALID_ARG)
+        del e
+        assert live == before
