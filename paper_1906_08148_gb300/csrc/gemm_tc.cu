@@ -68,8 +68,8 @@
 // between them is a look at a barrier in shared memory that takes some 250 cycles
 // beside the operand reads.  Measured on the 3-D lattices (GEMM only, CUDA events),
 // with the waits taken out of each role's way as the comments below say: 4 slices,
-// n = 65536, tau = 1e-6, 115.6 -> 93 ms (1.6 PFLOP/s executed, near the chip's
-// power-limited rate); 3 slices, n = 16384, 8.19 -> 6.37 ms; FP16 with 128-leaves,
+// n = 65536, tau = 1e-6, 115.6 -> 93 ms (1.42 PFLOP/s executed, one-column steps
+// counted at half width: 83 % of the chip's power-limited rate); 3 slices, n = 16384, 8.19 -> 6.37 ms; FP16 with 128-leaves,
 // n = 20000, tau = 1e-4, 7.67 -> 5.80 ms.  With single parts left out the first takes
 // 68 ms (MMAs alone), 51 (copies alone), 80 (without epilogue), 85 (without copies).
 #include "convert.cuh"
@@ -86,6 +86,7 @@ namespace spamm {
 // control warpgroup then gives up 96 of them per thread and the epilogue
 // takes 48 more, enough for its two-float accumulators and one slot's columns:
 // 128 x 72 + 256 x 216 = 64512, the launch total, so the increase never waits.
+// (-Xptxas -v: the 4-slice kernel spills 48 bytes, the other two none.)
 constexpr int kQuadThreads = 384;
 constexpr uint32_t kLaunchRegs = 168, kCtlRegs = 72, kEpiRegs = 216;
 static_assert(128 * kCtlRegs + 256 * kEpiRegs == kQuadThreads * kLaunchRegs, "register split must match the launch");

@@ -310,6 +310,10 @@ void prep_terms(spamm_ctx ctx, spamm_prec prec, const PrepReq* req, int k) {
   }
   pair.role0 = req[0].role;
   if (ntiles == 0) return;
+  // the blocks of a launch: staged, two fit an SM; from registers three in the FP16 form, for
+  // which this was measured, and two in the BF16 forms, whose third block per SM waits (their
+  // terms of 128-leaves, 2 x 8220 leaves: 1019 -> 846 us with 3 slices, 1203 -> 1032 with 4, against
+  // 256 threads per tile)
   const int64_t cap = (int64_t)ctx->num_sms * (bs == 64 ? 2 : 3);
   const unsigned grid = (unsigned)(ntiles < cap ? ntiles : cap);
   const bool staged = bs == 64;

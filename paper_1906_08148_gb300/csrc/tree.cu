@@ -597,7 +597,7 @@ void tree_set_counts(spamm_mat m, const uint64_t* host) {
 // The parents' squared norms of an output whose structure was built at plan
 // time, from its leaves' norms up, for every tree of a batch: levels of more than
 // kTopNodes nodes one launch each (all trees), the rest by one block per tree in
-// one launch.  The additions are place_parent's.
+// one launch.  The additions are child_sum's, in its order.
 struct NormTree {
   int64_t L;
   const uint64_t* count;  // nodes per level, on the device
