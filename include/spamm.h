@@ -33,6 +33,7 @@
  *   that stream before returning.
  * - Every call returns a spamm_status; nothing aborts or traps.  The message
  *   of the last failure on a context is available from spamm_last_error().
+ *   A call that failed has no work of its own in flight when it returns.
  *   A device-side wait that runs past its bound makes the call return
  *   SPAMM_E_TIMEOUT.
  * - A context is used by one host thread at a time.
